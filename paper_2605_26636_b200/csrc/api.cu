@@ -160,7 +160,8 @@ jv_status run_attn(const void* q, const void* k, const void* v, void* o, const j
     if (r != JV_OK || a.P == 0) return r;
     return from_cuda(launch_attn_generic(a, st, true));   // the P prefix queries, which attend everything
   }
-  if (a.strided) return JV_ERR_UNSUPPORTED;               // the generic kernels read contiguous tensors
+  if (a.strided) return JV_ERR_UNSUPPORTED;               // the fp32 and generic kernels read contiguous tensors
+  if (!g_force_generic.load() && attn_f32_supported(a)) return from_cuda(launch_attn_f32(a, st));
   return from_cuda(launch_attn_generic(a, st));
 }
 

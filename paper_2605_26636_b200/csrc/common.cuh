@@ -112,6 +112,9 @@ struct AttnArgs {
   int dtype;
 };
 cudaError_t launch_attn_generic(const AttnArgs& a, cudaStream_t st, bool prefix_rows_only = false);
+// fp32 tensors at D == 64: register-tiled fp32 kernel (full and windowed attention, prefix tokens)
+bool attn_f32_supported(const AttnArgs& a);
+cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st);
 // tcgen05 path: bf16, D == 64.  full = true: F over all N tokens; else W with (wh, ww)
 // windows whose width ww is a power of two <= 128 (a tile is a box of ww x 128/ww tokens).
 bool attn_tc_supported(const AttnArgs& a, bool full);

@@ -1,0 +1,55 @@
+"""The register-tiled fp32 attention kernel (head_dim 64) at the sizes where it can go wrong: both splits of a CTA into row
+warps and key groups, windows of a single key tile and ragged ones, prefix tokens alone in a tile.
+
+Tolerance: a score is a sum of 64 products in fp32, magnitude up to about 60 before scaling by 1 / 8: its error stays
+below 64 * 2^-24 * 60 / 8 = 3e-5, usually a tenth of that, and the result is off by that fraction of the values; the bar
+of every fp32 comparison here, 1e-4 of the rms, covers it."""
+import pytest
+import torch
+
+from paper_2605_26636_b200 import inputs
+from tests._util import TOL, dwc_to_device, guarded_empty, rel_err, sample_heads
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def jv():
+    from paper_2605_26636_b200 import jetvit
+    jetvit.lib()
+    yield jetvit
+    assert jetvit.device_status() == jetvit.JV_OK
+
+
+CASES = [  # B, H, P, Hg, Wg, win
+    (1, 1, 0, 1, 1, 1),          # one token
+    (1, 2, 0, 5, 13, 64),        # 65 tokens: two key tiles, the second of one key; one window
+    (1, 6, 0, 16, 16, 8),        # F: 16-row tiles, four key groups
+    (1, 2, 5, 9, 23, 8),         # edge windows, windows of 64 + 5 keys
+    (2, 8, 1, 17, 31, 16),       # 32-row tiles, two key groups
+    (4, 37, 0, 8, 8, 8),         # one key tile per window
+    (3, 50, 3, 12, 17, 7),       # windows whose width is not a power of two
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: "x".join(map(str, c)))
+def test_fp32_kernels(jv, oracle, case):
+    B, H, P, Hg, Wg, win = case
+    N = P + Hg * Wg
+    q, k, v = inputs.custom_qkv(B, H, N, 64, "f32", seed=3200 + N)
+    dq, dk, dv = (t.to(DEV) for t in (q, k, v))
+    heads = sample_heads(B, H, 6, N)
+    pick = lambda t: torch.stack([t[b, h] for b, h in heads]).unsqueeze(0)      # as one batch of sampled heads
+    qs, ks, vs = pick(q), pick(k), pick(v)
+    for name, call, ref in (
+            ("F", lambda o: jv.full_attn(dq, dk, dv, out=o), lambda: oracle.full_attn(qs, ks, vs)),
+            ("W", lambda o: jv.window_attn(dq, dk, dv, Hg, Wg, win, win, out=o, prefix=P),
+             lambda: oracle.window_attn(qs, ks, vs, Hg, Wg, win, win, prefix=P)),
+            ("L", lambda o: jv.linear_attn(dq, dk, dv, Hg, Wg, out=o, prefix=P),
+             lambda: oracle.linear_attn(qs, ks, vs, Hg, Wg, prefix=P))):
+        out, check = guarded_empty(q.shape, torch.float32, DEV)
+        out.fill_(float("nan"))
+        call(out)
+        check()
+        assert rel_err(pick(out.cpu()), ref()) <= TOL["f32"], (name, case)
