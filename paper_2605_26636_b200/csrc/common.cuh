@@ -141,6 +141,13 @@ struct LinArgs {
 cudaError_t launch_linear_generic(const LinArgs& a, const LinPlan& p, cudaStream_t st);
 bool linear_fast_supported(const LinArgs& a);
 cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t st);
+// fp32 tensors at D == 64, no convolution or 3 x 3 kernels (pooled or static)
+bool linear_f32_supported(const LinArgs& a);
+cudaError_t launch_linear_f32(const LinArgs& a, const LinPlan& p, cudaStream_t st);
+// the latency-tuned generator (D == 64): hidden layer and output layer, launched behind the grid that wrote the chunk
+// partials (layout of lin_common.cuh); the kernels are in ws + off_kernel when the output layer is complete, and a grid launched
+// with programmatic serialisation behind it that waits for it finds everything before it complete, too
+cudaError_t launch_dwc_generator_chain(const LinArgs& a, const LinPlan& p, const float* partial, cudaStream_t st);
 // bf16, D == 64, 3 x 3 kernels: the apply pass with the convolution fused in
 bool linear_conv_supported(const LinArgs& a);
 cudaError_t launch_linear_apply_conv(const LinArgs& a, const LinPlan& p, const float* partial, const float* w,

@@ -540,10 +540,11 @@ dwc_add_kernel(const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ 
 // sample: per tile of 1024 channels it forms the means (the chunk partials' v-sums, summed in chunk
 // order) in shared memory while the rows of W1 are already on their way, then warp w takes row r0 + w.
 constexpr int kGenTile = 1024;
+template <typename T>
 __global__ void __launch_bounds__(256)
 gen_hidden_kernel(const float* __restrict__ partial, const float* __restrict__ W1, const float* __restrict__ b1,
                   float* __restrict__ hidden, int H, int R, int nchunk, int state_elems, float inv_n, int early_trigger,
-                  const __nv_bfloat16* __restrict__ v, int P, int ntok) {
+                  const T* __restrict__ v, int P, int ntok) {
   __shared__ __align__(16) float s_sm[kGenTile];
   // early_trigger: the grids behind this one each wait for their predecessor before they read its
   // output, so they may be resident (set up, prefetching inputs of the call) while this one waits.
@@ -575,7 +576,7 @@ gen_hidden_kernel(const float* __restrict__ partial, const float* __restrict__ W
         const float* pv = partial + (size_t)(b * H + c / kD) * nchunk * state_elems + kOffVsum + c % kD;
         for (int k = 0; k < nchunk; ++k) m += __ldcg(pv + (size_t)k * state_elems);
         // the v-sums run over all tokens; the pooling is over the grid: take the prefix rows out again
-        for (int t = 0; t < P; ++t) m -= __bfloat162float(v[((size_t)(b * H + c / kD) * ntok + t) * kD + c % kD]);
+        for (int t = 0; t < P; ++t) m -= to_f32(v[((size_t)(b * H + c / kD) * ntok + t) * kD + c % kD]);
       }
       s_sm[threadIdx.x + 256 * i] = m * inv_n;
     }
@@ -676,6 +677,53 @@ gen_out_kernel(const float* __restrict__ hidden, const float* __restrict__ W2, c
   if (!wait_first) griddep_wait();
 }
 
+// Both layers are launched with programmatic serialisation behind the grid that wrote the chunk partials.
+cudaError_t enqueue_gen_hidden(const LinArgs& a, const LinPlan& p, const float* partial, int early_trigger, cudaStream_t st) {
+  const jv_shape& s = a.s;
+  const jv_dwc& d = *a.dwc;
+  float* hidden = (float*)((char*)a.ws + p.off_hidden);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cfg.gridDim = dim3(ceil_div(d.R, 8), s.B);
+  cfg.blockDim = dim3(256);
+  const float inv_n = 1.f / (float)(s.Hg * s.Wg);      // pooling: the mean over the grid tokens
+  cudaError_t e;
+  if (s.dtype == JV_F32)
+    e = cudaLaunchKernelEx(&cfg, gen_hidden_kernel<float>, partial, d.W1, d.b1, hidden, (int)s.H, (int)d.R, p.nchunk,
+                           p.state_elems, inv_n, early_trigger, (const float*)a.v, (int)s.P, shape_tokens(s));
+  else
+    e = cudaLaunchKernelEx(&cfg, gen_hidden_kernel<__nv_bfloat16>, partial, d.W1, d.b1, hidden, (int)s.H, (int)d.R, p.nchunk,
+                           p.state_elems, inv_n, early_trigger, (const __nv_bfloat16*)a.v, (int)s.P, shape_tokens(s));
+  count_launch();
+  return e;
+}
+
+cudaError_t enqueue_gen_out(const LinArgs& a, const LinPlan& p, int wait_first, cudaStream_t st) {
+  const jv_shape& s = a.s;
+  const jv_dwc& d = *a.dwc;
+  const int T = s.H * kD * d.k * d.k;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cfg.gridDim = dim3(ceil_div(T, 32));
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = (size_t)(s.B < 8 ? s.B : 8) * d.R * sizeof(float);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, (d.R % 4 == 0) ? gen_out_kernel<true> : gen_out_kernel<false>,
+                                           (const float*)((char*)a.ws + p.off_hidden), d.W2, d.b2,
+                                           (float*)((char*)a.ws + p.off_kernel), (int)s.B, T, (int)d.R, wait_first);
+  count_launch();
+  return e;
+}
+
 }  // namespace
 
 bool linear_fast_supported(const LinArgs& a) {
@@ -685,6 +733,14 @@ bool linear_fast_supported(const LinArgs& a) {
   // attention proper and the fused 3 x 3 convolution; the pooling's prefix correction reads V directly)
   if (in_strided(a.s) && a.dwc && (a.dwc->token_wise || a.dwc->k != 3 || a.s.P > 0)) return false;
   return a.s.dtype == JV_BF16 && a.s.D == kD && encode_fn() != nullptr;
+}
+
+cudaError_t launch_dwc_generator_chain(const LinArgs& a, const LinPlan& p, const float* partial, cudaStream_t st) {
+  if (a.dwc->R > 0) {                                  // R == 0: static kernels, the output layer just broadcasts b2
+    const cudaError_t e = enqueue_gen_hidden(a, p, partial, 1, st);
+    if (e != cudaSuccess) return e;
+  }
+  return enqueue_gen_out(a, p, 1, st);
 }
 
 cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t st) {
@@ -759,7 +815,6 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
     return err;
   };
 
-  float* hidden = (float*)(ws + p.off_hidden);
   const bool fused_conv = a.dwc && linear_conv_supported(a);
   if (fused_conv && s.P > 0) {
     // Prefix tokens: the convolution does not see them, their output is the attention output alone.
@@ -771,40 +826,17 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
     e = enqueue_apply(mqp, mop, s.P);
     if (e != cudaSuccess) return e;
   }
-  if (a.dwc && a.dwc->R > 0) {      // R == 0: static kernels, the output layer just broadcasts b2
-    const jv_dwc& d = *a.dwc;
-    cudaLaunchConfig_t hcfg = {};
-    hcfg.stream = st;
-    hcfg.attrs = attr;
-    hcfg.numAttrs = 1;
-    hcfg.gridDim = dim3(ceil_div(d.R, 8), s.B);
-    hcfg.blockDim = dim3(256);
-    e = cudaLaunchKernelEx(&hcfg, gen_hidden_kernel, (const float*)partial, d.W1, d.b1, hidden, (int)s.H, (int)d.R,
-                           p.nchunk, p.state_elems, 1.f / (float)(s.Hg * s.Wg), fused_conv ? 1 : 0, (const __nv_bfloat16*)a.v,
-                           (int)s.P, N);
-    count_launch();
-    if (e != cudaSuccess) return e;
-  }
-
   if (fused_conv) {
     // 3 x 3 kernels: state -> [hidden layer] -> output layer -> apply pass with the convolution fused in.
     // Every grid behind the state pass is launched with programmatic serialisation and waits for its
     // predecessor before it reads that one's output, so completion is transitive along the chain.
-    const jv_dwc& d = *a.dwc;
-    float* wk = (float*)(ws + p.off_kernel);
-    const int T = s.H * kD * d.k * d.k;
-    cudaLaunchConfig_t gcfg = {};
-    gcfg.stream = st;
-    gcfg.attrs = attr;
-    gcfg.numAttrs = 1;
-    gcfg.gridDim = dim3(ceil_div(T, 32));
-    gcfg.blockDim = dim3(256);
-    gcfg.dynamicSmemBytes = (size_t)(s.B < 8 ? s.B : 8) * d.R * sizeof(float);
-    e = cudaLaunchKernelEx(&gcfg, (d.R % 4 == 0) ? gen_out_kernel<true> : gen_out_kernel<false>, (const float*)hidden, d.W2,
-                           d.b2, wk, (int)s.B, T, (int)d.R, 1);
-    count_launch();
+    e = launch_dwc_generator_chain(a, p, partial, st);
     if (e != cudaSuccess) return e;
-    return launch_linear_apply_conv(a, p, partial, wk, status, true, st);
+    return launch_linear_apply_conv(a, p, partial, (const float*)(ws + p.off_kernel), status, true, st);
+  }
+  if (a.dwc && a.dwc->R > 0) {
+    e = enqueue_gen_hidden(a, p, partial, 0, st);
+    if (e != cudaSuccess) return e;
   }
 
   e = enqueue_apply(mq, mo, N);
@@ -813,19 +845,7 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
   if (a.dwc) {
     const __nv_bfloat16* v = (const __nv_bfloat16*)a.v;
     __nv_bfloat16* o = (__nv_bfloat16*)a.o;
-    const jv_dwc& d = *a.dwc;
-    float* wk = (float*)(ws + p.off_kernel);
-    const int T = s.H * kD * d.k * d.k;
-    cudaLaunchConfig_t gcfg = {};
-    gcfg.stream = st;
-    gcfg.attrs = attr;
-    gcfg.numAttrs = 1;
-    gcfg.gridDim = dim3(ceil_div(T, 32));
-    gcfg.blockDim = dim3(256);
-    gcfg.dynamicSmemBytes = (size_t)(s.B < 8 ? s.B : 8) * d.R * sizeof(float);
-    e = cudaLaunchKernelEx(&gcfg, (d.R % 4 == 0) ? gen_out_kernel<true> : gen_out_kernel<false>, (const float*)hidden, d.W2,
-                           d.b2, wk, (int)s.B, T, (int)d.R, 0);
-    count_launch();
+    e = enqueue_gen_out(a, p, 0, st);
     if (e != cudaSuccess) return e;
     const float* w = (const float*)(ws + p.off_kernel);
     const int run = 32;

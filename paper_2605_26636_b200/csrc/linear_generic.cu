@@ -17,11 +17,13 @@ LinPlan lin_plan(const jv_shape& s, const jv_dwc* dwc) {
   p.state_elems = (p.D1 * p.D1 + 3) / 4 * 4;
   // Chunks: as many as fit one wave of two CTAs per SM over all (batch, head) pairs, each a
   // multiple of 128 tokens and at least 512 tokens long so that the partials stay small next
-  // to K and V.  One wave means no tail, and chunks of equal length finish together.
+  // to K and V (fp32 tensors: 128, their state pass is bound by arithmetic and short chunks fill the
+  // chip).  One wave means no tail, and chunks of equal length finish together.
   int want = (2 * device_sm_count()) / BH;
   if (want < 1) want = 1;
   int chunk = ceil_div(ceil_div(N, want), 128) * 128;
-  if (chunk < 512) chunk = 512;
+  const int least = s.dtype == JV_F32 && s.D == 64 ? 128 : 512;
+  if (chunk < least) chunk = least;
   p.chunk_tokens = chunk;
   p.nchunk = ceil_div(N, chunk);
   size_t off = 0;

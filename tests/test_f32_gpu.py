@@ -1,5 +1,6 @@
-"""The register-tiled fp32 attention kernel (head_dim 64) at the sizes where it can go wrong: both splits of a CTA into row
-warps and key groups, windows of a single key tile and ragged ones, prefix tokens alone in a tile.
+"""The register-tiled fp32 kernels (attention and the linear block at head_dim 64) at the sizes where they can go wrong: both
+splits of a CTA into row warps and key groups, windows of a single key tile and ragged ones, prefix tokens alone in a
+tile; chunk and tile remainders of the linear block, one-column grids, rows shorter than a thread's run of tokens.
 
 Tolerance: a score is a sum of 64 products in fp32, magnitude up to about 60 before scaling by 1 / 8: its error stays
 below 64 * 2^-24 * 60 / 8 = 3e-5, usually a tenth of that, and the result is off by that fraction of the values; the bar
@@ -53,3 +54,19 @@ def test_fp32_kernels(jv, oracle, case):
         call(out)
         check()
         assert rel_err(pick(out.cpu()), ref()) <= TOL["f32"], (name, case)
+
+
+@pytest.mark.parametrize("static", [False, True], ids=["squeeze", "static"])
+@pytest.mark.parametrize("case", [(1, 1, 0, 1, 1), (1, 2, 0, 70, 1), (2, 3, 5, 11, 13), (1, 12, 1, 32, 32), (2, 2, 3, 3, 130)],
+                         ids=lambda c: "x".join(map(str, c)))
+def test_fp32_linear_with_convolution(jv, oracle, case, static):
+    B, H, P, Hg, Wg = case
+    q, k, v = inputs.custom_qkv(B, H, P + Hg * Wg, 64, "f32", seed=3300 + Hg + Wg)
+    d = inputs.dwc_weights(H * 64, 18, 3, 3301)                 # R = 18: rows of W2 that no float4 divides
+    if static:
+        d = {"k": 3, "R": 0, "b2": inputs.normal((H * 64 * 9,), inputs.SEED_BASE + 3302) * 0.2}
+    out, check = guarded_empty(q.shape, torch.float32, DEV)
+    out.fill_(float("nan"))
+    jv.linear_attn(*(t.to(DEV) for t in (q, k, v)), Hg, Wg, dwc=dwc_to_device(d, DEV), out=out, prefix=P)
+    check()
+    assert rel_err(out, oracle.linear_attn(q, k, v, Hg, Wg, dwc=d, prefix=P)) <= TOL["f32"]
