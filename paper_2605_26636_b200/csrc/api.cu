@@ -175,6 +175,7 @@ jv_status run_linear(const void* q, const void* k, const void* v, void* o, const
   }
   const LinPlan p = lin_plan(*s, dwc);
   if (!g_force_generic.load() && linear_fast_supported(a)) return from_cuda(launch_linear_fast(a, p, st));
+  if (!g_force_generic.load() && linear_d128_supported(a)) return from_cuda(launch_linear_d128(a, p, st));
   if (!g_force_generic.load() && linear_f32_supported(a)) return from_cuda(launch_linear_f32(a, p, st));
   if (in_strided(*s)) return JV_ERR_UNSUPPORTED;          // the generic kernels read contiguous tensors
   return from_cuda(launch_linear_generic(a, p, st));

@@ -141,6 +141,9 @@ struct LinArgs {
 cudaError_t launch_linear_generic(const LinArgs& a, const LinPlan& p, cudaStream_t st);
 bool linear_fast_supported(const LinArgs& a);
 cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t st);
+// bf16 tensors at D == 128 without the convolution
+bool linear_d128_supported(const LinArgs& a);
+cudaError_t launch_linear_d128(const LinArgs& a, const LinPlan& p, cudaStream_t st);
 // fp32 tensors at D == 64, no convolution or 3 x 3 kernels (pooled or static)
 bool linear_f32_supported(const LinArgs& a);
 cudaError_t launch_linear_f32(const LinArgs& a, const LinPlan& p, cudaStream_t st);
