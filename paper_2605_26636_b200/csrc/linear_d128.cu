@@ -1,9 +1,9 @@
 // Linear attention (Sec. 3.2.1, Eq. 2 reordered) at head_dim 128 on the tensor cores: bf16 tensors, no convolution.
 //
-//   lin128_state_kernel   per (head, token chunk): KV = relu(K)^T V, z = relu(K)^T 1 (mma.sync m16n8k16, TMA ring).
-//                         The chunks of a head are one thread-block cluster: their partial states are summed in
-//                         chunk order through distributed shared memory (no atomics: bit-reproducible), and the
-//                         finished state is written once, as the apply pass wants it: KV as a sum of kSplit bf16
+//   lin128_state_kernel   per (head, token chunk): KV = relu(K)^T V (tcgen05.mma, both operands as they lie in memory,
+//                         ReLU in place in shared memory), z = relu(K)^T 1 in fp32.  The chunks of a head are one
+//                         thread-block cluster: every CTA sends each row of its partial state to the CTA that
+//                         finishes that row, which sums the chunks in order (no atomics: bit-reproducible); the finished state is written once, as the apply pass wants it: KV as a sum of kSplit bf16
 //                         matrices, each already in the 128-byte-swizzled layout of its MMA operand, z in fp32.
 //   lin128_apply_kernel   o = relu(q) KV / (relu(q) . z + eps) per 128-token tile: one bulk copy of the state, ReLU in place in
 //                         shared memory, tcgen05.mma with the accumulator in tensor memory, TMA stores.
@@ -12,9 +12,9 @@
 // summed state is 66 KB per head: summing chunk partials in every apply CTA, as at head_dim 64, would read more than Q,
 // hence the cluster reduction.  KV as three bf16 terms keeps the 24 bits of the fp32 state, so the product
 // is as exact as the fp32 kernels' that served these calls before.
-// Measured, 2 x 8 heads, 64 x 64 tokens: MEASURED
-#include <cooperative_groups.h>
-
+// Measured, 2 x 8 heads, 64 x 64 tokens: 32.6 us (67 MB) against 1330 us on the shape-generic kernels; 8 x 8 heads: 72 us
+// = 3.7 TB/s.  With the state pass on mma.sync, which needs 2300 clocks of the legacy matrix path per 64 tokens (their
+// copy needs 1400), and the partials read by plain remote loads it was 43 us.
 #include "lin_common.cuh"
 
 namespace jv {
@@ -37,38 +37,45 @@ constexpr size_t kStateBytes = (size_t)kKvBytes + kC * sizeof(float);   // per (
 constexpr int kTok1 = 64;                             // tokens per tile
 constexpr int kHalf1 = kTok1 * 128;                   // 64 tokens x 64 channels: 8 KB
 constexpr int kStage1 = 4 * kHalf1;                   // K (two halves), V (two halves)
-constexpr int kStages1 = 3;
-constexpr int kMmaWarps = 8;
-constexpr int kThreads1 = (kMmaWarps + 1) * 32;
-constexpr int kLdRed = kC + 4;                        // padded row of the partial state in shared memory (over the ring)
+constexpr int kStages1 = 4;
+constexpr int kReluWarps = 8;
+constexpr int kThreads1 = (kReluWarps + 2) * 32;      // + TMA producer, MMA issuer
 constexpr int kMaxCluster = 8;
+constexpr int kLdRed = kC + 4;                        // padded row of a partial state: 16-byte accesses of 8 rows touch all banks
+constexpr int kRedRows = kC + kMaxCluster;            // nchunk shares of ceil(128 / nchunk) rows
 struct __align__(8) Bars1 {
-  uint64_t full[kStages1], empty[kStages1];
+  uint64_t full[kStages1], empty[kStages1];           // TMA landed / the tile's MMAs are complete
+  uint64_t relu_done[kStages1];                       // 256 arrivals: K rectified
+  uint64_t acc_full;                                  // all MMAs of the chunk are complete
+  uint64_t red_full;                                  // the chunks' partials of this CTA's rows have landed
+  uint32_t tmem_base;
   volatile uint32_t abort_flag;
-  float z[kC];
 };
-constexpr size_t kSmem1 = (size_t)kStages1 * kStage1 + sizeof(Bars1) + 1024;
-static_assert((size_t)kC * kLdRed * sizeof(float) <= (size_t)kStages1 * kStage1, "the partial state fits over the ring");
+// shared memory: ring, then this chunk's partial state over it (rows of 128 columns of KV, then z)
+//                | partial states of this CTA's rows, one per chunk | z of this chunk per token group | barriers
+constexpr size_t kOffRed = (size_t)kStages1 * kStage1, kOffZg = kOffRed + (size_t)kRedRows * kLdRed * sizeof(float);
+constexpr size_t kOffBars1 = kOffZg + (size_t)16 * kC * sizeof(float);
+constexpr size_t kSmem1 = kOffBars1 + sizeof(Bars1) + 1024;
+static_assert(kSmem1 <= 232448, "shared memory of one CTA");
+constexpr uint32_t kIdesc1 = idesc(128, 128, 1, 1);   // D fp32, A and B bf16, both MN-major, M = 128, N = 128
 
-__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+// MN-major operand of 128 columns as two swizzled halves of 64: the leading-dimension offset is the distance of the halves
+__device__ __forceinline__ uint64_t smem_desc_mn128(uint32_t addr, uint32_t half_bytes) {
+  return (smem_desc(addr) & ~(0x3FFFull << 16)) | ((uint64_t)(half_bytes >> 4) << 16);
 }
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
 }
 
-__global__ void __launch_bounds__(kThreads1, 2)
+__global__ void __launch_bounds__(kThreads1, 1)
 lin128_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV,
                     unsigned char* __restrict__ state, int* status, int N, int chunk_tokens) {
-  namespace cg = cooperative_groups;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t smem = smem_u32(smem_al);
-  Bars1* bars = reinterpret_cast<Bars1*>(smem_al + (size_t)kStages1 * kStage1);
-  cg::cluster_group cluster = cg::this_cluster();
+  Bars1* bars = reinterpret_cast<Bars1*>(smem_al + kOffBars1);
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int bh = blockIdx.y, chunk = blockIdx.x, nchunk = gridDim.x;   // the cluster is the whole grid row
   const int t_begin = min(N, chunk * chunk_tokens), t_end = min(N, t_begin + chunk_tokens);
@@ -78,29 +85,30 @@ lin128_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages1; ++s) {
       mbar_init(&bars->full[s], 1);
-      mbar_init(&bars->empty[s], kMmaWarps);
+      mbar_init(&bars->empty[s], 1);
+      mbar_init(&bars->relu_done[s], kReluWarps * 32);
     }
+    mbar_init(&bars->acc_full, 1);
+    mbar_init(&bars->red_full, 1);
     // an earlier kernel gave up: no copies, no waits (but this CTA still takes part in the cluster's barriers)
     bars->abort_flag = *reinterpret_cast<volatile int*>(status) != 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  __syncthreads();
-  bool ok = bars->abort_flag == 0;
-
-  // warp w of the eight: rows 32 (w / 2) .. + 31 of KV, columns 64 (w % 2) .. + 63
-  const int rg = warp >> 1, ch = warp & 1;
-  float acc[2][8][4], accz[2][4];
-#pragma unroll
-  for (int m = 0; m < 2; ++m) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) acc[m][j][i] = 0.f;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) accz[m][i] = 0.f;
+  if (warp == 0) {
+    __syncwarp();
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tmem_base)), "r"(kC) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  if (warp == kMmaWarps) {
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // (1) this CTA may be copied to
+  const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+  bool ok = bars->abort_flag == 0;
+  float* zg = reinterpret_cast<float*>(smem_al + kOffZg);              // [16 token groups][128]
+
+  if (warp == kReluWarps) {
     // ================= TMA producer =================
     int issued = 0;
     for (int it = 0; it < ntiles && ok; ++it) {
@@ -124,80 +132,120 @@ lin128_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
       for (int g = max(0, issued - kStages1); g < issued; ++g)
         while (!mbar_try(&bars->full[g % kStages1], (g / kStages1) & 1) && globaltimer() - t0 < kWaitLimitNs) {}
     }
-    __syncwarp();
+  } else if (warp == kReluWarps + 1) {
+    // ================= MMA issuer: KV += relu(K)^T V, 64 tokens at a time =================
+    for (int it = 0; it < ntiles && ok; ++it) {
+      const int s = it % kStages1;
+      ok = warp_wait(&bars->relu_done[s], (it / kStages1) & 1, &bars->abort_flag, status);
+      if (!ok) break;
+      tc_fence_after();
+      if (elect_one()) {
+        const uint64_t da = smem_desc_mn128(smem + s * kStage1, kHalf1), db = smem_desc_mn128(smem + s * kStage1 + 2 * kHalf1, kHalf1);
+#pragma unroll
+        for (int ks = 0; ks < kTok1 / 16; ++ks)
+          mma_ss_1(tmem, desc_advance(da, ks * 2048), desc_advance(db, ks * 2048), kIdesc1, (it > 0 || ks > 0) ? 1u : 0u);
+      }
+      __syncwarp();
+      tc_commit(&bars->empty[s]);
+    }
+    if (ok && ntiles > 0) tc_commit(&bars->acc_full);
+    if (!ok && lane == 0) {                                 // bounded time for the tensor core before tensor memory is released
+      const unsigned long long t0 = globaltimer();
+      while (globaltimer() - t0 < 1000000ull) {}
+    }
   } else {
-    const uint32_t ones = (lane < 4) ? 0x3F803F80u : 0u;    // B fragment of a ones column
+    // ================= rectifier warps: thread owns 16-byte chunk cc of tokens 4 tg .. 4 tg + 3 of every tile: ReLU in
+    // place, and z of its eight channels exactly in fp32 =================
+    const int cc = threadIdx.x & 15, tg = threadIdx.x >> 4;
+    float z[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) z[e] = 0.f;
     for (int it = 0; it < ntiles && ok; ++it) {
       const int s = it % kStages1;
       ok = warp_wait(&bars->full[s], (it / kStages1) & 1, &bars->abort_flag, status);
       if (!ok) break;
-      const uint32_t ks = smem + s * kStage1 + (rg >> 1) * kHalf1, vsm = smem + s * kStage1 + (2 + ch) * kHalf1;
+      unsigned char* kt = smem_al + (size_t)s * kStage1 + (cc >> 3) * kHalf1;
+      uint4 x[4];
 #pragma unroll
-      for (int kk = 0; kk < kTok1 / 16; ++kk) {
-        uint32_t a[2][4];
-        const int ta = kk * 16 + (lane & 7) + ((lane >> 4) & 1) * 8;
+      for (int j = 0; j < 4; ++j) x[j] = *reinterpret_cast<const uint4*>(kt + tile_off(4 * tg + j, cc & 7));
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {                       // A = relu(K)^T; K is stored [token][a] -> .trans
-          ldmatrix_x4_trans(a[m], ks + tile_off(ta, 4 * (rg & 1) + 2 * m + ((lane >> 3) & 1)));
-#pragma unroll
-          for (int i = 0; i < 4; ++i) a[m][i] = relu_bf16x2(a[m][i]);
-        }
-        const int tb = kk * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-#pragma unroll
-        for (int jp = 0; jp < 4; ++jp) {
-          uint32_t b[4];                                    // V stored [token][e] -> .trans; two n-tiles per load
-          ldmatrix_x4_trans(b, vsm + tile_off(tb, 2 * jp + (lane >> 4)));
-#pragma unroll
-          for (int m = 0; m < 2; ++m) {
-            mma_bf16(acc[m][2 * jp], a[m], b[0], b[1]);
-            mma_bf16(acc[m][2 * jp + 1], a[m], b[2], b[3]);
-          }
-        }
-        if (ch == 0) {
-#pragma unroll
-          for (int m = 0; m < 2; ++m) mma_bf16(accz[m], a[m], ones, ones);
-        }
+      for (int j = 0; j < 4; ++j) {
+        x[j].x = relu_bf16x2(x[j].x); x[j].y = relu_bf16x2(x[j].y); x[j].z = relu_bf16x2(x[j].z); x[j].w = relu_bf16x2(x[j].w);
+        *reinterpret_cast<uint4*>(kt + tile_off(4 * tg + j, cc & 7)) = x[j];
+        const float2 f0 = bf16x2_to_f2(x[j].x), f1 = bf16x2_to_f2(x[j].y), f2 = bf16x2_to_f2(x[j].z), f3 = bf16x2_to_f2(x[j].w);
+        z[0] += f0.x; z[1] += f0.y; z[2] += f1.x; z[3] += f1.y;
+        z[4] += f2.x; z[5] += f2.y; z[6] += f3.x; z[7] += f3.y;
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->empty[s]);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      mbar_arrive(&bars->relu_done[s]);
     }
+    *reinterpret_cast<float4*>(zg + tg * kC + 8 * cc) = make_float4(z[0], z[1], z[2], z[3]);
+    *reinterpret_cast<float4*>(zg + tg * kC + 8 * cc + 4) = make_float4(z[4], z[5], z[6], z[7]);
+    if (ok && ntiles > 0) ok = warp_wait(&bars->acc_full, 0, &bars->abort_flag, status);
+    tc_fence_after();
   }
-  // every copy has been waited for by the MMA warps (or landed above): the ring becomes the partial state
   __syncthreads();
-  float* red = reinterpret_cast<float*>(smem_al);
-  const int g = lane >> 2, tq = lane & 3;
-  if (warp < kMmaWarps) {
+  // The partial state goes to shared memory (over the ring: its copies have landed and its MMAs are complete), thread
+  // (quadrant q4, lane) holding row 32 q4 + lane, warps 0-3 its columns 0-63 and z, warps 4-7 columns 64-127; from there one
+  // bulk copy takes every CTA of the cluster the rows that it finishes.  (Stored to the other CTAs straight from
+  // the registers, 16 bytes of a row per lane, the 64 KB took 6000 clocks.)
+  const int share = (kC + nchunk - 1) / nchunk;
+  if (warp < kReluWarps) {
+    const int q4 = warp & 3, h = warp >> 2, row = 32 * q4 + lane;
+    float* dst = reinterpret_cast<float*>(smem_al) + row * kLdRed + 64 * h;
 #pragma unroll
-    for (int m = 0; m < 2; ++m) {
-      const int a0 = 32 * rg + 16 * m + g;
+    for (int j = 0; j < 2; ++j) {
+      uint32_t v[32];
+      if (ntiles > 0) {
+        tmem_ld32(tmem + ((uint32_t)(q4 << 5) << 16) + 64 * h + 32 * j, v);
+        tmem_wait_ld(v);
+      } else {
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        *reinterpret_cast<float2*>(red + a0 * kLdRed + 64 * ch + 8 * j + 2 * tq) = make_float2(acc[m][j][0], acc[m][j][1]);
-        *reinterpret_cast<float2*>(red + (a0 + 8) * kLdRed + 64 * ch + 8 * j + 2 * tq) = make_float2(acc[m][j][2], acc[m][j][3]);
+        for (int i = 0; i < 32; ++i) v[i] = 0u;
       }
-      if (ch == 0 && tq == 0) {
-        bars->z[a0] = accz[m][0];
-        bars->z[a0 + 8] = accz[m][2];
-      }
+#pragma unroll
+      for (int i = 0; i < 32; i += 4)
+        *reinterpret_cast<uint4*>(dst + 32 * j + i) = make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    }
+    if (h == 0) {
+      float z = 0.f;
+#pragma unroll
+      for (int g = 0; g < 16; ++g) z += zg[g * kC + row];
+      dst[kC] = z;
+    }
+    tc_fence_before();
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  __syncthreads();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // (1)
+  const int row0 = chunk * share, rows = max(0, min(share, kC - row0));
+  if (warp == 0 && elect_one()) {
+    if (rows > 0) mbar_expect_tx(&bars->red_full, (uint32_t)(nchunk * rows * kLdRed * 4));
+    for (int c = 0; c < nchunk; ++c) {
+      const int n = min(share, kC - c * share);
+      if (n > 0)
+        asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(map_rank(smem + (uint32_t)kOffRed + (uint32_t)(chunk * share * kLdRed * 4), c)),
+                       "r"(smem + (uint32_t)(c * share * kLdRed * 4)), "r"((uint32_t)(n * kLdRed * 4)),
+                       "r"(map_rank(smem_u32(&bars->red_full), c)) : "memory");
     }
   }
-  cluster.sync();
-  // this CTA finishes rows chunk * rows .. + rows - 1 of the head's state, eight columns per thread
-  const int rows = kC / nchunk, row0 = chunk * rows;
+  __syncwarp();
+  if (rows > 0) warp_wait(&bars->red_full, 0, &bars->abort_flag, status);   // (every CTA sends, also one that gave up)
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // (2) received: the senders may leave
+  // this CTA's rows: the chunks' partials summed in chunk order, eight columns per thread and step
+  const float* red = reinterpret_cast<const float*>(smem_al + kOffRed);
   unsigned char* st = state + (size_t)bh * kStateBytes;
   for (int i = threadIdx.x; i < rows * (kC / 8); i += kThreads1) {
-    const int row = row0 + i / (kC / 8), c8 = i % (kC / 8);
+    const int r = i / (kC / 8), c8 = i % (kC / 8);
     float x[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) x[e] = 0.f;
-#pragma unroll
-    for (int c = 0; c < kMaxCluster; ++c) {
-      if (c < nchunk) {
-        const float* src = cluster.map_shared_rank(red, c) + row * kLdRed + 8 * c8;
-        const float4 lo = *reinterpret_cast<const float4*>(src), hi = *reinterpret_cast<const float4*>(src + 4);
-        x[0] += lo.x; x[1] += lo.y; x[2] += lo.z; x[3] += lo.w;
-        x[4] += hi.x; x[5] += hi.y; x[6] += hi.z; x[7] += hi.w;
-      }
+    for (int c = 0; c < nchunk; ++c) {
+      const float* src = red + (c * share + r) * kLdRed + 8 * c8;
+      const float4 lo = *reinterpret_cast<const float4*>(src), hi = *reinterpret_cast<const float4*>(src + 4);
+      x[0] += lo.x; x[1] += lo.y; x[2] += lo.z; x[3] += lo.w;
+      x[4] += hi.x; x[5] += hi.y; x[6] += hi.z; x[7] += hi.w;
     }
 #pragma unroll
     for (int s = 0; s < kSplit; ++s) {                      // the bf16 nearest to what the terms before it left over
@@ -209,15 +257,18 @@ lin128_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
         x[2 * e] -= f.x;
         x[2 * e + 1] -= f.y;
       }
-      *reinterpret_cast<uint4*>(st + (size_t)(2 * s + (c8 >> 3)) * kKvHalf + tile_off(row, c8 & 7)) = make_uint4(w[0], w[1], w[2], w[3]);
+      *reinterpret_cast<uint4*>(st + (size_t)(2 * s + (c8 >> 3)) * kKvHalf + tile_off(row0 + r, c8 & 7)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
   for (int i = threadIdx.x; i < rows; i += kThreads1) {
     float z = 0.f;
-    for (int c = 0; c < nchunk; ++c) z += cluster.map_shared_rank(bars->z, c)[row0 + i];
+    for (int c = 0; c < nchunk; ++c) z += red[(c * share + i) * kLdRed + kC];
     reinterpret_cast<float*>(st + kKvBytes)[row0 + i] = z;
   }
-  cluster.sync();                                           // no CTA leaves while its partial may still be read
+  tc_fence_after();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kC) : "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // (2)
 }
 
 // ---- apply pass ---------------------------------------------------------------------
@@ -225,7 +276,7 @@ constexpr int kTok2 = 128;                            // tokens per tile
 constexpr int kHalf2 = kTok2 * 128;                   // 128 tokens x 64 channels: 16 KB
 constexpr int kTile2 = 2 * kHalf2;
 constexpr int kSlots = 3;                             // Q tiles; a slot becomes its tile's output staging
-constexpr int kThreads2 = 288;                        // 4 rectifier warps, 1 producer / issuer warp, 4 epilogue warps
+constexpr int kThreads2 = 320;                        // 4 rectifier warps, MMA issuer, 4 epilogue warps, TMA producer
 constexpr uint32_t kTmemCols = 256;                   // two 128-column fp32 accumulators
 struct __align__(8) Bars2 {
   uint64_t q_full[kSlots], q_free[kSlots];            // TMA landed / the four store groups have read the slot
@@ -239,7 +290,7 @@ constexpr size_t kOffQ = kKvBytes, kOffZ2 = kOffQ + (size_t)kSlots * kTile2, kOf
 constexpr size_t kOffBars2 = kOffDen + (size_t)kSlots * kTok2 * sizeof(float);
 constexpr size_t kSmem2 = kOffBars2 + sizeof(Bars2) + 1024;
 static_assert(kSmem2 <= 232448, "shared memory of one CTA");
-constexpr uint32_t kIdesc = idesc(128, 64, 1);        // D fp32, A and B bf16, B MN-major, M = 128, N = 64
+constexpr uint32_t kIdesc2 = idesc(128, 128, 1);      // D fp32, A and B bf16, B MN-major, M = 128, N = 128
 
 __global__ void __launch_bounds__(kThreads2, 1)
 lin128_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapO,
@@ -282,8 +333,8 @@ lin128_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
   const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
   bool ok = true;
 
-  if (warp == 4) {
-    // ================= TMA producer and MMA issuer =================
+  if (warp == 9) {
+    // ================= TMA producer =================
     int issued = 0;
     bool kv_issued = false;
     auto load_tile = [&](int it) {
@@ -306,14 +357,26 @@ lin128_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
       if (elect_one()) {
         mbar_expect_tx(&bars->kv_full, kKvBytes + kC * 4);
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(smem), "l"(state + (size_t)bh * kStateBytes), "r"(kKvBytes), "r"(smem_u32(&bars->kv_full)) : "memory");
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                      ::"r"(smem_u32(z_sm)), "l"(state + (size_t)bh * kStateBytes + kKvBytes), "r"(kC * 4),
                        "r"(smem_u32(&bars->kv_full)) : "memory");
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(smem), "l"(state + (size_t)bh * kStateBytes), "r"(kKvBytes), "r"(smem_u32(&bars->kv_full)) : "memory");
       }
       __syncwarp();
-      ok = warp_wait(&bars->kv_full, 0, &bars->abort_flag, status);
     }
+    for (int it = kSlots; it < ntiles && ok; ++it) {
+      ok = warp_wait(&bars->q_free[it % kSlots], ((it / kSlots) - 1) & 1, &bars->abort_flag, status);
+      if (ok) load_tile(it);
+    }
+    if (!ok && lane == 0) {                            // let the copies in flight land before the CTA leaves
+      const unsigned long long t0 = globaltimer();
+      for (int g = max(0, issued - kSlots); g < issued; ++g)
+        while (!mbar_try(&bars->q_full[g % kSlots], (g / kSlots) & 1) && globaltimer() - t0 < kWaitLimitNs) {}
+      while (kv_issued && !mbar_try(&bars->kv_full, 0) && globaltimer() - t0 < kWaitLimitNs) {}
+    }
+  } else if (warp == 4) {
+    // ================= MMA issuer =================
+    ok = warp_wait(&bars->kv_full, 0, &bars->abort_flag, status);
     for (int it = 0; it < ntiles && ok; ++it) {
       const int s = it % kSlots, b = it & 1;
       ok = warp_wait(&bars->relu_done[s], (it / kSlots) & 1, &bars->abort_flag, status);
@@ -321,32 +384,18 @@ lin128_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
       if (!ok) break;
       tc_fence_after();
       if (elect_one()) {
-        const uint32_t qa = smem + (uint32_t)kOffQ + s * kTile2;
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h)                    // 64-column halves of the accumulator
-#pragma unroll 1
-          for (int x = 0; x < kSplit; ++x) {
-            const uint64_t da = smem_desc(qa), db = smem_desc(smem + (2 * x + h) * kKvHalf);
+        const uint64_t da = smem_desc(smem + (uint32_t)kOffQ + s * kTile2);
 #pragma unroll
-            for (int ks = 0; ks < kC / 16; ++ks)
-              mma_ss_1(tmem + b * kC + 64 * h, desc_advance(da, (ks >> 2) * kHalf2 + (ks & 3) * 32), desc_advance(db, ks * 2048),
-                       kIdesc, (x > 0 || ks > 0) ? 1u : 0u);
-          }
+        for (int x = 0; x < kSplit; ++x) {
+          const uint64_t db = smem_desc_mn128(smem + 2 * x * kKvHalf, kKvHalf);
+#pragma unroll
+          for (int ks = 0; ks < kC / 16; ++ks)
+            mma_ss_1(tmem + b * kC, desc_advance(da, (ks >> 2) * kHalf2 + (ks & 3) * 32), desc_advance(db, ks * 2048), kIdesc2,
+                     (x > 0 || ks > 0) ? 1u : 0u);
+        }
       }
       __syncwarp();
       tc_commit(&bars->d_full[b]);
-      const int nx = it + kSlots - 1;                  // into the slot of tile it - 1, once its stores have read it
-      if (it > 0 && nx < ntiles) {
-        ok = warp_wait(&bars->q_free[nx % kSlots], ((it - 1) / kSlots) & 1, &bars->abort_flag, status);
-        if (!ok) break;
-        load_tile(nx);
-      }
-    }
-    if (!ok && lane == 0) {                            // let the copies in flight land before the CTA leaves
-      const unsigned long long t0 = globaltimer();
-      for (int g = max(0, issued - kSlots); g < issued; ++g)
-        while (!mbar_try(&bars->q_full[g % kSlots], (g / kSlots) & 1) && globaltimer() - t0 < kWaitLimitNs) {}
-      while (kv_issued && !mbar_try(&bars->kv_full, 0) && globaltimer() - t0 < kWaitLimitNs) {}
     }
   } else if (warp < 4) {
     // ================= rectifier warps: thread r owns token row r of every tile =================
@@ -484,11 +533,12 @@ cudaError_t launch_linear_d128(const LinArgs& a, const LinPlan& p, cudaStream_t 
   });
   if (e != cudaSuccess) return e;
 
-  // chunks per head: a cluster of 1, 2, 4 or 8 CTAs (the portable limit), at most one wave of two CTAs per SM, and
-  // no more chunks than 64-token tiles
+  // chunks per head: a cluster of up to 8 CTAs (the portable limit), one CTA per SM over all heads
   const int tiles = ceil_div(N, kTok1);
-  int nchunk = 1;
-  while (2 * nchunk <= kMaxCluster && 2 * nchunk * BH <= 2 * num_sms && 2 * nchunk <= tiles) nchunk *= 2;
+  int nchunk = num_sms / BH;
+  if (nchunk > kMaxCluster) nchunk = kMaxCluster;
+  if (nchunk > tiles) nchunk = tiles;
+  if (nchunk < 1) nchunk = 1;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = nchunk;

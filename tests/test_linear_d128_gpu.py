@@ -1,5 +1,5 @@
-"""Linear attention at head_dim 128 on its tensor-core kernels: every cluster size of the state pass (one, two, four and eight
-chunks per head, chunks past the end among them), ragged 64- and 128-token tiles, one tile and many per CTA of the apply pass.
+"""Linear attention at head_dim 128 on its tensor-core kernels: cluster sizes of the state pass from one to eight
+chunks per head (chunks past the end among them), ragged 64- and 128-token tiles, one tile and many per CTA of the apply pass.
 
 The state enters the product as three bf16 terms (24 bits), so the result differs from the oracle by the rounding of
 the bf16 store; the bars are those of every bf16 comparison."""
@@ -25,10 +25,12 @@ CASES = [  # B, H, P, Hg, Wg
     (1, 1, 0, 1, 1),
     (1, 2, 0, 5, 13),        # 65 tokens: two tiles, two chunks
     (1, 3, 0, 8, 16),        # 128 tokens: exactly one apply tile
-    (1, 2, 5, 17, 33),       # prefix tokens, 9 + tiles over eight chunks, the last ones empty
+    (1, 2, 5, 17, 33),       # prefix tokens, 9 + tiles over eight chunks
     (2, 8, 0, 64, 64),
     (1, 8, 1, 37, 37),
-    (5, 20, 0, 20, 24),      # 100 heads: two chunks, one CTA per head in the apply pass
+    (3, 8, 0, 33, 40),       # 24 heads: six chunks
+    (5, 10, 0, 20, 24),      # 50 heads: two chunks
+    (1, 21, 0, 10, 64),      # seven chunks of two tiles: the last ones empty, shares of 19 rows
     (2, 80, 0, 9, 15),       # 160 heads: one chunk
 ]
 
