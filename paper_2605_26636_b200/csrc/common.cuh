@@ -147,14 +147,18 @@ cudaError_t launch_linear_d128(const LinArgs& a, const LinPlan& p, cudaStream_t 
 // fp32 tensors at D == 64, no convolution or 3 x 3 kernels (pooled or static)
 bool linear_f32_supported(const LinArgs& a);
 cudaError_t launch_linear_f32(const LinArgs& a, const LinPlan& p, cudaStream_t st);
-// the latency-tuned generator (D == 64): hidden layer and output layer, launched behind the grid that wrote the chunk
-// partials (layout of lin_common.cuh); the kernels are in ws + off_kernel when the output layer is complete, and a grid launched
-// with programmatic serialisation behind it that waits for it finds everything before it complete, too
-cudaError_t launch_dwc_generator_chain(const LinArgs& a, const LinPlan& p, const float* partial, cudaStream_t st);
+// the kernel generator at D == 64, launched behind the grid that wrote the chunk partials (layout of lin_common.cuh); a grid
+// launched with programmatic serialisation behind it that waits for it finds the kernels and everything before them
+// complete.  prefix: the rows of o of the P <= kGenPrefix prefix tokens, too (bf16).
+constexpr int kGenPrefix = 16;
+cudaError_t launch_dwc_generator_fast(const LinArgs& a, const LinPlan& p, const float* partial, bool prefix, cudaStream_t st);
+// where the convolution kernels of a call are: generated ones in ws + off_kernel, static ones in place; *w_batch: floats
+// from sample to sample.  To be called ahead of the state pass (static kernels off 16 bytes are copied into ws).
+cudaError_t dwc_static_kernels(const LinArgs& a, const LinPlan& p, const float** w, int* w_batch, cudaStream_t st);
 // bf16, D == 64, 3 x 3 kernels: the apply pass with the convolution fused in
 bool linear_conv_supported(const LinArgs& a);
 cudaError_t launch_linear_apply_conv(const LinArgs& a, const LinPlan& p, const float* partial, const float* w,
-                                     int* status, bool programmatic, cudaStream_t st);
+                                     int w_batch, int* status, bool programmatic, cudaStream_t st);
 // shared by both linear paths: hidden = SiLU(W1 s + b1), w = W2 hidden + b2, with
 // s = vsum / N read from vsum[bh * bh_stride + e]
 cudaError_t launch_dwc_generator(const LinArgs& a, const LinPlan& p, const float* vsum, int bh_stride,

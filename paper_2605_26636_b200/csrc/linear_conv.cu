@@ -69,7 +69,8 @@ constexpr size_t kConvSmem = kOffBars + sizeof(ConvBars) + 1024;   // + alignmen
 
 struct ConvParams {
   const float* partial;     // chunk partials of the state pass
-  const float* w;           // convolution kernels [B][C][3][3] fp32 (generated, or broadcast static ones)
+  const float* w;           // convolution kernels [C][3][3] fp32 of sample b at w + b * w_batch (0: static, shared ones)
+  int w_batch;
   int* status;
   int H, BH, Hg, Wg, nchunk, state_elems;
   int ncb, nrb;             // patches per grid row / per grid column
@@ -395,7 +396,7 @@ lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
       const int sq = it % kNQ, sv = it % kNV;
       if (new_head) {
         const int b = ti.bh / p.H, h = ti.bh - b * p.H;
-        const float4* wp = reinterpret_cast<const float4*>(p.w + ((size_t)b * p.H * kD + (size_t)h * kD + 4 * c4) * 9);
+        const float4* wp = reinterpret_cast<const float4*>(p.w + (size_t)b * p.w_batch + ((size_t)h * kD + 4 * c4) * 9);
         float wf[36];                                  // [channel][tap] as stored
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
@@ -406,7 +407,7 @@ lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
         for (int pr = 0; pr < 2; ++pr)
 #pragma unroll
           for (int tap = 0; tap < 9; ++tap) wq[pr][tap] = pack_bf16(wf[9 * (2 * pr) + tap], wf[9 * (2 * pr + 1) + tap]);
-        if (ti.bh + 1 < p.BH) {   // the kernels of the (batch, head) after this one: into L2 ahead of the switch
+        if (h + 1 < p.H) {        // the kernels of the head after this one: into L2 ahead of the switch
           const float* wn = reinterpret_cast<const float*>(wp) + kD * 9;
           asm volatile("prefetch.global.L2 [%0];" ::"l"(wn));
           asm volatile("prefetch.global.L2 [%0];" ::"l"(wn + 32));
@@ -524,7 +525,7 @@ bool linear_conv_supported(const LinArgs& a) {
 // pass, `w` the kernels [B][C][3][3]; both are written by grids ahead of this one in the stream,
 // which this grid waits for (griddepcontrol.wait) before it reads them.
 cudaError_t launch_linear_apply_conv(const LinArgs& a, const LinPlan& p, const float* partial, const float* w,
-                                     int* status, bool programmatic, cudaStream_t st) {
+                                     int w_batch, int* status, bool programmatic, cudaStream_t st) {
   const jv_shape& s = a.s;
   const int BH = s.B * s.H;
   CUtensorMap mq, mv, mo;
@@ -541,6 +542,7 @@ cudaError_t launch_linear_apply_conv(const LinArgs& a, const LinPlan& p, const f
   ConvParams cp;
   cp.partial = partial;
   cp.w = w;
+  cp.w_batch = w_batch;
   cp.status = status;
   cp.H = s.H;
   cp.BH = BH;

@@ -2,7 +2,7 @@
 // throughout, register-tiled, with the 3 x 3 convolution inside the apply pass.
 //
 //   lin_f32_state_kernel   per (head, token chunk): KV = relu(K)^T V, z, v-sum -> partial (layout of lin_common.cuh)
-//   generator              the two latency-tuned layers of linear_fast.cu
+//   generator              dwc_generator.cu
 //   lin_f32_apply_kernel   per 64 tokens: sums the chunk partials of its head in chunk order, then
 //                          o = relu(q) KV / (relu(q).z + eps) + 3 x 3 convolution of V
 //
@@ -101,10 +101,10 @@ lin_f32_state_kernel(const float* __restrict__ k, const float* __restrict__ v, f
   out[kOffZ + tid] = colsum;                                      // z (64), then the v-sum (64)
 }
 
-// w: kernels [B][C][3][3] or nullptr (no convolution)
+// w: kernels [C][3][3] of sample b at w + b * w_batch, or nullptr (no convolution)
 __global__ void __launch_bounds__(kThreads)
 lin_f32_apply_kernel(const float* __restrict__ q, const float* __restrict__ v, float* __restrict__ o,
-                     const float* __restrict__ partial, const float* __restrict__ w, int H, int P, int Hg, int Wg, int nchunk,
+                     const float* __restrict__ partial, const float* __restrict__ w, int w_batch, int H, int P, int Hg, int Wg, int nchunk,
                      int state_elems, float eps) {
   extern __shared__ __align__(16) float smem_f[];
   float* qs = smem_f;                                             // relu(q) [64][kLdA]
@@ -182,7 +182,7 @@ lin_f32_apply_kernel(const float* __restrict__ q, const float* __restrict__ v, f
   const int tt = t0 + 8 * ty;                                     // this thread's eight consecutive tokens
   if (w != nullptr) {
     float wf[4][9];                                               // [channel][tap]
-    const float4* wp = reinterpret_cast<const float4*>(w + ((size_t)(bh / H) * H * kD + (size_t)(bh % H) * kD + 4 * tx) * 9);
+    const float4* wp = reinterpret_cast<const float4*>(w + (size_t)(bh / H) * w_batch + ((size_t)(bh % H) * kD + 4 * tx) * 9);
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
       const float4 x = __ldcg(wp + i);
@@ -232,7 +232,6 @@ lin_f32_apply_kernel(const float* __restrict__ q, const float* __restrict__ v, f
 }  // namespace
 
 bool linear_f32_supported(const LinArgs& a) {
-  if (a.dwc && a.dwc->R > 0 && (((uintptr_t)a.dwc->W1 | (uintptr_t)a.dwc->W2) & 15) != 0) return false;   // 128-bit loads of the weights
   return a.s.dtype == JV_F32 && a.s.D == kD && !in_strided(a.s) && !(a.dwc && (a.dwc->token_wise || a.dwc->k != 3));
 }
 
@@ -245,15 +244,14 @@ cudaError_t launch_linear_f32(const LinArgs& a, const LinPlan& p, cudaStream_t s
     return cudaFuncSetAttribute(lin_f32_state_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStateSmem);
   });
   if (e != cudaSuccess) return e;
+  const float* w = nullptr;
+  int w_batch = 0;
+  if (a.dwc && (e = dwc_static_kernels(a, p, &w, &w_batch, st)) != cudaSuccess) return e;
   lin_f32_state_kernel<<<dim3(p.nchunk, BH), kThreads, kStateSmem, st>>>((const float*)a.k, (const float*)a.v, partial, N,
                                                                          p.chunk_tokens, p.state_elems);
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const float* w = nullptr;
-  if (a.dwc) {
-    if ((e = launch_dwc_generator_chain(a, p, partial, st)) != cudaSuccess) return e;
-    w = (const float*)((char*)a.ws + p.off_kernel);
-  }
+  if (a.dwc && (e = launch_dwc_generator_fast(a, p, partial, false, st)) != cudaSuccess) return e;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -264,7 +262,7 @@ cudaError_t launch_linear_f32(const LinArgs& a, const LinPlan& p, cudaStream_t s
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, lin_f32_apply_kernel, (const float*)a.q, (const float*)a.v, (float*)a.o, (const float*)partial, w,
+  e = cudaLaunchKernelEx(&cfg, lin_f32_apply_kernel, (const float*)a.q, (const float*)a.v, (float*)a.o, (const float*)partial, w, w_batch,
                          (int)s.H, (int)s.P, (int)s.Hg, (int)s.Wg, p.nchunk, p.state_elems, a.eps);
   count_launch();
   return e;

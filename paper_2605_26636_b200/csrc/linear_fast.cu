@@ -21,10 +21,9 @@
 // its first Q loads overlap the tail of the state kernel, and it waits for that grid
 // (griddepcontrol.wait) only before touching the partials.
 //
-// With the convolution on, the generator's two layers (tiny kernels laid out for latency) run
-// between the state pass and the apply pass.  3 x 3 kernels: the apply pass is the fused
-// apply + convolution kernel of linear_conv.cu.  5 x 5 kernels: the apply pass above, the output
-// layer beside it, and a read-modify-write convolution pass over o behind both.
+// With the convolution on, the kernel generator (dwc_generator.cu) runs between the state pass and the
+// apply pass.  3 x 3 kernels: the apply pass is the fused apply + convolution kernel of linear_conv.cu.  5 x 5
+// kernels: the apply pass above and a read-modify-write convolution pass over o behind it.
 //
 // Partial layout per (batch, head, chunk), in floats:
 //   [0, 4096) KV[a][e], [4096, 4160) z[a], [4160, 4224) vsum[e]
@@ -274,11 +273,7 @@ lin_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
 
-  // A grid launched behind this one with programmatic serialisation (the output layer of the
-  // convolution's generator) may start once this grid lets its dependents go.  It reads what the
-  // grids before this one wrote, so no warp here does that before it knows that those grids are
-  // complete: the rectifier warps after their griddepcontrol.wait, the other warps after the first
-  // barrier that the rectifier warps have arrived on.
+  griddep_launch_dependents();                         // (a grid behind this one waits for it before it reads o)
 
   if (warp == 4) {
     // ================= TMA producer and MMA issuer (one elected lane) =================
@@ -308,7 +303,6 @@ lin_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
       }
       const int s = it % kApplyStages, b = it & 1;
       ok = warp_wait(&bars->relu_done[s], (it / kApplyStages) & 1, &bars->abort_flag, status);
-      if (it == 0) griddep_launch_dependents();
       if (ok && it >= 2) ok = warp_wait(&bars->d_empty[b], ((it >> 1) - 1) & 1, &bars->abort_flag, status);
       if (!ok) break;
       tc_fence_after();
@@ -335,8 +329,7 @@ lin_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     }
   } else if (warp < 4) {
     // ================= rectifier warps: thread r = 32 warp + lane owns token row r of every tile =================
-    griddep_wait();                                    // the grids before this one (state pass, generator's hidden layer) are complete
-    griddep_launch_dependents();
+    griddep_wait();                                    // the grids before this one (state pass, generator) are complete
     bool ok = *reinterpret_cast<volatile int*>(status) == 0;
     if (!ok) bars->abort_flag = 1;                     // an earlier kernel gave up: every role of this CTA falls through at once
     {  // second pass of the reduction: chunk partials summed in a fixed order; KV -> bf16 MMA operand, z in fp32
@@ -436,7 +429,6 @@ lin_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
       // The tile's MMAs were issued after all 128 rectifier threads had published its rows and
       // denominators, so the accumulator being complete means the denominators are in place.
       ok = warp_wait(&bars->d_full[b], (it >> 1) & 1, &bars->abort_flag, status);
-      if (it == 0) griddep_launch_dependents();
       if (!ok) break;
       tc_fence_after();
       const float inv = 1.f / (den_sm[(it & (kDenRing - 1)) * kApplyTok + row] + eps);
@@ -497,7 +489,7 @@ lin_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
 template <int K>
 __global__ void __launch_bounds__(256)
 dwc_add_kernel(const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ o, const float* __restrict__ w,
-               int H, int Hg, int Wg, int run) {
+               int w_batch, int H, int Hg, int Wg, int run) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int N = Hg * Wg, bh = blockIdx.y, b = bh / H, h = bh % H;
   const int t0 = (blockIdx.x * 8 + warp) * run;
@@ -505,7 +497,7 @@ dwc_add_kernel(const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ 
   const int t1 = min(N, t0 + run);
   constexpr int P = (K - 1) / 2;
   float w0[K * K], w1[K * K];
-  const float* wp = w + ((size_t)b * H * kD + (size_t)h * kD + 2 * lane) * K * K;
+  const float* wp = w + (size_t)b * w_batch + ((size_t)h * kD + 2 * lane) * K * K;
 #pragma unroll
   for (int i = 0; i < K * K; ++i) { w0[i] = wp[i]; w1[i] = wp[K * K + i]; }
   const __nv_bfloat16* vb = v + (size_t)bh * N * kD + 2 * lane;
@@ -532,198 +524,6 @@ dwc_add_kernel(const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ 
   }
 }
 
-// ---- kernel generator of the squeeze dynamic convolution (Sec. 3.2.1), tuned for latency ------
-// Both layers sit on the critical path between the state pass and the apply pass, so each is laid
-// out as ONE round trip of independent loads followed by arithmetic.
-//
-// hidden[b][r] = SiLU(b1[r] + sum_c W1[r][c] * mean_v[b][c]).  A block serves 8 values of r for one
-// sample: per tile of 1024 channels it forms the means (the chunk partials' v-sums, summed in chunk
-// order) in shared memory while the rows of W1 are already on their way, then warp w takes row r0 + w.
-constexpr int kGenTile = 1024;
-template <typename T>
-__global__ void __launch_bounds__(256)
-gen_hidden_kernel(const float* __restrict__ partial, const float* __restrict__ W1, const float* __restrict__ b1,
-                  float* __restrict__ hidden, int H, int R, int nchunk, int state_elems, float inv_n, int early_trigger,
-                  const T* __restrict__ v, int P, int ntok) {
-  __shared__ __align__(16) float s_sm[kGenTile];
-  // early_trigger: the grids behind this one each wait for their predecessor before they read its
-  // output, so they may be resident (set up, prefetching inputs of the call) while this one waits.
-  if (early_trigger) griddep_launch_dependents();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * 8 + warp, b = blockIdx.y, C = H * kD;
-  const bool r_ok = r < R;
-  const float* wrow = W1 + (size_t)(r_ok ? r : 0) * C;
-  float dot = 0.f;
-  bool waited = false;
-  for (int c0 = 0; c0 < C; c0 += kGenTile) {           // C is a multiple of 64
-    float4 wv[kGenTile / 128];                         // this lane's part of the row: W1 is an input of the call
-#pragma unroll
-    for (int i = 0; i < kGenTile / 128; ++i) {
-      const int c = c0 + 4 * lane + 128 * i;
-      wv[i] = (r_ok && c < C) ? __ldg(reinterpret_cast<const float4*>(wrow + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    if (!waited) {
-      griddep_wait();                                  // the state pass is complete
-      if (!early_trigger) griddep_launch_dependents(); // the apply grid may set up and load Q meanwhile
-      waited = true;
-    }
-    __syncthreads();                                   // the previous tile's means have been consumed
-#pragma unroll
-    for (int i = 0; i < kGenTile / 256; ++i) {
-      const int c = c0 + threadIdx.x + 256 * i;
-      float m = 0.f;
-      if (c < C) {
-        const float* pv = partial + (size_t)(b * H + c / kD) * nchunk * state_elems + kOffVsum + c % kD;
-        for (int k = 0; k < nchunk; ++k) m += __ldcg(pv + (size_t)k * state_elems);
-        // the v-sums run over all tokens; the pooling is over the grid: take the prefix rows out again
-        for (int t = 0; t < P; ++t) m -= to_f32(v[((size_t)(b * H + c / kD) * ntok + t) * kD + c % kD]);
-      }
-      s_sm[threadIdx.x + 256 * i] = m * inv_n;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < kGenTile / 128; ++i) {
-      const float4 sv = *reinterpret_cast<const float4*>(s_sm + 4 * lane + 128 * i);
-      dot = fmaf(wv[i].x, sv.x, fmaf(wv[i].y, sv.y, fmaf(wv[i].z, sv.z, fmaf(wv[i].w, sv.w, dot))));
-    }
-  }
-  dot = warp_sum(dot);
-  if (lane == 0 && r_ok) {
-    const float x = dot + (b1 ? b1[r] : 0.f);
-    hidden[(size_t)b * R + r] = x / (1.f + expf(-x));
-  }
-}
-// w[b][t] = b2[t] + sum_r W2[t][r] * hidden[b][r]; 8 lanes per output t, 32 outputs per block, all
-// samples (8 at a time, their hidden vectors in shared memory).  kVec (R a multiple of 4): a lane's
-// part of the W2 row is fetched as float4, the whole row in flight at once.
-template <bool kVec>
-__global__ void __launch_bounds__(256)
-gen_out_kernel(const float* __restrict__ hidden, const float* __restrict__ W2, const float* __restrict__ b2,
-               float* __restrict__ w, int B, int T, int R, int wait_first) {
-  extern __shared__ __align__(16) float h_sm[];        // [min(B, 8)][R]: small, so that the grid can be resident early
-  // wait_first = 0: launched behind the apply grid, which lets its dependents go only after it has
-  // seen the hidden layer's grid complete: hidden is final here and this grid runs beside the apply
-  // pass; it waits at its end (below).  wait_first = 1: launched directly behind the hidden layer
-  // (or the state pass, with static kernels), ahead of the fused apply + convolution grid: it waits
-  // for its predecessor before it reads hidden.
-  griddep_launch_dependents();                         // the grid behind this one may set up and prefetch
-  const int t = blockIdx.x * 32 + (threadIdx.x >> 3), part = threadIdx.x & 7;
-  const bool t_ok = t < T;
-  const float* wrow = W2 + (size_t)(t_ok ? t : 0) * R;
-  constexpr int kPer = kVec ? 4 : 16;                  // loads per lane and 128 values of r
-  bool waited = wait_first == 0;
-  for (int b0 = 0; b0 < B; b0 += 8) {
-    float acc[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) acc[i] = 0.f;
-    const int nb = min(8, B - b0);
-    for (int r0 = 0; r0 < R; r0 += 128) {
-      float wv[16];                                    // W2 is an input of the call: on its way before the wait
-      if (kVec) {
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-          const int r = r0 + 4 * part + 32 * i;
-          const float4 x = r < R ? __ldg(reinterpret_cast<const float4*>(wrow + r)) : make_float4(0.f, 0.f, 0.f, 0.f);
-          wv[4 * i] = x.x; wv[4 * i + 1] = x.y; wv[4 * i + 2] = x.z; wv[4 * i + 3] = x.w;
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-          const int r = r0 + part + 8 * i;
-          wv[i] = r < R ? __ldg(wrow + r) : 0.f;
-        }
-      }
-      if (r0 == 0) {                                   // this group of samples' hidden vectors -> shared memory
-        if (!waited) { griddep_wait(); waited = true; }
-        __syncthreads();
-        for (int i = threadIdx.x; i < nb * R; i += 256) h_sm[i] = __ldcg(hidden + (size_t)b0 * R + i);
-        __syncthreads();
-      }
-#pragma unroll
-      for (int bb = 0; bb < 8; ++bb) {
-        if (bb < nb) {
-          const float* hp = h_sm + bb * R + r0;
-          if (kVec) {
-#pragma unroll
-            for (int i = 0; i < kPer; ++i) {
-              const int r = 4 * part + 32 * i;
-              if (r0 + r < R) {
-                const float4 hv = *reinterpret_cast<const float4*>(hp + r);
-                acc[bb] = fmaf(wv[4 * i], hv.x, fmaf(wv[4 * i + 1], hv.y, fmaf(wv[4 * i + 2], hv.z, fmaf(wv[4 * i + 3], hv.w, acc[bb]))));
-              }
-            }
-          } else {
-#pragma unroll
-            for (int i = 0; i < kPer; ++i) {
-              const int r = part + 8 * i;
-              if (r0 + r < R) acc[bb] = fmaf(wv[i], hp[r], acc[bb]);
-            }
-          }
-        }
-      }
-    }
-    if (R == 0 && !waited) { griddep_wait(); waited = true; }   // static kernels: nothing to read, but completion must chain
-#pragma unroll
-    for (int bb = 0; bb < 8; ++bb) {
-      float sres = acc[bb];
-      sres += __shfl_xor_sync(0xffffffffu, sres, 1);
-      sres += __shfl_xor_sync(0xffffffffu, sres, 2);
-      sres += __shfl_xor_sync(0xffffffffu, sres, 4);
-      if (t_ok && part == 0 && bb < nb) w[(size_t)(b0 + bb) * T + t] = sres + (b2 ? b2[t] : 0.f);
-    }
-  }
-  // wait_first = 0: the convolution pass is launched behind this grid and adds into what the apply
-  // pass writes: this grid must not retire before the apply grid has.
-  if (!wait_first) griddep_wait();
-}
-
-// Both layers are launched with programmatic serialisation behind the grid that wrote the chunk partials.
-cudaError_t enqueue_gen_hidden(const LinArgs& a, const LinPlan& p, const float* partial, int early_trigger, cudaStream_t st) {
-  const jv_shape& s = a.s;
-  const jv_dwc& d = *a.dwc;
-  float* hidden = (float*)((char*)a.ws + p.off_hidden);
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cfg.gridDim = dim3(ceil_div(d.R, 8), s.B);
-  cfg.blockDim = dim3(256);
-  const float inv_n = 1.f / (float)(s.Hg * s.Wg);      // pooling: the mean over the grid tokens
-  cudaError_t e;
-  if (s.dtype == JV_F32)
-    e = cudaLaunchKernelEx(&cfg, gen_hidden_kernel<float>, partial, d.W1, d.b1, hidden, (int)s.H, (int)d.R, p.nchunk,
-                           p.state_elems, inv_n, early_trigger, (const float*)a.v, (int)s.P, shape_tokens(s));
-  else
-    e = cudaLaunchKernelEx(&cfg, gen_hidden_kernel<__nv_bfloat16>, partial, d.W1, d.b1, hidden, (int)s.H, (int)d.R, p.nchunk,
-                           p.state_elems, inv_n, early_trigger, (const __nv_bfloat16*)a.v, (int)s.P, shape_tokens(s));
-  count_launch();
-  return e;
-}
-
-cudaError_t enqueue_gen_out(const LinArgs& a, const LinPlan& p, int wait_first, cudaStream_t st) {
-  const jv_shape& s = a.s;
-  const jv_dwc& d = *a.dwc;
-  const int T = s.H * kD * d.k * d.k;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cfg.gridDim = dim3(ceil_div(T, 32));
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = (size_t)(s.B < 8 ? s.B : 8) * d.R * sizeof(float);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, (d.R % 4 == 0) ? gen_out_kernel<true> : gen_out_kernel<false>,
-                                           (const float*)((char*)a.ws + p.off_hidden), d.W2, d.b2,
-                                           (float*)((char*)a.ws + p.off_kernel), (int)s.B, T, (int)d.R, wait_first);
-  count_launch();
-  return e;
-}
-
 }  // namespace
 
 bool linear_fast_supported(const LinArgs& a) {
@@ -733,14 +533,6 @@ bool linear_fast_supported(const LinArgs& a) {
   // attention proper and the fused 3 x 3 convolution; the pooling's prefix correction reads V directly)
   if (in_strided(a.s) && a.dwc && (a.dwc->token_wise || a.dwc->k != 3 || a.s.P > 0)) return false;
   return a.s.dtype == JV_BF16 && a.s.D == kD && encode_fn() != nullptr;
-}
-
-cudaError_t launch_dwc_generator_chain(const LinArgs& a, const LinPlan& p, const float* partial, cudaStream_t st) {
-  if (a.dwc->R > 0) {                                  // R == 0: static kernels, the output layer just broadcasts b2
-    const cudaError_t e = enqueue_gen_hidden(a, p, partial, 1, st);
-    if (e != cudaSuccess) return e;
-  }
-  return enqueue_gen_out(a, p, 1, st);
 }
 
 cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t st) {
@@ -774,6 +566,10 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
     return cudaFuncSetAttribute(lin_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kApplySmem);
   });
   if (e != cudaSuccess) return e;
+  const bool fused_conv = a.dwc && linear_conv_supported(a);
+  const float* w = nullptr;           // convolution kernels [B][C][k][k], w_batch floats from sample to sample
+  int w_batch = 0;
+  if (a.dwc && (e = dwc_static_kernels(a, p, &w, &w_batch, st)) != cudaSuccess) return e;
   const int num_sms = device_sm_count();
   dim3 g1(p.nchunk, BH);
   if (a.dwc)
@@ -788,12 +584,8 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
 
-  // With the convolution on, the generator's hidden layer (tiny; it needs the state pass only) goes
-  // between the state pass and the apply pass, and its output layer behind the apply pass, beside
-  // which it runs.  Every launch from here to the output layer uses programmatic serialisation;
-  // each grid waits for its predecessor (griddepcontrol.wait) before it reads what that one wrote,
-  // the output layer at its very end, so that stream order still means "apply pass complete" for
-  // the convolution pass that follows it.
+  // Every grid behind the state pass is launched with programmatic serialisation and waits for its
+  // predecessor (griddepcontrol.wait) before it reads what that one wrote, so completion is transitive along the chain.
   // apply pass over the first ntokens tokens of every (batch, head): one wave of two CTAs per SM, spans
   // of whole 128-token tiles; launched so that its set-up overlaps the tail of the grid before it
   auto enqueue_apply = [&](const CUtensorMap& map_q, const CUtensorMap& map_o, int ntokens) -> cudaError_t {
@@ -815,47 +607,30 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
     return err;
   };
 
-  const bool fused_conv = a.dwc && linear_conv_supported(a);
-  if (fused_conv && s.P > 0) {
-    // Prefix tokens: the convolution does not see them, their output is the attention output alone.
-    // The plain apply pass over the first P tokens of every (batch, head), right behind the state pass
-    // (which it waits for; the grids behind it wait for it in turn).
-    CUtensorMap mqp, mop;
-    if (!make_map_tokens_in(&mqp, a.q, s.B, s.H, s.P, kApplyTok, in) || !make_map_tokens(&mop, a.o, BH, s.P, 32, N))
-      return cudaErrorInvalidValue;
-    e = enqueue_apply(mqp, mop, s.P);
-    if (e != cudaSuccess) return e;
-  }
+  if (!a.dwc) return enqueue_apply(mq, mo, N);
   if (fused_conv) {
-    // 3 x 3 kernels: state -> [hidden layer] -> output layer -> apply pass with the convolution fused in.
-    // Every grid behind the state pass is launched with programmatic serialisation and waits for its
-    // predecessor before it reads that one's output, so completion is transitive along the chain.
-    e = launch_dwc_generator_chain(a, p, partial, st);
-    if (e != cudaSuccess) return e;
-    return launch_linear_apply_conv(a, p, partial, (const float*)(ws + p.off_kernel), status, true, st);
+    // 3 x 3 kernels: state -> generator (with generated kernels) -> apply pass with the convolution fused in.
+    // Prefix tokens: the convolution does not see them, their output is the attention output alone.  A few of them are
+    // done beside the generator (a launch of their own cost 8.5 us of a 40 us block of 6 heads), more by the plain apply pass.
+    if (s.P > kGenPrefix) {
+      CUtensorMap mqp, mop;
+      if (!make_map_tokens_in(&mqp, a.q, s.B, s.H, s.P, kApplyTok, in) || !make_map_tokens(&mop, a.o, BH, s.P, 32, N))
+        return cudaErrorInvalidValue;
+      if ((e = enqueue_apply(mqp, mop, s.P)) != cudaSuccess) return e;
+    }
+    if ((e = launch_dwc_generator_fast(a, p, partial, s.P > 0 && s.P <= kGenPrefix, st)) != cudaSuccess) return e;
+    return launch_linear_apply_conv(a, p, partial, w, w_batch, status, true, st);
   }
-  if (a.dwc && a.dwc->R > 0) {
-    e = enqueue_gen_hidden(a, p, partial, 0, st);
-    if (e != cudaSuccess) return e;
-  }
-
-  e = enqueue_apply(mq, mo, N);
-  if (e != cudaSuccess) return e;
-
-  if (a.dwc) {
-    const __nv_bfloat16* v = (const __nv_bfloat16*)a.v;
-    __nv_bfloat16* o = (__nv_bfloat16*)a.o;
-    e = enqueue_gen_out(a, p, 0, st);
-    if (e != cudaSuccess) return e;
-    const float* w = (const float*)(ws + p.off_kernel);
-    const int run = 32;
-    dim3 g4(ceil_div(ceil_div(N, run), 8), BH);
-    // 5 x 5 kernels (3 x 3 ones took the fused path above): a read-modify-write pass over o
-    if (a.dwc->k == 3) dwc_add_kernel<3><<<g4, 256, 0, st>>>(v, o, w, s.H, s.Hg, s.Wg, run);
-    else
-      dwc_add_kernel<5><<<g4, 256, 0, st>>>(v, o, w, s.H, s.Hg, s.Wg, run);
-    count_launch();
-  }
+  // 5 x 5 kernels: generator, apply pass, a read-modify-write pass over o
+  if ((e = launch_dwc_generator_fast(a, p, partial, false, st)) != cudaSuccess) return e;
+  if ((e = enqueue_apply(mq, mo, N)) != cudaSuccess) return e;
+  const int run = 32;
+  dim3 g4(ceil_div(ceil_div(N, run), 8), BH);
+  const __nv_bfloat16* v = (const __nv_bfloat16*)a.v;
+  __nv_bfloat16* o = (__nv_bfloat16*)a.o;
+  if (a.dwc->k == 3) dwc_add_kernel<3><<<g4, 256, 0, st>>>(v, o, w, w_batch, s.H, s.Hg, s.Wg, run);
+  else dwc_add_kernel<5><<<g4, 256, 0, st>>>(v, o, w, w_batch, s.H, s.Hg, s.Wg, run);
+  count_launch();
   return cudaGetLastError();
 }
 
