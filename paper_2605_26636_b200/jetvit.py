@@ -31,6 +31,9 @@ class JvDwc(ctypes.Structure):
                 ("token_wise", ctypes.c_int32)]
 
 
+_DwcPtrs = ctypes.POINTER(ctypes.POINTER(JvDwc))
+
+
 class JetVitError(RuntimeError):
     def __init__(self, status: int, where: str):
         self.status = status
@@ -133,15 +136,36 @@ def make_shape(t: torch.Tensor, Hg: int, Wg: int, prefix: int = 0) -> JvShape:
 def _check_tensors(*ts: torch.Tensor):
     """q, k, v[, o]: one shape, dtype and device; q, k, v in one layout; o (a fourth tensor) contiguous."""
     ref = ts[0]
+    shape, dtype, dev, dense, strides = ref.shape, ref.dtype, ref.get_device(), ref.is_contiguous(), ref.stride()
     for i, t in enumerate(ts):
+        # these cheap attributes settle nearly every call; what they do not settle goes through the checks below, one by one
+        if dev >= 0 and t.shape == shape and t.dtype is dtype and t.get_device() == dev \
+                and (t.is_contiguous() if dense or i >= 3 else t.stride() == strides):
+            continue
         if not t.is_cuda:
             raise ValueError("tensors must live on a CUDA device (there is no CPU path)")
-        if t.shape != ref.shape or t.dtype != ref.dtype or t.device != ref.device:
+        if t.shape != shape or t.dtype != dtype or t.device != ref.device:
             raise ValueError("q, k, v, o must be [B,H,N,D] tensors of one shape, dtype and device")
         if i < 3 and _in_layout(t) != _in_layout(ref):
             raise ValueError("q, k and v must share one layout (all contiguous, or all views with the same token stride)")
         if i >= 3 and not t.is_contiguous():
             raise ValueError("o must be a contiguous [B,H,N,D] tensor")
+
+
+class _current_device:
+    """``with torch.cuda.device(d)`` that costs nothing when d is the current device already."""
+    __slots__ = ("ctx",)
+
+    def __init__(self, device: torch.device):
+        self.ctx = None if device.index == torch.cuda.current_device() else torch.cuda.device(device)
+
+    def __enter__(self):
+        if self.ctx is not None:
+            self.ctx.__enter__()
+
+    def __exit__(self, *exc):
+        if self.ctx is not None:
+            self.ctx.__exit__(*exc)
 
 
 def _empty_out(q: torch.Tensor) -> torch.Tensor:
@@ -163,9 +187,16 @@ def make_dwc(d: Optional[dict], device) -> Optional[JvDwc]:
                  int(d.get("token_wise", 0)))
 
 
+# the current stream's handle without building a Stream object, where torch has the call
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def workspace_bytes(mixer: str, shape: JvShape, dwc: Optional[JvDwc] = None) -> int:
@@ -194,7 +225,7 @@ def linear_attn(q, k, v, Hg: int, Wg: int, eps: float = 1e-6, dwc: Optional[dict
     _check_tensors(q, k, v, out)
     shape = make_shape(q, Hg, Wg, prefix)
     d = make_dwc(dwc, q.device)
-    with torch.cuda.device(q.device):
+    with _current_device(q.device):
         if ws is None:
             ws = alloc_workspace("L", shape, d, q.device)
             if ws is not None and stream is not None:
@@ -213,7 +244,7 @@ def linear_attn_focused(q, k, v, Hg: int, Wg: int, focus_p: float, eps: float = 
     _check_tensors(q, k, v, out)
     shape = make_shape(q, Hg, Wg, prefix)
     d = make_dwc(dwc, q.device)
-    with torch.cuda.device(q.device):
+    with _current_device(q.device):
         if ws is None:
             ws = alloc_workspace("f", shape, d, q.device)
             if ws is not None and stream is not None:
@@ -238,7 +269,7 @@ def linear_attn_static(q, k, v, Hg: int, Wg: int, eps: float = 1e-6, dwc: Option
     _check_tensors(q, k, v, out)
     shape = make_shape(q, Hg, Wg, prefix)
     d = make_dwc(dwc, q.device)
-    with torch.cuda.device(q.device):
+    with _current_device(q.device):
         st = lib().jv_linear_attn_static(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(),
                                          ctypes.byref(shape), float(eps),
                                          ctypes.byref(d) if d is not None else None, _stream(stream))
@@ -252,7 +283,7 @@ def window_attn(q, k, v, Hg: int, Wg: int, win_h: int, win_w: int, scale: float 
     out = _empty_out(q) if out is None else out
     _check_tensors(q, k, v, out)
     shape = make_shape(q, Hg, Wg, prefix)
-    with torch.cuda.device(q.device):
+    with _current_device(q.device):
         st = lib().jv_window_attn(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), ctypes.byref(shape),
                                   int(win_h), int(win_w), float(scale), None, 0, _stream(stream))
     _raise(st, "jv_window_attn")
@@ -267,7 +298,7 @@ def full_attn(q, k, v, Hg: Optional[int] = None, Wg: Optional[int] = None, scale
     if Hg is None or Wg is None:
         Hg, Wg = 1, q.shape[2]
     shape = make_shape(q, Hg, Wg)
-    with torch.cuda.device(q.device):
+    with _current_device(q.device):
         st = lib().jv_full_attn(q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(), ctypes.byref(shape),
                                 float(scale), None, 0, _stream(stream))
     _raise(st, "jv_full_attn")
@@ -283,18 +314,20 @@ def hybrid_mixers(schedule: str, q: Sequence[torch.Tensor], k, v, Hg: int, Wg: i
     if not (len(q) == len(k) == len(v) == n):
         raise ValueError("need one q, k, v per schedule entry")
     out = [_empty_out(t) for t in q] if out is None else list(out)
+    q0 = q[0] if n else None
     for l in range(n):
         _check_tensors(q[l], k[l], v[l], out[l])
-        if q[l].shape != q[0].shape or q[l].dtype != q[0].dtype or _in_layout(q[l]) != _in_layout(q[0]):
+        if l and (q[l].shape != q0.shape or q[l].dtype != q0.dtype
+                  or q[l].stride() != q0.stride() and _in_layout(q[l]) != _in_layout(q0)):
             raise ValueError("all layers share one shape, dtype and input layout")
     shape = make_shape(q[0], Hg, Wg, prefix)
-    arr = lambda ts: (ctypes.c_void_p * n)(*[t.data_ptr() for t in ts])
+    vps = ctypes.c_void_p * n
+    arr = lambda ts: vps(*[t.data_ptr() for t in ts])
     dstructs = [make_dwc(d, q[0].device) for d in dwc] if dwc is not None else None
     dptr = None
     if dstructs is not None:
-        dptr = (ctypes.POINTER(JvDwc) * n)(*[ctypes.pointer(d) if d is not None else ctypes.POINTER(JvDwc)()
-                                             for d in dstructs])
-    with torch.cuda.device(q[0].device):
+        dptr = ctypes.cast(vps(*[None if d is None else ctypes.addressof(d) for d in dstructs]), _DwcPtrs)
+    with _current_device(q[0].device):
         if ws is None:
             need = 0
             for l, m in enumerate(schedule):
@@ -334,7 +367,7 @@ def qkv_proj(x, w, bias, H: int, Hg: int, Wg: int, out=None, stream=None, prefix
     if tuple(q.shape) != (B, H, N, 64) or q.dtype != x.dtype:
         raise ValueError("q, k, v must be [B, H, N, 64] bf16")
     shape = JvShape(B, H, Hg, Wg, 64, JV_BF16, prefix)
-    with torch.cuda.device(x.device):
+    with _current_device(x.device):
         st = lib().jv_qkv_proj(x.data_ptr(), w.data_ptr(), None if bias is None else bias.data_ptr(), q.data_ptr(),
                                k.data_ptr(), v.data_ptr(), ctypes.byref(shape), _stream(stream))
     _raise(st, "jv_qkv_proj")
@@ -353,7 +386,7 @@ def out_proj(o, w, bias, Hg: int, Wg: int, out=None, stream=None, prefix: int = 
     if not (y.is_cuda and y.is_contiguous() and tuple(y.shape) == (B, N, C) and y.dtype == o.dtype):
         raise ValueError("y must be a contiguous [B, N, C] bf16 CUDA tensor")
     shape = JvShape(B, H, Hg, Wg, 64, JV_BF16, prefix)
-    with torch.cuda.device(o.device):
+    with _current_device(o.device):
         st = lib().jv_out_proj(o.data_ptr(), w.data_ptr(), None if bias is None else bias.data_ptr(), y.data_ptr(),
                                ctypes.byref(shape), _stream(stream))
     _raise(st, "jv_out_proj")
