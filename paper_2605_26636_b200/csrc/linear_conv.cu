@@ -11,8 +11,8 @@
 //
 // Warp roles (19 warps):
 //   warps 0-3    rectifiers: per head, the deterministic second pass of the state reduction (chunk
-//                partials summed in a fixed order -> KV as bf16 MMA operand, z in fp32); per tile,
-//                ReLU of the Q tile in place (one thread per token) and that token's denominator
+//                partials summed in a fixed order -> KV as bf16 MMA operand, z as three bf16 terms, its 24 bits);
+//                per tile, relu(Q) from the Q slot into tensor memory as the MMA's A operand (one thread per token)
 //   warp 4       TMA producer: Q patches into a ring of kNQ slots, V halos into a ring of kNV slots
 //   warps 5-8    epilogue: accumulator (tensor memory) x 1/denominator -> bf16, written over the Q
 //                tile it came from (the slot doubles as the output staging tile)
@@ -20,9 +20,17 @@
 //                tokens of both rows, slides the 3 x 3 window over four input rows of the halo
 //                (bf16 x bf16 products summed in fp32), adds the result to the attention
 //                output waiting in the slot and rounds to bf16
-//   warp 17      MMA issuer: relu(Q) KV as tcgen05.mma M128 N64 K64, accumulators double-buffered
+//   warp 17      MMA issuer: relu(Q) KV as tcgen05.mma M128 N64 K64 and the denominators relu(Q) z as N16, accumulators
+//                double-buffered; also copies each head's convolution kernels into shared memory, a head ahead
 //   warp 18      store warp: one TMA store per finished tile (clipped at the grid edge), then the
 //                slot goes back to the producer
+//
+// What bounds it: shared-memory bandwidth.  A tile moves 56 KB through it for the copies in and out and the
+// convolution warps read V three times over (two output rows per warp); with relu(Q) rewritten in shared memory and read
+// from there by the MMAs, the denominators from z in shared memory and the kernels fetched lane by lane at each head
+// boundary a tile took 2250 clocks and a boundary 5000; now 1850 and 800.  8 x 16 heads, 64 x 64 tokens: 45 -> 39 us of the
+// block's 84.6 -> 78.7.  More convolution warps (sixteen, half the tokens each: 87.0 us for the block), packed fp32
+// multiply-adds on widened values (98.9 us: register moves) and fewer instructions elsewhere did not help.
 //
 // Every mbarrier wait is bounded; a wait that runs out sets the device status word and the CTA-wide
 // abort flag, every role falls through, tensor memory is released.
@@ -39,13 +47,15 @@ constexpr int kTileBytes = kPatchH * kPatchW * kD * 2;   // 16 KB
 constexpr int kKvBytes = kD * kD * 2;                 // bf16 KV[a][e], 128-byte swizzle
 constexpr int kHaloBytes = (kPatchH + 2) * (kPatchW + 2) * kD * 2;   // 23040
 constexpr int kHaloSlot = 23552;                      // padded to a multiple of 512
-constexpr int kNQ = 5;                                // Q / output ring
-constexpr int kNV = 3;                                // V halo ring
-constexpr int kDenRing = 8;                           // denominators of the tiles between ReLU and epilogue (> kNQ)
+constexpr int kNQ = 6;                                // Q / output ring
+constexpr int kNV = 4;                                // V halo ring
+constexpr int kZtBytes = 16 * kD * 2;                 // z as an MMA operand: 16 rows of 64 channels, z = row 0 + row 1 + row 2
 constexpr int kWarps = 19, kThreadsConv = kWarps * 32;
 constexpr int kWarpProducer = 4, kWarpEpi0 = 5, kWarpConv0 = 9, kWarpMma = 17, kWarpStore = 18;
-constexpr uint32_t kTmemCols = 128;                   // two 64-column fp32 accumulators
+constexpr uint32_t kTmemCols = 256;                   // two buffers (below)
+constexpr uint32_t kAccStride = 128, kColZ = 64, kColA = 96;   // buffer b at 128 b: output, denominators, relu(Q) as A operand
 constexpr uint32_t kIdesc = idesc(128, 64, 1);        // D fp32, A and B bf16, B MN-major, M = 128, N = 64
+constexpr uint32_t kIdescZ = idesc(128, 16, 0);       // the denominators: B = z, K-major, N = 16
 
 struct __align__(8) ConvBars {
   uint64_t q_full[kNQ], q_free[kNQ];                  // TMA landed / the tile's store has read the slot
@@ -55,17 +65,20 @@ struct __align__(8) ConvBars {
   uint64_t v_full[kNV], v_free[kNV];                  // TMA landed / the 8 convolution warps are done with the halo
   uint64_t d_full[2], d_empty[2];                     // accumulator complete (tcgen05.commit) / read by the epilogue (128)
   uint64_t kv_free[2];                                // the MMAs that read this KV buffer are complete (tcgen05.commit)
+  uint64_t w_full[2], w_free[2];                      // a head's convolution kernels have landed / the 8 convolution warps have read them
   uint64_t workers;                                   // the 128 rectifier threads among themselves
   uint32_t tmem_base;
   volatile uint32_t abort_flag;
 };
-// shared memory: Q ring | KV x 2 | V halo ring | z x 2 | denominators | barriers
+// shared memory: Q ring | KV x 2 | z x 2 | kernels x 2 | V halo ring | barriers
 constexpr size_t kOffKv = (size_t)kNQ * kTileBytes;
-constexpr size_t kOffHalo = kOffKv + 2 * kKvBytes;
-constexpr size_t kOffZsm = kOffHalo + (size_t)kNV * kHaloSlot;
-constexpr size_t kOffDen = kOffZsm + 2 * kD * sizeof(float);
-constexpr size_t kOffBars = kOffDen + (size_t)kDenRing * 128 * sizeof(float);
+constexpr size_t kOffZt = kOffKv + 2 * kKvBytes;
+constexpr size_t kOffW = kOffZt + 2 * kZtBytes;
+constexpr int kWBytes = kD * 9 * 4;                   // a head's convolution kernels [64][3][3] fp32
+constexpr size_t kOffHalo = kOffW + ((2 * kWBytes + 511) / 512) * 512;
+constexpr size_t kOffBars = kOffHalo + (size_t)kNV * kHaloSlot;
 constexpr size_t kConvSmem = kOffBars + sizeof(ConvBars) + 1024;   // + alignment slack
+static_assert(kConvSmem <= 232448, "shared memory of one CTA");
 
 struct ConvParams {
   const float* partial;     // chunk partials of the state pass
@@ -92,6 +105,11 @@ __device__ __forceinline__ void add_bf16x2(float& lo, float& hi, uint32_t a) {
       "mov.b32 {al, ah}, %2;\n"
       "add.rn.f32.bf16 %0, al, %0;\nadd.rn.f32.bf16 %1, ah, %1;\n}\n"
       : "+f"(lo), "+f"(hi) : "r"(a));
+}
+
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
 }
 
 // Walks the tiles of a CTA's range in order: (batch*head, patch row, patch column).
@@ -121,8 +139,6 @@ lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
   // 1024-byte alignment by an offset from the array itself, so that accesses stay shared-space loads and stores
   unsigned char* smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t smem = smem_u32(smem_al);
-  float* z_sm = reinterpret_cast<float*>(smem_al + kOffZsm);          // [2][64]
-  float* den_sm = reinterpret_cast<float*>(smem_al + kOffDen);        // [kDenRing][128]
   ConvBars* bars = reinterpret_cast<ConvBars*>(smem_al + kOffBars);
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
@@ -147,6 +163,8 @@ lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
       mbar_init(&bars->d_full[b], 1);
       mbar_init(&bars->d_empty[b], 128);
       mbar_init(&bars->kv_free[b], 1);
+      mbar_init(&bars->w_full[b], 1);
+      mbar_init(&bars->w_free[b], 8);
     }
     mbar_init(&bars->workers, 128);
     bars->abort_flag = 0;
@@ -211,27 +229,57 @@ lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
         while (!mbar_try(&bars->v_full[g % kNV], (g / kNV) & 1) && globaltimer() - t0 < kWaitLimitNs) {}
     }
   } else if (warp == kWarpMma) {
-    // ================= MMA issuer =================
+    // ================= MMA issuer; also fetches the convolution kernels, a head ahead =================
     TileIter ti;
     ti.init(t_begin, p.ncb, p.nrb);
     bool ok = true;
     int nh = 0;                                        // heads seen so far by this CTA: KV buffer nh & 1
+    const int bh_last = (t_end - 1) / (p.ncb * p.nrb);
+    griddep_wait();                                    // the kernels come from the grid before this one
+    auto load_w = [&](int bh, int buf) {
+      if (elect_one()) {
+        const int b = bh / p.H;
+        mbar_expect_tx(&bars->w_full[buf], kWBytes);
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(smem + (uint32_t)kOffW + buf * kWBytes), "l"(p.w + (size_t)b * p.w_batch + (size_t)(bh - b * p.H) * kD * 9),
+                       "r"(kWBytes), "r"(smem_u32(&bars->w_full[buf])) : "memory");
+      }
+      __syncwarp();
+    };
+    int issued_w = 1;
+    load_w(ti.bh, 0);
+    bool head_starts = true;
     for (int it = 0; it < ntiles; ++it) {
       const int sq = it % kNQ, b = it & 1, hb = nh & 1;
+      if (head_starts && ti.bh < bh_last) {            // the next head's kernels (their buffer: read at the start of the head before)
+        if (nh >= 1) {
+          ok = warp_wait(&bars->w_free[hb ^ 1], ((nh - 1) >> 1) & 1, &bars->abort_flag, p.status);
+          if (!ok) break;
+        }
+        load_w(ti.bh + 1, hb ^ 1);
+        ++issued_w;
+      }
       ok = warp_wait(&bars->relu_done[sq], (it / kNQ) & 1, &bars->abort_flag, p.status);
       if (ok && it >= 2) ok = warp_wait(&bars->d_empty[b], ((it >> 1) - 1) & 1, &bars->abort_flag, p.status);
       if (!ok) break;
       tc_fence_after();
-      const uint32_t qa = smem + sq * kTileBytes, kv = smem + (uint32_t)kOffKv + hb * kKvBytes;
+      const uint32_t kv = smem + (uint32_t)kOffKv + hb * kKvBytes, zt = smem + (uint32_t)kOffZt + hb * kZtBytes;
 #pragma unroll
-      for (int ks = 0; ks < kD / 16; ++ks)
-        mma_ss(tmem + b * kD, smem_desc(qa + ks * 32), smem_desc(kv + ks * 2048), kIdesc, ks > 0 ? 1u : 0u);
+      for (int ks = 0; ks < kD / 16; ++ks) {
+        mma_ts(tmem + b * kAccStride, tmem + b * kAccStride + kColA + 8 * ks, smem_desc(kv + ks * 2048), kIdesc, ks > 0 ? 1u : 0u);
+        mma_ts(tmem + b * kAccStride + kColZ, tmem + b * kAccStride + kColA + 8 * ks, smem_desc(zt + ks * 32), kIdescZ, ks > 0 ? 1u : 0u);
+      }
       tc_commit(&bars->d_full[b]);
-      const bool head_ends = ti.next(p.ncb, p.nrb);
-      if (head_ends) {                                 // the KV buffer may be rebuilt once these MMAs are complete
+      head_starts = ti.next(p.ncb, p.nrb);
+      if (head_starts) {                                 // the KV buffer may be rebuilt once these MMAs are complete
         tc_commit(&bars->kv_free[hb]);
         ++nh;
       }
+    }
+    if (!ok && lane == 0) {   // let the copies in flight land before the CTA leaves
+      const unsigned long long t0 = globaltimer();
+      for (int g = max(0, issued_w - 2); g < issued_w; ++g)
+        while (!mbar_try(&bars->w_full[g & 1], (g >> 1) & 1) && globaltimer() - t0 < kWaitLimitNs) {}
     }
   } else if (warp < 4) {
     // ================= rectifier warps: thread r = 32 warp + lane owns token row r of every tile =================
@@ -240,29 +288,33 @@ lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
     if (!ok) bars->abort_flag = 1;                     // an earlier kernel gave up: every role of this CTA falls through at once
     const int row = threadIdx.x;
     uint32_t wpar = 0;
+    for (int i = threadIdx.x; i < 2 * kZtBytes / 16; i += 128)        // (rows 3 .. 15 of both z operands stay zero)
+      *reinterpret_cast<uint4*>(smem_al + kOffZt + 16 * i) = make_uint4(0u, 0u, 0u, 0u);
+    asm volatile("bar.sync 1, 128;" ::: "memory");
     // Second pass of the state reduction for (batch, head) bh into KV / z buffer hb: the chunk
     // partials are summed in chunk order (no atomics: bit-reproducible); KV goes to shared memory as
-    // the bf16 MMA operand (128-byte swizzle), z stays fp32.  All loads of a chunk are in flight together.
+    // the bf16 MMA operand (128-byte swizzle), z as three bf16 terms (its 24 bits).  All loads of a chunk are in flight together.
     auto build_state = [&](int bh, int hb) {
       unsigned char* kv_ptr = smem_al + kOffKv + (size_t)hb * kKvBytes;
       const float* P = p.partial + (size_t)bh * p.nchunk * p.state_elems;
       float4 acc[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-      float zs = 0.f;
-      for (int k = 0; k < p.nchunk; ++k) {
-        const float* Pk = P + (size_t)k * p.state_elems;
-        float4 t[8];
+      auto load = [&](float4 (&t)[8], const float* Pk) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {                  // 16-byte chunk pairs tid, tid + 128, ... of the 64 x 64 matrix
           const float* src = Pk + (threadIdx.x + 128 * i) * 8;
           t[2 * i] = __ldcg(reinterpret_cast<const float4*>(src));
           t[2 * i + 1] = __ldcg(reinterpret_cast<const float4*>(src + 4));
         }
-        const float zk = threadIdx.x < kD ? __ldcg(Pk + kOffZ + threadIdx.x) : 0.f;
+      };
+      load(acc, P);
+      float zs = threadIdx.x < kD ? __ldcg(P + kOffZ + threadIdx.x) : 0.f;
+      for (int k = 1; k < p.nchunk; ++k) {
+        const float* Pk = P + (size_t)k * p.state_elems;
+        float4 t[8];
+        load(t, Pk);
+        if (threadIdx.x < kD) zs += __ldcg(Pk + kOffZ + threadIdx.x);
 #pragma unroll
         for (int j = 0; j < 8; ++j) { acc[j].x += t[j].x; acc[j].y += t[j].y; acc[j].z += t[j].z; acc[j].w += t[j].w; }
-        zs += zk;
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -274,7 +326,15 @@ lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
         pk.w = pack_bf16(acc[2 * i + 1].z, acc[2 * i + 1].w);
         *reinterpret_cast<uint4*>(kv_ptr + tile_off(c >> 3, c & 7)) = pk;
       }
-      if (threadIdx.x < kD) z_sm[hb * kD + threadIdx.x] = zs;
+      if (threadIdx.x < kD) {
+        unsigned char* zt = smem_al + kOffZt + (size_t)hb * kZtBytes + (threadIdx.x & 7) * 2;
+#pragma unroll
+        for (int n = 0; n < 3; ++n) {                  // the bf16 nearest to what the terms before it left over
+          const __nv_bfloat16 t = __float2bfloat16_rn(zs);
+          zs -= __bfloat162float(t);
+          *reinterpret_cast<__nv_bfloat16*>(zt + tile_off(n, threadIdx.x >> 3)) = t;
+        }
+      }
     };
     // all 128 rectifier threads: what they wrote is complete and visible to the tensor core
     auto workers_sync = [&]() -> bool {
@@ -316,28 +376,25 @@ lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
       }
       ok = warp_wait(&bars->q_full[sq], (it / kNQ) & 1, &bars->abort_flag, p.status);
       if (!ok) break;
-      {  // ReLU of this thread's row in place; its denominator relu(q).z exactly in fp32
-        unsigned char* q = smem_al + (size_t)sq * kTileBytes + row * 128;
-        const float* z = z_sm + hb * kD;
-        uint4 v[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) v[c] = *reinterpret_cast<const uint4*>(q + ((c ^ (row & 7)) << 4));
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      // ReLU of this thread's row, as the MMA's A operand into tensor memory (the buffer is free once the MMAs of the
+      // tile before the last are complete); the row's denominator relu(q).z comes from the tensor core, too
+      if (it >= 2) {
+        ok = warp_wait(&bars->d_full[it & 1], ((it >> 1) - 1) & 1, &bars->abort_flag, p.status);
+        if (!ok) break;
+        tc_fence_after();
+      }
+      {
+        const unsigned char* q = smem_al + (size_t)sq * kTileBytes + row * 128;
+        uint32_t v[32];
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-          v[c].x = relu_bf16x2(v[c].x); v[c].y = relu_bf16x2(v[c].y); v[c].z = relu_bf16x2(v[c].z); v[c].w = relu_bf16x2(v[c].w);
-          const float4 za = *reinterpret_cast<const float4*>(z + 8 * c), zb = *reinterpret_cast<const float4*>(z + 8 * c + 4);
-          const float2 f0 = bf16x2_to_f2(v[c].x), f1 = bf16x2_to_f2(v[c].y), f2 = bf16x2_to_f2(v[c].z), f3 = bf16x2_to_f2(v[c].w);
-          acc[0] = fmaf(f0.x, za.x, fmaf(f0.y, za.y, acc[0]));
-          acc[1] = fmaf(f1.x, za.z, fmaf(f1.y, za.w, acc[1]));
-          acc[2] = fmaf(f2.x, zb.x, fmaf(f2.y, zb.y, acc[2]));
-          acc[3] = fmaf(f3.x, zb.z, fmaf(f3.y, zb.w, acc[3]));
+          const uint4 x = *reinterpret_cast<const uint4*>(q + ((c ^ (row & 7)) << 4));
+          v[4 * c] = relu_bf16x2(x.x); v[4 * c + 1] = relu_bf16x2(x.y); v[4 * c + 2] = relu_bf16x2(x.z); v[4 * c + 3] = relu_bf16x2(x.w);
         }
-#pragma unroll
-        for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(q + ((c ^ (row & 7)) << 4)) = v[c];
-        den_sm[(it & (kDenRing - 1)) * 128 + row] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+        tmem_st32(tmem + ((uint32_t)(warp << 5) << 16) + (it & 1) * kAccStride + kColA, v);
+        tmem_wait_st();
       }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      tc_fence_before();
       mbar_arrive(&bars->relu_done[sq]);
       ++head_tile;
       if (ti.next(p.ncb, p.nrb)) { ++nh; head_tile = 0; }
@@ -349,18 +406,19 @@ lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
     bool ok = true;
     for (int it = 0; it < ntiles && ok; ++it) {
       const int sq = it % kNQ, b = it & 1;
-      // The tile's MMAs were issued after all 128 rectifier threads had published its rows and
-      // denominators, so the accumulator being complete means the denominators are in place; it
-      // also means that the tensor core is done reading the Q tile, which is overwritten below.
+      // The accumulator being complete also means that the tensor core is done reading the Q tile, which is
+      // overwritten below.
       ok = warp_wait(&bars->d_full[b], (it >> 1) & 1, &bars->abort_flag, p.status);
       if (!ok) break;
       tc_fence_after();
-      const float inv = 1.f / (den_sm[(it & (kDenRing - 1)) * 128 + row] + p.eps);
-      uint32_t v0[32], v1[32];
-      tmem_ld32(tmem + lane_base + b * kD, v0);
-      tmem_ld32(tmem + lane_base + b * kD + 32, v1);
+      uint32_t v0[32], v1[32], vz[4];
+      tmem_ld4(tmem + lane_base + b * kAccStride + kColZ, vz);
+      tmem_ld32(tmem + lane_base + b * kAccStride, v0);
+      tmem_ld32(tmem + lane_base + b * kAccStride + 32, v1);
       tmem_wait_ld(v0);
       tmem_wait_ld(v1);
+      asm volatile("" : "+r"(vz[0]), "+r"(vz[1]), "+r"(vz[2]));      // (no use of them ahead of the waits)
+      const float inv = 1.f / ((__uint_as_float(vz[0]) + __uint_as_float(vz[1])) + __uint_as_float(vz[2]) + p.eps);
       tc_fence_before();
       mbar_arrive(&bars->d_empty[b]);                  // the accumulator buffer may be overwritten
       unsigned char* st = smem_al + (size_t)sq * kTileBytes + row * 128;
@@ -386,32 +444,31 @@ lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
     const int cw = warp - kWarpConv0;
     const int rp = cw >> 1, c4 = lane & 15;
     const int xt = 8 * (cw & 1) + 4 * (lane >> 4);    // first of this lane's 4 token columns inside the patch
-    griddep_wait();                                    // the kernels w come from the grid before this one
     bool ok = true;
-    uint32_t wq[2][9];                                 // kernels of this lane's channels as bf16 pairs, [channel pair][tap]
+    int nh = 0;                                        // heads seen so far: buffer of the kernels
+    uint32_t wq[2][9];                                 // kernels of this lane's channels, [channel pair][tap]
     TileIter ti;
     ti.init(t_begin, p.ncb, p.nrb);
     bool new_head = true;
     for (int it = 0; it < ntiles && ok; ++it) {
       const int sq = it % kNQ, sv = it % kNV;
       if (new_head) {
-        const int b = ti.bh / p.H, h = ti.bh - b * p.H;
-        const float4* wp = reinterpret_cast<const float4*>(p.w + (size_t)b * p.w_batch + ((size_t)h * kD + 4 * c4) * 9);
+        ok = warp_wait(&bars->w_full[nh & 1], (nh >> 1) & 1, &bars->abort_flag, p.status);
+        if (!ok) break;
+        const float4* wp = reinterpret_cast<const float4*>(smem_al + kOffW + (size_t)(nh & 1) * kWBytes + c4 * 144);
         float wf[36];                                  // [channel][tap] as stored
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-          const float4 t4 = __ldcg(wp + k);   // written by the grid before this one: read through L2
+          const float4 t4 = wp[k];
           wf[4 * k] = t4.x; wf[4 * k + 1] = t4.y; wf[4 * k + 2] = t4.z; wf[4 * k + 3] = t4.w;
         }
 #pragma unroll
         for (int pr = 0; pr < 2; ++pr)
 #pragma unroll
           for (int tap = 0; tap < 9; ++tap) wq[pr][tap] = pack_bf16(wf[9 * (2 * pr) + tap], wf[9 * (2 * pr + 1) + tap]);
-        if (h + 1 < p.H) {        // the kernels of the head after this one: into L2 ahead of the switch
-          const float* wn = reinterpret_cast<const float*>(wp) + kD * 9;
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(wn));
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(wn + 32));
-        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->w_free[nh & 1]);
+        ++nh;
       }
       ok = warp_wait(&bars->v_full[sv], (it / kNV) & 1, &bars->abort_flag, p.status);
       if (ok) ok = warp_wait(&bars->la_done[sq], (it / kNQ) & 1, &bars->abort_flag, p.status);
