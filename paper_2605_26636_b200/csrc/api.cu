@@ -148,17 +148,22 @@ jv_status run_attn(const void* q, const void* k, const void* v, void* o, const j
   if (!g_force_generic.load() && !one_window && attn_w4_supported(a)) {
     int* status = device_status_ptr();
     if (!status) return JV_ERR_CUDA;
-    const jv_status r = from_cuda(launch_attn_w4(a, status, st));
-    if (r != JV_OK || a.P == 0) return r;
-    return from_cuda(launch_attn_generic(a, st, true));   // the P prefix queries, which attend everything
+    if (a.P > 0) {                                        // the P prefix queries, which attend everything
+      const int free_sms = device_sm_count() - attn_w4_ctas(a);
+      const jv_status r = from_cuda(launch_attn_prefix(a, free_sms > 0 ? free_sms : 2 * device_sm_count(), st));
+      if (r != JV_OK) return r;
+    }
+    return from_cuda(launch_attn_w4(a, status, st));
   }
   if (!g_force_generic.load() && attn_tc_supported(a, full)) {
     int* status = device_status_ptr();
     if (!status) return JV_ERR_CUDA;
     if (a.strided && a.P > 0) return JV_ERR_UNSUPPORTED;  // the prefix queries' kernel reads contiguous tensors
-    const jv_status r = from_cuda(launch_attn_tc(a, full, status, st));
-    if (r != JV_OK || a.P == 0) return r;
-    return from_cuda(launch_attn_generic(a, st, true));   // the P prefix queries, which attend everything
+    if (a.P > 0) {
+      const jv_status r = from_cuda(launch_attn_prefix(a, 2 * device_sm_count(), st));
+      if (r != JV_OK) return r;
+    }
+    return from_cuda(launch_attn_tc(a, full, status, st));
   }
   if (a.strided) return JV_ERR_UNSUPPORTED;               // the fp32 and generic kernels read contiguous tensors
   if (!g_force_generic.load() && attn_f32_supported(a)) return from_cuda(launch_attn_f32(a, st));

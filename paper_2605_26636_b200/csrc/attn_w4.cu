@@ -32,7 +32,7 @@
 // check one step into their next item, off the critical path.
 //
 // Measured (8 x 16 heads, 64 x 64 tokens, 16 x 16 windows, back to back): 66.7 us = 4.0 TB/s; with five prefix tokens (their
-// queries' kernel included) 109 us.  With one Q buffer per tile, K and V in whole tiles and the output staged over V it was 71.0
+// queries' kernel, then 41.5 us, included) 109 us.  With one Q buffer per tile, K and V in whole tiles and the output staged over V it was 71.0
 // and 118.9: a window's Q could only be copied once the window before had issued its last scores, and there was no
 // room for a third V stage beside the prefix rows.  32 x 12 heads, 16 x 16 tokens, 8 x 8 windows: 20 us less than on attn_tc.cu, where
 // half of a tile's rows, and half of the exponentials of the rest, are of no use.
@@ -156,10 +156,6 @@ attn_w4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   Barriers* bar = reinterpret_cast<Barriers*>(smem + kSmemTiles + Layout<kPrefix>::kPre);
   const uint32_t sQ = smem_u32(smem), sK = sQ + kQT * 2 * kTileBytes, sV = sK + kSlots * kKS * kSubBytes;
   const uint32_t sPre = sQ + (uint32_t)kSmemTiles;   // slot s: prefix rows of K at s * 4 KB, of V 2 KB behind them
-
-  // a grid launched behind this one with programmatic serialisation (the prefix queries of W, which
-  // depend on nothing here) may run beside it
-  if (kPrefix) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
@@ -616,6 +612,8 @@ attn_w4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   }
 
   // ================= common teardown =================
+  // with prefix tokens this launch overlaps the one ahead of it (their queries) and must not end before it
+  if (kPrefix) asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncwarp();
   tc_fence_before();
   __syncthreads();
@@ -641,6 +639,17 @@ bool attn_w4_supported(const AttnArgs& a) {
   return encode_fn() != nullptr;
 }
 
+// CTAs of a launch.  Fewer items than SMs: one to a CTA.  With prefix tokens and less than a wave of items, both slots of
+// half as many CTAs work, if that leaves the prefix queries' launch SMs of its own: the two run side by side (42 heads
+// of 28 x 28 tokens: 16.5 us; behind one another, with the items over all SMs, 20.9).
+int attn_w4_ctas(const AttnArgs& a) {
+  const int box_w = a.ww * a.wh == 64 ? 2 * a.ww : a.ww, box_h = kTile / box_w;
+  const int64_t total = (int64_t)ceil_div(a.Wg, box_w) * ceil_div(a.Hg, 2 * box_h) * a.BH;
+  const int sms = device_sm_count();
+  if (a.P > 0 && total <= kSlots * sms && total + a.BH > sms) return (int)((total + kSlots - 1) / kSlots);
+  return (int)(total < sms ? total : sms);
+}
+
 template <bool kPrefix, int kWpt>
 cudaError_t launch_w4(const CUtensorMap (&maps)[6], const W4Params& p, int grid, cudaStream_t st) {
   static OncePerDevice smem_opt_in;   // > 48 KB of dynamic shared memory: a per-device function attribute
@@ -649,10 +658,19 @@ cudaError_t launch_w4(const CUtensorMap (&maps)[6], const W4Params& p, int grid,
                                 (int)Layout<kPrefix>::kBytes);
   });
   if (e != cudaSuccess) return e;
-  attn_w4_kernel<kPrefix, kWpt><<<grid, kThreads, Layout<kPrefix>::kBytes, st>>>(maps[0], maps[1], maps[2], maps[3], maps[4],
-                                                                                 maps[5], p);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = Layout<kPrefix>::kBytes;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = kPrefix ? 1 : 0;                      // the prefix queries' launch is right ahead of this one
+  const cudaError_t r = cudaLaunchKernelEx(&cfg, attn_w4_kernel<kPrefix, kWpt>, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], p);
   count_launch();
-  return cudaGetLastError();
+  return r;
 }
 
 cudaError_t launch_attn_w4(const AttnArgs& a, int* status, cudaStream_t st) {
@@ -721,8 +739,7 @@ cudaError_t launch_attn_w4(const AttnArgs& a, int* status, cudaStream_t st) {
   p.H = a.H;
   p.div_H = make_fastdiv((uint32_t)a.H);
   p.scale_log2 = a.scale * 1.4426950408889634f;
-  const int num_sms = device_sm_count();
-  const int grid = p.total < num_sms ? p.total : num_sms;   // fewer items than SMs: one to a CTA
+  const int grid = attn_w4_ctas(a);
   if (a.P > 0)
     return wpt == 0 ? launch_w4<true, 0>(maps, p, grid, st) : wpt == 1 ? launch_w4<true, 1>(maps, p, grid, st) : launch_w4<true, 2>(maps, p, grid, st);
   return wpt == 0 ? launch_w4<false, 0>(maps, p, grid, st) : wpt == 1 ? launch_w4<false, 1>(maps, p, grid, st) : launch_w4<false, 2>(maps, p, grid, st);

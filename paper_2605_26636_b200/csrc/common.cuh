@@ -111,7 +111,10 @@ struct AttnArgs {
   float scale;
   int dtype;
 };
-cudaError_t launch_attn_generic(const AttnArgs& a, cudaStream_t st, bool prefix_rows_only = false);
+cudaError_t launch_attn_generic(const AttnArgs& a, cudaStream_t st);
+// the P prefix queries of window attention on their own, ahead of the launch of the windows, in at most `ctas` blocks where
+// that can be (bf16, D == 64, contiguous)
+cudaError_t launch_attn_prefix(const AttnArgs& a, int ctas, cudaStream_t st);
 // fp32 tensors at D == 64: register-tiled fp32 kernel (full and windowed attention, prefix tokens)
 bool attn_f32_supported(const AttnArgs& a);
 cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st);
@@ -121,6 +124,7 @@ bool attn_tc_supported(const AttnArgs& a, bool full);
 cudaError_t launch_attn_tc(const AttnArgs& a, bool full, int* status, cudaStream_t st);
 // tcgen05 path for windows of one or two 128-token tiles (bf16, D == 64, at most 16 prefix tokens): two windows per CTA
 bool attn_w4_supported(const AttnArgs& a);
+int attn_w4_ctas(const AttnArgs& a);   // CTAs (one per SM) of its launch
 cudaError_t launch_attn_w4(const AttnArgs& a, int* status, cudaStream_t st);
 // tcgen05 path at head_dim 128 (bf16, N >= 128, no prefix tokens in W): two query tiles per CTA.
 // full = true: F over all N tokens; else W with windows whose width is a power of two <= 128
