@@ -7,13 +7,20 @@
 //   out:  o [B, H, N, 64]  times  w [C, C]^T  ->  y [B, N, C]
 //         input feature h * 64 + e: one K block of 64 is one head of o
 //
-// One persistent CTA per SM loops over output tiles of 128 tokens x 256 features (feature
-// tile fastest, so the CTAs that run together share their token tile in L2 and the weights
-// stay L2-resident).  Warp roles:
-//   warp 0      TMA producer: A (128 tokens x 64) and B (256 features x 64) through a 4-stage ring
-//   warp 1      MMA issuer: 4 x tcgen05.mma M128 N256 K16 per stage into one of two
-//               accumulators in tensor memory (2 x 256 columns)
-//   warps 4-7   epilogue of the other accumulator: tensor memory -> registers, + bias, bf16,
+// One persistent CTA per SM loops over output tiles of 128 tokens x 256 features, or a pair of CTAs over tiles of 2 x 128 x 256
+// (template parameter kCtas; feature tile fastest, so what runs together shares its token tiles in L2 and the weights stay
+// L2-resident).  In a pair tcgen05.mma runs in its two-SM form (cta_group::2, M 256, N 256): each CTA holds one of the two token
+// tiles, which need not be neighbours, half of the tile's weights, and the accumulator rows of its own tokens.
+// What bounds a tile of one CTA is not the tensor pipe but shared memory: a K block of 64 is 48 KB written by the copies
+// and 48 KB read by the MMAs, 768 clocks for 512 clocks of MMA; with the weights shared by two CTAs it is 32 + 32 KB.
+// Measured (2 x 8192 tokens, 768 -> 2304 / 8 x 4096 tokens, 1024 -> 3072 features): 46.2 / 138 us = 1254 / 1493 TF in pairs,
+// 49.7 / 153 us singly; with four epilogue warps instead of eight and the bias fetched after the accumulator, 53.4 / 152.
+// Warp roles (both CTAs of a pair):
+//   warp 0      TMA producer: A (128 tokens x 64) and (half of) B (256 features x 64) through a ring of 4 (5) stages; the
+//               copies of both CTAs report to the leader's barrier
+//   warp 1      (leader, the even CTA) MMA issuer: 4 x tcgen05.mma K16 per stage into one of two
+//               accumulators in tensor memory (2 x 256 columns in each CTA); its commits arrive in both CTAs
+//   warps 4-11  epilogue of the other accumulator, two warps per tensor-memory quadrant: tensor memory -> registers, + bias, bf16,
 //               swizzled staging in shared memory, one TMA store per warp and 64-feature block
 // Token tiles never cross a batch element: rows past N are zero-filled on load and clipped on
 // store by TMA; feature blocks past the last one are skipped.
@@ -28,44 +35,55 @@ namespace {
 using namespace tc;
 
 constexpr int kD = 64;                       // head_dim = K block = feature block
-constexpr int kBM = 128;                     // tokens per tile
+constexpr int kBM = 128;                     // tokens per CTA and tile
 constexpr int kBN = 256;                     // features per tile
 constexpr int kABytes = kBM * kD * 2;        // 16 KB
-constexpr int kBBytes = kBN * kD * 2;        // 32 KB
-constexpr int kStageBytes = kABytes + kBBytes;
-constexpr int kStages = 4;
-constexpr int kThreads = 256;
+constexpr int kEpiWarps = 8;                 // two per tensor-memory quadrant, each with half of the tile's features
+constexpr int kThreads = (4 + kEpiWarps) * 32;
 constexpr uint32_t kTmemCols = 512;
 constexpr int kStagingBytes = 32 * kD * 2;   // one warp's 32 tokens x 64 features
+constexpr int kMaxStages = 5;
 
+// kCtas: CTAs per tile, 1 or 2 (a pair)
+template <int kCtas>
+struct Layout {
+  static constexpr int kBBytes = kBN / kCtas * kD * 2;             // this CTA's part of the features
+  static constexpr int kStageBytes = kABytes + kBBytes;
+  static constexpr int kStages = kCtas == 2 ? 5 : 4;
+  static constexpr int kBufs = kCtas == 2 ? 2 : 1;                 // staging buffers per epilogue warp
+  static constexpr size_t kTiles = (size_t)kStages * kStageBytes + (size_t)kEpiWarps * kBufs * kStagingBytes;
+};
 struct __align__(8) Barriers {
-  uint64_t full[kStages], empty[kStages];
+  uint64_t full[kMaxStages], empty[kMaxStages];    // full, acc_empty: the leader's count for the pair
   uint64_t acc_full[2], acc_empty[2];
   uint64_t drain;
   uint32_t tmem_base;
   volatile uint32_t abort_flag;
 };
-constexpr size_t kSmemTiles = (size_t)kStages * kStageBytes + 4 * 2 * kStagingBytes;
-constexpr size_t kSmemBytes = kSmemTiles + sizeof(Barriers) + 1024;
+template <int kCtas>
+constexpr size_t smem_bytes() { return Layout<kCtas>::kTiles + sizeof(Barriers) + 1024; }
+static_assert(smem_bytes<1>() <= 232448 && smem_bytes<2>() <= 232448, "shared memory of one CTA");
 
 struct ProjParams {
   const float* bias;       // [features] or nullptr
+  int bias_vec;            // bias is 16-byte aligned
   int* status;
   int tiles_m_per_batch;   // ceil(N / 128)
   int tiles_n;             // ceil(features / 256)
-  int total_tiles;         // B * tiles_m_per_batch * tiles_n
+  int tiles_m;             // B * tiles_m_per_batch
+  int total_tiles;         // ceil(tiles_m / 2) * tiles_n: tiles of a pair of CTAs
   int kblocks;             // C / 64
   int H;                   // heads
   int fblocks;             // features / 64
   int N;                   // tokens per batch element
   int silu;                // 1: x / (1 + exp(-x)) on the result (the kernel generator's hidden layer)
   int out_f16;             // 1: the result is stored as fp16 instead of bf16 (same size; the generator's intermediates)
-  uint32_t idesc;          // instruction descriptor: M128 N256, both operands K-major, bf16 or fp16 operands
+  uint32_t idesc;          // instruction descriptor: bf16 or fp16 operands
 };
 
-// Instruction descriptor: M128 N256, both operands K-major; bf16 operands, or fp16 ones (format 0 in both fields)
-constexpr uint32_t kIdesc = idesc(kBM, kBN, 0);
-constexpr uint32_t kIdescF16 = kIdesc & ~((1u << 7) | (1u << 10));
+// Instruction descriptors: M128 (one CTA) or M256 (a pair) x N256, both operands K-major; bf16 operands, or fp16 ones (format 0 in both fields)
+constexpr uint32_t kIdesc1 = idesc(kBM, kBN, 0), kIdesc2 = idesc(2 * kBM, kBN, 0);
+constexpr uint32_t kIdescF16Mask = ~((1u << 7) | (1u << 10));
 __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
   uint32_t r;
   asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
@@ -73,17 +91,50 @@ __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
 }
 
 struct Tile {
-  int b, tok0, f0;   // batch element, first token, first feature
+  int b, tok0, f0;   // batch element, this CTA's first token (N: it has no tile, an odd one out), first feature
 };
-__device__ __forceinline__ Tile decode_tile(const ProjParams& p, int i) {
-  const int tn = i % p.tiles_n, r = i / p.tiles_n;
-  const int tm = r % p.tiles_m_per_batch, b = r / p.tiles_m_per_batch;
+template <int kCtas>
+__device__ __forceinline__ Tile decode_tile(const ProjParams& p, int i, int rank) {
+  const int tn = i % p.tiles_n, m = kCtas * (i / p.tiles_n) + rank;
+  if (m >= p.tiles_m) return Tile{0, p.N, tn * kBN};
+  const int tm = m % p.tiles_m_per_batch, b = m / p.tiles_m_per_batch;
   return Tile{b, tm * kBM, tn * kBN};
 }
 
+// ---- one CTA, or the two-SM forms, whose addresses are of the cluster's shared memory -----------------------------------
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2) {
+  asm volatile("cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+               ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2) : "memory");
+}
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
+  asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+               ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1) : "memory");
+}
+__device__ __forceinline__ void mma_ss_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
+}
+// arrives on the barrier (at this offset in both CTAs of a pair) once the MMAs issued so far are complete
+template <bool kPair>
+__device__ __forceinline__ void commit(uint64_t* bar) {
+  if (!kPair) tc_commit(bar);
+  else if (elect_one())
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
 // kQKV: A = x as (C, N, B), outputs q, k, v as (64, N, B*H); else A = o as (64, N, B*H),
 // output y as (C, N, B).  B (the weights) is (C, features) in both.
-template <bool kQKV>
+template <bool kQKV, int kCtas>
 __global__ void __launch_bounds__(kThreads, 1)
 proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                const __grid_constant__ CUtensorMap mapD0, const __grid_constant__ CUtensorMap mapD1,
@@ -91,16 +142,15 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
   extern __shared__ unsigned char smem_raw[];
   // 1024-byte alignment by an offset from the array itself, so that accesses stay shared-space loads and stores
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  Barriers* bar = reinterpret_cast<Barriers*>(smem + kSmemTiles);
+  using L = Layout<kCtas>;
+  constexpr int kStages = L::kStages, kStageBytes = L::kStageBytes, kBufs = L::kBufs;
+  constexpr bool kPair = kCtas == 2;
+  Barriers* bar = reinterpret_cast<Barriers*>(smem + L::kTiles);
   const uint32_t sRing = smem_u32(smem), sStage = sRing + kStages * kStageBytes;
 
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
-  // a timeout flagged earlier (by any CTA or launch) makes the rest leave at once
-  if (threadIdx.x == 0) bar->tmem_base = *reinterpret_cast<volatile int*>(p.status);
-  __syncthreads();
-  if (bar->tmem_base != 0) return;
-  __syncthreads();
+  const int rank = kPair ? blockIdx.x & 1 : 0;   // in the pair: 0 leads
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -109,25 +159,47 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&bar->acc_full[a], 1);
-      mbar_init(&bar->acc_empty[a], 4);      // lane 0 of each epilogue warp
+      mbar_init(&bar->acc_empty[a], kCtas * kEpiWarps);      // lane 0 of each epilogue warp
     }
     mbar_init(&bar->drain, 1);
-    bar->abort_flag = 0;
+    // a timeout flagged earlier (by any CTA or launch) makes the rest leave at once: as the leader sees it, for both CTAs
+    bar->abort_flag = *reinterpret_cast<volatile int*>(p.status) != 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  uint32_t gave_up;
+  if (kPair) {
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(gave_up) : "r"(map_rank(smem_u32((const void*)&bar->abort_flag), 0)) : "memory");
+    cluster_arrive();                        // (the leader may not leave or raise its flag before the other CTA has read it)
+    cluster_wait();
+  } else {
+    __syncthreads();
+    gave_up = bar->abort_flag;
+    __syncthreads();
+  }
+  if (gave_up) return;
+  if (kPair && threadIdx.x == 0) bar->abort_flag = 0;
   if (warp == 0) {
     __syncwarp();
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bar->tmem_base)),
-                 "r"(kTmemCols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if (kPair) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bar->tmem_base)),
+                   "r"(kTmemCols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bar->tmem_base)),
+                   "r"(kTmemCols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bar->tmem_base, 0);
 
-  const int tile0 = blockIdx.x, tile_step = gridDim.x;
+  const int tile0 = blockIdx.x / kCtas, tile_step = gridDim.x / kCtas;
 
   if (warp == 0) {
     // ================= TMA producer =================
@@ -135,16 +207,22 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     int s = 0, issued = 0;
     uint32_t par = 1;
     for (int i = tile0; i < p.total_tiles && ok; i += tile_step) {
-      const Tile t = decode_tile(p, i);
+      const Tile t = decode_tile<kCtas>(p, i, rank);
       for (int kb = 0; kb < p.kblocks; ++kb) {
         ok = warp_wait(&bar->empty[s], par, &bar->abort_flag, p.status);
         if (!ok) break;
         if (elect_one()) {
           const uint32_t dst = sRing + s * kStageBytes;
-          mbar_expect_tx(&bar->full[s], kStageBytes);
-          if (kQKV) tma_load_3d(dst, &mapA, &bar->full[s], kb * kD, t.tok0, t.b);
-          else tma_load_3d(dst, &mapA, &bar->full[s], 0, t.tok0, t.b * p.H + kb % p.H);   // (more K blocks than planes: A repeats)
-          tma_load_2d(dst + kABytes, &mapB, &bar->full[s], kb * kD, t.f0);
+          const int a0 = kQKV ? kb * kD : 0, a2 = kQKV ? t.b : t.b * p.H + kb % p.H;   // (more K blocks than planes: A repeats)
+          if (rank == 0) mbar_expect_tx(&bar->full[s], kCtas * kStageBytes);           // what both CTAs' copies bring
+          if (kPair) {
+            const uint32_t full = map_rank(smem_u32(&bar->full[s]), 0);
+            tma_load_3d_pair(dst, &mapA, full, a0, t.tok0, a2);
+            tma_load_2d_pair(dst + kABytes, &mapB, full, kb * kD, t.f0 + rank * (kBN / 2));
+          } else {
+            tma_load_3d(dst, &mapA, &bar->full[s], a0, t.tok0, a2);
+            tma_load_2d(dst + kABytes, &mapB, &bar->full[s], kb * kD, t.f0);
+          }
         }
         __syncwarp();
         ++issued;
@@ -152,13 +230,14 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
       }
     }
     if (!ok && lane == 0) {
-      // let the copies still in flight land before the CTA leaves (bounded by the same limit)
+      // let the copies still in flight land before the CTA leaves (bounded by the same limit; the leader's barriers tell)
       const unsigned long long t0 = globaltimer();
-      for (int g = max(0, issued - kStages); g < issued; ++g)
+      for (int g = max(0, issued - kStages); g < issued && rank == 0; ++g)
         while (!mbar_try(&bar->full[g % kStages], (g / kStages) & 1) && globaltimer() - t0 < kWaitLimitNs) {}
+      while (rank != 0 && globaltimer() - t0 < 1000000ull) {}
     }
-  } else if (warp == 1) {
-    // ================= MMA issuer =================
+  } else if (warp == 1 && rank == 0) {
+    // ================= MMA issuer (of the pair) =================
     bool ok = true;
     int s = 0, n = 0;
     uint32_t ph = 0;
@@ -173,16 +252,21 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         if (!ok) break;
         tc_fence_after();
         const uint32_t sa = sRing + s * kStageBytes, sb = sa + kABytes;
+        if (elect_one()) {
+          const uint64_t da = smem_desc(sa), db = smem_desc(sb);
 #pragma unroll
-        for (int ks = 0; ks < kD / 16; ++ks)
-          mma_ss(d, smem_desc(sa + ks * 32), smem_desc(sb + ks * 32), p.idesc, (kb > 0 || ks > 0) ? 1u : 0u);
-        tc_commit(&bar->empty[s]);
+          for (int ks = 0; ks < kD / 16; ++ks)
+            if (kPair) mma_ss_pair(d, desc_advance(da, ks * 32), desc_advance(db, ks * 32), p.idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+            else mma_ss_1(d, desc_advance(da, ks * 32), desc_advance(db, ks * 32), p.idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+        }
+        __syncwarp();
+        commit<kPair>(&bar->empty[s]);
         if (++s == kStages) { s = 0; ph ^= 1; }
       }
-      if (ok) tc_commit(&bar->acc_full[a]);
+      if (ok) commit<kPair>(&bar->acc_full[a]);
     }
     // every MMA issued so far must have retired before tensor memory is released
-    tc_commit(&bar->drain);
+    commit<kPair>(&bar->drain);
     if (lane == 0) {
       const unsigned long long t0 = globaltimer();
       while (!mbar_try(&bar->drain, 0) && globaltimer() - t0 < kWaitLimitNs) {}
@@ -190,21 +274,21 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     __syncwarp();
   } else if (warp >= 4) {
     // ================= epilogue: one thread per token row =================
-    const int q4 = warp & 3;
+    const int q4 = warp & 3, half = (warp - 4) >> 2;   // the warp's tensor-memory quadrant; which half of the tile's features
     const uint32_t lane_base = (uint32_t)(q4 << 5) << 16;
-    unsigned char* stage_ptr = smem + kStages * kStageBytes + q4 * 2 * kStagingBytes;
-    const uint32_t stage_u32 = sStage + q4 * 2 * kStagingBytes;
+    unsigned char* stage_ptr = smem + kStages * kStageBytes + (warp - 4) * kBufs * kStagingBytes;
+    const uint32_t stage_u32 = sStage + (warp - 4) * kBufs * kStagingBytes;
     bool ok = true;
     int n = 0, nstore = 0;
     for (int i = tile0; i < p.total_tiles && ok; i += tile_step, ++n) {
-      const Tile t = decode_tile(p, i);
+      const Tile t = decode_tile<kCtas>(p, i, rank);
       const int a = n & 1;
       ok = warp_wait(&bar->acc_full[a], (n >> 1) & 1, &bar->abort_flag, p.status);
       if (!ok) break;
       tc_fence_after();
       const int tok = t.tok0 + 32 * q4;
 #pragma unroll 1
-      for (int j = 0; j < kBN / kD; ++j) {
+      for (int j = 2 * half; j < 2 * half + 2; ++j) {
         const int fb = t.f0 / kD + j;
         if (fb >= p.fblocks || tok >= p.N) break;   // no such features / none of this warp's rows exists
         uint32_t ob[32];
@@ -212,41 +296,37 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         for (int c = 0; c < 2; ++c) {
           uint32_t v[32];
           tmem_ld32(tmem + lane_base + a * kBN + j * kD + c * 32, v);
+          float4 bb[8];                       // the bias, on its way beside the accumulator
+#pragma unroll
+          for (int i4 = 0; i4 < 8; ++i4) {
+            const float* bp = p.bias + fb * kD + c * 32 + 4 * i4;
+            bb[i4] = !p.bias ? make_float4(0.f, 0.f, 0.f, 0.f)
+                     : p.bias_vec ? __ldg(reinterpret_cast<const float4*>(bp))
+                                  : make_float4(__ldg(bp), __ldg(bp + 1), __ldg(bp + 2), __ldg(bp + 3));
+          }
           tmem_wait_ld(v);
+#pragma unroll
+          for (int i4 = 0; i4 < 8; ++i4) {
+            v[4 * i4] = __float_as_uint(__uint_as_float(v[4 * i4]) + bb[i4].x);
+            v[4 * i4 + 1] = __float_as_uint(__uint_as_float(v[4 * i4 + 1]) + bb[i4].y);
+            v[4 * i4 + 2] = __float_as_uint(__uint_as_float(v[4 * i4 + 2]) + bb[i4].z);
+            v[4 * i4 + 3] = __float_as_uint(__uint_as_float(v[4 * i4 + 3]) + bb[i4].w);
+          }
           if (p.silu) {
 #pragma unroll
             for (int i2 = 0; i2 < 32; ++i2) {
-              const float z = __uint_as_float(v[i2]) + (p.bias ? __ldg(p.bias + fb * kD + c * 32 + i2) : 0.f);
+              const float z = __uint_as_float(v[i2]);
               v[i2] = __float_as_uint(z / (1.f + __expf(-z)));
             }
-#pragma unroll
-            for (int i2 = 0; i2 < 16; ++i2)
-              ob[16 * c + i2] = p.out_f16 ? pack_f16(__uint_as_float(v[2 * i2]), __uint_as_float(v[2 * i2 + 1]))
-                                          : pack_bf16(__uint_as_float(v[2 * i2]), __uint_as_float(v[2 * i2 + 1]));
-          } else if (p.out_f16) {
-#pragma unroll
-            for (int i2 = 0; i2 < 16; ++i2) {
-              const float b0 = p.bias ? __ldg(p.bias + fb * kD + c * 32 + 2 * i2) : 0.f;
-              const float b1 = p.bias ? __ldg(p.bias + fb * kD + c * 32 + 2 * i2 + 1) : 0.f;
-              ob[16 * c + i2] = pack_f16(__uint_as_float(v[2 * i2]) + b0, __uint_as_float(v[2 * i2 + 1]) + b1);
-            }
-          } else if (p.bias) {
-            const float4* b4 = reinterpret_cast<const float4*>(p.bias + fb * kD + c * 32);
-#pragma unroll
-            for (int i4 = 0; i4 < 8; ++i4) {
-              const float4 bb = __ldg(b4 + i4);
-              ob[16 * c + 2 * i4] = pack_bf16(__uint_as_float(v[4 * i4]) + bb.x, __uint_as_float(v[4 * i4 + 1]) + bb.y);
-              ob[16 * c + 2 * i4 + 1] = pack_bf16(__uint_as_float(v[4 * i4 + 2]) + bb.z, __uint_as_float(v[4 * i4 + 3]) + bb.w);
-            }
-          } else {
-#pragma unroll
-            for (int i2 = 0; i2 < 16; ++i2)
-              ob[16 * c + i2] = pack_bf16(__uint_as_float(v[2 * i2]), __uint_as_float(v[2 * i2 + 1]));
           }
+#pragma unroll
+          for (int i2 = 0; i2 < 16; ++i2)
+            ob[16 * c + i2] = p.out_f16 ? pack_f16(__uint_as_float(v[2 * i2]), __uint_as_float(v[2 * i2 + 1]))
+                                        : pack_bf16(__uint_as_float(v[2 * i2]), __uint_as_float(v[2 * i2 + 1]));
         }
-        // the store issued two blocks ago must have finished reading this staging buffer
-        const int sbuf = nstore & 1;
-        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+        // the store that last used this staging buffer must have finished reading it
+        const int sbuf = kBufs == 2 ? nstore & 1 : 0;
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kBufs - 1) : "memory");
         __syncwarp();
 #pragma unroll
         for (int c = 0; c < 8; ++c)     // 16-byte chunk c of this row, at its 128-byte-swizzle position
@@ -270,7 +350,12 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
       // this accumulator may be overwritten once all four warps have read it
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bar->acc_empty[a]);
+      if (lane == 0) {
+        if (kPair)
+          asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(map_rank(smem_u32(&bar->acc_empty[a]), 0)) : "memory");
+        else
+          mbar_arrive(&bar->acc_empty[a]);
+      }
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   }
@@ -278,10 +363,17 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
   // ================= common teardown =================
   __syncwarp();
   tc_fence_before();
-  __syncthreads();
+  if (kPair) {
+    cluster_arrive();                        // neither CTA leaves, or frees tensor memory, while the other's commits and arrivals may come
+    cluster_wait();
+  } else {
+    __syncthreads();
+  }
   tc_fence_after();
-  if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  if (warp == 0) {
+    if (kPair) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  }
 }
 
 // ---- host side ----------------------------------------------------------------------
@@ -310,15 +402,57 @@ bool map2(CUtensorMap* m, const void* ptr, uint64_t inner, uint64_t rows, uint32
 
 bool proj_tc_available() { return encode_fn() != nullptr; }
 
-static cudaError_t proj_opt_in() {   // > 48 KB of dynamic shared memory: a per-device function attribute
-  static OncePerDevice once;
-  return once.run([] {
-    cudaError_t r = cudaFuncSetAttribute(proj_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-    if (r == cudaSuccess)
-      r = cudaFuncSetAttribute(proj_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-    return r;
+namespace {
+
+template <bool kQKV, int kCtas>
+cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& md0, const CUtensorMap& md1, const CUtensorMap& md2,
+                   const ProjParams& p, cudaStream_t st) {
+  static OncePerDevice opt_in;   // > 48 KB of dynamic shared memory: a per-device function attribute
+  cudaError_t e = opt_in.run([] {
+    return cudaFuncSetAttribute(proj_tc_kernel<kQKV, kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<kCtas>());
   });
+  if (e != cudaSuccess) return e;
+  const int slots = device_sm_count() / kCtas;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kCtas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kCtas * (p.total_tiles < slots ? p.total_tiles : slots));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem_bytes<kCtas>();
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = kCtas == 2 ? 1 : 0;
+  e = cudaLaunchKernelEx(&cfg, proj_tc_kernel<kQKV, kCtas>, ma, mb, md0, md1, md2, p);
+  count_launch();
+  return e;
 }
+
+// Pairs of CTAs where every pair has three tiles or more: a pair takes 2 us longer to start (cluster launch, two cluster
+// barriers) and a tile of it is a tenth faster or more.  Measured, single / pair: 30 tiles of a pair 9.1 / 11.1 us, 54: 15.3 / 17.3,
+// 96: 18.9 / 20.9, 192: 23.0 / 23.0, 288: 33.2 / 33.2, 576: 49.7 / 46.2, 512 of 16 K blocks: 57.5 / 53.1, 1536: 153 / 138.
+bool pair_tiles(int64_t tiles_m, int tiles_n) {
+  return (tiles_m + 1) / 2 * tiles_n >= 3 * (device_sm_count() / 2);
+}
+
+// Fills in what depends on the problem's size; false if there are too many tiles.
+bool plan(ProjParams& p, bool pair, int B, int N, int features, int kblocks, bool f16) {
+  const int ctas = pair ? 2 : 1;
+  p.tiles_m_per_batch = ceil_div(N, kBM);
+  p.tiles_n = ceil_div(features, kBN);
+  p.tiles_m = B * p.tiles_m_per_batch;
+  const int64_t total = (int64_t)ceil_div(p.tiles_m, ctas) * p.tiles_n;
+  p.total_tiles = (int)total;
+  p.kblocks = kblocks;
+  p.fblocks = features / kD;
+  p.N = N;
+  p.idesc = (pair ? kIdesc2 : kIdesc1) & (f16 ? kIdescF16Mask : ~0u);
+  return total <= 0x7fffffffll;
+}
+
+}  // namespace
 
 // The kernel on its own terms (see common.cuh).  kQKV of the kernel means "A is [B, N, K]" for the loads
 // and "D is planes" for the stores, which go together in the two projections; the other two
@@ -330,34 +464,21 @@ cudaError_t launch_proj_gemm(bool planes_in, bool planes_out, const void* A, con
                              cudaStream_t st) {
   if (!encode_fn() || planes_in == planes_out || F % kD != 0) return cudaErrorNotSupported;
   const uint64_t K = (uint64_t)kblocks * kD;
+  const bool pair = pair_tiles((int64_t)B * ceil_div(N, kBM), ceil_div(F, kBN));
   CUtensorMap ma, mb, md;
-  bool ok = map2(&mb, W, K, (uint64_t)F, kBN);
+  bool ok = map2(&mb, W, K, (uint64_t)F, pair ? kBN / 2 : kBN);
   if (planes_in) ok = ok && map3(&ma, A, kD, (uint64_t)N, (uint64_t)B * a_planes, kBM) && map3(&md, D, (uint64_t)F, (uint64_t)N, (uint64_t)B, 32);
   else ok = ok && map3(&ma, A, K, (uint64_t)N, (uint64_t)B, kBM) && map3(&md, D, kD, (uint64_t)N, (uint64_t)B * (F / kD), 32);
-  if (!ok) return cudaErrorInvalidValue;
-  cudaError_t e = proj_opt_in();
-  if (e != cudaSuccess) return e;
-  const int num_sms = device_sm_count();
   ProjParams p;
+  if (!ok || !plan(p, pair, B, N, F, kblocks, f16_in)) return cudaErrorInvalidValue;
   p.bias = bias;
+  p.bias_vec = ((uintptr_t)bias & 15) == 0;
   p.status = status;
-  p.tiles_m_per_batch = ceil_div(N, kBM);
-  p.tiles_n = ceil_div(F, kBN);
-  const int64_t total = (int64_t)B * p.tiles_m_per_batch * p.tiles_n;
-  if (total > 0x7fffffffll) return cudaErrorInvalidValue;
-  p.total_tiles = (int)total;
-  p.kblocks = kblocks;
   p.H = planes_in ? a_planes : F / kD;
-  p.fblocks = F / kD;
-  p.N = N;
   p.silu = silu ? 1 : 0;
   p.out_f16 = f16_out ? 1 : 0;
-  p.idesc = f16_in ? kIdescF16 : kIdesc;
-  const int grid = p.total_tiles < num_sms ? p.total_tiles : num_sms;
-  if (planes_in) proj_tc_kernel<false><<<grid, kThreads, kSmemBytes, st>>>(ma, mb, md, md, md, p);
-  else proj_tc_kernel<true><<<grid, kThreads, kSmemBytes, st>>>(ma, mb, md, md, md, p);
-  count_launch();
-  return cudaGetLastError();
+  if (planes_in) return pair ? launch<false, 2>(ma, mb, md, md, md, p, st) : launch<false, 1>(ma, mb, md, md, md, p, st);
+  return pair ? launch<true, 2>(ma, mb, md, md, md, p, st) : launch<true, 1>(ma, mb, md, md, md, p, st);
 }
 
 cudaError_t launch_proj_tc(bool qkv, const void* x, const void* w, const float* bias, void* d0, void* d1, void* d2,
@@ -365,8 +486,9 @@ cudaError_t launch_proj_tc(bool qkv, const void* x, const void* w, const float* 
   if (!encode_fn()) return cudaErrorNotSupported;
   const uint64_t N = (uint64_t)shape_tokens(s), C = (uint64_t)s.H * kD, BH = (uint64_t)s.B * s.H;   // prefix and grid tokens alike
   const uint64_t features = qkv ? 3 * C : C;
+  const bool pair = pair_tiles((int64_t)s.B * ceil_div((int)N, kBM), ceil_div((int)features, kBN));
   CUtensorMap ma, mb, md0, md1, md2;
-  bool ok = map2(&mb, w, C, features, kBN);
+  bool ok = map2(&mb, w, C, features, pair ? kBN / 2 : kBN);
   if (qkv) {
     ok = ok && map3(&ma, x, C, N, s.B, kBM) && map3(&md0, d0, kD, N, BH, 32) && map3(&md1, d1, kD, N, BH, 32) &&
          map3(&md2, d2, kD, N, BH, 32);
@@ -375,31 +497,16 @@ cudaError_t launch_proj_tc(bool qkv, const void* x, const void* w, const float* 
     md1 = md0;
     md2 = md0;
   }
-  if (!ok) return cudaErrorInvalidValue;
-
-  cudaError_t e = proj_opt_in();
-  if (e != cudaSuccess) return e;
-  const int num_sms = device_sm_count();
   ProjParams p;
+  if (!ok || !plan(p, pair, s.B, (int)N, (int)features, s.H, false)) return cudaErrorInvalidValue;
   p.bias = bias;
+  p.bias_vec = ((uintptr_t)bias & 15) == 0;
   p.status = status;
-  p.tiles_m_per_batch = ceil_div((int)N, kBM);
-  p.tiles_n = ceil_div((int)features, kBN);
-  const int64_t total = (int64_t)s.B * p.tiles_m_per_batch * p.tiles_n;
-  if (total > 0x7fffffffll) return cudaErrorInvalidValue;
-  p.total_tiles = (int)total;
-  p.kblocks = s.H;
   p.H = s.H;
-  p.fblocks = (int)(features / kD);
-  p.N = (int)N;
   p.silu = 0;
   p.out_f16 = 0;
-  p.idesc = kIdesc;
-  const int grid = p.total_tiles < num_sms ? p.total_tiles : num_sms;
-  if (qkv) proj_tc_kernel<true><<<grid, kThreads, kSmemBytes, st>>>(ma, mb, md0, md1, md2, p);
-  else proj_tc_kernel<false><<<grid, kThreads, kSmemBytes, st>>>(ma, mb, md0, md1, md2, p);
-  count_launch();
-  return cudaGetLastError();
+  if (qkv) return pair ? launch<true, 2>(ma, mb, md0, md1, md2, p, st) : launch<true, 1>(ma, mb, md0, md1, md2, p, st);
+  return pair ? launch<false, 2>(ma, mb, md0, md1, md2, p, st) : launch<false, 1>(ma, mb, md0, md1, md2, p, st);
 }
 
 }  // namespace jv
