@@ -153,15 +153,19 @@ bool linear_f32_supported(const LinArgs& a);
 cudaError_t launch_linear_f32(const LinArgs& a, const LinPlan& p, cudaStream_t st);
 // the kernel generator at D == 64, launched behind the grid that wrote the chunk partials (layout of lin_common.cuh); a grid
 // launched with programmatic serialisation behind it that waits for it finds the kernels and everything before them
-// complete.  prefix: the rows of o of the P <= kGenPrefix prefix tokens, too (bf16).
+// complete.  prefix: the rows of o of the P <= kGenPrefix prefix tokens, too (bf16).  *state, *nchunk: where such a grid finds
+// the heads' states, and in how many partials each.
 constexpr int kGenPrefix = 16;
-cudaError_t launch_dwc_generator_fast(const LinArgs& a, const LinPlan& p, const float* partial, bool prefix, cudaStream_t st);
+cudaError_t launch_dwc_generator_fast(const LinArgs& a, const LinPlan& p, const float* partial, bool prefix, const float** state,
+                                      int* nchunk, cudaStream_t st);
+// the chunk partials of every head summed in chunk order (what the generator does beside its hidden layer) by a launch of its own
+cudaError_t launch_sum_chunks(const LinArgs& a, const LinPlan& p, const float* partial, const float** state, cudaStream_t st);
 // where the convolution kernels of a call are: generated ones in ws + off_kernel, static ones in place; *w_batch: floats
 // from sample to sample.  To be called ahead of the state pass (static kernels off 16 bytes are copied into ws).
 cudaError_t dwc_static_kernels(const LinArgs& a, const LinPlan& p, const float** w, int* w_batch, cudaStream_t st);
 // bf16, D == 64, 3 x 3 kernels: the apply pass with the convolution fused in
 bool linear_conv_supported(const LinArgs& a);
-cudaError_t launch_linear_apply_conv(const LinArgs& a, const LinPlan& p, const float* partial, const float* w,
+cudaError_t launch_linear_apply_conv(const LinArgs& a, const LinPlan& p, const float* partial, int nchunk, const float* w,
                                      int w_batch, int* status, bool programmatic, cudaStream_t st);
 // shared by both linear paths: hidden = SiLU(W1 s + b1), w = W2 hidden + b2, with
 // s = vsum / N read from vsum[bh * bh_stride + e]

@@ -10,6 +10,11 @@
 // (One kernel for both layers, hidden formed by a cluster of eight CTAs, saved the launch but lost more in the
 // exchange of the partial sums through distributed shared memory: 10.8 us against 9.7 for 8 samples of 1024 channels.)
 //
+// Where a head has three chunks or more, blocks beside the hidden layer's sum them (in chunk order) into the head's state, off
+// the critical path, for whoever reads the state behind the generator: the apply pass read the chunks one round trip
+// after another at its start (1 x 16 heads of 128 x 128 tokens, 16 chunks: 62.0 us for the block, 50.0 so; 2 x 12 heads of 64 x 128,
+// 11 chunks: 50.0 and 41.8).
+//
 // The rows of up to kGenPrefix prefix tokens, which the convolution does not see, are work of the same kind (a few
 // products with a head's summed state): blocks behind the output layer's own take them.
 #include "lin_common.cuh"
@@ -29,13 +34,14 @@ constexpr size_t kMaxSmem = 48 * 1024;                // (no opt-in needed; smal
 
 struct GenParams {
   const float *partial, *W1, *b1, *W2, *b2;
-  float *hidden, *w;
+  float *hidden, *w, *state;                          // state: the chunks' sum, in the layout of a partial
   const void *v, *q;                                  // q, o: prefix rows only
   __nv_bfloat16* o;
   int B, H, R, P, ntok, nchunk, state_elems;
   int T;                                              // outputs per sample: C k k
   int group;                                          // samples per pass over the output layer (shared memory)
   int rows;                                           // of W2 per thread, 1 .. kRows
+  int nhid, nred;                                     // blocks of the hidden layer per sample; blocks per head that sum the chunks
   int nmain;                                          // blocks of the output layer; the ones behind take prefix rows
   float inv_n, eps;
 };
@@ -125,14 +131,15 @@ __device__ __forceinline__ void prefix_rows(const GenParams& p, int bh, float* s
   constexpr int kPer = kD / kAGroups;                 // rows of KV per thread
   const int e = threadIdx.x & 63, ag = threadIdx.x >> 6;
   const size_t row0 = (size_t)bh * p.ntok;
+  const int nchunk = p.nred ? 1 : p.nchunk;
   const __nv_bfloat16* q = (const __nv_bfloat16*)p.q + row0 * kD;
   for (int i = threadIdx.x; i < p.P * kD; i += kThreadsOut) qs[i] = fmaxf(__bfloat162float(q[i]), 0.f);
   griddep_wait();
-  const float* src = p.partial + (size_t)bh * p.nchunk * p.state_elems;
+  const float* src = p.nred ? p.state + (size_t)bh * p.state_elems : p.partial + (size_t)bh * p.nchunk * p.state_elems;
   float kv[kPer], z = 0.f;
 #pragma unroll
   for (int i = 0; i < kPer; ++i) kv[i] = 0.f;
-  for (int c = 0; c < p.nchunk; ++c, src += p.state_elems) {          // in chunk order
+  for (int c = 0; c < nchunk; ++c, src += p.state_elems) {            // in chunk order
 #pragma unroll
     for (int i = 0; i < kPer; ++i) kv[i] += __ldcg(src + (kPer * ag + i) * kD + e);
     if (threadIdx.x < kD) z += __ldcg(src + kOffZ + threadIdx.x);
@@ -157,6 +164,27 @@ __device__ __forceinline__ void prefix_rows(const GenParams& p, int bh, float* s
   }
 }
 
+// One of the nred blocks that sum the chunks of head h of sample b
+__device__ __forceinline__ void sum_chunks(const GenParams& p, int b, int h, int part) {
+  constexpr int kVecs = (kD * kD + kD) / 4;           // KV and z
+  griddep_wait();                                     // the state pass is complete
+  const size_t bh = (size_t)b * p.H + h;
+  const float4* src = reinterpret_cast<const float4*>(p.partial + bh * p.nchunk * p.state_elems);
+  float4* dst = reinterpret_cast<float4*>(p.state + bh * p.state_elems);
+  const int stride = p.state_elems / 4;
+  for (int i = part * kThreads + threadIdx.x; i < kVecs; i += p.nred * kThreads) {
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k0 = 0; k0 < p.nchunk; k0 += 8) {
+      float4 x[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) x[k] = k0 + k < p.nchunk ? __ldcg(src + (size_t)(k0 + k) * stride + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) { s.x += x[k].x; s.y += x[k].y; s.z += x[k].z; s.w += x[k].w; }
+    }
+    dst[i] = s;
+  }
+}
+
 // A block serves 8 values of r for one sample: per 1024 channels it forms the means in shared memory while the rows of
 // W1 are already on their way, then warp w takes row r0 + w.
 template <typename T, bool kVec>
@@ -164,6 +192,11 @@ __global__ void __launch_bounds__(kThreads, 2)
 gen_hidden_kernel(const GenParams p) {
   __shared__ __align__(16) float mean[kTileC];
   griddep_launch_dependents();                        // (the grid behind this one waits for it before it reads hidden)
+  if ((int)blockIdx.x >= p.nhid) {
+    const int i = blockIdx.x - p.nhid;
+    sum_chunks(p, blockIdx.y, i / p.nred, i % p.nred);
+    return;
+  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = blockIdx.x * 8 + warp, b = blockIdx.y, C = p.H * kD;
   const bool r_ok = r < p.R;
@@ -317,11 +350,34 @@ cudaError_t dwc_static_kernels(const LinArgs& a, const LinPlan& p, const float**
   return cudaMemcpyAsync((char*)a.ws + p.off_kernel, a.dwc->b2, (size_t)T * sizeof(float), cudaMemcpyDeviceToDevice, st);
 }
 
-cudaError_t launch_dwc_generator_fast(const LinArgs& a, const LinPlan& p, const float* partial, bool prefix, cudaStream_t st) {
+cudaError_t launch_sum_chunks(const LinArgs& a, const LinPlan& p, const float* partial, const float** state, cudaStream_t st) {
+  GenParams g = {};
+  g.partial = partial;
+  g.state = (float*)((char*)a.ws + p.off_state);
+  g.H = a.s.H;
+  g.nchunk = p.nchunk;
+  g.state_elems = p.state_elems;
+  g.nred = 4;
+  *state = g.state;
+  return enqueue(gen_hidden_kernel<__nv_bfloat16, true>, dim3(g.nred * a.s.H, a.s.B), kThreads, 0, g, st);
+}
+
+cudaError_t launch_dwc_generator_fast(const LinArgs& a, const LinPlan& p, const float* partial, bool prefix, const float** state,
+                                      int* nchunk, cudaStream_t st) {
   const jv_shape& s = a.s;
   const jv_dwc& d = *a.dwc;
-  if (d.R == 0 && !prefix) return cudaSuccess;
+  // static kernels: a launch only for sums of enough chunks (its 3 us against the readers' round trips)
+  const bool reduce = p.nchunk >= (d.R > 0 ? 3 : 8);
+  *state = partial;
+  *nchunk = p.nchunk;
+  if (d.R == 0 && !prefix && !reduce) return cudaSuccess;
   GenParams g = {};
+  g.state = (float*)((char*)a.ws + p.off_state);
+  if (reduce) {
+    g.nred = p.nchunk >= 8 ? 4 : 1;
+    *state = g.state;
+    *nchunk = 1;
+  }
   g.partial = partial;
   g.W1 = d.W1;
   g.b1 = d.b1;
@@ -344,13 +400,17 @@ cudaError_t launch_dwc_generator_fast(const LinArgs& a, const LinPlan& p, const 
   g.eps = a.eps;
   const bool vec = d.R % 4 == 0 && (((uintptr_t)d.W1 | (uintptr_t)d.W2) & 15) == 0;
   size_t smem = 0;
-  if (d.R > 0) {
-    const dim3 grid(ceil_div(d.R, 8), s.B);
+  if (d.R > 0 || reduce) {
+    g.nhid = ceil_div(d.R, 8);
+    const dim3 grid(g.nhid + g.nred * s.H, s.B);
     const cudaError_t e = s.dtype == JV_F32 ? (vec ? enqueue(gen_hidden_kernel<float, true>, grid, kThreads, 0, g, st)
                                                    : enqueue(gen_hidden_kernel<float, false>, grid, kThreads, 0, g, st))
                                             : (vec ? enqueue(gen_hidden_kernel<__nv_bfloat16, true>, grid, kThreads, 0, g, st)
                                                    : enqueue(gen_hidden_kernel<__nv_bfloat16, false>, grid, kThreads, 0, g, st));
     if (e != cudaSuccess) return e;
+  }
+  if (d.R == 0 && !prefix) return cudaSuccess;
+  if (d.R > 0) {
     size_t group = kMaxSmem / (d.R * sizeof(float));  // (R <= 1024: at least 12)
     group &= ~(size_t)7;
     g.group = (size_t)s.B < group ? s.B : (int)group;

@@ -578,10 +578,10 @@ bool linear_conv_supported(const LinArgs& a) {
 }
 
 // Enqueues the fused apply + convolution pass over the grid tokens (prefix tokens, which the
-// convolution does not see, are left to the plain apply pass).  `partial` holds the chunk partials of the state
-// pass, `w` the kernels [B][C][3][3]; both are written by grids ahead of this one in the stream,
+// convolution does not see, are left to the plain apply pass).  `partial` holds the states, each
+// as nchunk partials, `w` the kernels [B][C][3][3]; both are written by grids ahead of this one in the stream,
 // which this grid waits for (griddepcontrol.wait) before it reads them.
-cudaError_t launch_linear_apply_conv(const LinArgs& a, const LinPlan& p, const float* partial, const float* w,
+cudaError_t launch_linear_apply_conv(const LinArgs& a, const LinPlan& p, const float* partial, int nchunk, const float* w,
                                      int w_batch, int* status, bool programmatic, cudaStream_t st) {
   const jv_shape& s = a.s;
   const int BH = s.B * s.H;
@@ -605,7 +605,7 @@ cudaError_t launch_linear_apply_conv(const LinArgs& a, const LinPlan& p, const f
   cp.BH = BH;
   cp.Hg = s.Hg;
   cp.Wg = s.Wg;
-  cp.nchunk = p.nchunk;
+  cp.nchunk = nchunk;
   cp.state_elems = p.state_elems;
   cp.ncb = ceil_div(s.Wg, kPatchW);
   cp.nrb = ceil_div(s.Hg, kPatchH);

@@ -251,7 +251,9 @@ cudaError_t launch_linear_f32(const LinArgs& a, const LinPlan& p, cudaStream_t s
                                                                          p.chunk_tokens, p.state_elems);
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (a.dwc && (e = launch_dwc_generator_fast(a, p, partial, false, st)) != cudaSuccess) return e;
+  const float* state = partial;
+  int nchunk = p.nchunk;
+  if (a.dwc && (e = launch_dwc_generator_fast(a, p, partial, false, &state, &nchunk, st)) != cudaSuccess) return e;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -262,8 +264,8 @@ cudaError_t launch_linear_f32(const LinArgs& a, const LinPlan& p, cudaStream_t s
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, lin_f32_apply_kernel, (const float*)a.q, (const float*)a.v, (float*)a.o, (const float*)partial, w, w_batch,
-                         (int)s.H, (int)s.P, (int)s.Hg, (int)s.Wg, p.nchunk, p.state_elems, a.eps);
+  e = cudaLaunchKernelEx(&cfg, lin_f32_apply_kernel, (const float*)a.q, (const float*)a.v, (float*)a.o, state, w, w_batch,
+                         (int)s.H, (int)s.P, (int)s.Hg, (int)s.Wg, nchunk, p.state_elems, a.eps);
   count_launch();
   return e;
 }

@@ -588,7 +588,7 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
   // predecessor (griddepcontrol.wait) before it reads what that one wrote, so completion is transitive along the chain.
   // apply pass over the first ntokens tokens of every (batch, head): one wave of two CTAs per SM, spans
   // of whole 128-token tiles; launched so that its set-up overlaps the tail of the grid before it
-  auto enqueue_apply = [&](const CUtensorMap& map_q, const CUtensorMap& map_o, int ntokens) -> cudaError_t {
+  auto enqueue_apply = [&](const CUtensorMap& map_q, const CUtensorMap& map_o, int ntokens, const float* state, int nchunk) -> cudaError_t {
     int nspan = (2 * num_sms) / BH;
     if (nspan < 1) nspan = 1;
     int span = ceil_div(ceil_div(ntokens, nspan), kApplyTok) * kApplyTok;
@@ -601,13 +601,20 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t err = cudaLaunchKernelEx(&cfg, lin_apply_kernel, map_q, map_o, (const float*)partial, status, ntokens,
-                                               span, p.nchunk, p.state_elems, a.eps, (int)s.H);
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, lin_apply_kernel, map_q, map_o, state, status, ntokens,
+                                               span, nchunk, p.state_elems, a.eps, (int)s.H);
     count_launch();
     return err;
   };
 
-  if (!a.dwc) return enqueue_apply(mq, mo, N);
+  if (!a.dwc) {
+    // Many chunks: their sum by a launch of its own instead of by every apply CTA at its start.  Measured, without / with it: 16 chunks
+    // 39.0 / 36.9 us (16 heads of 128 x 128) and 19.6 / 16.5 (6 of 90 x 90), 11: 31.6 / 30.9, 8: 34.9 / 35.4, 6: 28.8 / 30.8.
+    if (p.nchunk < 10) return enqueue_apply(mq, mo, N, partial, p.nchunk);
+    const float* state;
+    if ((e = launch_sum_chunks(a, p, partial, &state, st)) != cudaSuccess) return e;
+    return enqueue_apply(mq, mo, N, state, 1);
+  }
   if (fused_conv) {
     // 3 x 3 kernels: state -> generator (with generated kernels) -> apply pass with the convolution fused in.
     // Prefix tokens: the convolution does not see them, their output is the attention output alone.  A few of them are
@@ -616,14 +623,18 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
       CUtensorMap mqp, mop;
       if (!make_map_tokens_in(&mqp, a.q, s.B, s.H, s.P, kApplyTok, in) || !make_map_tokens(&mop, a.o, BH, s.P, 32, N))
         return cudaErrorInvalidValue;
-      if ((e = enqueue_apply(mqp, mop, s.P)) != cudaSuccess) return e;
+      if ((e = enqueue_apply(mqp, mop, s.P, partial, p.nchunk)) != cudaSuccess) return e;
     }
-    if ((e = launch_dwc_generator_fast(a, p, partial, s.P > 0 && s.P <= kGenPrefix, st)) != cudaSuccess) return e;
-    return launch_linear_apply_conv(a, p, partial, w, w_batch, status, true, st);
+    const float* state;
+    int nchunk;
+    if ((e = launch_dwc_generator_fast(a, p, partial, s.P > 0 && s.P <= kGenPrefix, &state, &nchunk, st)) != cudaSuccess) return e;
+    return launch_linear_apply_conv(a, p, state, nchunk, w, w_batch, status, true, st);
   }
   // 5 x 5 kernels: generator, apply pass, a read-modify-write pass over o
-  if ((e = launch_dwc_generator_fast(a, p, partial, false, st)) != cudaSuccess) return e;
-  if ((e = enqueue_apply(mq, mo, N)) != cudaSuccess) return e;
+  const float* state;
+  int nchunk;
+  if ((e = launch_dwc_generator_fast(a, p, partial, false, &state, &nchunk, st)) != cudaSuccess) return e;
+  if ((e = enqueue_apply(mq, mo, N, state, nchunk)) != cudaSuccess) return e;
   const int run = 32;
   dim3 g4(ceil_div(ceil_div(N, run), 8), BH);
   const __nv_bfloat16* v = (const __nv_bfloat16*)a.v;
