@@ -38,12 +38,14 @@ constexpr size_t smem_bytes() {
 template <int R, int G>
 __global__ void __launch_bounds__(32 * R * G, 3)
 attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ o,
-                int Hg, int Wg, int P, int wh, int ww, int nwx, bool prefix_rows, float scale) {
+                int Hg, int Wg, int P, int wh, int ww, int nwx, bool prefix_rows, bool overlap, float scale) {
   extern __shared__ __align__(16) float smem_f[];
   float* qs = smem_f;                                        // [16 R][kLd]
   float* ps = qs + R * kRowsWarp * kLd;                      // [R G warps][16][kLd]: probabilities, then the warp's output
   float* ks = ps + R * G * kRowsWarp * kLd;                  // [G][64][kLd]: the group's K tile, then its V tile
-  if (prefix_rows) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // overlap: the launch ahead is that of the prefix queries (it has waited for what came before it); waited for at the end
+  if (!overlap) griddep_wait();
+  griddep_launch_dependents();
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tx = lane & 15, ty = lane >> 4;
   const int grp = warp / R, rw = warp % R;                   // key group, row warp
@@ -240,33 +242,21 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
       *reinterpret_cast<float4*>(o + base + (size_t)tok * kDim + 4 * tx) = make_float4(x.x * inv, x.y * inv, x.z * inv, x.w * inv);
     }
   }
-  // a launch that overlaps the one before it (see launch_attn_f32) ends only after it
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (overlap) griddep_wait();
 }
 
 template <int R, int G>
 cudaError_t launch(const AttnArgs& a, bool prefix_rows, bool overlap, cudaStream_t st) {
   static OncePerDevice opt_in;
-  cudaError_t e = opt_in.run([&] {
+  const cudaError_t e = opt_in.run([&] {
     return cudaFuncSetAttribute(attn_f32_kernel<R, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<R, G>());
   });
   if (e != cudaSuccess) return e;
   const int wh = a.wh < a.Hg ? a.wh : a.Hg, ww = a.ww < a.Wg ? a.ww : a.Wg;
   const int nwx = ceil_div(a.Wg, ww), nwin = nwx * ceil_div(a.Hg, wh);
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = prefix_rows ? dim3(ceil_div(a.P, R * kRowsWarp), 1, a.BH) : dim3(ceil_div(wh * ww, R * kRowsWarp), nwin, a.BH);
-  cfg.blockDim = dim3(32 * R * G);
-  cfg.dynamicSmemBytes = smem_bytes<R, G>();
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = overlap ? 1 : 0;
-  e = cudaLaunchKernelEx(&cfg, attn_f32_kernel<R, G>, (const float*)a.q, (const float*)a.k, (const float*)a.v, (float*)a.o, a.Hg,
-                         a.Wg, a.P, wh, ww, nwx, prefix_rows, a.scale);
-  count_launch();
-  return e;
+  const dim3 grid = prefix_rows ? dim3(ceil_div(a.P, R * kRowsWarp), 1, a.BH) : dim3(ceil_div(wh * ww, R * kRowsWarp), nwin, a.BH);
+  return launch_programmatic(attn_f32_kernel<R, G>, grid, 32 * R * G, smem_bytes<R, G>(), st, (const float*)a.q, (const float*)a.k,
+                             (const float*)a.v, (float*)a.o, a.Hg, a.Wg, a.P, wh, ww, nwx, prefix_rows, overlap, a.scale);
 }
 
 }  // namespace

@@ -126,12 +126,6 @@ attn_f4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
-  // a timeout flagged earlier (by any CTA or launch) makes the rest leave at once
-  if (threadIdx.x == 0) bar->tmem_base = *reinterpret_cast<volatile int*>(p.status);
-  __syncthreads();
-  if (bar->tmem_base != 0) return;
-  __syncthreads();
-
   if (threadIdx.x == 0) {
     for (int t = 0; t < kQT; ++t) {
       mbar_init(&bar->q_full[t], 1);
@@ -161,6 +155,17 @@ attn_f4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bar->tmem_base, 0);
+
+  griddep_wait();                 // what is read and written from here on may belong to the launch ahead
+  griddep_launch_dependents();
+  // a timeout flagged earlier (by any CTA or launch) makes the rest leave at once
+  if (threadIdx.x == 0 && *reinterpret_cast<volatile int*>(p.status) != 0) bar->abort_flag = 1;
+  __syncthreads();
+  if (bar->abort_flag) {
+    if (warp == 0)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    return;
+  }
 
   const int item0 = blockIdx.x, item_step = gridDim.x;
   const int ntiles = p.ntiles, nsteps = 2 * p.ntiles;
@@ -510,10 +515,8 @@ cudaError_t launch_attn_f4(const AttnArgs& a, int* status, cudaStream_t st) {
   p.div_H = make_fastdiv((uint32_t)a.H);
   p.scale_log2 = a.scale * 1.4426950408889634f;
   const int grid = p.total_items < num_sms ? p.total_items : num_sms;
-  if (split) attn_f4_kernel<true><<<grid, kThreads, kSmemBytes, st>>>(maps[0], maps[1], maps[2], maps[3], p);
-  else attn_f4_kernel<false><<<grid, kThreads, kSmemBytes, st>>>(maps[0], maps[1], maps[2], maps[3], p);
-  count_launch();
-  return cudaGetLastError();
+  return launch_programmatic(split ? attn_f4_kernel<true> : attn_f4_kernel<false>, dim3(grid), kThreads, kSmemBytes, st, maps[0], maps[1],
+                             maps[2], maps[3], p);
 }
 
 }  // namespace jv

@@ -49,7 +49,8 @@ attn_prefix_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16
                         const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ o, int N, int P, float scale_log2) {
   namespace cg = cooperative_groups;
   __shared__ float part[kWarps + 1][kRows][kLd];      // one partial per warp, then the block's own
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");    // the windows' launch overlaps this one
+  griddep_wait();
+  griddep_launch_dependents();                        // the windows' launch overlaps this one
   cg::cluster_group cluster = cg::this_cluster();
   const int nsplit = cluster.num_blocks(), split = cluster.block_rank();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -204,21 +205,9 @@ cudaError_t launch_attn_prefix(const AttnArgs& a, int ctas, cudaStream_t st) {
   // splits of the keys: at least one 16-key step per warp
   int split = 1;
   while (split < 8 && 2 * split * a.BH * groups <= ctas && split * kWarps * kKeys < N) split *= 2;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = split;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.BH * split, groups);
-  cfg.blockDim = dim3(kWarps * 32);
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, attn_prefix_rows_kernel, (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k,
-                                           (const __nv_bfloat16*)a.v, (__nv_bfloat16*)a.o, N, a.P, a.scale * 1.4426950408889634f);
-  count_launch();
-  return e;
+  return launch_programmatic_cluster(attn_prefix_rows_kernel, split, dim3(a.BH * split, groups), kWarps * 32, 0, st,
+                                     (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v,
+                                     (__nv_bfloat16*)a.o, N, a.P, a.scale * 1.4426950408889634f);
 }
 
 }  // namespace jv

@@ -139,17 +139,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   // broadcast from lane 0: lets the compiler keep everything derived from the warp index uniform
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
-  // a grid launched behind this one with programmatic serialisation (the prefix queries of W, which
-  // depend on nothing here) may run beside it
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
-  // Once any CTA has flagged a timeout the rest of the grid (and later launches, until the
-  // host reads the status) leave at once instead of each running into the same limit.
-  if (threadIdx.x == 0) bar->tmem_base = *reinterpret_cast<volatile int*>(p.status);
-  __syncthreads();
-  if (bar->tmem_base != 0) return;
-  __syncthreads();
-
   if (threadIdx.x == 0) {
     for (int b = 0; b < 2; ++b) {
       mbar_init(&bar->q_full[b], 1);
@@ -184,6 +173,17 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bar->tmem_base, 0);
+
+  griddep_wait();                 // what is read and written from here on may belong to the launch ahead
+  griddep_launch_dependents();
+  // a timeout flagged earlier (by any CTA or launch) makes the rest leave at once
+  if (threadIdx.x == 0 && *reinterpret_cast<volatile int*>(p.status) != 0) bar->abort_flag = 1;
+  __syncthreads();
+  if (bar->abort_flag) {
+    if (warp == 0)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    return;
+  }
 
   const int item0 = blockIdx.x, item_step = gridDim.x;
 
@@ -786,9 +786,7 @@ cudaError_t launch_attn_tc(const AttnArgs& a, bool full, int* status, cudaStream
   // persistent: one CTA per SM (shared memory and the 512 tensor-memory columns allow no more)
   const int num_sms = device_sm_count();
   const int grid = p.total_items < num_sms ? p.total_items : num_sms;
-  attn_tc_kernel<<<grid, kThreads, kSmemBytes, st>>>(maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], p);
-  count_launch();
-  return cudaGetLastError();
+  return launch_programmatic(attn_tc_kernel, dim3(grid), kThreads, kSmemBytes, st, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], p);
 }
 
 }  // namespace jv

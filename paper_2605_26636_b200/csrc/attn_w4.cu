@@ -159,12 +159,6 @@ attn_w4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
-  // a timeout flagged earlier (by any CTA or launch) makes the rest leave at once
-  if (threadIdx.x == 0) bar->tmem_base = *reinterpret_cast<volatile int*>(p.status);
-  __syncthreads();
-  if (bar->tmem_base != 0) return;
-  __syncthreads();
-
   if (threadIdx.x == 0) {
     for (int t = 0; t < kQT; ++t) {
       for (int b = 0; b < 2; ++b) {
@@ -202,6 +196,19 @@ attn_w4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bar->tmem_base, 0);
+
+  // With prefix tokens the launch ahead is that of their queries, which this one overlaps (it has waited for what came before
+  // it before it let this one go); this one waits for it at its end.
+  if (!kPrefix) griddep_wait();   // what is read and written from here on may belong to the launch ahead
+  griddep_launch_dependents();
+  // a timeout flagged earlier (by any CTA or launch) makes the rest leave at once
+  if (threadIdx.x == 0 && *reinterpret_cast<volatile int*>(p.status) != 0) bar->abort_flag = 1;
+  __syncthreads();
+  if (bar->abort_flag) {
+    if (warp == 0)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    return;
+  }
 
   const int item_step = kSlots * gridDim.x;
 
@@ -613,7 +620,7 @@ attn_w4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 
   // ================= common teardown =================
   // with prefix tokens this launch overlaps the one ahead of it (their queries) and must not end before it
-  if (kPrefix) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (kPrefix) griddep_wait();
   __syncwarp();
   tc_fence_before();
   __syncthreads();
@@ -658,19 +665,8 @@ cudaError_t launch_w4(const CUtensorMap (&maps)[6], const W4Params& p, int grid,
                                 (int)Layout<kPrefix>::kBytes);
   });
   if (e != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = Layout<kPrefix>::kBytes;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = kPrefix ? 1 : 0;                      // the prefix queries' launch is right ahead of this one
-  const cudaError_t r = cudaLaunchKernelEx(&cfg, attn_w4_kernel<kPrefix, kWpt>, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], p);
-  count_launch();
-  return r;
+  return launch_programmatic(attn_w4_kernel<kPrefix, kWpt>, dim3(grid), kThreads, Layout<kPrefix>::kBytes, st, maps[0], maps[1], maps[2],
+                             maps[3], maps[4], maps[5], p);
 }
 
 cudaError_t launch_attn_w4(const AttnArgs& a, int* status, cudaStream_t st) {

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <utility>
 
 #include "jetvit.h"
 
@@ -45,6 +46,57 @@ class OncePerDevice {
  private:
   std::atomic<int> done_[kMaxDevices] = {};
 };
+
+// ---- programmatic launches ----------------------------------------------------
+// Every kernel of the tensor-core and fp32 paths is launched with programmatic stream serialisation: it may start, and do
+// what depends on nothing (barriers, tensor memory, first loads of weights), while the launch ahead of it drains, which takes
+// 2 to 4 us off every boundary between two launches.  The rules:
+//   - a kernel waits (griddep_wait) before it reads what an earlier launch may have written and before it writes anything;
+//     a launch is then complete only after the one ahead of it, so completion is transitive along the stream;
+//   - it lets the next launch go (griddep_launch_dependents) only after its tensor memory is allocated (the next one's
+//     allocation would otherwise wait for memory that this one could never get), and, where the next one reads the call's
+//     inputs before its own wait, only after its own wait: whoever produced them is complete then.
+__device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... Params, typename... Args>
+cudaError_t launch_programmatic(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args&&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+  count_launch();
+  return e;
+}
+// the same for a grid of clusters of `cluster` blocks along x
+template <typename... Params, typename... Args>
+cudaError_t launch_programmatic_cluster(void (*kernel)(Params...), int cluster, dim3 grid, int threads, size_t smem, cudaStream_t st,
+                                        Args&&... args) {
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+  count_launch();
+  return e;
+}
 
 // ---- element access -------------------------------------------------------
 __device__ __forceinline__ float to_f32(float x) { return x; }
@@ -166,7 +218,7 @@ cudaError_t dwc_static_kernels(const LinArgs& a, const LinPlan& p, const float**
 // bf16, D == 64, 3 x 3 kernels: the apply pass with the convolution fused in
 bool linear_conv_supported(const LinArgs& a);
 cudaError_t launch_linear_apply_conv(const LinArgs& a, const LinPlan& p, const float* partial, int nchunk, const float* w,
-                                     int w_batch, int* status, bool programmatic, cudaStream_t st);
+                                     int w_batch, int* status, cudaStream_t st);
 // shared by both linear paths: hidden = SiLU(W1 s + b1), w = W2 hidden + b2, with
 // s = vsum / N read from vsum[bh * bh_stride + e]
 cudaError_t launch_dwc_generator(const LinArgs& a, const LinPlan& p, const float* vsum, int bh_stride,

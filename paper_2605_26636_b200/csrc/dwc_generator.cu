@@ -318,23 +318,6 @@ gen_out_kernel(const GenParams p) {
   }
 }
 
-template <typename... Args>
-cudaError_t enqueue(void (*kernel)(Args...), dim3 grid, int threads, size_t smem, const GenParams& p, cudaStream_t st) {
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p);
-  count_launch();
-  return e;
-}
-
 }  // namespace
 
 cudaError_t dwc_static_kernels(const LinArgs& a, const LinPlan& p, const float** w, int* w_batch, cudaStream_t st) {
@@ -359,7 +342,7 @@ cudaError_t launch_sum_chunks(const LinArgs& a, const LinPlan& p, const float* p
   g.state_elems = p.state_elems;
   g.nred = 4;
   *state = g.state;
-  return enqueue(gen_hidden_kernel<__nv_bfloat16, true>, dim3(g.nred * a.s.H, a.s.B), kThreads, 0, g, st);
+  return launch_programmatic(gen_hidden_kernel<__nv_bfloat16, true>, dim3(g.nred * a.s.H, a.s.B), kThreads, 0, st, g);
 }
 
 cudaError_t launch_dwc_generator_fast(const LinArgs& a, const LinPlan& p, const float* partial, bool prefix, const float** state,
@@ -403,10 +386,10 @@ cudaError_t launch_dwc_generator_fast(const LinArgs& a, const LinPlan& p, const 
   if (d.R > 0 || reduce) {
     g.nhid = ceil_div(d.R, 8);
     const dim3 grid(g.nhid + g.nred * s.H, s.B);
-    const cudaError_t e = s.dtype == JV_F32 ? (vec ? enqueue(gen_hidden_kernel<float, true>, grid, kThreads, 0, g, st)
-                                                   : enqueue(gen_hidden_kernel<float, false>, grid, kThreads, 0, g, st))
-                                            : (vec ? enqueue(gen_hidden_kernel<__nv_bfloat16, true>, grid, kThreads, 0, g, st)
-                                                   : enqueue(gen_hidden_kernel<__nv_bfloat16, false>, grid, kThreads, 0, g, st));
+    const cudaError_t e = s.dtype == JV_F32 ? (vec ? launch_programmatic(gen_hidden_kernel<float, true>, grid, kThreads, 0, st, g)
+                                                   : launch_programmatic(gen_hidden_kernel<float, false>, grid, kThreads, 0, st, g))
+                                            : (vec ? launch_programmatic(gen_hidden_kernel<__nv_bfloat16, true>, grid, kThreads, 0, st, g)
+                                                   : launch_programmatic(gen_hidden_kernel<__nv_bfloat16, false>, grid, kThreads, 0, st, g));
     if (e != cudaSuccess) return e;
   }
   if (d.R == 0 && !prefix) return cudaSuccess;
@@ -428,7 +411,7 @@ cudaError_t launch_dwc_generator_fast(const LinArgs& a, const LinPlan& p, const 
   // one sample, two, four or eight at a time
   auto* out = !vec ? gen_out_kernel<false, 4> : s.B == 1 ? gen_out_kernel<true, 1> : s.B == 2 ? gen_out_kernel<true, 2>
               : s.B <= 4 ? gen_out_kernel<true, 4> : gen_out_kernel<true, 8>;
-  return enqueue(out, dim3(blocks), kThreadsOut, smem, g, st);
+  return launch_programmatic(out, dim3(blocks), kThreadsOut, smem, st, g);
 }
 
 }  // namespace jv

@@ -14,9 +14,6 @@ constexpr int kD = 64;
 // [4160, 4224) vsum[e]
 constexpr int kOffZ = kD * kD, kOffVsum = kD * kD + kD;
 
-__device__ __forceinline__ void griddep_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 __device__ __forceinline__ uint32_t relu_bf16x2(uint32_t x) {
   __nv_bfloat162 v = *reinterpret_cast<__nv_bfloat162*>(&x);
   v = __hmax2(v, __float2bfloat162_rn(0.f));

@@ -181,6 +181,7 @@ lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
+  griddep_launch_dependents();
 
   if (warp == kWarpProducer) {
     // ================= TMA producer =================
@@ -582,7 +583,7 @@ bool linear_conv_supported(const LinArgs& a) {
 // as nchunk partials, `w` the kernels [B][C][3][3]; both are written by grids ahead of this one in the stream,
 // which this grid waits for (griddepcontrol.wait) before it reads them.
 cudaError_t launch_linear_apply_conv(const LinArgs& a, const LinPlan& p, const float* partial, int nchunk, const float* w,
-                                     int w_batch, int* status, bool programmatic, cudaStream_t st) {
+                                     int w_batch, int* status, cudaStream_t st) {
   const jv_shape& s = a.s;
   const int BH = s.B * s.H;
   CUtensorMap mq, mv, mo;
@@ -612,19 +613,8 @@ cudaError_t launch_linear_apply_conv(const LinArgs& a, const LinPlan& p, const f
   cp.total_tiles = BH * cp.ncb * cp.nrb;
   cp.eps = a.eps;
   const int num_sms = device_sm_count();
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cp.total_tiles < num_sms ? cp.total_tiles : num_sms);
-  cfg.blockDim = dim3(kThreadsConv);
-  cfg.dynamicSmemBytes = kConvSmem;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = programmatic ? 1 : 0;
-  e = cudaLaunchKernelEx(&cfg, lin_apply_conv_kernel, mq, mv, mo, cp);
-  count_launch();
-  return e;
+  return launch_programmatic(lin_apply_conv_kernel, dim3(cp.total_tiles < num_sms ? cp.total_tiles : num_sms), kThreadsConv, kConvSmem, st,
+                             mq, mv, mo, cp);
 }
 
 }  // namespace jv

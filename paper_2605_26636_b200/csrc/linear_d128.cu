@@ -21,8 +21,6 @@ namespace jv {
 namespace {
 
 using namespace tc;
-using lin::griddep_launch_dependents;
-using lin::griddep_wait;
 using lin::relu_bf16x2;
 using lin::bf16x2_to_f2;
 using lin::tile_off;
@@ -81,7 +79,6 @@ lin128_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
   const int t_begin = min(N, chunk * chunk_tokens), t_end = min(N, t_begin + chunk_tokens);
   const int ntiles = (t_end - t_begin + kTok1 - 1) / kTok1;            // 0 for a chunk past the end
 
-  griddep_launch_dependents();
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages1; ++s) {
       mbar_init(&bars->full[s], 1);
@@ -90,8 +87,7 @@ lin128_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     }
     mbar_init(&bars->acc_full, 1);
     mbar_init(&bars->red_full, 1);
-    // an earlier kernel gave up: no copies, no waits (but this CTA still takes part in the cluster's barriers)
-    bars->abort_flag = *reinterpret_cast<volatile int*>(status) != 0;
+    bars->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -101,8 +97,12 @@ lin128_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
+  griddep_wait();                 // what is read and written from here on may belong to the launch ahead
+  // an earlier kernel gave up: no copies, no waits (but this CTA still takes part in the cluster's barriers)
+  if (threadIdx.x == 0 && *reinterpret_cast<volatile int*>(status) != 0) bars->abort_flag = 1;
   __syncthreads();
   tc_fence_after();
+  griddep_launch_dependents();    // (the apply pass reads Q ahead of its own wait)
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // (1) this CTA may be copied to
   const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
   bool ok = bars->abort_flag == 0;
@@ -330,6 +330,7 @@ lin128_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_const
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  griddep_launch_dependents();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_base, 0);
   bool ok = true;
 
@@ -539,39 +540,16 @@ cudaError_t launch_linear_d128(const LinArgs& a, const LinPlan& p, cudaStream_t 
   if (nchunk > kMaxCluster) nchunk = kMaxCluster;
   if (nchunk > tiles) nchunk = tiles;
   if (nchunk < 1) nchunk = 1;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = nchunk;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nchunk, BH);
-  cfg.blockDim = dim3(kThreads1);
-  cfg.dynamicSmemBytes = kSmem1;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, lin128_state_kernel, mk, mv, state, status, N, ceil_div(tiles, nchunk) * kTok1);
-  count_launch();
+  e = launch_programmatic_cluster(lin128_state_kernel, nchunk, dim3(nchunk, BH), kThreads1, kSmem1, st, mk, mv, state, status, N,
+                                  ceil_div(tiles, nchunk) * kTok1);
   if (e != cudaSuccess) return e;
 
   // one wave of one CTA per SM over (head, span of whole 128-token tiles); its set-up and first Q tiles overlap the state pass
   int nspan = num_sms / BH;
   if (nspan < 1) nspan = 1;
   const int span = ceil_div(ceil_div(N, nspan), kTok2) * kTok2;
-  cudaLaunchAttribute attr2[1];
-  attr2[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr2[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg2 = {};
-  cfg2.gridDim = dim3(ceil_div(N, span), BH);
-  cfg2.blockDim = dim3(kThreads2);
-  cfg2.dynamicSmemBytes = kSmem2;
-  cfg2.stream = st;
-  cfg2.attrs = attr2;
-  cfg2.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg2, lin128_apply_kernel, mq, mo, (const unsigned char*)state, status, N, span, a.eps);
-  count_launch();
-  return e;
+  return launch_programmatic(lin128_apply_kernel, dim3(ceil_div(N, span), BH), kThreads2, kSmem2, st, mq, mo, (const unsigned char*)state,
+                             status, N, span, a.eps);
 }
 
 }  // namespace jv

@@ -32,6 +32,7 @@ __global__ void __launch_bounds__(kThreads)
 lin_f32_state_kernel(const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ partial, int N,
                      int chunk_tokens, int state_elems) {
   extern __shared__ __align__(16) float smem_f[];
+  griddep_wait();
   griddep_launch_dependents();
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;      // rows a = 8 ty + i, columns e = 4 tx + j of KV
   const int t_begin = blockIdx.x * chunk_tokens, t_end = min(N, t_begin + chunk_tokens);
@@ -112,6 +113,7 @@ lin_f32_apply_kernel(const float* __restrict__ q, const float* __restrict__ v, f
   float* zs = kv + kD * kLdA;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;      // tokens 8 ty + i, channels 4 tx + j
   const int N = P + Hg * Wg, bh = blockIdx.y, t0 = blockIdx.x * kTok;
+  griddep_launch_dependents();
   const size_t base = (size_t)bh * N * kD;
 #pragma unroll
   for (int i = 0; i < kTok / 8; ++i) {                            // q is an input of the call: loaded ahead of the wait
@@ -247,27 +249,15 @@ cudaError_t launch_linear_f32(const LinArgs& a, const LinPlan& p, cudaStream_t s
   const float* w = nullptr;
   int w_batch = 0;
   if (a.dwc && (e = dwc_static_kernels(a, p, &w, &w_batch, st)) != cudaSuccess) return e;
-  lin_f32_state_kernel<<<dim3(p.nchunk, BH), kThreads, kStateSmem, st>>>((const float*)a.k, (const float*)a.v, partial, N,
-                                                                         p.chunk_tokens, p.state_elems);
-  count_launch();
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  e = launch_programmatic(lin_f32_state_kernel, dim3(p.nchunk, BH), kThreads, kStateSmem, st, (const float*)a.k, (const float*)a.v,
+                          partial, N, p.chunk_tokens, p.state_elems);
+  if (e != cudaSuccess) return e;
   const float* state = partial;
   int nchunk = p.nchunk;
   if (a.dwc && (e = launch_dwc_generator_fast(a, p, partial, false, &state, &nchunk, st)) != cudaSuccess) return e;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ceil_div(N, kTok), BH);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kApplySmem;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, lin_f32_apply_kernel, (const float*)a.q, (const float*)a.v, (float*)a.o, state, w, w_batch,
-                         (int)s.H, (int)s.P, (int)s.Hg, (int)s.Wg, nchunk, p.state_elems, a.eps);
-  count_launch();
-  return e;
+  return launch_programmatic(lin_f32_apply_kernel, dim3(ceil_div(N, kTok), BH), kThreads, kApplySmem, st, (const float*)a.q,
+                             (const float*)a.v, (float*)a.o, state, w, w_batch, (int)s.H, (int)s.P, (int)s.Hg, (int)s.Wg, nchunk,
+                             p.state_elems, a.eps);
 }
 
 }  // namespace jv

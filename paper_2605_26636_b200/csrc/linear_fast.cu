@@ -80,9 +80,6 @@ lin_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant
   const int t_begin = chunk * chunk_tokens, t_end = min(N, t_begin + chunk_tokens);
   const int ntiles = (t_end - t_begin + kTileTok - 1) / kTileTok;
 
-  // let the grid that depends on this one (the apply pass) start its set-up as SMs free up
-  griddep_launch_dependents();
-
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStateStages; ++s) {
       mbar_init(&ring->full[s], 1);
@@ -93,6 +90,8 @@ lin_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
+  griddep_wait();
+  griddep_launch_dependents();    // the grids behind this one read the call's inputs ahead of their own waits
   if (*reinterpret_cast<volatile int*>(status) != 0) return;   // an earlier kernel gave up: leave at once
 
   if (warp == 4) {
@@ -572,17 +571,9 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
   if (a.dwc && (e = dwc_static_kernels(a, p, &w, &w_batch, st)) != cudaSuccess) return e;
   const int num_sms = device_sm_count();
   dim3 g1(p.nchunk, BH);
-  if (a.dwc)
-    lin_state_kernel<true><<<g1, kThreads, kStateSmem, st>>>(mk, mv, partial, status, N, p.chunk_tokens, p.state_elems, (int)s.H);
-  else
-    lin_state_kernel<false><<<g1, kThreads, kStateSmem, st>>>(mk, mv, partial, status, N, p.chunk_tokens, p.state_elems, (int)s.H);
-  count_launch();
-  e = cudaGetLastError();
+  e = launch_programmatic(a.dwc ? lin_state_kernel<true> : lin_state_kernel<false>, g1, kThreads, kStateSmem, st, mk, mv, partial, status,
+                          N, p.chunk_tokens, p.state_elems, (int)s.H);
   if (e != cudaSuccess) return e;
-
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
 
   // Every grid behind the state pass is launched with programmatic serialisation and waits for its
   // predecessor (griddepcontrol.wait) before it reads what that one wrote, so completion is transitive along the chain.
@@ -594,17 +585,8 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
     int span = ceil_div(ceil_div(ntokens, nspan), kApplyTok) * kApplyTok;
     if (span < 4 * kApplyTok) span = 4 * kApplyTok;
     nspan = ceil_div(ntokens, span);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nspan, BH);
-    cfg.blockDim = dim3(kApplyThreads);
-    cfg.dynamicSmemBytes = kApplySmem;
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t err = cudaLaunchKernelEx(&cfg, lin_apply_kernel, map_q, map_o, state, status, ntokens,
-                                               span, nchunk, p.state_elems, a.eps, (int)s.H);
-    count_launch();
-    return err;
+    return launch_programmatic(lin_apply_kernel, dim3(nspan, BH), kApplyThreads, kApplySmem, st, map_q, map_o, state, status, ntokens,
+                               span, nchunk, p.state_elems, a.eps, (int)s.H);
   };
 
   if (!a.dwc) {
@@ -628,7 +610,7 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
     const float* state;
     int nchunk;
     if ((e = launch_dwc_generator_fast(a, p, partial, s.P > 0 && s.P <= kGenPrefix, &state, &nchunk, st)) != cudaSuccess) return e;
-    return launch_linear_apply_conv(a, p, state, nchunk, w, w_batch, status, true, st);
+    return launch_linear_apply_conv(a, p, state, nchunk, w, w_batch, status, st);
   }
   // 5 x 5 kernels: generator, apply pass, a read-modify-write pass over o
   const float* state;

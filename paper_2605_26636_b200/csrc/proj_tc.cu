@@ -162,11 +162,24 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
       mbar_init(&bar->acc_empty[a], kCtas * kEpiWarps);      // lane 0 of each epilogue warp
     }
     mbar_init(&bar->drain, 1);
-    // a timeout flagged earlier (by any CTA or launch) makes the rest leave at once: as the leader sees it, for both CTAs
-    bar->abort_flag = *reinterpret_cast<volatile int*>(p.status) != 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if (warp == 0) {
+    __syncwarp();
+    if (kPair) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bar->tmem_base)),
+                   "r"(kTmemCols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bar->tmem_base)),
+                   "r"(kTmemCols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+  }
+  griddep_wait();                            // what is read and written from here on may belong to the launch ahead
+  // a timeout flagged earlier (by any CTA or launch) makes the rest leave at once: as the leader sees it, for both CTAs
+  if (threadIdx.x == 0) bar->abort_flag = *reinterpret_cast<volatile int*>(p.status) != 0;
   uint32_t gave_up;
   if (kPair) {
     __syncwarp();
@@ -180,24 +193,20 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     gave_up = bar->abort_flag;
     __syncthreads();
   }
-  if (gave_up) return;
-  if (kPair && threadIdx.x == 0) bar->abort_flag = 0;
-  if (warp == 0) {
-    __syncwarp();
-    if (kPair) {
-      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bar->tmem_base)),
-                   "r"(kTmemCols) : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    } else {
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bar->tmem_base)),
-                   "r"(kTmemCols) : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-  }
+  if (threadIdx.x == 0) bar->abort_flag = 0;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bar->tmem_base, 0);
+  griddep_launch_dependents();
+  auto free_tmem = [&]() {
+    if (kPair) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  };
+  if (gave_up) {
+    if (warp == 0) free_tmem();
+    return;
+  }
 
   const int tile0 = blockIdx.x / kCtas, tile_step = gridDim.x / kCtas;
 
@@ -370,10 +379,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     __syncthreads();
   }
   tc_fence_after();
-  if (warp == 0) {
-    if (kPair) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
-    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
-  }
+  if (warp == 0) free_tmem();
 }
 
 // ---- host side ----------------------------------------------------------------------
@@ -408,26 +414,14 @@ template <bool kQKV, int kCtas>
 cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& md0, const CUtensorMap& md1, const CUtensorMap& md2,
                    const ProjParams& p, cudaStream_t st) {
   static OncePerDevice opt_in;   // > 48 KB of dynamic shared memory: a per-device function attribute
-  cudaError_t e = opt_in.run([] {
+  const cudaError_t e = opt_in.run([] {
     return cudaFuncSetAttribute(proj_tc_kernel<kQKV, kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<kCtas>());
   });
   if (e != cudaSuccess) return e;
   const int slots = device_sm_count() / kCtas;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kCtas;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kCtas * (p.total_tiles < slots ? p.total_tiles : slots));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem_bytes<kCtas>();
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = kCtas == 2 ? 1 : 0;
-  e = cudaLaunchKernelEx(&cfg, proj_tc_kernel<kQKV, kCtas>, ma, mb, md0, md1, md2, p);
-  count_launch();
-  return e;
+  const dim3 grid(kCtas * (p.total_tiles < slots ? p.total_tiles : slots));
+  if (kCtas == 1) return launch_programmatic(proj_tc_kernel<kQKV, kCtas>, grid, kThreads, smem_bytes<kCtas>(), st, ma, mb, md0, md1, md2, p);
+  return launch_programmatic_cluster(proj_tc_kernel<kQKV, kCtas>, kCtas, grid, kThreads, smem_bytes<kCtas>(), st, ma, mb, md0, md1, md2, p);
 }
 
 // Pairs of CTAs where every pair has three tiles or more: a pair takes 2 us longer to start (cluster launch, two cluster
