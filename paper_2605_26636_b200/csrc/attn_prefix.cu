@@ -205,9 +205,13 @@ cudaError_t launch_attn_prefix(const AttnArgs& a, int ctas, cudaStream_t st) {
   // splits of the keys: at least one 16-key step per warp
   int split = 1;
   while (split < 8 && 2 * split * a.BH * groups <= ctas && split * kWarps * kKeys < N) split *= 2;
-  return launch_programmatic_cluster(attn_prefix_rows_kernel, split, dim3(a.BH * split, groups), kWarps * 32, 0, st,
-                                     (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v,
-                                     (__nv_bfloat16*)a.o, N, a.P, a.scale * 1.4426950408889634f);
+  const dim3 grid(a.BH * split, groups);
+  // A launch of more than one block per SM starts only when the chip is empty: dropped in while the launch ahead drains, its
+  // blocks fill the first SMs two to one and leave the last without (8 x 16 heads, 64 x 64: 97.3 us for the call, 91.0 so; 6 heads,
+  // 48 blocks: 12.1 us programmatically, 14.4 so).
+  return launch_cluster((int)(grid.x * grid.y) <= device_sm_count(), attn_prefix_rows_kernel, split, grid, kWarps * 32, 0, st,
+                        (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, (__nv_bfloat16*)a.o, N, a.P,
+                        a.scale * 1.4426950408889634f);
 }
 
 }  // namespace jv

@@ -540,7 +540,7 @@ cudaError_t launch_linear_d128(const LinArgs& a, const LinPlan& p, cudaStream_t 
   if (nchunk > kMaxCluster) nchunk = kMaxCluster;
   if (nchunk > tiles) nchunk = tiles;
   if (nchunk < 1) nchunk = 1;
-  e = launch_programmatic_cluster(lin128_state_kernel, nchunk, dim3(nchunk, BH), kThreads1, kSmem1, st, mk, mv, state, status, N,
+  e = launch_cluster(true, lin128_state_kernel, nchunk, dim3(nchunk, BH), kThreads1, kSmem1, st, mk, mv, state, status, N,
                                   ceil_div(tiles, nchunk) * kTok1);
   if (e != cudaSuccess) return e;
 

@@ -421,7 +421,7 @@ cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorM
   const int slots = device_sm_count() / kCtas;
   const dim3 grid(kCtas * (p.total_tiles < slots ? p.total_tiles : slots));
   if (kCtas == 1) return launch_programmatic(proj_tc_kernel<kQKV, kCtas>, grid, kThreads, smem_bytes<kCtas>(), st, ma, mb, md0, md1, md2, p);
-  return launch_programmatic_cluster(proj_tc_kernel<kQKV, kCtas>, kCtas, grid, kThreads, smem_bytes<kCtas>(), st, ma, mb, md0, md1, md2, p);
+  return launch_cluster(true, proj_tc_kernel<kQKV, kCtas>, kCtas, grid, kThreads, smem_bytes<kCtas>(), st, ma, mb, md0, md1, md2, p);
 }
 
 // Pairs of CTAs where every pair has three tiles or more: a pair takes 2 us longer to start (cluster launch, two cluster
