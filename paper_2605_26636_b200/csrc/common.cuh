@@ -62,13 +62,15 @@ __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wa
 template <typename... Params, typename... Args>
 cudaError_t launch_cluster(bool programmatic, void (*kernel)(Params...), int cluster, dim3 grid, int threads, size_t smem, cudaStream_t st,
                            Args&&... args) {
-  cudaLaunchAttribute attr[2];                         // a grid of clusters of `cluster` blocks along x (1: no clusters)
+  // a grid of clusters of `cluster` blocks along x; 0: no clusters.  (A kernel that copies between shared memories of a cluster
+  // needs the attribute for a cluster of one, too.)
+  cudaLaunchAttribute attr[2];
   int n = 0;
   if (programmatic) {
     attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[n++].val.programmaticStreamSerializationAllowed = 1;
   }
-  if (cluster > 1) {
+  if (cluster > 0) {
     attr[n].id = cudaLaunchAttributeClusterDimension;
     attr[n].val.clusterDim.x = cluster;
     attr[n].val.clusterDim.y = 1;
@@ -87,7 +89,7 @@ cudaError_t launch_cluster(bool programmatic, void (*kernel)(Params...), int clu
 }
 template <typename... Params, typename... Args>
 cudaError_t launch_programmatic(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args&&... args) {
-  return launch_cluster(true, kernel, 1, grid, threads, smem, st, std::forward<Args>(args)...);
+  return launch_cluster(true, kernel, 0, grid, threads, smem, st, std::forward<Args>(args)...);
 }
 
 // ---- element access -------------------------------------------------------
