@@ -636,7 +636,6 @@ attn_w4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 bool attn_w4_supported(const AttnArgs& a) {
   if (a.dtype != JV_BF16 || a.D != kD) return false;
   if (a.P > kPreRows || (a.P > 0 && a.strided)) return false;
-  if (a.wh >= a.Hg && a.ww >= a.Wg) return false;         // one window: full attention's kernels
   const int ww = a.ww;
   if (ww < 1 || ww > 32 || (ww & (ww - 1)) != 0) return false;   // a warp's 32 rows are whole box rows
   const int bh = kTile / ww;
