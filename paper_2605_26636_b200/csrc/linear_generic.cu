@@ -16,13 +16,15 @@ LinPlan lin_plan(const jv_shape& s, const jv_dwc* dwc) {
   p.D1 = s.D + 1;
   p.state_elems = (p.D1 * p.D1 + 3) / 4 * 4;
   // Chunks: as many as fit one wave of two CTAs per SM over all (batch, head) pairs, each a
-  // multiple of 128 tokens and at least 512 tokens long so that the partials stay small next
-  // to K and V (fp32 tensors: 128, their state pass is bound by arithmetic and short chunks fill the
-  // chip).  One wave means no tail, and chunks of equal length finish together.
+  // multiple of 128 tokens; one wave means no tail, and chunks of equal length finish together.  At least
+  // 512 tokens long where every CTA of the apply pass sums the partials of its head at its start, 128 where
+  // they are summed once per head (beside the kernel generator; fp32 tensors): short chunks fill the chip.  Measured, at least
+  // 512 / 128 tokens: with the convolution, 6 heads of 37 x 37 18.7 / 15.2 us, 16 of 40 x 40 17.4 / 14.3, 12 of 60 x 60 22.4 / 20.6;
+  // without it, 16 of 40 x 40: 11.2 / 13.0.
   int want = (2 * device_sm_count()) / BH;
   if (want < 1) want = 1;
   int chunk = ceil_div(ceil_div(N, want), 128) * 128;
-  const int least = s.dtype == JV_F32 && s.D == 64 ? 128 : 512;
+  const int least = s.D == 64 && (s.dtype == JV_F32 || (dwc && !dwc->token_wise)) ? 128 : 512;
   if (chunk < least) chunk = least;
   p.chunk_tokens = chunk;
   p.nchunk = ceil_div(N, chunk);
