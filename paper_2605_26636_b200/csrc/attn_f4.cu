@@ -57,9 +57,11 @@ struct F4Params {
   int* status;
   int N;                 // tokens per (batch, head)
   int ntiles;            // key (and query) tiles per head: ceil(N / 128)
-  int qgroups;           // groups of four query tiles per head
+  int qt;                // query tiles per group: 4 or 3
+  int qgroups;           // groups per head
   int n_full;            // items [0, n_full) are whole groups, (batch*head, group) with the group fastest;
-  int total_items;       // items [n_full, total_items) are half groups (two query tiles), see launch_attn_f4
+  int total_items;       // items [n_full, total_items) are pieces of groups, see plan_f4
+  int lg_piece;          // query tiles of a piece: 1 or 2
   FastDiv div_qgroups;
   int H;                 // heads per batch element: the inputs are addressed by (head, batch)
   FastDiv div_H;
@@ -81,18 +83,18 @@ constexpr uint32_t kIdescQK = idesc(kTile, kSub, 0);
 constexpr uint32_t kIdescPV = idesc(kTile, kD, 1);
 
 struct Item {
-  int bh, qt0, nt;  // (batch, head), the first of the item's query tiles, and how many it has (4 or 2)
+  int bh, qt0, nt;  // (batch, head), the first of the item's query tiles, and how many it has
 };
-// kHalves: the launch has half groups (n_full < total_items); without them the decode is one division.
-template <bool kHalves>
+// kPieces: the launch has groups of three or pieces of groups; without them the decode is one division.
+template <bool kPieces>
 __device__ __forceinline__ Item decode_item(const F4Params& p, int i) {
   Item it;
-  if (kHalves) {
-    const int half = i - p.n_full;                 // >= 0: a half group
-    const int g = half < 0 ? i : p.n_full + (half >> 1);
+  if (kPieces) {
+    const int k = i - p.n_full, lg = 2 - p.lg_piece;   // k >= 0: piece k of the groups from n_full on, 1 << lg to a group
+    const int g = k < 0 ? i : p.n_full + (k >> lg);
     it.bh = fdiv(g, p.div_qgroups);
-    it.qt0 = kQT * (g - it.bh * p.qgroups) + (half < 0 ? 0 : 2 * (half & 1));
-    it.nt = half < 0 ? kQT : 2;
+    it.qt0 = p.qt * (g - it.bh * p.qgroups) + (k < 0 ? 0 : (k & ((1 << lg) - 1)) << p.lg_piece);
+    it.nt = k < 0 ? p.qt : 1 << p.lg_piece;
   } else {
     it.bh = fdiv(i, p.div_qgroups);
     it.qt0 = kQT * (i - it.bh * p.qgroups);
@@ -101,18 +103,18 @@ __device__ __forceinline__ Item decode_item(const F4Params& p, int i) {
   return it;
 }
 // query tile t of the item exists: inside the item and inside the head
-template <bool kHalves>
+template <bool kPieces>
 __device__ __forceinline__ bool tile_exists(const Item& it, int t, int ntiles) {
-  return (!kHalves || t < it.nt) && it.qt0 + t < ntiles;
+  return (!kPieces || t < it.nt) && it.qt0 + t < ntiles;
 }
 
 // ---- the kernel ------------------------------------------------------------------
 // CTA c works on items c, c + gridDim.x, ...  Every role walks the same item sequence on its own;
 // ring stages and barrier parities follow running counters.  A query tile past the last one of
 // the head (the last item of a head whose tile count is not a multiple of four), or past the item's
-// own two tiles (a half group), is skipped by its softmax warps; its issuer still takes part in the
-// ring protocol so that arrival counts hold.  A half group without any tile is skipped by every role.
-template <bool kHalves>
+// own (a group of three, a piece), is skipped by its softmax warps; its issuer still takes part in the
+// ring protocol so that arrival counts hold.  A piece without any tile is skipped by every role.
+template <bool kPieces>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_f4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapO,
@@ -178,13 +180,13 @@ attn_f4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     uint32_t par = 1;          // parity of the "empty" phase this pass over the ring waits for
     int issued_v = 0;          // for the abort path: V copies issued so far
     for (int i = item0; i < p.total_items && ok; i += item_step) {
-      const Item it = decode_item<kHalves>(p, i);
-      if (kHalves && !tile_exists<kHalves>(it, 0, ntiles)) continue;
+      const Item it = decode_item<kPieces>(p, i);
+      if (kPieces && !tile_exists<kPieces>(it, 0, ntiles)) continue;
       const int b = fdiv(it.bh, p.div_H), h = it.bh - b * p.H;   // coordinates of the input tensor maps
       for (int t = 0; t < kQT && ok; ++t) {
         ok = warp_wait<kSuspendNs>(&bar->q_empty[t], (n & 1) ^ 1, &bar->abort_flag, p.status);
         if (!ok) break;
-        if (tile_exists<kHalves>(it, t, ntiles) && elect_one()) {
+        if (tile_exists<kPieces>(it, t, ntiles) && elect_one()) {
           mbar_expect_tx(&bar->q_full[t], kTileBytes);
           tma_load_4d(sQ + t * kTileBytes, &mapQ, &bar->q_full[t], 0, (it.qt0 + t) * kTile, h, b);
         }
@@ -231,9 +233,9 @@ attn_f4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     uint32_t pcnt[2] = {0, 0};              // steps published so far per tile: parity of p_full
     uint32_t qcnt[2] = {0, 0};              // items in which the tile existed: parity of q_full
     for (int i = item0; i < p.total_items && ok; i += item_step) {
-      const Item it = decode_item<kHalves>(p, i);
-      if (kHalves && !tile_exists<kHalves>(it, 0, ntiles)) continue;
-      const bool ex[2] = {tile_exists<kHalves>(it, tb, ntiles), tile_exists<kHalves>(it, tb + 1, ntiles)};
+      const Item it = decode_item<kPieces>(p, i);
+      if (kPieces && !tile_exists<kPieces>(it, 0, ntiles)) continue;
+      const bool ex[2] = {tile_exists<kPieces>(it, tb, ntiles), tile_exists<kPieces>(it, tb + 1, ntiles)};
       for (int u = 0; u <= nsteps && ok; ++u) {
         const bool has_qk = u < nsteps, has_pv = u > 0;
         if (has_qk && (u & 1) == 0) {       // first half of a key tile: its K must have landed
@@ -319,8 +321,8 @@ attn_f4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     uint32_t ocnt = 0;                // items seen by this tile: parity of o_full
 
     for (int i = item0; i < p.total_items && ok; i += item_step) {
-      const Item it = decode_item<kHalves>(p, i);
-      if (!tile_exists<kHalves>(it, t, ntiles)) continue;   // this query tile does not exist
+      const Item it = decode_item<kPieces>(p, i);
+      if (!tile_exists<kPieces>(it, t, ntiles)) continue;   // this query tile does not exist
       float m = -INFINITY, l = 0.f;
       for (int u = 0; u < nsteps; ++u) {
         ok = warp_wait<kSuspendNs>(&bar->s_full[t], scnt & 1, &bar->abort_flag, p.status);
@@ -455,15 +457,40 @@ attn_f4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 }  // namespace
 
 // Long sequences only: with fewer than eight key tiles the two-tile kernel's deeper pipeline wins.
+namespace {
+// How a launch is cut into items.  A group of four query tiles keeps a CTA's sub-cores busiest, but items are dealt out
+// round-robin and the last round is as long as its longest item, so a problem of one or two rounds may be better off with smaller
+// items, which each take longer per tile.  Measured per 64-key step and item, groups of four = 1: three tiles 0.87, two 0.72,
+// one 0.61; a pair on the two-tile kernel (attn_tc.cu), whose scores are double-buffered, 0.63.
+struct F4Plan {
+  int qt, n_full, total_items, lg_piece;
+  float cost;           // in rounds of groups of four
+};
+F4Plan plan_f4(int ntiles, int BH) {
+  const int sms = device_sm_count();
+  const int g4 = ceil_div(ntiles, 4) * BH, g3 = ceil_div(ntiles, 3) * BH, rem = g4 % sms;
+  // groups of four, those of the last round in pieces if all of the pieces fit it
+  F4Plan a{4, g4, g4, 1, (float)(g4 / sms)};
+  if (rem > 0 && 4 * rem <= sms) a = F4Plan{4, g4 - rem, g4 + 3 * rem, 0, a.cost + 0.61f};
+  else if (rem > 0 && 2 * rem <= sms) a = F4Plan{4, g4 - rem, g4 + rem, 1, a.cost + 0.72f};
+  else if (rem > 0) a.cost += 1.f;
+  const F4Plan b{3, g3, g3, 1, 0.87f * ceil_div(g3, sms)};
+  return b.cost < a.cost ? b : a;
+}
+}  // namespace
+
 bool attn_f4_supported(const AttnArgs& a) {
   if (a.dtype != JV_BF16 || a.D != kD) return false;
   const int64_t N = (int64_t)a.Hg * a.Wg;
   const int64_t ntiles = (N + kTile - 1) / kTile;
+  if (ntiles * a.BH > 0x7fffffffll) return false;
   // Shorter sequences: where the last group of four is (almost) full and there are groups for half the SMs.  Measured, this kernel /
   // the two-tile kernel: 96 heads of 400 tokens 17.1 / 20.5 us, 288 of 324: 21.0 / 29.4, 48 of 900: 27.5 / 33.2; 96 of 576 (a last group of
   // one) 28.4 / 23.7, 48 of 700 (of two) 21.3 / 16.2, 16 of 800 17.3 / 16.6, 6 of 1000 18.8 / 17.6.
   if (N < 8 * kTile && ((ntiles & 3) == 1 || (ntiles & 3) == 2 || 2 * (ntiles + 3) / 4 * a.BH < device_sm_count())) return false;
-  if ((ntiles + kQT - 1) / kQT * a.BH > 0x7fffffffll) return false;
+  // Few query tiles: pairs on the two-tile kernel, if that has fewer rounds' worth of work (12 heads of 3025 tokens 46.6 / 50.7 us,
+  // 6 of 4272 63.0 / 68.6, 16 of 2106 34.8 / 37.6, 6 of 1370 23.0 / 24.8).
+  if (0.63f * ceil_div(ceil_div((int)ntiles, 2) * a.BH, device_sm_count()) < plan_f4((int)ntiles, a.BH).cost) return false;
   return encode_fn() != nullptr;
 }
 
@@ -504,21 +531,18 @@ cudaError_t launch_attn_f4(const AttnArgs& a, int* status, cudaStream_t st) {
   p.status = status;
   p.N = N;
   p.ntiles = ceil_div(N, kTile);
-  p.qgroups = ceil_div(p.ntiles, kQT);
-  // Items are dealt out round-robin, so the last round is as long as a full one however few CTAs it
-  // keeps busy.  When it would keep at most half of them busy, its groups are split into half groups
-  // of two query tiles (a serial per-tile chain makes those finish in a little over half the time).
-  const int groups = p.qgroups * a.BH;
-  const int rem = groups % num_sms;
-  const int split = (rem > 0 && rem <= num_sms / 2) ? rem : 0;
-  p.n_full = groups - split;
-  p.total_items = groups + split;
+  const F4Plan plan = plan_f4(p.ntiles, a.BH);
+  p.qt = plan.qt;
+  p.qgroups = ceil_div(p.ntiles, p.qt);
+  p.n_full = plan.n_full;
+  p.total_items = plan.total_items;
+  p.lg_piece = plan.lg_piece;
   p.div_qgroups = make_fastdiv((uint32_t)p.qgroups);
   p.H = a.H;
   p.div_H = make_fastdiv((uint32_t)a.H);
   p.scale_log2 = a.scale * 1.4426950408889634f;
   const int grid = p.total_items < num_sms ? p.total_items : num_sms;
-  return launch_programmatic(split ? attn_f4_kernel<true> : attn_f4_kernel<false>, dim3(grid), kThreads, kSmemBytes, st, maps[0], maps[1],
+  return launch_programmatic(p.qt < kQT || p.total_items > p.n_full ? attn_f4_kernel<true> : attn_f4_kernel<false>, dim3(grid), kThreads, kSmemBytes, st, maps[0], maps[1],
                              maps[2], maps[3], p);
 }
 

@@ -1,4 +1,4 @@
-"""Full attention on sequences below 1024 tokens: at most two tiles on the window kernel (one token, a tile less one, a tile,
+"""Full attention by length and heads.  Below 1024 tokens: at most two tiles on the window kernel (one token, a tile less one, a tile,
 a tile and one, two tiles), the rest by heads and tiles on the four-tile or the two-tile kernel; q, k, v contiguous and in a
 fused activation."""
 import pytest
@@ -42,3 +42,22 @@ def test_short_sequences(jv, oracle, case, fused):
     pick = lambda t: torch.stack([t[b, h] for b, h in heads]).unsqueeze(0)
     assert rel_err(pick(out.cpu()), oracle.full_attn(pick(q), pick(k), pick(v))) <= TOL["bf16"], case
     assert bool(torch.isfinite(out).all())
+
+
+# B, H, N: groups of three (the last of a head with two tiles, and whole), single tiles and pairs of tiles in the last round
+# (the last piece of a head empty, or its last tile ragged), pairs on the two-tile kernel
+SPLITS = [(1, 16, 2880), (1, 16, 3070), (2, 19, 2048), (2, 19, 1600), (1, 26, 4096), (2, 13, 4000), (1, 12, 3025)]
+
+
+@pytest.mark.parametrize("case", SPLITS, ids=lambda c: "x".join(map(str, c)))
+def test_items_of_three_tiles_and_pieces(jv, oracle, case):
+    B, H, N = case
+    q, k, v = inputs.custom_qkv(B, H, N, 64, "bf16", seed=4200 + N + H)
+    out, check = guarded_empty(q.shape, torch.bfloat16, DEV)
+    out.fill_(float("nan"))
+    jv.full_attn(*(t.to(DEV) for t in (q, k, v)), out=out)
+    check()
+    assert bool(torch.isfinite(out).all())
+    heads = [(0, 0), (B - 1, H - 1)]                   # the last head's groups are the ones cut into pieces
+    pick = lambda t: torch.stack([t[b, h] for b, h in heads]).unsqueeze(0)
+    assert rel_err(pick(out.cpu()), oracle.full_attn(pick(q), pick(k), pick(v))) <= TOL["bf16"], case
