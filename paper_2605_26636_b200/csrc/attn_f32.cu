@@ -4,19 +4,22 @@
 // What bounds it: the FMA pipes (4 * 64 flop per query-key pair; 128 multiply-adds per clock and SM).  A warp
 // owns 16 query rows and walks tiles of 64 keys; a lane owns 8 rows x 4 keys of the scores (keys lane % 16 + 16 j)
 // and 8 rows x 4 channels of the output.  Multiply-adds are packed pairs (fma.rn.f32x2: even and odd channels
-// in QK^T, two neighbouring channels in PV), fed by 128-bit shared-memory loads: 12 loads per 64 packed
-// multiply-adds, half of what the shared-memory port could deliver, so the FMA pipes stay the limit.  The rows of a
+// in QK^T, two neighbouring rows in PV), fed by 128-bit shared-memory loads: 12 loads per 64 packed
+// multiply-adds, three quarters of what the shared-memory port could deliver.  The rows of a
 // warp see all keys of a tile inside that warp: row maxima are 16-lane shuffles and the probabilities pass from the
-// score layout to the PV layout through the warp's own shared memory, without a CTA barrier.
+// score layout to the PV layout through the warp's own shared memory, without a CTA barrier.  They are kept by key, so that
+// a load gives pairs of rows and a value is doubled once for eight rows (kept by row, with pairs of channels, every
+// probability had to be doubled: 98 us where this takes 93).
 //
 // A CTA is R row warps x G key groups: group g takes the key tiles g, g + G, ... through its own buffer (K, then V in its
 // place: with three CTAs on an SM the others compute while one waits for a copy), and the groups' partial softmaxes are
 // merged at the end.
 //
 // Measured (12 heads, 32 x 32 tokens; the kernel of one warp per query row, which served these calls before and still
-// serves other head dims, in brackets): full attention 100 us (729), 16 x 16 windows 31 us (195); 6 heads, 16 x 16
-// tokens, full attention 10 us (63).  Full attention runs at 32 TFLOP/s of the 73 that a loop of nothing but multiply-adds
-// reaches: two of five instructions are not multiply-adds, and the registers leave room for three warps per scheduler.
+// serves other head dims, in brackets): full attention 93 us (729), 16 x 16 windows 27 us (195); 6 heads, 16 x 16
+// tokens, full attention 8 us (63).  Full attention runs at 35 TFLOP/s (41 where the grid fills the chip evenly) of the 73 that
+// a loop of nothing but multiply-adds reaches: one of three instructions is not a multiply-add, and the registers leave room
+// for three warps per scheduler.
 #include "f32_common.cuh"
 
 namespace jv {
@@ -28,21 +31,24 @@ constexpr int kDim = 64;
 constexpr int kKeys = 64;        // keys per tile
 constexpr int kRowsWarp = 16;    // query rows per warp
 constexpr int kLd = 68;          // floats per shared-memory row: 16-byte reads of 8 consecutive rows touch all banks
+constexpr int kLdP = 20;         // floats per key of the transposed probabilities (16 rows): 16-byte writes of 8 keys likewise
+constexpr int kWarpBuf = kKeys * kLdP;  // floats of a warp's own buffer
+static_assert(kWarpBuf >= kRowsWarp * kLd, "the buffer takes the warp's output as well");
 
 template <int R, int G>
 constexpr size_t smem_bytes() {
-  return (size_t)(R * kRowsWarp + R * G * kRowsWarp + G * kKeys) * kLd * sizeof(float);
+  return ((size_t)(R * kRowsWarp + G * kKeys) * kLd + R * G * kWarpBuf) * sizeof(float);
 }
 
 // prefix_rows: the launch serves the P prefix queries (keys: all tokens) instead of the windows.
 template <int R, int G>
-__global__ void __launch_bounds__(32 * R * G, 3)
+__global__ void __launch_bounds__(32 * R * G, G == 4 ? 2 : 3)  // what shared memory leaves room for
 attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ o,
                 int Hg, int Wg, int P, int wh, int ww, int nwx, bool prefix_rows, bool overlap, float scale) {
   extern __shared__ __align__(16) float smem_f[];
   float* qs = smem_f;                                        // [16 R][kLd]
-  float* ps = qs + R * kRowsWarp * kLd;                      // [R G warps][16][kLd]: probabilities, then the warp's output
-  float* ks = ps + R * G * kRowsWarp * kLd;                  // [G][64][kLd]: the group's K tile, then its V tile
+  float* ps = qs + R * kRowsWarp * kLd;                      // [R G warps]: probabilities [64 keys][kLdP], then the warp's output [16][kLd]
+  float* ks = ps + R * G * kWarpBuf;                  // [G][64][kLd]: the group's K tile, then its V tile
   // overlap: the launch ahead is that of the prefix queries (it has waited for what came before it); waited for at the end
   if (!overlap) griddep_wait();
   griddep_launch_dependents();
@@ -89,7 +95,7 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
   };
 
   float* kg = ks + grp * kKeys * kLd;
-  float* pw = ps + warp * kRowsWarp * kLd;
+  float* pw = ps + warp * kWarpBuf;
   const int ntiles = (cnt + kKeys - 1) / kKeys;
 
   if (grp == 0) {                                            // Q: group 0 copies the CTA's rows
@@ -110,13 +116,16 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
 
   const float* qr = qs + (rw * kRowsWarp + ty * 8) * kLd;
   float m[8], l[8];
-  f32x2 acc[8][2];
+  f32x2 acc[4][4];                                           // rows 2 i and 2 i + 1, channel 4 tx + e
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     m[i] = -INFINITY;
     l[i] = 0.f;
-    acc[i][0] = acc[i][1] = 0ull;
   }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) acc[i][e] = 0ull;
 
   for (int t = grp; t < ntiles; t += G) {
     copy_wait<0>();                                          // K of this tile
@@ -146,51 +155,56 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
 
     const bool ragged = (t + 1) * kKeys > cnt;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      float s[4];
+    for (int h = 0; h < 2; ++h) {                            // four rows at a time
+      float p[4][4], alpha[4];                               // [key][row]
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float2 e = unpack2(s2[i][j]);
-        s[j] = (e.x + e.y) * scale;
-        if (ragged && t * kKeys + tx + 16 * j >= cnt) s[j] = -INFINITY;
+      for (int r = 0; r < 4; ++r) {
+        const int i = 4 * h + r;
+        float s[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float2 e = unpack2(s2[i][j]);
+          s[j] = (e.x + e.y) * scale;
+          if (ragged && t * kKeys + tx + 16 * j >= cnt) s[j] = -INFINITY;
+        }
+        float mx = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
+#pragma unroll
+        for (int w = 1; w < 16; w <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
+        const float mn = fmaxf(m[i], mx);                    // finite: every tile holds at least one key
+        alpha[r] = expf(m[i] - mn);                          // exp(-inf) = 0 on the first tile
+        m[i] = mn;
+        float sum = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          p[j][r] = expf(s[j] - mn);
+          sum += p[j][r];
+        }
+        l[i] = fmaf(l[i], alpha[r], sum);
       }
-      float mx = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
 #pragma unroll
-      for (int w = 1; w < 16; w <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
-      const float mn = fmaxf(m[i], mx);                      // finite: every tile holds at least one key
-      const float alpha = expf(m[i] - mn);                   // exp(-inf) = 0 on the first tile
-      m[i] = mn;
-      float sum = 0.f;
+      for (int j = 0; j < 4; ++j)
+        *reinterpret_cast<float4*>(pw + (tx + 16 * j) * kLdP + ty * 8 + 4 * h) = make_float4(p[j][0], p[j][1], p[j][2], p[j][3]);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float p = expf(s[j] - mn);
-        sum += p;
-        pw[(ty * 8 + i) * kLd + tx + 16 * j] = p;
+      for (int r = 0; r < 2; ++r) {
+        const f32x2 a2 = pack2(alpha[2 * r], alpha[2 * r + 1]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[2 * h + r][e] = mul2(acc[2 * h + r][e], a2);
       }
-      l[i] = fmaf(l[i], alpha, sum);
-      const f32x2 a2 = pack2(alpha, alpha);
-      acc[i][0] = mul2(acc[i][0], a2);
-      acc[i][1] = mul2(acc[i][1], a2);
     }
     copy_wait<0>();                                          // V of this tile
     group_sync();                                            // (also orders the warp's own probabilities)
-#pragma unroll 4
-    for (int c = 0; c < kKeys; c += 4) {
-      ulonglong2 vv[4];
+#pragma unroll 8
+    for (int c = 0; c < kKeys; ++c) {
+      const float4 v4 = *reinterpret_cast<const float4*>(kg + c * kLd + 4 * tx);
+      const ulonglong2 pa = *reinterpret_cast<const ulonglong2*>(pw + c * kLdP + ty * 8);
+      const ulonglong2 pb = *reinterpret_cast<const ulonglong2*>(pw + c * kLdP + ty * 8 + 4);
+      const f32x2 vv[4] = {pack2(v4.x, v4.x), pack2(v4.y, v4.y), pack2(v4.z, v4.z), pack2(v4.w, v4.w)};
 #pragma unroll
-      for (int j = 0; j < 4; ++j) vv[j] = *reinterpret_cast<const ulonglong2*>(kg + (c + j) * kLd + 4 * tx);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float4 pp = *reinterpret_cast<const float4*>(pw + (ty * 8 + i) * kLd + c);
-        const f32x2 p0 = pack2(pp.x, pp.x), p1 = pack2(pp.y, pp.y), p2 = pack2(pp.z, pp.z), p3 = pack2(pp.w, pp.w);
-        fma2(acc[i][0], p0, vv[0].x);
-        fma2(acc[i][1], p0, vv[0].y);
-        fma2(acc[i][0], p1, vv[1].x);
-        fma2(acc[i][1], p1, vv[1].y);
-        fma2(acc[i][0], p2, vv[2].x);
-        fma2(acc[i][1], p2, vv[2].y);
-        fma2(acc[i][0], p3, vv[3].x);
-        fma2(acc[i][1], p3, vv[3].y);
+      for (int e = 0; e < 4; ++e) {
+        fma2(acc[0][e], pa.x, vv[e]);
+        fma2(acc[1][e], pa.y, vv[e]);
+        fma2(acc[2][e], pb.x, vv[e]);
+        fma2(acc[3][e], pb.y, vv[e]);
       }
     }
     group_sync();                                            // the group is done with V (and the warp with its P)
@@ -206,10 +220,13 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     float* dst = pw + (ty * 8 + i) * kLd;
-    ulonglong2 x;
-    x.x = acc[i][0];
-    x.y = acc[i][1];
-    *reinterpret_cast<ulonglong2*>(dst + 4 * tx) = x;
+    float x[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float2 y = unpack2(acc[i / 2][e]);
+      x[e] = i % 2 ? y.y : y.x;
+    }
+    *reinterpret_cast<float4*>(dst + 4 * tx) = make_float4(x[0], x[1], x[2], x[3]);
     if (tx == 0) {
       dst[64] = m[i];
       dst[65] = l[i];
@@ -223,12 +240,12 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
     if (row < nq) {
       float M = -INFINITY;
 #pragma unroll
-      for (int g = 0; g < G; ++g) M = fmaxf(M, ps[((g * R + rw) * kRowsWarp + r) * kLd + 64]);
+      for (int g = 0; g < G; ++g) M = fmaxf(M, ps[(g * R + rw) * kWarpBuf + r * kLd + 64]);
       float L = 0.f;
       float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int g = 0; g < G; ++g) {
-        const float* src = ps + ((g * R + rw) * kRowsWarp + r) * kLd;
+        const float* src = ps + (g * R + rw) * kWarpBuf + r * kLd;
         const float f = expf(src[64] - M);                   // a group without a tile: exp(-inf) = 0
         const float4 y = *reinterpret_cast<const float4*>(src + 4 * tx);
         L = fmaf(src[65], f, L);
@@ -265,9 +282,12 @@ bool attn_f32_supported(const AttnArgs& a) { return a.dtype == JV_F32 && a.D == 
 
 // The P prefix queries go first, with the keys of a row tile split over four groups (their chain is the
 // longest: all N keys); the windows' launch overlaps them, as neither reads what the other writes.
-// 32 rows x 2 groups per CTA, unless that leaves the chip nearly empty: then 16 rows x 4 groups, which halves a CTA's
-// chain.  Measured, 32 x 2 against 16 x 4: 48 CTAs of 32 rows 16 / 10 us, 156 CTAs 39 / 34 us, 258 CTAs 98 / 110 us, 384 CTAs
-// 103 / 115 us; windows of one or two key tiles have no work for four groups (432 CTAs, 8 x 8 windows: 18 / 33 us).
+// 32 rows x 2 groups per CTA (three on an SM) or 16 rows x 4 groups (two): the second halves the chain of a CTA, and its
+// finer grain leaves less of the last round empty; the first is 10 % faster where both fill the chip.  Measured, 32 x 2 against
+// 16 x 4 with up to two CTAs of 32 rows per SM: 48 CTAs 13 / 8 us, 150 CTAs 57 / 33, 256 CTAs 92 / 69.  Beyond that by
+// rounds, at 9 to 5 for one round of either: 300 CTAs 78 / 60 us (3 and 5 rounds), 384 CTAs 93 / 99 (3 and 6), 512 CTAs
+// 122 / 116 (4 and 7), 688 CTAs 202 / 222 (5 and 10).  Windows of one or two key tiles have no work for four groups (432
+// CTAs, 8 x 8 windows: 18 / 33 us).
 cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st) {
   const int wh = a.wh < a.Hg ? a.wh : a.Hg, ww = a.ww < a.Wg ? a.ww : a.Wg;
   const bool prefix = a.P > 0;
@@ -276,7 +296,8 @@ cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
   }
   const int64_t ctas = (int64_t)ceil_div(a.Wg, ww) * ceil_div(a.Hg, wh) * a.BH * ceil_div(wh * ww, 2 * kRowsWarp);
-  if (4 * ctas <= 5 * device_sm_count() && wh * ww + a.P > 2 * kKeys) return launch<1, 4>(a, false, prefix, st);
+  const int64_t sms = device_sm_count(), rounds2 = (ctas + sms - 1) / sms, rounds1 = (2 * ctas + sms - 1) / sms;
+  if (wh * ww + a.P > 2 * kKeys && (rounds2 <= 2 || 5 * rounds1 <= 9 * rounds2)) return launch<1, 4>(a, false, prefix, st);
   return launch<2, 2>(a, false, prefix, st);
 }
 
