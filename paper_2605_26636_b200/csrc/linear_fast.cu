@@ -620,8 +620,7 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
   dim3 g4(ceil_div(ceil_div(N, run), 8), BH);
   const __nv_bfloat16* v = (const __nv_bfloat16*)a.v;
   __nv_bfloat16* o = (__nv_bfloat16*)a.o;
-  if (a.dwc->k == 3) dwc_add_kernel<3><<<g4, 256, 0, st>>>(v, o, w, w_batch, s.H, s.Hg, s.Wg, run);
-  else dwc_add_kernel<5><<<g4, 256, 0, st>>>(v, o, w, w_batch, s.H, s.Hg, s.Wg, run);
+  dwc_add_kernel<5><<<g4, 256, 0, st>>>(v, o, w, w_batch, s.H, s.Hg, s.Wg, run);
   count_launch();
   return cudaGetLastError();
 }

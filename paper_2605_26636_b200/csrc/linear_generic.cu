@@ -233,13 +233,6 @@ cudaError_t launch_generic_t(const LinArgs& a, const LinPlan& p, cudaStream_t st
 
 }  // namespace
 
-cudaError_t launch_lin_reduce(const float* partial, float* state, int nchunk, int state_elems, size_t total,
-                              cudaStream_t st) {
-  lin_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(partial, state, nchunk, state_elems, total);
-  count_launch();
-  return cudaGetLastError();
-}
-
 cudaError_t launch_dwc_generator(const LinArgs& a, const LinPlan& p, const float* vsum, int bh_stride,
                                  cudaStream_t st) {
   const jv_shape& s = a.s;

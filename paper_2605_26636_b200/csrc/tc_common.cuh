@@ -153,15 +153,7 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
   if (elect_one())
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// D[tmem] (+)= A[smem] * B[smem]
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-  if (elect_one())
-  asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
-}
-// The same, to be called by ONE lane (the caller holds the election): a run of MMAs issued back to
+// D[tmem] (+)= A[smem] * B[smem], to be called by ONE lane (the caller holds the election): a run of MMAs issued back to
 // back by one thread, without an election and a branch around each of them.
 __device__ __forceinline__ void mma_ss_1(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
   asm volatile(
