@@ -149,6 +149,11 @@ jv_status run_attn(const void* q, const void* k, const void* v, void* o, const j
       return from_cuda(launch_attn_w4(w, status, st));
     }
   }
+  if (!g_force_generic.load() && one_window && attn_split_supported(a)) {
+    int* status = device_status_ptr();
+    if (!status) return JV_ERR_CUDA;
+    return from_cuda(launch_attn_split(a, status, st));
+  }
   if (!g_force_generic.load() && one_window && attn_f4_supported(a)) {
     int* status = device_status_ptr();
     if (!status) return JV_ERR_CUDA;

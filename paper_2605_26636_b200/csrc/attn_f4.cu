@@ -1,4 +1,4 @@
-// Full softmax attention (Eq. 1) for long sequences on the 5th-generation tensor cores:
+// Full softmax attention (Eq. 1) on the 5th-generation tensor cores:
 // four 128-row query tiles per CTA, so that every SM sub-core holds four softmax warps.
 // bf16 tensors, head_dim 64.
 //
@@ -454,10 +454,6 @@ attn_f4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 }
 
 // ---- host side ----------------------------------------------------------------------
-}  // namespace
-
-// Long sequences only: with fewer than eight key tiles the two-tile kernel's deeper pipeline wins.
-namespace {
 // How a launch is cut into items.  A group of four query tiles keeps a CTA's sub-cores busiest, but items are dealt out
 // round-robin and the last round is as long as its longest item, so a problem of one or two rounds may be better off with smaller
 // items, which each take longer per tile.  Measured per 64-key step and item, groups of four = 1: three tiles 0.87, two 0.72,
@@ -477,7 +473,13 @@ F4Plan plan_f4(int ntiles, int BH) {
   const F4Plan b{3, g3, g3, 1, 0.87f * ceil_div(g3, sms)};
   return b.cost < a.cost ? b : a;
 }
+float tc_cost(int ntiles, int BH) { return 0.63f * ceil_div(ceil_div(ntiles, 2) * BH, device_sm_count()); }
 }  // namespace
+
+float attn_f4_cost(int ntiles, int BH) {
+  const float f4 = plan_f4(ntiles, BH).cost, tc = tc_cost(ntiles, BH);
+  return tc < f4 ? tc : f4;
+}
 
 bool attn_f4_supported(const AttnArgs& a) {
   if (a.dtype != JV_BF16 || a.D != kD) return false;
@@ -490,11 +492,11 @@ bool attn_f4_supported(const AttnArgs& a) {
   if (N < 8 * kTile && ((ntiles & 3) == 1 || (ntiles & 3) == 2 || 2 * (ntiles + 3) / 4 * a.BH < device_sm_count())) return false;
   // Few query tiles: pairs on the two-tile kernel, if that has fewer rounds' worth of work (12 heads of 3025 tokens 46.6 / 50.7 us,
   // 6 of 4272 63.0 / 68.6, 16 of 2106 34.8 / 37.6, 6 of 1370 23.0 / 24.8).
-  if (0.63f * ceil_div(ceil_div((int)ntiles, 2) * a.BH, device_sm_count()) < plan_f4((int)ntiles, a.BH).cost) return false;
+  if (tc_cost((int)ntiles, a.BH) < plan_f4((int)ntiles, a.BH).cost) return false;
   return encode_fn() != nullptr;
 }
 
-cudaError_t launch_attn_f4(const AttnArgs& a, int* status, cudaStream_t st) {
+cudaError_t launch_attn_f4(const AttnArgs& a, int* status, cudaStream_t st, int whole_groups) {
   EncodeFn enc = encode_fn();
   if (!enc) return cudaErrorNotSupported;
   const int N = a.Hg * a.Wg;
@@ -531,9 +533,9 @@ cudaError_t launch_attn_f4(const AttnArgs& a, int* status, cudaStream_t st) {
   p.status = status;
   p.N = N;
   p.ntiles = ceil_div(N, kTile);
-  const F4Plan plan = plan_f4(p.ntiles, a.BH);
+  const F4Plan plan = whole_groups > 0 ? F4Plan{kQT, whole_groups, whole_groups, 1, 0.f} : plan_f4(p.ntiles, a.BH);
   p.qt = plan.qt;
-  p.qgroups = ceil_div(p.ntiles, p.qt);
+  p.qgroups = whole_groups > 0 ? p.ntiles / kQT : ceil_div(p.ntiles, p.qt);
   p.n_full = plan.n_full;
   p.total_items = plan.total_items;
   p.lg_piece = plan.lg_piece;

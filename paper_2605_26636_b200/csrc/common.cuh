@@ -176,9 +176,16 @@ cudaError_t launch_attn_w4(const AttnArgs& a, int* status, cudaStream_t st);
 // full = true: F over all N tokens; else W with windows whose width is a power of two <= 128
 bool attn_d128_supported(const AttnArgs& a, bool full);
 cudaError_t launch_attn_d128(const AttnArgs& a, bool full, int* status, cudaStream_t st);
-// tcgen05 path for full attention over long sequences (bf16, D == 64, N >= 1024): four query tiles per CTA
+// tcgen05 path for full attention (bf16, D == 64), one query tile per CTA with its keys over four slots: all of a call, or what is left of
+// it behind whole rounds of the four-tile kernel, by the cost of either
+bool attn_split_supported(const AttnArgs& a);
+cudaError_t launch_attn_split(const AttnArgs& a, int* status, cudaStream_t st);
+// tcgen05 path for full attention (bf16, D == 64): four query tiles per CTA
 bool attn_f4_supported(const AttnArgs& a);
-cudaError_t launch_attn_f4(const AttnArgs& a, int* status, cudaStream_t st);
+// whole_groups > 0: only that many groups of four query tiles, of the floor(tiles / 4) whole ones of every head, head by head
+cudaError_t launch_attn_f4(const AttnArgs& a, int* status, cudaStream_t st, int whole_groups = 0);
+// time of a call on this kernel or the two-tile one, whichever is shorter, in rounds of items of four query tiles
+float attn_f4_cost(int ntiles, int BH);
 
 struct LinArgs {
   const void *q, *k, *v;
@@ -217,8 +224,6 @@ cudaError_t launch_linear_apply_conv(const LinArgs& a, const LinPlan& p, const f
 // s = vsum / N read from vsum[bh * bh_stride + e]
 cudaError_t launch_dwc_generator(const LinArgs& a, const LinPlan& p, const float* vsum, int bh_stride,
                                  cudaStream_t st);
-cudaError_t launch_lin_reduce(const float* partial, float* state, int nchunk, int state_elems, size_t total,
-                              cudaStream_t st);
 
 // Focused feature map of Eq. 3 over every token row of q and k -> qf, kf (same shape and type)
 cudaError_t launch_focus_map(const void* q, const void* k, void* qf, void* kf, const jv_shape& s, float p, cudaStream_t st);
