@@ -168,8 +168,7 @@ jv_status run_attn(const void* q, const void* k, const void* v, void* o, const j
     int* status = device_status_ptr();
     if (!status) return JV_ERR_CUDA;
     if (a.P > 0) {                                        // the P prefix queries, which attend everything
-      const int free_sms = device_sm_count() - attn_w4_ctas(a);
-      const jv_status r = from_cuda(launch_attn_prefix(a, free_sms > 0 ? free_sms : 2 * device_sm_count(), st));
+      const jv_status r = from_cuda(launch_attn_prefix(a, device_sm_count() - attn_w4_ctas(a), st));
       if (r != JV_OK) return r;
     }
     return from_cuda(launch_attn_w4(a, status, st));
@@ -179,7 +178,7 @@ jv_status run_attn(const void* q, const void* k, const void* v, void* o, const j
     if (!status) return JV_ERR_CUDA;
     if (a.strided && a.P > 0) return JV_ERR_UNSUPPORTED;  // the prefix queries' kernel reads contiguous tensors
     if (a.P > 0) {
-      const jv_status r = from_cuda(launch_attn_prefix(a, 2 * device_sm_count(), st));
+      const jv_status r = from_cuda(launch_attn_prefix(a, 0, st));
       if (r != JV_OK) return r;
     }
     return from_cuda(launch_attn_tc(a, full, status, st));

@@ -199,17 +199,27 @@ attn_prefix_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16
 // only after it: this one is short and, on small problems, leaves most SMs free.  Behind the windows it took 2 us of its own
 // even there (6 heads, 37 x 37 tokens), and a persistent kernel of the windows leaves it no SM until it ends.
 // ctas: how many blocks it should have at most (it has at least one per (batch, head) and group).
-cudaError_t launch_attn_prefix(const AttnArgs& a, int ctas, cudaStream_t st) {
+//
+// Beside the windows, on the SMs that their launch leaves free, if there is a block for every head and none has more than 24 steps to
+// walk; else on the whole chip ahead of them.  Measured, beside / ahead: 24 heads, 48 x 48 tokens, 40 SMs free, 18 steps: 15.5 / 20.6 us
+// for the call; 16 heads, 64 x 64, 20 SMs free, 33 steps: 23.1 / 20.6.
+// Ahead, the launch is a plain one: dropped in while the launch before it drains, its blocks fill the first SMs two to one
+// and leave the last without.  Programmatically / plainly: 8 x 16 heads, 64 x 64 tokens 97.5 / 90.9 us for the call, 16 heads, 128 x 128
+// tokens 64.8 / 58.5, 24 heads, 40 x 60 22.0 / 22.9; beside, 6 heads, 37 x 37: 11.9 / 14.1.
+cudaError_t launch_attn_prefix(const AttnArgs& a, int free_sms, cudaStream_t st) {
   if (a.dtype != JV_BF16 || a.D != kD || a.strided) return cudaErrorNotSupported;   // (the callers are the bf16 tensor-core paths)
   const int N = a.P + a.Hg * a.Wg, groups = ceil_div(a.P, kRows);
-  // splits of the keys: at least one 16-key step per warp
-  int split = 1;
-  while (split < 8 && 2 * split * a.BH * groups <= ctas && split * kWarps * kKeys < N) split *= 2;
+  // splits of the keys over at most `ctas` blocks: at least one 16-key step per warp
+  auto split_for = [&](int64_t ctas) {
+    int split = 1;
+    while (split < 8 && 2ll * split * a.BH * groups <= ctas && split * kWarps * kKeys < N) split *= 2;
+    return split;
+  };
+  int split = split_for(free_sms);
+  const bool beside = (int64_t)a.BH * groups <= free_sms && ceil_div(N, split * kWarps * kKeys) <= 24;
+  if (!beside) split = split_for(2 * device_sm_count());
   const dim3 grid(a.BH * split, groups);
-  // A launch of more than one block per SM starts only when the chip is empty: dropped in while the launch ahead drains, its
-  // blocks fill the first SMs two to one and leave the last without (8 x 16 heads, 64 x 64: 97.3 us for the call, 91.0 so; 6 heads,
-  // 48 blocks: 12.1 us programmatically, 14.4 so).
-  return launch_cluster((int)(grid.x * grid.y) <= device_sm_count(), attn_prefix_rows_kernel, split, grid, kWarps * 32, 0, st,
+  return launch_cluster(beside, attn_prefix_rows_kernel, split, grid, kWarps * 32, 0, st,
                         (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, (__nv_bfloat16*)a.o, N, a.P,
                         a.scale * 1.4426950408889634f);
 }

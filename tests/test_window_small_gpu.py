@@ -34,6 +34,8 @@ CASES = [  # B, H, P, Hg, Wg, wh, ww, fused activation
     (1, 2, 7, 31, 20, 16, 8, False),
     (3, 5, 0, 41, 23, 16, 8, False),
     (8, 16, 5, 33, 47, 16, 16, False),
+    (1, 16, 5, 64, 64, 16, 16, False),   # the prefix queries ahead of the windows although a few SMs are free
+    (1, 24, 1, 40, 60, 16, 16, False),
 ]
 
 
