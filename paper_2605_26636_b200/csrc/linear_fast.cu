@@ -62,10 +62,10 @@ struct __align__(8) Ring {
 };
 
 // ---- pass 1: partial state of one token chunk ------------------------------------
-constexpr int kStateStages = 6;               // 6 x (K tile + V tile) = 96 KB per CTA, two CTAs per SM
-constexpr size_t kStateSmem = (size_t)kStateStages * 2 * kTileBytes + 1024 + sizeof(Ring);
+// kStages x (K tile + V tile): 6 = 96 KB per CTA, two CTAs per SM; 3 = 48 KB, four
+constexpr size_t state_smem(int stages) { return (size_t)stages * 2 * kTileBytes + 1024 + sizeof(Ring); }
 
-template <bool kVsum>
+template <bool kVsum, int kStages>
 __global__ void __launch_bounds__(kThreads)
 lin_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV,
                  float* __restrict__ partial, int* status, int N, int chunk_tokens, int state_elems, int H) {
@@ -73,7 +73,7 @@ lin_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant
   // 1024-byte alignment by an offset from the array itself, so that accesses stay shared-space loads and stores
   unsigned char* smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t smem = smem_u32(smem_al);      // stage s: K tile at s * 16 KB, V tile at s * 16 KB + 8 KB
-  Ring* ring = reinterpret_cast<Ring*>(smem_al + (size_t)kStateStages * 2 * kTileBytes);
+  Ring* ring = reinterpret_cast<Ring*>(smem_al + (size_t)kStages * 2 * kTileBytes);
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int bh = blockIdx.y, chunk = blockIdx.x;
   const int in_b = bh / H, in_h = bh - in_b * H;      // coordinates of the input tensor maps
@@ -81,7 +81,7 @@ lin_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant
   const int ntiles = (t_end - t_begin + kTileTok - 1) / kTileTok;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStateStages; ++s) {
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(&ring->full[s], 1);
       mbar_init(&ring->empty[s], 4);          // one arrival per MMA warp
     }
@@ -115,12 +115,12 @@ lin_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant
       }
       __syncwarp();
       ++issued;
-      if (++s == kStateStages) { s = 0; par ^= 1; }
+      if (++s == kStages) { s = 0; par ^= 1; }
     }
     if (!ok && lane == 0) {   // let the copies in flight land before the CTA leaves
       const unsigned long long t0 = globaltimer();
-      for (int g = max(0, issued - kStateStages); g < issued; ++g)
-        while (!mbar_try(&ring->full[g % kStateStages], (g / kStateStages) & 1) && globaltimer() - t0 < kWaitLimitNs) {}
+      for (int g = max(0, issued - kStages); g < issued; ++g)
+        while (!mbar_try(&ring->full[g % kStages], (g / kStages) & 1) && globaltimer() - t0 < kWaitLimitNs) {}
     }
     return;
   }
@@ -169,7 +169,7 @@ lin_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&ring->empty[s]);
-    if (++s == kStateStages) { s = 0; par ^= 1; }
+    if (++s == kStages) { s = 0; par ^= 1; }
   }
   if (!ok) return;
 
@@ -560,8 +560,11 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
   static OncePerDevice smem_opt_in;   // > 48 KB of dynamic shared memory: a per-device function attribute
   cudaError_t e = smem_opt_in.run([] {
     cudaError_t r;
-    if ((r = cudaFuncSetAttribute(lin_state_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStateSmem)) != cudaSuccess) return r;
-    if ((r = cudaFuncSetAttribute(lin_state_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStateSmem)) != cudaSuccess) return r;
+    const cudaFuncAttribute attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if ((r = cudaFuncSetAttribute(lin_state_kernel<false, 6>, attr, (int)state_smem(6))) != cudaSuccess) return r;
+    if ((r = cudaFuncSetAttribute(lin_state_kernel<true, 6>, attr, (int)state_smem(6))) != cudaSuccess) return r;
+    if ((r = cudaFuncSetAttribute(lin_state_kernel<false, 3>, attr, (int)state_smem(3))) != cudaSuccess) return r;
+    if ((r = cudaFuncSetAttribute(lin_state_kernel<true, 3>, attr, (int)state_smem(3))) != cudaSuccess) return r;
     return cudaFuncSetAttribute(lin_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kApplySmem);
   });
   if (e != cudaSuccess) return e;
@@ -571,7 +574,12 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
   if (a.dwc && (e = dwc_static_kernels(a, p, &w, &w_batch, st)) != cudaSuccess) return e;
   const int num_sms = device_sm_count();
   dim3 g1(p.nchunk, BH);
-  e = launch_programmatic(a.dwc ? lin_state_kernel<true> : lin_state_kernel<false>, g1, kThreads, kStateSmem, st, mk, mv, partial, status,
+  // More heads than two CTAs per SM take: rings half as deep, four CTAs, so that the rest does not wait for a second wave.  Two / four,
+  // the block with a static convolution: 384 heads of 256 tokens 23.7 / 21.3 us, 300 of 576 37.0 / 33.7, 312 of 4096 181.9 / 151.7.
+  const bool many = (int64_t)p.nchunk * BH > 2 * num_sms;
+  auto* state_kernel = a.dwc ? (many ? lin_state_kernel<true, 3> : lin_state_kernel<true, 6>)
+                             : (many ? lin_state_kernel<false, 3> : lin_state_kernel<false, 6>);
+  e = launch_programmatic(state_kernel, g1, kThreads, state_smem(many ? 3 : 6), st, mk, mv, partial, status,
                           N, p.chunk_tokens, p.state_elems, (int)s.H);
   if (e != cudaSuccess) return e;
 
