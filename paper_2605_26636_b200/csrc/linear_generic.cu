@@ -23,6 +23,11 @@ LinPlan lin_plan(const jv_shape& s, const jv_dwc* dwc) {
   // without it, 16 of 40 x 40: 11.2 / 13.0.
   int want = (2 * device_sm_count()) / BH;
   if (want < 1) want = 1;
+  // With one chunk per head and up to 1.5 heads per SM some SMs have twice the work of the others: two chunks, which fit
+  // four CTAs to an SM, if that leaves them long enough.  One / two chunks, the block with generated kernels: 168 heads of 4480 tokens 117.7 /
+  // 103.3 us, 192 of 4096 114.6 / 105.2, 160 of 1600 55.0 / 52.0, 192 of 1024 44.3 / 43.6; 288 of 1600 78.0 / 80.4, 192 of 576
+  // 31.2 / 32.6; without a convolution no difference.
+  if (want == 1 && N >= 1024 && 2 * BH <= 3 * device_sm_count() && s.D == 64 && s.dtype == JV_BF16 && dwc && !dwc->token_wise) want = 2;
   int chunk = ceil_div(ceil_div(N, want), 128) * 128;
   const int least = s.D == 64 && (s.dtype == JV_F32 || (dwc && !dwc->token_wise)) ? 128 : 512;
   if (chunk < least) chunk = least;
