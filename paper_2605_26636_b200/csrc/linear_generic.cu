@@ -16,7 +16,7 @@ LinPlan lin_plan(const jv_shape& s, const jv_dwc* dwc) {
   p.D1 = s.D + 1;
   p.state_elems = (p.D1 * p.D1 + 3) / 4 * 4;
   // Chunks: as many as fit one wave of two CTAs per SM over all (batch, head) pairs, each a
-  // multiple of 128 tokens; one wave means no tail, and chunks of equal length finish together.  At least
+  // multiple of 128 (fp32: 64) tokens; one wave means no tail, and chunks of equal length finish together.  At least
   // 512 tokens long where every CTA of the apply pass sums the partials of its head at its start, 128 where
   // they are summed once per head (beside the kernel generator; fp32 tensors): short chunks fill the chip.  Measured, at least
   // 512 / 128 tokens: with the convolution, 6 heads of 37 x 37 18.7 / 15.2 us, 16 of 40 x 40 17.4 / 14.3, 12 of 60 x 60 22.4 / 20.6;
@@ -28,8 +28,12 @@ LinPlan lin_plan(const jv_shape& s, const jv_dwc* dwc) {
   // 103.3 us, 192 of 4096 114.6 / 105.2, 160 of 1600 55.0 / 52.0, 192 of 1024 44.3 / 43.6; 288 of 1600 78.0 / 80.4, 192 of 576
   // 31.2 / 32.6; without a convolution no difference.
   if (want == 1 && N >= 1024 && 2 * BH <= 3 * device_sm_count() && s.D == 64 && s.dtype == JV_BF16 && dwc && !dwc->token_wise) want = 2;
-  int chunk = ceil_div(ceil_div(N, want), 128) * 128;
-  const int least = s.D == 64 && (s.dtype == JV_F32 || (dwc && !dwc->token_wise)) ? 128 : 512;
+  // fp32 tensors: chunks of 64 tokens and up with a convolution, and on short sequences, where the sums at the start of every apply CTA stay short.
+  // Least chunk 128 / 64: 6 heads of 256 tokens 12.0 / 9.7 us, 12 of 400 15.4 / 13.2; 12 of 1024 with the convolution 25.4 / 21.8, without
+  // it 12 of 1369 22.0 / 27.2.
+  const int unit = s.D == 64 && s.dtype == JV_F32 && (N <= 512 || (dwc && !dwc->token_wise)) ? 64 : 128;
+  int chunk = ceil_div(ceil_div(N, want), unit) * unit;
+  const int least = s.D == 64 && (s.dtype == JV_F32 || (dwc && !dwc->token_wise)) ? unit : 512;
   if (chunk < least) chunk = least;
   p.chunk_tokens = chunk;
   p.nchunk = ceil_div(N, chunk);

@@ -57,7 +57,7 @@ def test_fp32_kernels(jv, oracle, case):
 
 
 @pytest.mark.parametrize("static", [False, True], ids=["squeeze", "static"])
-@pytest.mark.parametrize("case", [(1, 1, 0, 1, 1), (1, 2, 0, 70, 1), (2, 3, 5, 11, 13), (1, 12, 1, 32, 32), (2, 2, 3, 3, 130)],
+@pytest.mark.parametrize("case", [(1, 1, 0, 1, 1), (1, 2, 0, 70, 1), (2, 3, 5, 11, 13), (1, 12, 1, 32, 32), (2, 2, 3, 3, 130), (2, 12, 0, 32, 32)],
                          ids=lambda c: "x".join(map(str, c)))
 def test_fp32_linear_with_convolution(jv, oracle, case, static):
     B, H, P, Hg, Wg = case
