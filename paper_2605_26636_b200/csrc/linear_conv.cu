@@ -25,12 +25,13 @@
 //   warp 18      store warp: one TMA store per finished tile (clipped at the grid edge), then the
 //                slot goes back to the producer
 //
-// What bounds it: shared-memory bandwidth.  A tile moves 56 KB through it for the copies in and out and the
-// convolution warps read V three times over (two output rows per warp); with relu(Q) rewritten in shared memory and read
-// from there by the MMAs, the denominators from z in shared memory and the kernels fetched lane by lane at each head
-// boundary a tile took 2250 clocks and a boundary 5000; now 1850 and 800.  8 x 16 heads, 64 x 64 tokens: 45 -> 39 us of the
-// block's 84.6 -> 78.7.  More convolution warps (sixteen, half the tokens each: 87.0 us for the block), packed fp32
-// multiply-adds on widened values (98.9 us: register moves) and fewer instructions elsewhere did not help.
+// What bounds it: no unit by itself.  8 x 16 heads, 64 x 64 tokens: 39 us for the 201 MB that the pass moves, 5.2 TB/s of them, a
+// part from L2, where a plain copy of that size reaches 5.5; DRAM is half busy, issue slots 54 %, shared memory about 1300 of a tile's 1850
+// clocks.  It took 45 while shared memory bound it: relu(Q) rewritten there and read from there by the MMAs, the
+// denominators from z in shared memory, the kernels fetched lane by lane at each head boundary (2250 clocks a tile and 5000 a
+// boundary; now 1850 and 800).  More convolution warps (sixteen, half the tokens each: 87.0 us for the block, then 84.6), packed fp32
+// multiply-adds on widened values (98.9 us: register moves), and four rows by four columns per lane with four warps to a tile (a
+// quarter fewer reads of V: 75.2 us, now 74.5, and 88.3 instead of 85.2 for a stack of 6 heads) did not help.
 //
 // Every mbarrier wait is bounded; a wait that runs out sets the device status word and the CTA-wide
 // abort flag, every role falls through, tensor memory is released.
