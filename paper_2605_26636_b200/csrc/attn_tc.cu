@@ -129,6 +129,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
                const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapO,
                const __grid_constant__ CUtensorMap mapKp, const __grid_constant__ CUtensorMap mapVp, const TcParams p) {
   extern __shared__ unsigned char smem_raw[];
+  if (threadIdx.x == 32) {
+    prefetch_map(&mapQ);
+    prefetch_map(&mapK);
+    prefetch_map(&mapV);
+    prefetch_map(&mapO);
+  }
   // 1024-byte alignment by an offset from the array itself, so that accesses stay shared-space loads and stores
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   Barriers* bar = reinterpret_cast<Barriers*>(smem + kSmemTiles);

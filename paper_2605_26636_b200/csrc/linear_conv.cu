@@ -137,6 +137,11 @@ __global__ void __launch_bounds__(kThreadsConv, 1)
 lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapV,
                       const __grid_constant__ CUtensorMap mapO, const ConvParams p) {
   extern __shared__ unsigned char smem_raw[];
+  if (threadIdx.x == 32) {
+    prefetch_map(&mapQ);
+    prefetch_map(&mapV);
+    prefetch_map(&mapO);
+  }
   // 1024-byte alignment by an offset from the array itself, so that accesses stay shared-space loads and stores
   unsigned char* smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t smem = smem_u32(smem_al);

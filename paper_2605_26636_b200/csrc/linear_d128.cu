@@ -71,6 +71,10 @@ __global__ void __launch_bounds__(kThreads1, 1)
 lin128_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV,
                     unsigned char* __restrict__ state, int* status, int N, int chunk_tokens) {
   extern __shared__ unsigned char smem_raw[];
+  if (threadIdx.x == 32) {
+    prefetch_map(&mapK);
+    prefetch_map(&mapV);
+  }
   unsigned char* smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t smem = smem_u32(smem_al);
   Bars1* bars = reinterpret_cast<Bars1*>(smem_al + kOffBars1);
@@ -296,6 +300,10 @@ __global__ void __launch_bounds__(kThreads2, 1)
 lin128_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapO,
                     const unsigned char* __restrict__ state, int* status, int N, int span_tokens, float eps) {
   extern __shared__ unsigned char smem_raw[];
+  if (threadIdx.x == 32) {
+    prefetch_map(&mapQ);
+    prefetch_map(&mapO);
+  }
   unsigned char* smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t smem = smem_u32(smem_al);
   float* z_sm = reinterpret_cast<float*>(smem_al + kOffZ2);

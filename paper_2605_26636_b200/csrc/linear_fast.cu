@@ -70,6 +70,10 @@ __global__ void __launch_bounds__(kThreads)
 lin_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV,
                  float* __restrict__ partial, int* status, int N, int chunk_tokens, int state_elems, int H) {
   extern __shared__ unsigned char smem_raw[];
+  if (threadIdx.x == 32) {
+    prefetch_map(&mapK);
+    prefetch_map(&mapV);
+  }
   // 1024-byte alignment by an offset from the array itself, so that accesses stay shared-space loads and stores
   unsigned char* smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t smem = smem_u32(smem_al);      // stage s: K tile at s * 16 KB, V tile at s * 16 KB + 8 KB
@@ -231,6 +235,10 @@ lin_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                  const float* __restrict__ partial, int* status, int N, int span_tokens, int nchunk, int state_elems,
                  float eps, int H) {
   extern __shared__ unsigned char smem_raw[];
+  if (threadIdx.x == 32) {
+    prefetch_map(&mapQ);
+    prefetch_map(&mapO);
+  }
   // 1024-byte alignment by an offset from the array itself, so that accesses stay shared-space loads and stores
   unsigned char* smem_al = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t smem = smem_u32(smem_al);                                       // Q ring

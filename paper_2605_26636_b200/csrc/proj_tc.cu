@@ -140,6 +140,11 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
                const __grid_constant__ CUtensorMap mapD0, const __grid_constant__ CUtensorMap mapD1,
                const __grid_constant__ CUtensorMap mapD2, const ProjParams p) {
   extern __shared__ unsigned char smem_raw[];
+  if (threadIdx.x == 32) {
+    prefetch_map(&mapA);
+    prefetch_map(&mapB);
+    prefetch_map(&mapD0);
+  }
   // 1024-byte alignment by an offset from the array itself, so that accesses stay shared-space loads and stores
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   using L = Layout<kCtas>;

@@ -112,6 +112,13 @@ __device__ __forceinline__ bool warp_wait_limit(uint64_t* bar, uint32_t parity, 
   return __all_sync(0xffffffffu, mbar_wait<0>(bar, parity, abort_flag, status, limit_ns));
 }
 
+// Brings a tensor map into the descriptor cache: by one thread, ahead of the wait for the launch before, so that the first copies
+// need not fetch theirs (a launch's parameters are new memory every time).  Six layers of 6 heads on 37 x 37 tokens 84.8 -> 84.2 us, three
+// of 384 heads on 16 x 16 tokens 69.6 -> 69.4; long launches the same.
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
