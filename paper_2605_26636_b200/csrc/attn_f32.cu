@@ -42,7 +42,7 @@ constexpr size_t smem_bytes() {
 
 // prefix_rows: the launch serves the P prefix queries (keys: all tokens) instead of the windows.
 template <int R, int G>
-__global__ void __launch_bounds__(32 * R * G, G == 4 ? 2 : 3)  // what shared memory leaves room for
+__global__ void __launch_bounds__(32 * R * G, G == 8 ? 1 : G == 4 ? 2 : 3)  // what shared memory leaves room for
 attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ o,
                 int Hg, int Wg, int P, int wh, int ww, int nwx, bool prefix_rows, bool overlap, float scale) {
   extern __shared__ __align__(16) float smem_f[];
@@ -280,8 +280,10 @@ cudaError_t launch(const AttnArgs& a, bool prefix_rows, bool overlap, cudaStream
 
 bool attn_f32_supported(const AttnArgs& a) { return a.dtype == JV_F32 && a.D == kDim && !a.strided; }
 
-// The P prefix queries go first, with the keys of a row tile split over four groups (their chain is the
-// longest: all N keys); the windows' launch overlaps them, as neither reads what the other writes.
+// The P prefix queries go first, with the keys of a row tile split over eight or four groups (their chain is the
+// longest: all N keys); the windows' launch overlaps them, as neither reads what the other writes.  Eight groups take an SM each: for
+// few heads or long sequences.  Four / eight groups, us for the call: 6 heads, 16 x 16 tokens, 8 x 8 windows 11.8 / 10.2, 6 of 37 x 37 33.2 /
+// 27.7, 24 of 37 x 37, 16 x 16 windows 106 / 87; 24 of 24 x 24 47.7 / 50.1.
 // 32 rows x 2 groups per CTA (three on an SM) or 16 rows x 4 groups (two): the second halves the chain of a CTA, and its
 // finer grain leaves less of the last round empty; the first is 10 % faster where both fill the chip.  Measured, 32 x 2 against
 // 16 x 4 with up to two CTAs of 32 rows per SM: 48 CTAs 13 / 8 us, 150 CTAs 57 / 33, 256 CTAs 92 / 69.  Beyond that by
@@ -292,7 +294,9 @@ cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st) {
   const int wh = a.wh < a.Hg ? a.wh : a.Hg, ww = a.ww < a.Wg ? a.ww : a.Wg;
   const bool prefix = a.P > 0;
   if (prefix) {
-    const cudaError_t e = launch<1, 4>(a, true, false, st);
+    const int N = a.P + a.Hg * a.Wg;
+    const bool eight = 8 * a.BH <= device_sm_count() || N >= 1024;
+    const cudaError_t e = eight ? launch<1, 8>(a, true, false, st) : launch<1, 4>(a, true, false, st);
     if (e != cudaSuccess) return e;
   }
   const int64_t ctas = (int64_t)ceil_div(a.Wg, ww) * ceil_div(a.Hg, wh) * a.BH * ceil_div(wh * ww, 2 * kRowsWarp);
