@@ -473,6 +473,7 @@ lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
         for (int pr = 0; pr < 2; ++pr)
 #pragma unroll
           for (int tap = 0; tap < 9; ++tap) wq[pr][tap] = pack_bf16(wf[9 * (2 * pr) + tap], wf[9 * (2 * pr + 1) + tap]);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the reads, before the next head's copy over them
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars->w_free[nh & 1]);
         ++nh;

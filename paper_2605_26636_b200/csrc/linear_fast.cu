@@ -171,6 +171,10 @@ lin_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant
       }
       mma_bf16(acc[8], a, ones, ones);
     }
+    // The stage goes back to the copies only once its reads are complete: they and the copies are of different proxies, and an
+    // arrival alone lets the last ldmatrix be overtaken by a copy that has nothing to fetch (the rows past N of a head's last
+    // tile are zeros from the copy engine itself; without the fence 44 of 60 calls on 576 heads of 2500 tokens had a wrong state).
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncwarp();
     if (lane == 0) mbar_arrive(&ring->empty[s]);
     if (++s == kStages) { s = 0; par ^= 1; }
