@@ -59,3 +59,27 @@ def test_small_windows(jv, oracle, case):
     heads = sample_heads(B, H, 4, N)
     pick = lambda t: torch.stack([t[b, h] for b, h in heads]).unsqueeze(0)
     assert rel_err(pick(out.cpu()), oracle.window_attn(pick(q), pick(k), pick(v), Hg, Wg, wh, ww, prefix=P)) <= TOL["bf16"], case
+
+
+def test_a_dominant_key_of_an_8x8_window_weighs_exactly_one(jv):
+    """Every window has one key 2^4 to 2^8 above another one, in the other half of its rows, and nothing else of weight; all values are
+    1.5.  With the larger one's probability taken against itself it is 1 in bf16 too, the smaller one's rounding is 2^-8 of
+    2^-4 at most, and the result rounds to 1.5 (the neighbours are 2^-7 away).  Against the smaller one the larger one's probability is
+    rounded itself, by up to 2^-8 of the whole."""
+    B, H, Hg, Wg = 2, 16, 40, 56
+    gen = torch.Generator().manual_seed(8901)
+    nwin = B * H * (Hg // 8) * (Wg // 8)
+    score = torch.full((nwin, 64), -40.0)                   # in powers of two: the softmax scale below is ln 2
+    low = torch.randint(0, 32, (nwin,), generator=gen)      # keys 0 .. 31 are the window's upper four rows
+    high = torch.randint(32, 64, (nwin,), generator=gen)
+    swap = torch.rand(nwin, generator=gen) < 0.25
+    low, high = torch.where(swap, high, low), torch.where(swap, low, high)
+    score[torch.arange(nwin), low] = 0.0
+    score[torch.arange(nwin), high] = torch.randint(4 * 32, 8 * 32, (nwin,), generator=gen) / 32.0   # exact in bf16
+    k0 = score.view(B, H, Hg // 8, Wg // 8, 8, 8).permute(0, 1, 2, 4, 3, 5).reshape(B, H, Hg * Wg)
+    q, k = (torch.zeros(B, H, Hg * Wg, 64) for _ in range(2))
+    q[..., 0] = 1.0
+    k[..., 0] = k0
+    q, k, v = (t.bfloat16().to(DEV) for t in (q, k, torch.full_like(q, 1.5)))
+    out = jv.window_attn(q, k, v, Hg, Wg, 8, 8, scale=0.6931471805599453)
+    assert bool((out == 1.5).all()), int((out != 1.5).sum())
