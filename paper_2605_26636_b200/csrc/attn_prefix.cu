@@ -57,8 +57,10 @@ attn_prefix_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16
   const int r0 = blockIdx.y * kRows, nr = min(kRows, P - r0);
   const size_t base = (size_t)(blockIdx.x / nsplit) * N * kD;
   const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-  auto row16 = [&](const __nv_bfloat16* src, int row, int ch, bool in) -> uint4 {       // eight channels of a token
-    return in ? __ldg(reinterpret_cast<const uint4*>(src + base + (size_t)row * kD + ch)) : zero;
+  // Eight channels of a token.  A coherent load: beside the windows this launch may start while the one ahead of it still
+  // writes q, k and v, and a non-coherent one promises that nobody does for as long as the kernel runs.
+  auto row16 = [&](const __nv_bfloat16* src, int row, int ch, bool in) -> uint4 {
+    return in ? __ldcg(reinterpret_cast<const uint4*>(src + base + (size_t)row * kD + ch)) : zero;
   };
   auto load = [&](Tile& x, int t0) {
 #pragma unroll

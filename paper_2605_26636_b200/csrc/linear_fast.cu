@@ -344,6 +344,7 @@ lin_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     bool ok = *reinterpret_cast<volatile int*>(status) == 0;
     if (!ok) bars->abort_flag = 1;                     // an earlier kernel gave up: every role of this CTA falls through at once
     {  // second pass of the reduction: chunk partials summed in a fixed order; KV -> bf16 MMA operand, z in fp32
+      // (coherent loads: the launch ahead writes the partials while this one is running already)
       const float* P = partial + (size_t)bh * nchunk * state_elems;
 #pragma unroll
       for (int i = 0; i < (kD * 8) / kConsumers; ++i) {
@@ -355,8 +356,8 @@ lin_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
           for (int k = 0; k < 4; ++k) {
             const bool in = k0 + k < nchunk;
             const float* src = P + (size_t)(in ? k0 + k : 0) * state_elems + row * kD + ch * 8;
-            xa[k] = in ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
-            ya[k] = in ? *reinterpret_cast<const float4*>(src + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+            xa[k] = in ? __ldcg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            ya[k] = in ? __ldcg(reinterpret_cast<const float4*>(src + 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
           }
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
@@ -375,7 +376,7 @@ lin_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
       }
       if (threadIdx.x < kD) {
         float zs = 0.f;
-        for (int k = 0; k < nchunk; ++k) zs += P[(size_t)k * state_elems + kOffZ + threadIdx.x];
+        for (int k = 0; k < nchunk; ++k) zs += __ldcg(P + (size_t)k * state_elems + kOffZ + threadIdx.x);
         z_sm[threadIdx.x] = zs;
       }
     }

@@ -310,13 +310,13 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         for (int c = 0; c < 2; ++c) {
           uint32_t v[32];
           tmem_ld32(tmem + lane_base + a * kBN + j * kD + c * 32, v);
-          float4 bb[8];                       // the bias, on its way beside the accumulator
+          float4 bb[8];                       // the bias, on its way beside the accumulator (coherent loads: the launch ahead may write it)
 #pragma unroll
           for (int i4 = 0; i4 < 8; ++i4) {
             const float* bp = p.bias + fb * kD + c * 32 + 4 * i4;
             bb[i4] = !p.bias ? make_float4(0.f, 0.f, 0.f, 0.f)
-                     : p.bias_vec ? __ldg(reinterpret_cast<const float4*>(bp))
-                                  : make_float4(__ldg(bp), __ldg(bp + 1), __ldg(bp + 2), __ldg(bp + 3));
+                     : p.bias_vec ? *reinterpret_cast<const float4*>(bp)
+                                  : make_float4(bp[0], bp[1], bp[2], bp[3]);
           }
           tmem_wait_ld(v);
 #pragma unroll
