@@ -213,6 +213,7 @@ attn_w4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   if (bar->abort_flag) {
     if (warp == 0)
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    if (kPrefix) griddep_wait();    // (no launch ends before the one ahead of it)
     return;
   }
 

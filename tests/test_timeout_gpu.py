@@ -77,3 +77,21 @@ def test_selftest_rejects_bad_limits(jv):
     with pytest.raises(jv.JetVitError):
         jv.selftest_wait_timeout(5_000_000)
     assert jv.device_status() == jv.JV_OK
+
+
+def test_windows_that_leave_at_once_end_behind_their_prefix_queries(jv):
+    """Window attention with prefix tokens while the status word is set: the windows' launch, which runs beside that of the prefix queries,
+    leaves at once.  It must not be complete before the other one is, or what is enqueued behind the call could
+    be overwritten by it."""
+    H, Hg, Wg, P = 6, 37, 37, 5
+    q, k, v = (t.to(DEV) for t in inputs.custom_qkv(1, H, P + Hg * Wg, 64, "bf16", seed=37))
+    o = torch.empty_like(q)
+    assert jv.device_status() == jv.JV_OK
+    jv.selftest_wait_timeout(1000)
+    for _ in range(20):
+        jv.window_attn(q, k, v, Hg, Wg, 16, 16, out=o, prefix=P)
+        o.fill_(1234.5)
+        seen = o.clone()
+        assert bool((seen == 1234.5).all()) and bool((o == 1234.5).all())
+    assert jv.device_status() == jv.JV_ERR_TIMEOUT
+    assert jv.device_status() == jv.JV_OK
