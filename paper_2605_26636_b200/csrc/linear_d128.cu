@@ -235,7 +235,14 @@ lin128_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
     }
   }
   __syncwarp();
-  if (rows > 0) warp_wait(&bars->red_full, 0, &bars->abort_flag, status);   // (every CTA sends, also one that gave up)
+  if (rows > 0) {
+    // Every CTA sends, also one that gave up, and none may leave while copies into its shared memory are on their way: this wait
+    // is bounded by time alone, whatever the abort flag says.
+    const unsigned long long t0 = globaltimer();
+    bool landed;
+    while (!(landed = mbar_try(&bars->red_full, 0)) && globaltimer() - t0 < kWaitLimitNs) {}
+    if (!landed) atomicOr(status, kStatusTimeout);
+  }
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // (2) received: the senders may leave
   // this CTA's rows: the chunks' partials summed in chunk order, eight columns per thread and step
   const float* red = reinterpret_cast<const float*>(smem_al + kOffRed);

@@ -95,3 +95,23 @@ def test_windows_that_leave_at_once_end_behind_their_prefix_queries(jv):
         assert bool((seen == 1234.5).all()) and bool((o == 1234.5).all())
     assert jv.device_status() == jv.JV_ERR_TIMEOUT
     assert jv.device_status() == jv.JV_OK
+
+
+@pytest.mark.parametrize("H", [8, 21, 50])                # clusters of eight, seven and two CTAs
+def test_head_dim_128_state_pass_while_the_word_is_set(jv, oracle, H):
+    """The CTAs of a cluster exchange their partial states also when they have given up, and each stays until what is sent to it has
+    landed: many such calls in a row leave the device in order and the output alone."""
+    Hg, Wg = 31, 21
+    qh, kh, vh = inputs.custom_qkv(1, H, Hg * Wg, 128, "bf16", seed=128 + H)
+    q, k, v = (t.to(DEV) for t in (qh, kh, vh))
+    o = torch.full_like(q, 1234.5)
+    assert jv.device_status() == jv.JV_OK
+    jv.selftest_wait_timeout(1000)
+    for _ in range(20):
+        jv.linear_attn(q, k, v, Hg, Wg, out=o)
+    torch.cuda.synchronize()
+    assert bool((o == 1234.5).all())
+    assert jv.device_status() == jv.JV_ERR_TIMEOUT
+    jv.linear_attn(q, k, v, Hg, Wg, out=o)
+    assert rel_err(o[:, :2], oracle.linear_attn(qh[:, :2], kh[:, :2], vh[:, :2], Hg, Wg)) <= TOL["bf16"]
+    assert jv.device_status() == jv.JV_OK
