@@ -31,7 +31,7 @@
  *             Kernels bound every wait (2 s); one that gives up sets a sticky
  *             per-device status word and returns, and jv_device_status()
  *             reports JV_ERR_TIMEOUT.  While the word is set, the tensor-core
- *             kernels (bf16, D = 64) that are launched leave at once WITHOUT
+ *             kernels (bf16, D = 64 or 128) that are launched leave WITHOUT
  *             writing their output: calls keep returning JV_OK (they only
  *             enqueue) and o keeps its old contents until jv_device_status()
  *             has been called, which reads and clears the word.  A caller that

@@ -168,7 +168,7 @@ jv_status run_attn(const void* q, const void* k, const void* v, void* o, const j
     int* status = device_status_ptr();
     if (!status) return JV_ERR_CUDA;
     if (a.P > 0) {                                        // the P prefix queries, which attend everything
-      const jv_status r = from_cuda(launch_attn_prefix(a, device_sm_count() - attn_w4_ctas(a), st));
+      const jv_status r = from_cuda(launch_attn_prefix(a, device_sm_count() - attn_w4_ctas(a), status, st));
       if (r != JV_OK) return r;
     }
     return from_cuda(launch_attn_w4(a, status, st));
@@ -178,7 +178,7 @@ jv_status run_attn(const void* q, const void* k, const void* v, void* o, const j
     if (!status) return JV_ERR_CUDA;
     if (a.strided && a.P > 0) return JV_ERR_UNSUPPORTED;  // the prefix queries' kernel reads contiguous tensors
     if (a.P > 0) {
-      const jv_status r = from_cuda(launch_attn_prefix(a, 0, st));
+      const jv_status r = from_cuda(launch_attn_prefix(a, 0, status, st));
       if (r != JV_OK) return r;
     }
     return from_cuda(launch_attn_tc(a, full, status, st));

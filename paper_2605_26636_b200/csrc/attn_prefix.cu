@@ -46,11 +46,13 @@ struct Tile {
 
 __global__ void __launch_bounds__(kWarps * 32, 2)
 attn_prefix_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
-                        const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ o, int N, int P, float scale_log2) {
+                        const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ o, const int* status, int N, int P,
+                        float scale_log2) {
   namespace cg = cooperative_groups;
   __shared__ float part[kWarps + 1][kRows][kLd];      // one partial per warp, then the block's own
   griddep_wait();
   griddep_launch_dependents();                        // the windows' launch overlaps this one
+  const bool gave_up = *reinterpret_cast<const volatile int*>(status) != 0;   // an earlier kernel gave up: o stays as it is
   cg::cluster_group cluster = cg::this_cluster();
   const int nsplit = cluster.num_blocks(), split = cluster.block_rank();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -189,8 +191,10 @@ attn_prefix_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16
     combine(nsplit, [&](int i) { return cluster.map_shared_rank(&part[kWarps][r][0], i); }, M, L, x0, x1);
     const float inv = 1.f / L;
     __nv_bfloat16* dst = o + base + (size_t)(r0 + r) * kD;
-    dst[lane] = __float2bfloat16_rn(x0 * inv);
-    dst[32 + lane] = __float2bfloat16_rn(x1 * inv);
+    if (!gave_up) {
+      dst[lane] = __float2bfloat16_rn(x0 * inv);
+      dst[32 + lane] = __float2bfloat16_rn(x1 * inv);
+    }
   }
   cluster.sync();                                     // no block leaves while its shared memory may still be read
 }
@@ -208,7 +212,7 @@ attn_prefix_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16
 // Ahead, the launch is a plain one: dropped in while the launch before it drains, its blocks fill the first SMs two to one
 // and leave the last without.  Programmatically / plainly: 8 x 16 heads, 64 x 64 tokens 97.5 / 90.9 us for the call, 16 heads, 128 x 128
 // tokens 64.8 / 58.5, 24 heads, 40 x 60 22.0 / 22.9; beside, 6 heads, 37 x 37: 11.9 / 14.1.
-cudaError_t launch_attn_prefix(const AttnArgs& a, int free_sms, cudaStream_t st) {
+cudaError_t launch_attn_prefix(const AttnArgs& a, int free_sms, const int* status, cudaStream_t st) {
   if (a.dtype != JV_BF16 || a.D != kD || a.strided) return cudaErrorNotSupported;   // (the callers are the bf16 tensor-core paths)
   const int N = a.P + a.Hg * a.Wg, groups = ceil_div(a.P, kRows);
   // splits of the keys over at most `ctas` blocks: at least one 16-key step per warp
@@ -222,7 +226,7 @@ cudaError_t launch_attn_prefix(const AttnArgs& a, int free_sms, cudaStream_t st)
   if (!beside) split = split_for(2 * device_sm_count());
   const dim3 grid(a.BH * split, groups);
   return launch_cluster(beside, attn_prefix_rows_kernel, split, grid, kWarps * 32, 0, st,
-                        (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, (__nv_bfloat16*)a.o, N, a.P,
+                        (const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, (__nv_bfloat16*)a.o, status, N, a.P,
                         a.scale * 1.4426950408889634f);
 }
 

@@ -160,7 +160,7 @@ struct AttnArgs {
 cudaError_t launch_attn_generic(const AttnArgs& a, cudaStream_t st);
 // the P prefix queries of window attention on their own, ahead of the launch of the windows, which leaves `free_sms` SMs
 // to it (bf16, D == 64, contiguous)
-cudaError_t launch_attn_prefix(const AttnArgs& a, int free_sms, cudaStream_t st);
+cudaError_t launch_attn_prefix(const AttnArgs& a, int free_sms, const int* status, cudaStream_t st);
 // fp32 tensors at D == 64: register-tiled fp32 kernel (full and windowed attention, prefix tokens)
 bool attn_f32_supported(const AttnArgs& a);
 cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st);

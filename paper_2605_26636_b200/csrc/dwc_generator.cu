@@ -35,8 +35,9 @@ constexpr size_t kMaxSmem = 48 * 1024;                // (no opt-in needed; smal
 struct GenParams {
   const float *partial, *W1, *b1, *W2, *b2;
   float *hidden, *w, *state;                          // state: the chunks' sum, in the layout of a partial
-  const void *v, *q;                                  // q, o: prefix rows only
+  const void *v, *q;                                  // q, o, status: prefix rows only
   __nv_bfloat16* o;
+  const int* status;
   int B, H, R, P, ntok, nchunk, state_elems;
   int T;                                              // outputs per sample: C k k
   int group;                                          // samples per pass over the output layer (shared memory)
@@ -135,6 +136,7 @@ __device__ __forceinline__ void prefix_rows(const GenParams& p, int bh, float* s
   const __nv_bfloat16* q = (const __nv_bfloat16*)p.q + row0 * kD;
   for (int i = threadIdx.x; i < p.P * kD; i += kThreadsOut) qs[i] = fmaxf(__bfloat162float(q[i]), 0.f);
   griddep_wait();
+  const bool gave_up = *reinterpret_cast<const volatile int*>(p.status) != 0;   // an earlier kernel gave up: o stays as it is
   const float* src = p.nred ? p.state + (size_t)bh * p.state_elems : p.partial + (size_t)bh * p.nchunk * p.state_elems;
   float kv[kPer], z = 0.f;
 #pragma unroll
@@ -160,7 +162,7 @@ __device__ __forceinline__ void prefix_rows(const GenParams& p, int bh, float* s
     float s = 0.f;
 #pragma unroll
     for (int g = 0; g < kAGroups; ++g) s += red[(g * kGenPrefix + t) * kD + e];
-    p.o[(row0 + t) * kD + e] = __float2bfloat16_rn(s / den);
+    if (!gave_up) p.o[(row0 + t) * kD + e] = __float2bfloat16_rn(s / den);
   }
 }
 
@@ -404,6 +406,8 @@ cudaError_t launch_dwc_generator_fast(const LinArgs& a, const LinPlan& p, const 
   }
   int blocks = g.nmain;
   if (prefix) {
+    g.status = device_status_ptr();
+    if (!g.status) return cudaErrorUnknown;
     blocks += s.B * s.H;
     const size_t need = (size_t)((1 + kAGroups) * kGenPrefix + 1) * kD * sizeof(float);
     if (smem < need) smem = need;

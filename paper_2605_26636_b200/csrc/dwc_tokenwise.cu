@@ -88,8 +88,9 @@ __global__ void convert_weights_kernel(const float* __restrict__ W1, __nv_bfloat
 // go through shared memory so that lane l ends up with the 18 values of its channels 2 l, 2 l + 1.
 __global__ void __launch_bounds__(256)
 dwc_tok_apply_kernel(const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ o, const __half* __restrict__ wk,
-                     int H, int P, int Hg, int Wg) {
+                     const int* status, int H, int P, int Hg, int Wg) {
   __shared__ uint32_t wsm[8][9 * 32];
+  if (*reinterpret_cast<const volatile int*>(status) != 0) return;   // an earlier kernel gave up: o stays as it is
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ntok = P + Hg * Wg, N = Hg * Wg;
   const int bh = blockIdx.y, b = bh / H, h = bh - b * H;
@@ -168,7 +169,7 @@ cudaError_t launch_dwc_tokenwise_fast(const LinArgs& a, const LinPlan& p, int* s
   e = launch_proj_gemm(false, true, hidden, w2, d.b2, wk, s.B, ntok, d.R / 64, 0, F, false, true, true, status, st);
   if (e != cudaSuccess) return e;
   dim3 grid(ceil_div(s.Hg * s.Wg, 8), s.B * s.H);
-  dwc_tok_apply_kernel<<<grid, 256, 0, st>>>((const __nv_bfloat16*)a.v, (__nv_bfloat16*)a.o, wk, s.H, s.P, s.Hg, s.Wg);
+  dwc_tok_apply_kernel<<<grid, 256, 0, st>>>((const __nv_bfloat16*)a.v, (__nv_bfloat16*)a.o, wk, status, s.H, s.P, s.Hg, s.Wg);
   count_launch();
   return cudaGetLastError();
 }

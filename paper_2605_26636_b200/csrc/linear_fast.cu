@@ -501,7 +501,8 @@ lin_apply_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
 template <int K>
 __global__ void __launch_bounds__(256)
 dwc_add_kernel(const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ o, const float* __restrict__ w,
-               int w_batch, int H, int Hg, int Wg, int run) {
+               int w_batch, const int* status, int H, int Hg, int Wg, int run) {
+  if (*reinterpret_cast<const volatile int*>(status) != 0) return;   // an earlier kernel gave up: o stays as it is
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int N = Hg * Wg, bh = blockIdx.y, b = bh / H, h = bh % H;
   const int t0 = (blockIdx.x * 8 + warp) * run;
@@ -645,7 +646,7 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
   dim3 g4(ceil_div(ceil_div(N, run), 8), BH);
   const __nv_bfloat16* v = (const __nv_bfloat16*)a.v;
   __nv_bfloat16* o = (__nv_bfloat16*)a.o;
-  dwc_add_kernel<5><<<g4, 256, 0, st>>>(v, o, w, w_batch, s.H, s.Hg, s.Wg, run);
+  dwc_add_kernel<5><<<g4, 256, 0, st>>>(v, o, w, w_batch, status, s.H, s.Hg, s.Wg, run);
   count_launch();
   return cudaGetLastError();
 }

@@ -115,3 +115,56 @@ def test_head_dim_128_state_pass_while_the_word_is_set(jv, oracle, H):
     jv.linear_attn(q, k, v, Hg, Wg, out=o)
     assert rel_err(o[:, :2], oracle.linear_attn(qh[:, :2], kh[:, :2], vh[:, :2], Hg, Wg)) <= TOL["bf16"]
     assert jv.device_status() == jv.JV_OK
+
+
+@pytest.mark.parametrize("P", [1, 5, 16, 20])             # 20: the linear block's prefix rows by the apply pass, W on the kernel of large windows
+def test_prefix_rows_stay_while_the_word_is_set(jv, oracle, P):
+    """The rows of the prefix tokens have kernels of their own in W and in the linear block with a convolution; they leave o alone as the
+    others do.  The linear block's scratch holds NaN: its state pass leaves without writing it."""
+    H, Hg, Wg = 4, 33, 29
+    qh, kh, vh = inputs.custom_qkv(1, H, P + Hg * Wg, 64, "bf16", seed=90 + P)
+    q, k, v = (t.to(DEV) for t in (qh, kh, vh))
+    dh = inputs.dwc_weights(H * 64, 16, 3, 91)
+    d = dwc_to_device(dh, DEV)
+    static = {"k": 3, "R": 0, "b2": d["b2"]}
+    ws = jv.alloc_workspace("L", jv.make_shape(q, Hg, Wg, P), jv.make_dwc(d, DEV), DEV)
+    calls = [lambda o: jv.linear_attn(q, k, v, Hg, Wg, dwc=d, out=o, ws=ws, prefix=P),
+             lambda o: jv.linear_attn(q, k, v, Hg, Wg, dwc=static, out=o, ws=ws, prefix=P),
+             lambda o: jv.linear_attn(q, k, v, Hg, Wg, out=o, ws=ws, prefix=P),
+             lambda o: jv.window_attn(q, k, v, Hg, Wg, 16, 16, out=o, prefix=P),
+             lambda o: jv.window_attn(q, k, v, Hg, Wg, 8, 8, out=o, prefix=P)]
+    assert jv.device_status() == jv.JV_OK
+    ws.fill_(255)
+    jv.selftest_wait_timeout(1000)
+    outs = [torch.full_like(q, 1234.5) for _ in calls]
+    for fn, o in zip(calls, outs):
+        fn(o)
+        fn(o)
+    torch.cuda.synchronize()
+    for i, o in enumerate(outs):
+        assert bool((o == 1234.5).all()), (i, (o != 1234.5).nonzero()[:4].tolist())
+    assert jv.device_status() == jv.JV_ERR_TIMEOUT
+    assert rel_err(calls[0](outs[0]), oracle.linear_attn(qh, kh, vh, Hg, Wg, dwc=dh, prefix=P)) <= TOL["bf16"]
+    assert rel_err(calls[3](outs[3]), oracle.window_attn(qh, kh, vh, Hg, Wg, 16, 16, prefix=P)) <= TOL["bf16"]
+    assert jv.device_status() == jv.JV_OK
+
+
+@pytest.mark.parametrize("k,R,token_wise", [(5, 16, 0), (3, 64, 1)])
+def test_convolutions_that_add_to_the_output_stay_away_while_the_word_is_set(jv, oracle, k, R, token_wise):
+    """5 x 5 kernels and token-wise ones are a pass of their own that reads o and adds to it."""
+    H, Hg, Wg = 2, 24, 20
+    qh, kh, vh = inputs.custom_qkv(1, H, Hg * Wg, 64, "bf16", seed=95 + k)
+    q, kk, v = (t.to(DEV) for t in (qh, kh, vh))
+    dh = dict(inputs.dwc_weights(H * 64, R, k, 96), token_wise=token_wise)
+    d = dwc_to_device(dh, DEV)
+    o = torch.full_like(q, 1234.5)
+    assert jv.device_status() == jv.JV_OK
+    jv.selftest_wait_timeout(1000)
+    jv.linear_attn(q, kk, v, Hg, Wg, dwc=d, out=o)
+    torch.cuda.synchronize()
+    assert bool((o == 1234.5).all())
+    assert jv.device_status() == jv.JV_ERR_TIMEOUT
+    ref = oracle.linear_attn(qh, kh, vh, Hg, Wg, dwc=dh)
+    # o is rounded to bf16 twice on these paths: the bars of tests/test_parity_gpu.py for them
+    assert rel_err(jv.linear_attn(q, kk, v, Hg, Wg, dwc=d, out=o), ref, rms_tol=4.5e-3) <= TOL["bf16"]
+    assert jv.device_status() == jv.JV_OK
