@@ -361,7 +361,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         }
         ++nstore;
       }
-      // this accumulator may be overwritten once all four warps have read it
+      // this accumulator may be overwritten once all epilogue warps have read it
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
@@ -375,6 +375,12 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
   }
 
   // ================= common teardown =================
+  // The leader's commits arrive in the other CTA's shared memory, too: that one stays until the last of them has
+  // (bounded by time; the leader has waited for its own).
+  if (kPair && rank != 0 && warp == 4 && lane == 0) {
+    const unsigned long long t0 = globaltimer();
+    while (!mbar_try(&bar->drain, 0) && globaltimer() - t0 < kWaitLimitNs) {}
+  }
   __syncwarp();
   tc_fence_before();
   if (kPair) {

@@ -42,3 +42,21 @@ def test_projection_on_pairs(jv, oracle, H, which):
         for got, want in zip(outs, refs):
             assert rel_err(got[sl], want) <= TOL["bf16"]
     assert all(bool(torch.isfinite(o).all()) for o in outs)
+
+
+def test_pairs_one_behind_the_other(jv):
+    """Many launches of pairs in a row, each reading what the one before wrote: no CTA of a pair may leave while the other's commits are
+    still to arrive in it, nor start on tensor memory that is not free yet.  All rounds give the same bits."""
+    B, H, Hg, Wg = 3, 12, 50, 62
+    C = 64 * H
+    x = inputs.normal((B, Hg * Wg, C), inputs.SEED_BASE + 9950, "bf16").to(DEV)
+    w, b = (t.to(DEV) for t in inputs.proj_weights(3 * C, C, 9951))
+    wo, bo = (t.to(DEV) for t in inputs.proj_weights(C, C, 9952))
+    qkv = jv.qkv_proj(x, w, b, H, Hg, Wg)
+    y = jv.out_proj(qkv[0], wo, bo, Hg, Wg)
+    ref = [t.clone() for t in (*qkv, y)]
+    for _ in range(50):
+        jv.qkv_proj(x, w, b, H, Hg, Wg, out=qkv)
+        jv.out_proj(qkv[0], wo, bo, Hg, Wg, out=y)
+    for got, want in zip((*qkv, y), ref):
+        assert torch.equal(got, want)
