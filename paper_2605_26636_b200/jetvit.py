@@ -363,9 +363,9 @@ def qkv_proj(x, w, bias, H: int, Hg: int, Wg: int, out=None, stream=None, prefix
         raise ValueError("x must be [B, prefix + Hg*Wg, 64*H]")
     _check_proj(x, w, bias, H, 3 * C)
     q, k, v = out if out is not None else (torch.empty((B, H, N, 64), dtype=x.dtype, device=x.device) for _ in range(3))
-    _check_tensors(q, k, v)
-    if tuple(q.shape) != (B, H, N, 64) or q.dtype != x.dtype:
-        raise ValueError("q, k, v must be [B, H, N, 64] bf16")
+    for t in (q, k, v):            # outputs: written contiguously, whatever layout the mixers take as inputs
+        if not (t.is_cuda and t.is_contiguous() and tuple(t.shape) == (B, H, N, 64) and t.dtype == x.dtype and t.device == x.device):
+            raise ValueError("q, k, v must be contiguous [B, H, N, 64] bf16 tensors on x's device")
     shape = JvShape(B, H, Hg, Wg, 64, JV_BF16, prefix)
     with _current_device(x.device):
         st = lib().jv_qkv_proj(x.data_ptr(), w.data_ptr(), None if bias is None else bias.data_ptr(), q.data_ptr(),
