@@ -170,13 +170,14 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
         float mx = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
 #pragma unroll
         for (int w = 1; w < 16; w <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
-        const float mn = fmaxf(m[i], mx);                    // finite: every tile holds at least one key
-        alpha[r] = expf(m[i] - mn);                          // exp(-inf) = 0 on the first tile
+        const float mn = fmaxf(m[i], mx);
+        const float ref = mn == -INFINITY ? 0.f : mn;        // all scores of this group so far are -inf: weight 0, not NaN
+        alpha[r] = expf(m[i] - ref);                         // exp(-inf) = 0 on the first tile
         m[i] = mn;
         float sum = 0.f;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          p[j][r] = expf(s[j] - mn);
+          p[j][r] = expf(s[j] - ref);
           sum += p[j][r];
         }
         l[i] = fmaf(l[i], alpha[r], sum);
@@ -246,7 +247,7 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
 #pragma unroll
       for (int g = 0; g < G; ++g) {
         const float* src = ps + (g * R + rw) * kWarpBuf + r * kLd;
-        const float f = expf(src[64] - M);                   // a group without a tile: exp(-inf) = 0
+        const float f = expf(src[64] - M);                   // a group without a tile, or a key: exp(-inf) = 0
         const float4 y = *reinterpret_cast<const float4*>(src + 4 * tx);
         L = fmaf(src[65], f, L);
         x.x = fmaf(y.x, f, x.x);

@@ -119,21 +119,22 @@ attn_prefix_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16
         sc[n][c] = t0 + 8 * n + 2 * t + (c & 1) < N ? sc[n][c] * scale_log2 : -INFINITY;
         mx[c >> 1] = fmaxf(mx[c >> 1], sc[n][c]);
       }
-    float alpha[2];
+    float alpha[2], ref[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
       mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
-      const float m_new = fmaxf(m[h], mx[h]);                        // finite: the tile holds at least one key
-      alpha[h] = exp2f(m[h] - m_new);
+      const float m_new = fmaxf(m[h], mx[h]);
+      ref[h] = m_new == -INFINITY ? 0.f : m_new;                     // all scores of this warp so far are -inf: weight 0, not NaN
+      alpha[h] = exp2f(m[h] - ref[h]);
       m[h] = m_new;
       l[h] *= alpha[h];                                              // (this lane's share of the sum)
     }
     uint32_t pa[4];                                                  // A fragment of P
 #pragma unroll
     for (int n = 0; n < 2; ++n) {
-      const float p0 = exp2f(sc[n][0] - m[0]), p1 = exp2f(sc[n][1] - m[0]);
-      const float p2 = exp2f(sc[n][2] - m[1]), p3 = exp2f(sc[n][3] - m[1]);
+      const float p0 = exp2f(sc[n][0] - ref[0]), p1 = exp2f(sc[n][1] - ref[0]);
+      const float p2 = exp2f(sc[n][2] - ref[1]), p3 = exp2f(sc[n][3] - ref[1]);
       l[0] += p0 + p1;
       l[1] += p2 + p3;
       pa[2 * n] = pack_bf16x2(p0, p1);                               // row g
@@ -170,7 +171,7 @@ attn_prefix_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16
     for (int i = 0; i < n; ++i) M = fmaxf(M, src_of(i)[0]);
     for (int i = 0; i < n; ++i) {
       const float* src = src_of(i);
-      const float f = src[0] == -INFINITY ? 0.f : exp2f(src[0] - M);   // a source that saw no key
+      const float f = src[0] == -INFINITY ? 0.f : exp2f(src[0] - M);   // a source that saw no key, or none of weight
       L = fmaf(src[1], f, L);
       x0 = fmaf(src[2 + lane], f, x0);
       x1 = fmaf(src[2 + 32 + lane], f, x1);

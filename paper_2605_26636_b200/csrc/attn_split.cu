@@ -290,7 +290,7 @@ attn_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
       max32(va, mx4);
       const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
       float o_scale = 1.f;
-      if (mx > m + kLazy) {          // always true on the first step (m = -inf, mx finite: a box holds at least one key)
+      if (mx > m + kLazy) {          // always true on the first step, unless all of its scores are -inf
         o_scale = ex2((m - mx) * sl2);
         l *= o_scale;
         m = mx;
@@ -311,7 +311,7 @@ attn_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
         tmem_wait_ld(va);
       }
       // pass 2: exponentials against the reference, P over the scores just consumed
-      const float mneg = -m * sl2;
+      const float mneg = m == -INFINITY ? 0.f : -m * sl2;    // (all scores of the slot so far -inf: probabilities of 2^-126 at most, not NaN)
       const uint64_t mnegx2 = pack2(mneg, mneg);
       uint64_t lsum[4] = {0ull, 0ull, 0ull, 0ull};
       uint32_t pk[16];

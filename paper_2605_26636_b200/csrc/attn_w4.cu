@@ -554,7 +554,8 @@ attn_w4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
           }
         }
         // ---- pass 2: exponentials against the reference, P over the scores just consumed
-        const float mneg = -m * sl2;
+        // (kWpt == 2: half a window's scores may all be -inf; probabilities of 2^-126 at most then, not NaN)
+        const float mneg = kWpt == 2 && m == -INFINITY ? 0.f : -m * sl2;
         const uint64_t mnegx2 = pack2(mneg, mneg);
         uint64_t lsum[4] = {0ull, 0ull, 0ull, 0ull};
         uint32_t pk[16];
@@ -591,7 +592,7 @@ attn_w4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       ok = warp_wait<kSuspendNs>(&bar->o_full[t], n & 1, &bar->abort_flag, p.status);
       if (!ok) break;
       tc_fence_after();
-      const float inv = 1.f / l;
+      const float inv = kWpt == 2 && m == -INFINITY ? __uint_as_float(0x7fc00000u) : 1.f / l;   // no key of any weight: NaN
       const int wx0 = it.x0, wy0 = it.y0 + x * p.box_h + sub_y;           // origin of this warp's sub-box
       const bool store = wx0 < it.x_end && wy0 < it.y_end;                // else none of its rows exists
       unsigned char* stg = smem + (size_t)(2 * t + (n & 1)) * kTileBytes + q4 * 4096;
