@@ -338,7 +338,8 @@ lin_apply_conv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_con
 #pragma unroll
         for (int n = 0; n < 3; ++n) {                  // the bf16 nearest to what the terms before it left over
           const __nv_bfloat16 t = __float2bfloat16_rn(zs);
-          zs -= __bfloat162float(t);
+          const float f = __bfloat162float(t);
+          zs = isinf(f) ? 0.f : zs - f;                // (infinity leaves nothing over: inf - inf would be NaN)
           *reinterpret_cast<__nv_bfloat16*>(zt + tile_off(n, threadIdx.x >> 3)) = t;
         }
       }

@@ -265,8 +265,8 @@ lin128_state_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_const
       for (int e = 0; e < 4; ++e) {
         w[e] = pack_bf16(x[2 * e], x[2 * e + 1]);
         const float2 f = bf16x2_to_f2(w[e]);
-        x[2 * e] -= f.x;
-        x[2 * e + 1] -= f.y;
+        x[2 * e] = isinf(f.x) ? 0.f : x[2 * e] - f.x;       // (infinity leaves nothing over: inf - inf would be NaN)
+        x[2 * e + 1] = isinf(f.y) ? 0.f : x[2 * e + 1] - f.y;
       }
       *reinterpret_cast<uint4*>(st + (size_t)(2 * s + (c8 >> 3)) * kKvHalf + tile_off(row0 + r, c8 & 7)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
