@@ -494,8 +494,9 @@ bool attn_f4_supported(const AttnArgs& a) {
   if (ntiles * a.BH > 0x7fffffffll) return false;
   // Shorter sequences: where the last group of four is (almost) full and there are groups for half the SMs.  Measured, this kernel /
   // the two-tile kernel: 96 heads of 400 tokens 17.1 / 20.5 us, 288 of 324: 21.0 / 29.4, 48 of 900: 27.5 / 33.2; 96 of 576 (a last group of
-  // one) 28.4 / 23.7, 48 of 700 (of two) 21.3 / 16.2, 16 of 800 17.3 / 16.6, 6 of 1000 18.8 / 17.6.
-  if (N < 8 * kTile && ((ntiles & 3) == 1 || (ntiles & 3) == 2 || 2 * (ntiles + 3) / 4 * a.BH < device_sm_count())) return false;
+  // one) 28.4 / 23.7, 48 of 700 (of two) 21.3 / 16.2, 16 of 800 17.3 / 16.6, 6 of 1000 18.8 / 17.6.  (50 to 73 heads of 300 to 512 tokens and 30 to 36 of 800 to 1000
+  // take the same time whether the line lies at half the SMs or a third: other rules decide there.)
+  if (N < 8 * kTile && ((ntiles & 3) == 1 || (ntiles & 3) == 2 || 2 * ((ntiles + 3) / 4) * a.BH < device_sm_count())) return false;
   // Few query tiles: pairs on the two-tile kernel, if that has fewer rounds' worth of work (12 heads of 3025 tokens 46.6 / 50.7 us,
   // 6 of 4272 63.0 / 68.6, 16 of 2106 34.8 / 37.6, 6 of 1370 23.0 / 24.8).
   if (tc_cost((int)ntiles, a.BH) < plan_f4((int)ntiles, a.BH).cost) return false;
