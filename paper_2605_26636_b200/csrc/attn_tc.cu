@@ -704,6 +704,8 @@ bool attn_tc_supported(const AttnArgs& a, bool full) {
   Geometry g;
   if (!geometry(a, full, &g)) return false;
   if (a.P > kTile) return false;                        // the prefix keys are one key tile
+  // that tile's map holds whole box rows: of a window wider than all of a short head's tokens they would reach past the tensor's end
+  if (a.P > 0 && ceil_div(a.P, g.box_w) * g.box_w > a.P + a.Hg * a.Wg) return false;
   if ((int64_t)g.nwx * g.nwy * ceil_div(g.tiles_per_window, 2) * a.BH > 0x7fffffffll) return false;
   // 128-byte rows keep every TMA stride a multiple of 16 bytes; the base must be 16-byte aligned (checked by the ABI)
   return encode_fn() != nullptr;
@@ -743,7 +745,7 @@ cudaError_t launch_attn_tc(const AttnArgs& a, bool full, int* status, cudaStream
   }
   // The prefix rows of K and V in the shape of a key box: prefix token r at box position
   // (r % box_w, r / box_w).  Positions past P inside the last box row read grid tokens (they exist:
-  // a grid holds at least one box row of tokens) and are masked by the softmax; rows past that are
+  // see attn_tc_supported) and are masked by the softmax; rows past that are
   // outside the map and arrive as zeros.
   // (prefix tokens come with contiguous inputs only: the caller has checked)
   maps[4] = maps[1];

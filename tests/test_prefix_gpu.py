@@ -129,3 +129,16 @@ def test_projections_with_prefix_tokens(jv, oracle):
         assert rel_err(got, want) <= TOL["bf16"]
     y = jv.out_proj(q, wo.to(DEV), bo.to(DEV), Hg, Wg, prefix=P)
     assert rel_err(y, oracle.out_proj(q.cpu(), wo, bo)) <= TOL["bf16"]
+
+
+@pytest.mark.parametrize("P,Hg,Wg,wh,ww", [(1, 2, 5, 1, 16), (3, 3, 2, 2, 128), (5, 7, 3, 3, 32), (1, 5, 3, 3, 16)])
+def test_windows_wider_than_all_tokens_of_a_head(jv, oracle, P, Hg, Wg, wh, ww):
+    """The tensor-core kernel fetches prefix keys in whole rows of its tile box.  Where a head has fewer tokens than such a row those would lie
+    past the end of k and v: such calls (all but the last one) are the shape-generic kernel's, in one launch."""
+    N = P + Hg * Wg
+    q, k, v = inputs.custom_qkv(1, 2, N, 64, "bf16", seed=77 + N)
+    dq, dk, dv = _dev((q, k, v))
+    launches = jv.launch_count()
+    o = jv.window_attn(dq, dk, dv, Hg, Wg, wh, ww, prefix=P)
+    assert jv.launch_count() - launches == (1 if -(-P // ww) * ww > N else 2)
+    assert rel_err(o, oracle.window_attn(q, k, v, Hg, Wg, wh, ww, prefix=P)) <= TOL["bf16"]
