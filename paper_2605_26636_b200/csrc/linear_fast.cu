@@ -603,10 +603,14 @@ cudaError_t launch_linear_fast(const LinArgs& a, const LinPlan& p, cudaStream_t 
   // of whole 128-token tiles (with at least four tiles to a span, 6 heads of 37 x 37 tokens took 11.6 us for the block, not 10.2)
   auto enqueue_apply = [&](const CUtensorMap& map_q, const CUtensorMap& map_o, int ntokens, const float* state, int nchunk) -> cudaError_t {
     int nspan = (2 * num_sms) / BH;
-    // More heads than SMs: one wave of whole heads leaves some SMs with twice the work of the others; long heads are cut, at about 1400 tokens a
-    // span, below which a span's start costs more than that.  One span / three: 192 heads of 4096 tokens 83.4 / 77.0 us for the block, 168 of
-    // 4480 82.2 / 75.3, 312 of 4096 135.0 / 125.9, 160 of 1600 34.4 / 34.0, 192 of 1024 26.5 / 27.3.
-    if (BH > num_sms) nspan = ntokens / 1365;
+    // More heads than SMs: whole heads, two to an SM, leave some SMs with twice the work of the others.  Where the last wave of them is
+    // less than two thirds full, heads of three spans of 1365 tokens or more are cut (a span's start costs more than shorter ones give).
+    // One span / three, 4096 tokens: 160 heads 75.9 / 70.4 us for the block, 192: 85.7 / 79.3, 384: 161.9 / 150.7; 224: 92.4 / 98.8, 288: 110.9 /
+    // 117.4, 480: 183.9 / 189.2.  One / two, 2752 tokens: 192 heads 60.5 / 62.5.
+    if (BH > num_sms) {
+      const int64_t waves = ceil_div(BH, 2 * num_sms);
+      nspan = ntokens >= 3 * 1365 && 3ll * BH < 2 * waves * 2 * num_sms ? ntokens / 1365 : 1;
+    }
     if (nspan < 1) nspan = 1;
     int span = ceil_div(ceil_div(ntokens, nspan), kApplyTok) * kApplyTok;
     nspan = ceil_div(ntokens, span);

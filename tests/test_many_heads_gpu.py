@@ -1,5 +1,5 @@
 """The linear block with more heads than the state pass has CTAs at two to an SM (its rings are then half as deep): fewer tiles than a
-ring holds, the last one of a few tokens, and several times round it; two chunks, two spans per head; prefix tokens, strided inputs."""
+ring holds, the last one of a few tokens, and several times round it; two chunks, one or three spans per head; prefix tokens, strided inputs."""
 import pytest
 import torch
 
@@ -20,7 +20,7 @@ def jv():
 
 @pytest.mark.parametrize("conv", [False, True], ids=["none", "squeeze"])
 @pytest.mark.parametrize("case", [(50, 6, 0, 5, 13, True), (99, 3, 1, 8, 8, False), (25, 12, 0, 24, 24, True), (31, 10, 5, 17, 23, False), (20, 8, 3, 32, 33, False),
-                                  (10, 16, 0, 53, 52, False)],
+                                  (10, 16, 0, 53, 52, False), (10, 16, 2, 65, 66, False)],
                          ids=lambda c: "x".join(map(str, c)))
 def test_many_heads(jv, oracle, case, conv):
     B, H, P, Hg, Wg, fused = case
