@@ -16,7 +16,7 @@
 // merged at the end.
 //
 // Measured (12 heads, 32 x 32 tokens; the kernel of one warp per query row, which served these calls before and still
-// serves other head dims, in brackets): full attention 93 us (729), 16 x 16 windows 27 us (195); 6 heads, 16 x 16
+// serves other head dims and windows of at most eight tokens, in brackets): full attention 93 us (729), 16 x 16 windows 27 us (195); 6 heads, 16 x 16
 // tokens, full attention 8 us (63).  Full attention runs at 35 TFLOP/s (41 where the grid fills the chip evenly) of the 73 that
 // a loop of nothing but multiply-adds reaches: one of three instructions is not a multiply-add, and the registers leave room
 // for three warps per scheduler.
@@ -291,6 +291,11 @@ bool attn_f32_supported(const AttnArgs& a) { return a.dtype == JV_F32 && a.D == 
 // rounds, at 9 to 5 for one round of either: 300 CTAs 78 / 60 us (3 and 5 rounds), 384 CTAs 93 / 99 (3 and 6), 512 CTAs
 // 122 / 116 (4 and 7), 688 CTAs 202 / 222 (5 and 10).  Windows of one or two key tiles have no work for four groups (432
 // CTAs, 8 x 8 windows: 18 / 33 us).
+// Windows of at most eight tokens leave most of a 32 x 64 tile of scores empty: the kernel of one warp per query row, eight to a block, is the
+// better one.  This one / that one, 96 heads of 32 x 32 tokens: 2 x 2 windows 484 / 270 us, 2 x 4 256 / 148, 3 x 3 245 / 254; 12 heads of 64 x 64, 2 x 2
+// 235 / 135.  With prefix tokens, whose queries stay here: as long as a window's keys and they are one tile of that kernel, and the windows fill
+// the chip several times (it does not overlap the prefix queries): 12 heads of 64 x 64, 2 x 2, 5 prefix tokens 299 / 207, 40: 301 / 337; 6 heads of
+// 16 x 16, 1 x 1 36.7 / 30.8, 1 x 2 20.4 / 23.3, 2 x 2 11.9 / 18.5; of 37 x 37, 1 x 7 50.5 / 47.1.
 cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st) {
   const int wh = a.wh < a.Hg ? a.wh : a.Hg, ww = a.ww < a.Wg ? a.ww : a.Wg;
   const bool prefix = a.P > 0;
@@ -300,8 +305,10 @@ cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st) {
     const cudaError_t e = eight ? launch<1, 8>(a, true, false, st) : launch<1, 4>(a, true, false, st);
     if (e != cudaSuccess) return e;
   }
-  const int64_t ctas = (int64_t)ceil_div(a.Wg, ww) * ceil_div(a.Hg, wh) * a.BH * ceil_div(wh * ww, 2 * kRowsWarp);
-  const int64_t sms = device_sm_count(), rounds2 = (ctas + sms - 1) / sms, rounds1 = (2 * ctas + sms - 1) / sms;
+  const int64_t sms = device_sm_count(), windows = (int64_t)ceil_div(a.Wg, ww) * ceil_div(a.Hg, wh) * a.BH;
+  if (wh * ww <= 8 && (!prefix || (a.P + wh * ww <= 32 && windows >= 8 * sms))) return launch_attn_generic(a, st, true);
+  const int64_t ctas = windows * ceil_div(wh * ww, 2 * kRowsWarp);
+  const int64_t rounds2 = (ctas + sms - 1) / sms, rounds1 = (2 * ctas + sms - 1) / sms;
   if (wh * ww + a.P > 2 * kKeys && (rounds2 <= 2 || 5 * rounds1 <= 9 * rounds2)) return launch<1, 4>(a, false, prefix, st);
   return launch<2, 2>(a, false, prefix, st);
 }

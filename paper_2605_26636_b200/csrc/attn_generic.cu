@@ -107,11 +107,13 @@ attn_generic_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
 
 }  // namespace
 
-cudaError_t launch_attn_generic(const AttnArgs& a, cudaStream_t st) {
+// windows_only: without the prefix queries
+cudaError_t launch_attn_generic(const AttnArgs& a, cudaStream_t st, bool windows_only) {
   const int wh = a.wh < a.Hg ? a.wh : a.Hg, ww = a.ww < a.Wg ? a.ww : a.Wg;
   const int nwy = ceil_div(a.Hg, wh), nwx = ceil_div(a.Wg, ww);
-  const int rows_max = a.P > wh * ww ? a.P : wh * ww;
-  dim3 grid(ceil_div(rows_max, kRows), nwy * nwx + (a.P > 0 ? 1 : 0), a.BH);
+  const bool prefix = a.P > 0 && !windows_only;
+  const int rows_max = prefix && a.P > wh * ww ? a.P : wh * ww;
+  dim3 grid(ceil_div(rows_max, kRows), nwy * nwx + (prefix ? 1 : 0), a.BH);
   const size_t smem = (size_t)(2 * kTile * (a.D + 1) + kRows * a.D) * sizeof(float);
   if (a.dtype == JV_F32)
     attn_generic_kernel<float><<<grid, kRows * 32, smem, st>>>(

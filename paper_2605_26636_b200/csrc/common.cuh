@@ -157,7 +157,7 @@ struct AttnArgs {
   float scale;
   int dtype;
 };
-cudaError_t launch_attn_generic(const AttnArgs& a, cudaStream_t st);
+cudaError_t launch_attn_generic(const AttnArgs& a, cudaStream_t st, bool windows_only = false);
 // the P prefix queries of window attention on their own, ahead of the launch of the windows, which leaves `free_sms` SMs
 // to it (bf16, D == 64, contiguous)
 cudaError_t launch_attn_prefix(const AttnArgs& a, int free_sms, const int* status, cudaStream_t st);

@@ -56,6 +56,34 @@ def test_fp32_kernels(jv, oracle, case):
         assert rel_err(pick(out.cpu()), ref()) <= TOL["f32"], (name, case)
 
 
+# Windows of up to eight tokens are the kernel of one warp per query row's, with prefix tokens where there are many of them (B = 4) and a window's keys
+# are at most 32; their prefix queries are not; windows of nine tokens are one launch of this kernel.
+@pytest.mark.parametrize("B,P", [(2, 0), (2, 1), (4, 1), (4, 24), (4, 31), (4, 70)])
+@pytest.mark.parametrize("wh,ww", [(1, 1), (2, 2), (2, 4), (8, 1), (3, 3), (1, 9)])
+def test_fp32_small_windows(jv, oracle, B, P, wh, ww):
+    H, Hg, Wg = 8, 15, 19
+    q, k, v = inputs.custom_qkv(B, H, P + Hg * Wg, 64, "f32", seed=3400 + P + wh)
+    out, check = guarded_empty(q.shape, torch.float32, DEV)
+    out.fill_(float("nan"))
+    launches = jv.launch_count()
+    jv.window_attn(*(t.to(DEV) for t in (q, k, v)), Hg, Wg, wh, ww, out=out, prefix=P)
+    assert jv.launch_count() - launches == (2 if P else 1)
+    check()
+    heads = sample_heads(B, H, 4, P + wh)
+    pick = lambda t: torch.stack([t[b, h] for b, h in heads]).unsqueeze(0)
+    assert rel_err(pick(out.cpu()), oracle.window_attn(pick(q), pick(k), pick(v), Hg, Wg, wh, ww, prefix=P)) <= TOL["f32"]
+
+
+@pytest.mark.parametrize("N", [1, 2, 7, 8, 9])
+def test_fp32_short_sequences(jv, oracle, N):
+    q, k, v = inputs.custom_qkv(2, 5, N, 64, "f32", seed=3500 + N)
+    out, check = guarded_empty(q.shape, torch.float32, DEV)
+    out.fill_(float("nan"))
+    jv.full_attn(*(t.to(DEV) for t in (q, k, v)), out=out)
+    check()
+    assert rel_err(out, oracle.full_attn(q, k, v)) <= TOL["f32"]
+
+
 @pytest.mark.parametrize("static", [False, True], ids=["squeeze", "static"])
 @pytest.mark.parametrize("case", [(1, 1, 0, 1, 1), (1, 2, 0, 70, 1), (2, 3, 5, 11, 13), (1, 12, 1, 32, 32), (2, 2, 3, 3, 130), (2, 12, 0, 32, 32)],
                          ids=lambda c: "x".join(map(str, c)))
