@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(256)
 dwc_tok_apply_kernel(const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ o, const __half* __restrict__ wk,
                      const int* status, int H, int P, int Hg, int Wg) {
   __shared__ uint32_t wsm[8][9 * 32];
-  if (*reinterpret_cast<const volatile int*>(status) != 0) return;   // an earlier kernel gave up: o stays as it is
+  const bool gave_up = *reinterpret_cast<const volatile int*>(status) != 0;   // an earlier kernel gave up: o stays as it is
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ntok = P + Hg * Wg, N = Hg * Wg;
   const int bh = blockIdx.y, b = bh / H, h = bh - b * H;
@@ -125,7 +125,7 @@ dwc_tok_apply_kernel(const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restr
   uint32_t* dst = reinterpret_cast<uint32_t*>(o + ((size_t)bh * ntok + P + i) * kD + 2 * lane);
   const uint32_t cur = *dst;
   __nv_bfloat162 r = __floats2bfloat162_rn(__uint_as_float(cur << 16) + a0, __uint_as_float(cur & 0xffff0000u) + a1);
-  *dst = *reinterpret_cast<uint32_t*>(&r);
+  if (!gave_up) *dst = *reinterpret_cast<uint32_t*>(&r);
 }
 
 }  // namespace

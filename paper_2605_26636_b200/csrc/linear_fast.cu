@@ -502,7 +502,7 @@ template <int K>
 __global__ void __launch_bounds__(256)
 dwc_add_kernel(const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ o, const float* __restrict__ w,
                int w_batch, const int* status, int H, int Hg, int Wg, int run) {
-  if (*reinterpret_cast<const volatile int*>(status) != 0) return;   // an earlier kernel gave up: o stays as it is
+  const bool gave_up = *reinterpret_cast<const volatile int*>(status) != 0;   // an earlier kernel gave up: o stays as it is
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int N = Hg * Wg, bh = blockIdx.y, b = bh / H, h = bh % H;
   const int t0 = (blockIdx.x * 8 + warp) * run;
@@ -533,7 +533,7 @@ dwc_add_kernel(const __nv_bfloat16* __restrict__ v, __nv_bfloat16* __restrict__ 
     }
     __nv_bfloat162* op = reinterpret_cast<__nv_bfloat162*>(ob + (size_t)t * kD);
     const float2 cur = __bfloat1622float2(*op);
-    *op = __floats2bfloat162_rn(cur.x + s0, cur.y + s1);
+    if (!gave_up) *op = __floats2bfloat162_rn(cur.x + s0, cur.y + s1);
   }
 }
 
