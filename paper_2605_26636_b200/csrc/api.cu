@@ -178,7 +178,7 @@ jv_status run_attn(const void* q, const void* k, const void* v, void* o, const j
     if (!status) return JV_ERR_CUDA;
     if (a.strided && a.P > 0) return JV_ERR_UNSUPPORTED;  // the prefix queries' kernel reads contiguous tensors
     if (a.P > 0) {
-      const jv_status r = from_cuda(launch_attn_prefix(a, 0, status, st));
+      const jv_status r = from_cuda(launch_attn_prefix(a, device_sm_count() - attn_tc_ctas(a, full), status, st));
       if (r != JV_OK) return r;
     }
     return from_cuda(launch_attn_tc(a, full, status, st));

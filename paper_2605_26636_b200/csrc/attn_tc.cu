@@ -28,7 +28,7 @@
 // attend the P prefix keys.  They come in as one more key tile behind the window's own (a box of
 // a second pair of tensor maps that view the prefix rows in the box's shape), with the keys past P
 // masked like keys outside the grid.  The P prefix queries themselves (which attend everything)
-// are not served here.
+// are not served here, but by the launch ahead, beside which this one runs.
 //
 // Every mbarrier wait is bounded: a wait that runs out sets the device status word,
 // raises a CTA-wide abort flag, and every role falls through to the common teardown
@@ -180,7 +180,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, bar->tmem_base, 0);
 
-  griddep_wait();                 // what is read and written from here on may belong to the launch ahead
+  // With prefix tokens the launch ahead is that of their queries, which this one overlaps (it has waited for what came before
+  // it before it let this one go); this one waits for it at its end.
+  if (p.P == 0) griddep_wait();   // what is read and written from here on may belong to the launch ahead
   griddep_launch_dependents();
   // a timeout flagged earlier (by any CTA or launch) makes the rest leave at once
   if (threadIdx.x == 0 && *reinterpret_cast<volatile int*>(p.status) != 0) bar->abort_flag = 1;
@@ -188,6 +190,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   if (bar->abort_flag) {
     if (warp == 0)
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    if (p.P > 0) griddep_wait();
     return;
   }
 
@@ -670,6 +673,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
   }
 
   // ================= common teardown =================
+  if (p.P > 0) griddep_wait();    // no launch ends before the one ahead of it
   __syncwarp();
   tc_fence_before();
   __syncthreads();
@@ -709,6 +713,14 @@ bool attn_tc_supported(const AttnArgs& a, bool full) {
   if ((int64_t)g.nwx * g.nwy * ceil_div(g.tiles_per_window, 2) * a.BH > 0x7fffffffll) return false;
   // 128-byte rows keep every TMA stride a multiple of 16 bytes; the base must be 16-byte aligned (checked by the ABI)
   return encode_fn() != nullptr;
+}
+
+int attn_tc_ctas(const AttnArgs& a, bool full) {
+  Geometry g;
+  if (!geometry(a, full, &g)) return 0;
+  const int64_t items = (int64_t)ceil_div(g.tiles_per_window, 2) * g.nwx * g.nwy * a.BH;
+  const int sms = device_sm_count();
+  return (int)(items < sms ? items : sms);
 }
 
 cudaError_t launch_attn_tc(const AttnArgs& a, bool full, int* status, cudaStream_t st) {
@@ -792,9 +804,7 @@ cudaError_t launch_attn_tc(const AttnArgs& a, bool full, int* status, cudaStream
   p.div_H = make_fastdiv((uint32_t)a.H);
   p.scale_log2 = a.scale * 1.4426950408889634f;
   // persistent: one CTA per SM (shared memory and the 512 tensor-memory columns allow no more)
-  const int num_sms = device_sm_count();
-  const int grid = p.total_items < num_sms ? p.total_items : num_sms;
-  return launch_programmatic(attn_tc_kernel, dim3(grid), kThreads, kSmemBytes, st, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], p);
+  return launch_programmatic(attn_tc_kernel, dim3(attn_tc_ctas(a, full)), kThreads, kSmemBytes, st, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], p);
 }
 
 }  // namespace jv

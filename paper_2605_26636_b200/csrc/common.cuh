@@ -167,6 +167,7 @@ cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st);
 // tcgen05 path: bf16, D == 64.  full = true: F over all N tokens; else W with (wh, ww)
 // windows whose width ww is a power of two <= 128 (a tile is a box of ww x 128/ww tokens).
 bool attn_tc_supported(const AttnArgs& a, bool full);
+int attn_tc_ctas(const AttnArgs& a, bool full);   // CTAs (one per SM) of its launch
 cudaError_t launch_attn_tc(const AttnArgs& a, bool full, int* status, cudaStream_t st);
 // tcgen05 path for windows of one or two 128-token tiles (bf16, D == 64, at most 16 prefix tokens): two windows per CTA
 bool attn_w4_supported(const AttnArgs& a);
