@@ -63,3 +63,53 @@ def test_block_with_prefix_tokens(jv, oracle, B, H, Hg, Wg, P):
     ref = check(chain, xs)
     q, k, v = (t[:1, :2].cpu() for t in qkv)               # of the last pass
     assert rel_err(ref[-2][:1, :2], oracle.window_attn(q, k, v, Hg, Wg, 16, 16, prefix=P)) <= TOL["bf16"]
+
+
+def test_full_attention_split_behind_whole_rounds(jv, oracle):
+    """40 heads of 17 query tiles: one whole round of the four-tile kernel and, beside its end, the split-key kernel on what is left.  The second
+    call reads what both of the first one's launches wrote."""
+    B, H, N = 2, 20, 2100
+    q, k, v = (t.to(DEV) for t in inputs.custom_qkv(B, H, N, 64, "bf16", seed=430))
+    sources = [torch.roll(q, 7 * i, dims=2) for i in range(PASSES)]
+    o1, o2 = torch.empty_like(q), torch.empty_like(q)
+    launches = jv.launch_count()
+    jv.full_attn(q, k, v, out=o1)
+    assert jv.launch_count() - launches == 2
+
+    def chain(src, step):
+        jv.full_attn(src, k, v, out=o1)
+        step()
+        jv.full_attn(o1, k, src, out=o2)
+        step()
+        return o1, o2
+
+    ref = check(chain, sources)
+    pick = lambda t: t[1:, 19:].cpu()
+    assert rel_err(pick(ref[-1]), oracle.full_attn(pick(ref[-2]), pick(k), pick(sources[-1]))) <= TOL["bf16"]
+
+
+@pytest.mark.parametrize("dtype,D,H,Hg,Wg,P", [("f32", 64, 6, 37, 37, 5), ("f32", 64, 12, 16, 16, 0), ("bf16", 128, 8, 32, 33, 0), ("bf16", 128, 3, 9, 7, 0)])
+def test_one_mixer_behind_the_other(jv, oracle, dtype, D, H, Hg, Wg, P):
+    """Window, linear (fp32: with generated kernels) and full attention, each on the one before, on the fp32 kernels and at head_dim 128."""
+    N = P + Hg * Wg
+    q, k, v = (t.to(DEV) for t in inputs.custom_qkv(1, H, N, D, dtype, seed=440 + N))
+    d = {a: (t.to(DEV) if hasattr(t, "to") else t) for a, t in inputs.dwc_weights(H * D, 48, 3, 441).items()} if dtype == "f32" else None
+    sources = [torch.roll(q, 5 * i, dims=2) for i in range(PASSES)]
+    outs = [torch.empty_like(q) for _ in range(3)]
+
+    def chain(src, step):
+        jv.window_attn(src, k, v, Hg, Wg, 16, 16, out=outs[0], prefix=P)
+        step()
+        jv.linear_attn(src, k, outs[0], Hg, Wg, dwc=d, out=outs[1], prefix=P)
+        step()
+        jv.full_attn(src, k, outs[1], out=outs[2])
+        step()
+        return outs
+
+    ref = check(chain, sources)
+    src, o1, o2, o3 = (t[:, :2].cpu() for t in (sources[-1], *ref[-3:]))
+    kk, vv = k[:, :2].cpu(), v[:, :2].cpu()
+    assert rel_err(o1, oracle.window_attn(src, kk, vv, Hg, Wg, 16, 16, prefix=P)) <= TOL[dtype]
+    if d is None:
+        assert rel_err(o2, oracle.linear_attn(src, kk, o1, Hg, Wg, prefix=P)) <= TOL[dtype]
+    assert rel_err(o3, oracle.full_attn(src, kk, o2)) <= TOL[dtype]

@@ -22,10 +22,10 @@ def jv():
 
 
 def test_a_wait_that_runs_out_sets_the_status_and_nothing_hangs(jv, oracle):
-    Hg, Wg = 40, 32                                   # N = 1280: F runs on the four-tile kernel
+    Hg, Wg = 40, 32                                   # two heads of 1280 tokens, or of 512: F with its keys over four slots
     qh, kh, vh = inputs.custom_qkv(1, 2, Hg * Wg, 64, "bf16", seed=31)
     q, k, v = (t.to(DEV) for t in (qh, kh, vh))
-    qs, ks, vs = (t[:, :, :512].contiguous() for t in (q, k, v))    # 512 tokens: F on the two-tile kernel
+    qs, ks, vs = (t[:, :, :512].contiguous() for t in (q, k, v))
     dh = inputs.dwc_weights(2 * 64, 16, 3, 32)
     d = dwc_to_device(dh, DEV)
     calls = {
@@ -68,6 +68,70 @@ def test_a_wait_that_runs_out_sets_the_status_and_nothing_hangs(jv, oracle):
         assert torch.equal(o.view(-1)[:n], good[name].view(-1)[:n]), name
     assert rel_err(good["L+dwc"], oracle.linear_attn(qh, kh, vh, Hg, Wg, dwc=dh)) <= TOL["bf16"]
     assert rel_err(good["F"], oracle.full_attn(qh, kh, vh)) <= TOL["bf16"]
+    assert jv.device_status() == jv.JV_OK
+
+
+def test_every_tensor_core_kernel_leaves_at_once(jv):
+    """One call for each of the kernels that look at the status word, twice while it is set (tensor memory that the first one had not given back
+    would make the second one wait until its limit): the output keeps its contents, the call after the word has been
+    cleared computes what it computed before."""
+    def qkv(B, H, N, D=64, seed=0):
+        return tuple(t.to(DEV) for t in inputs.custom_qkv(B, H, N, D, "bf16", seed=500 + seed))
+
+    def proj(B, N, H):
+        C = 64 * H
+        x = inputs.normal((B, N, C), 5100 + N, "bf16").to(DEV)
+        (w, b), (wo, bo) = inputs.proj_weights(3 * C, C, 5200), inputs.proj_weights(C, C, 5201)
+        return x, w.to(DEV), b.to(DEV), wo.to(DEV), bo.to(DEV)
+
+    d = dwc_to_device(inputs.dwc_weights(4 * 64, 16, 3, 501), DEV)
+    calls = {}
+
+    def mixer(name, q, fn):
+        calls[name] = (lambda o: fn(o[0]), [torch.empty_like(q)])
+
+    q1, k1, v1 = qkv(1, 48, 1024, seed=1)             # 96 groups of four query tiles
+    mixer("F, four-tile kernel", q1, lambda o: jv.full_attn(q1, k1, v1, out=o))
+    q2, k2, v2 = qkv(1, 24, 1024, seed=2)             # 96 pairs
+    mixer("F, two-tile kernel", q2, lambda o: jv.full_attn(q2, k2, v2, out=o))
+    q3, k3, v3 = qkv(2, 20, 2100, seed=3)
+    mixer("F, keys over four slots behind a round of the four-tile kernel", q3, lambda o: jv.full_attn(q3, k3, v3, out=o))
+    q4, k4, v4 = qkv(1, 300, 200, seed=4)
+    mixer("F, window kernel", q4, lambda o: jv.full_attn(q4, k4, v4, out=o))
+    q5, k5, v5 = qkv(1, 4, 5 + 40 * 36, seed=5)
+    for win in (8, 16, 32):
+        mixer(f"W {win} with prefix tokens", q5, lambda o, win=win: jv.window_attn(q5, k5, v5, 40, 36, win, win, out=o, prefix=5))
+    mixer("L with prefix tokens", q5, lambda o: jv.linear_attn(q5, k5, v5, 40, 36, dwc=d, out=o, prefix=5))
+    q6, k6, v6 = qkv(2, 8, 40 * 30, 128, seed=6)
+    mixer("F, head_dim 128", q6, lambda o: jv.full_attn(q6, k6, v6, out=o))
+    mixer("W, head_dim 128", q6, lambda o: jv.window_attn(q6, k6, v6, 40, 30, 16, 16, out=o))
+    mixer("L, head_dim 128", q6, lambda o: jv.linear_attn(q6, k6, v6, 40, 30, out=o))
+    for name, (B, N, H) in (("one CTA", (1, 300, 6)), ("pairs", (3, 3100, 8))):
+        x, w, b, wo, bo = proj(B, N, H)
+        outs = [torch.empty((B, H, N, 64), dtype=torch.bfloat16, device=DEV) for _ in range(3)]
+        calls[f"qkv_proj, {name}"] = (lambda o, x=x, w=w, b=b, H=H, N=N: jv.qkv_proj(x, w, b, H, 1, N, out=tuple(o)), outs)
+        src = torch.randn((B, H, N, 64), device=DEV).bfloat16()
+        calls[f"out_proj, {name}"] = (lambda o, src=src, wo=wo, bo=bo, N=N: jv.out_proj(src, wo, bo, 1, N, out=o[0]), [torch.empty_like(x)])
+
+    assert jv.device_status() == jv.JV_OK
+    good = {}
+    for name, (fn, outs) in calls.items():
+        fn(outs)
+        good[name] = [o.clone() for o in outs]
+    assert jv.device_status() == jv.JV_OK
+    jv.selftest_wait_timeout(1000)
+    for fn, outs in calls.values():
+        for o in outs:
+            o.fill_(1234.5)
+        fn(outs)
+        fn(outs)
+    torch.cuda.synchronize()
+    for name, (fn, outs) in calls.items():
+        assert all(bool((o == 1234.5).all()) for o in outs), name
+    assert jv.device_status() == jv.JV_ERR_TIMEOUT
+    for name, (fn, outs) in calls.items():
+        fn(outs)
+        assert all(torch.equal(a, b) for a, b in zip(outs, good[name])), name
     assert jv.device_status() == jv.JV_OK
 
 
