@@ -209,8 +209,8 @@ def test_other_model_shapes(jv, oracle, case):
 @pytest.mark.parametrize("case", [(1, 3, 32, 32), (1, 2, 37, 29), (2, 1, 35, 40), (1, 1, 31, 33)],
                          ids=lambda c: "x".join(map(str, c)))
 def test_full_attention_long_sequences(jv, oracle, case):
-    """N >= 1024 runs on the kernel with four query tiles per CTA: tile counts of 8, 9, 11 (the last item
-    of a head holds one or three tiles) with ragged last key tiles, and 1023 tokens just below the switch."""
+    """Few heads of about 1024 tokens (keys over four slots): 8, 9 and 11 query tiles a head, ragged last key tiles, and
+    1023 tokens.  The other kernels at these lengths: tests/test_full_attention_routes_gpu.py."""
     B, H, Hg, Wg = case
     q, k, v = inputs.custom_qkv(B, H, Hg * Wg, 64, "bf16", seed=Hg + Wg)
     out, check = guarded_empty(q.shape, torch.bfloat16, DEV)

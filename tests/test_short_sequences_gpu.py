@@ -1,6 +1,6 @@
 """Full attention by length and heads.  Below 1024 tokens: at most two tiles on the window kernel (one token, a tile less one, a tile,
-a tile and one, two tiles), the rest by heads and tiles on the four-tile or the two-tile kernel; q, k, v contiguous and in a
-fused activation."""
+a tile and one, two tiles), the rest by heads and tiles on the split-key, the four-tile or the two-tile kernel; q, k, v contiguous and
+in a fused activation."""
 import pytest
 import torch
 
@@ -44,8 +44,8 @@ def test_short_sequences(jv, oracle, case, fused):
     assert bool(torch.isfinite(out).all())
 
 
-# B, H, N: groups of three (the last of a head with two tiles, and whole), single tiles and pairs of tiles in the last round
-# (the last piece of a head empty, or its last tile ragged), pairs on the two-tile kernel
+# B, H, N: groups of three (the last of a head with two tiles, and whole), the split-key kernel behind a round of the four-tile one, pairs on the two-tile
+# kernel, the split-key kernel alone in two rounds
 SPLITS = [(1, 16, 2880), (1, 16, 3070), (2, 19, 2048), (2, 19, 1600), (1, 26, 4096), (2, 13, 4000), (1, 12, 3025)]
 
 

@@ -37,10 +37,10 @@ def bnhd_views(q, k, v):
 
 
 CASES = [  # B, H, Hg, Wg, win_h, win_w
-    (2, 3, 64, 64, 16, 16),      # two-tile windows; N = 4096: the four-tile full-attention kernel
+    (2, 3, 64, 64, 16, 16),      # two-tile windows; N = 4096: full attention with its keys over four slots
     (1, 2, 73, 73, 16, 16),      # ragged grid: edge windows, clipped tiles
     (2, 2, 24, 40, 8, 16),       # one-tile windows
-    (1, 4, 17, 33, 8, 8),        # windows of 64 tokens: the two-tile-per-CTA kernel; short full attention
+    (1, 4, 17, 33, 8, 8),        # windows of 64 tokens, four to an item; short full attention
     (3, 1, 40, 24, 40, 24),      # one window: W is F
 ]
 
