@@ -10,7 +10,7 @@
 //
 // Measured, before (the better of the four-tile and the two-tile kernel) / now, us: 6 heads of 1370 tokens 22.0 / 13.0, of 3038 tokens
 // 44.3 / 22.3, of 5329 71 / 64; 24 of 576 13.3 / 8.9; 16 of 1030 20.7 / 12.3.  Behind whole rounds of four tiles: 12 heads of 6988 tokens
-// 232 / 176, 64 of 5329 571 / 546, 16 of 16384 1204 / 1152.
+// 232 / 176, 64 of 5329 591 / 566 (in turn, in a loop at the power cap), 16 of 16384 1204 / 1152.
 //
 // Warp roles (19 warps): 0 TMA producer, 1 and 2 MMA issuers (slots 0, 1 and 2, 3), 3-18 softmax, one thread per query row
 // and slot, then the merge, one thread per query row and 16 channels.  A slot has its own rings of K and V in boxes of 64 keys; when
@@ -396,8 +396,8 @@ attn_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
 }
 
 // In steps of 64 keys of the four-tile kernel a round of tiles here takes a quarter of the steps of a head, and 3.5 more.  The
-// comparison with the other kernels (2 steps of overhead) is right to 4 % over 6 to 96 heads of 300 to 16384 tokens: 12 heads of 4111
-// tokens 77.7 us here / 78.4 there, 16 of 4096 100 / 88, 24 of 1024 22.6 / 20.9 (two tiles at a time), 32 of 1043 24.5 / 28.3.
+// comparison with the other kernels (2 steps of overhead) takes the faster side, or one within 2.5 % of it, over 6 to 192 heads of 320 to 8192
+// tokens: 16 of 4096 101 us here / 86 there, 24 of 1024 20.2 / 18.0 (two tiles at a time), 64 of 4096 334 / 345, 48 of 2500 110.6 / 108.7.
 // What of a call goes where: `groups` groups of four tiles to the four-tile kernel (whole rounds of it, or none), `tiles` here.
 struct SplitPlan {
   int groups, tiles;

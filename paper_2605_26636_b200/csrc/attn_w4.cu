@@ -31,11 +31,11 @@
 // producer may refill that buffer when the four warps that staged into it have seen their stores read it, which they
 // check one step into their next item, off the critical path.
 //
-// Measured (8 x 16 heads, 64 x 64 tokens, 16 x 16 windows, back to back): 66.7 us = 4.0 TB/s; with five prefix tokens (their
-// queries' kernel, then 41.5 us, included) 109 us.  With one Q buffer per tile, K and V in whole tiles and the output staged over V it was 71.0
-// and 118.9: a window's Q could only be copied once the window before had issued its last scores, and there was no
-// room for a third V stage beside the prefix rows.  32 x 12 heads, 16 x 16 tokens, 8 x 8 windows: 20 us less than on attn_tc.cu, where
-// half of a tile's rows, and half of the exponentials of the rest, are of no use.
+// Measured (8 x 16 heads, 64 x 64 tokens, 16 x 16 windows): 55 us = 4.85 TB/s in short runs, 65.5 in a long loop at the power cap; with five
+// prefix tokens (their queries' kernel, 29 us, included) 89 and 100.  With one Q buffer per tile, K and V in whole tiles and the output staged over
+// V it was 60 and 71 (114 and 119): a window's Q could only be copied once the window before had issued its last scores, and there was no
+// room for a third V stage beside the prefix rows.  8 x 8 windows, 32 x 12 heads of 16 x 16 tokens 12.8 us, 8 x 16 of 64 x 64 46.1 (on attn_tc.cu, where
+// half of a tile's rows, and half of the exponentials of the rest, are of no use, 186).
 //
 // Every mbarrier wait is bounded: a wait that runs out sets the device status word, raises a
 // CTA-wide abort flag, and every role falls through to the common teardown (tensor memory is

@@ -13,8 +13,9 @@
 // tiles, which need not be neighbours, half of the tile's weights, and the accumulator rows of its own tokens.
 // What bounds a tile of one CTA is not the tensor pipe but shared memory: a K block of 64 is 48 KB written by the copies
 // and 48 KB read by the MMAs, 768 clocks for 512 clocks of MMA; with the weights shared by two CTAs it is 32 + 32 KB.
-// Measured (2 x 8192 tokens, 768 -> 2304 / 8 x 4096 tokens, 1024 -> 3072 features): 46.2 / 138 us = 1254 / 1493 TF in pairs,
-// 49.7 / 153 us singly; with four epilogue warps instead of eight and the bias fetched after the accumulator, 53.4 / 152.
+// Measured (2 x 8192 tokens, 768 -> 2304 / 8 x 4096 tokens, 1024 -> 3072 features, in turn): 44.4 / 140 us = 1307 / 1475 TF in pairs, 48.2 / 157
+// singly, in short runs; 51.5 / 160 and 55.4 / 184 in a long loop at the power cap.  With four epilogue warps instead of eight and the bias fetched
+// after the accumulator (single CTAs, another run) 53.4 / 152, when this form took 49.7 / 153.
 // Warp roles (both CTAs of a pair):
 //   warp 0      TMA producer: A (128 tokens x 64) and (half of) B (256 features x 64) through a ring of 4 (5) stages; the
 //               copies of both CTAs report to the leader's barrier
@@ -436,8 +437,9 @@ cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorM
 }
 
 // Pairs of CTAs where every pair has three tiles or more: a pair takes 2 us longer to start (cluster launch, two cluster
-// barriers) and a tile of it is a tenth faster or more.  Measured, single / pair: 30 tiles of a pair 9.1 / 11.1 us, 54: 15.3 / 17.3,
-// 96: 18.9 / 20.9, 192: 23.0 / 23.0, 288: 33.2 / 33.2, 576: 49.7 / 46.2, 512 of 16 K blocks: 57.5 / 53.1, 1536: 153 / 138.
+// barriers) and a tile of it is a tenth faster or more.  Measured in turn in long loops, single / pair: 24 tiles of a pair 8.9 / 10.0 us, 72: 9.6 / 10.7,
+// 96: 13.6 / 14.2, 192: 18.5 / 18.5 and (16 K blocks) 22.5 / 21.6, 288: 23.9 / 23.9 and (24) 48.5 / 45.2, 576: 55.4 / 51.5, 512 (16): 66.8 / 61.0, 1536:
+// 184 / 160.
 bool pair_tiles(int64_t tiles_m, int tiles_n) {
   return (tiles_m + 1) / 2 * tiles_n >= 3 * (device_sm_count() / 2);
 }
