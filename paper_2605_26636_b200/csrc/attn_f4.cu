@@ -219,10 +219,12 @@ attn_f4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       ++n;
     }
     if (!ok && lane == 0) {
-      // let the copies still in flight land before the CTA leaves (bounded by the same limit)
+      // let the copies still in flight land before the CTA leaves (bounded by the same limit): those of V by their
+      // barriers, those of K and Q around them by a millisecond from here
       const unsigned long long t0 = globaltimer();
       for (int g = max(0, issued_v - kStages); g < issued_v; ++g)
         while (!mbar_try(&bar->v_full[g % kStages], (g / kStages) & 1) && globaltimer() - t0 < kWaitLimitNs) {}
+      while (globaltimer() - t0 < 1000000ull) {}
     }
   } else if (warp == 1 || warp == 2) {
     // ================= MMA issuers: warp 1 serves query tiles 0 and 1, warp 2 tiles 2 and 3 =================

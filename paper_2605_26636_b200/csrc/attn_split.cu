@@ -181,6 +181,7 @@ attn_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
     if (!ok && lane == 0) {
       // let the copies still in flight land before the CTA leaves (bounded by the same limit)
       const unsigned long long t0 = globaltimer();
+      while (!mbar_try(&bar->q_full, 0) && globaltimer() - t0 < kWaitLimitNs) {}
 #pragma unroll
       for (int t = 0; t < kSlots; ++t)
         for (int g = max(0, issued[t] - kStages); g < issued[t]; ++g) {

@@ -282,10 +282,12 @@ attn_w4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       ++n;
     }
     if (!ok && lane == 0) {
-      // let the copies still in flight land before the CTA leaves (bounded by the same limit)
+      // let the copies still in flight land before the CTA leaves (bounded by the same limit): those of V by their
+      // barriers, those of K and Q around them by a millisecond from here
       const unsigned long long t0 = globaltimer();
       for (int g = max(0, issued_v - kVS); g < issued_v; ++g)
         while (!mbar_try(&bar->v_full[s][g % kVS], (g / kVS) & 1) && globaltimer() - t0 < kWaitLimitNs) {}
+      while (globaltimer() - t0 < 1000000ull) {}
     }
   } else if (warp < 2 * kSlots) {
     // ================= MMA issuer of slot `warp - 2`: both query tiles of the slot's item =================
