@@ -15,11 +15,12 @@
 // place: with three CTAs on an SM the others compute while one waits for a copy), and the groups' partial softmaxes are
 // merged at the end.
 //
-// Measured (12 heads, 32 x 32 tokens; the kernel of one warp per query row, which served these calls before and still
-// serves other head dims and windows of at most eight tokens, in brackets): full attention 93 us (729), 16 x 16 windows 27 us (195); 6 heads, 16 x 16
-// tokens, full attention 8 us (63).  Full attention runs at 35 TFLOP/s (41 where the grid fills the chip evenly) of the 73 that
-// a loop of nothing but multiply-adds reaches: one of three instructions is not a multiply-add, and the registers leave room
-// for three warps per scheduler.
+// It serves what does not fill the chip with its row tiles, short rows of queries and the prefix queries of windows; the rest goes to the
+// tensor cores (attn_f32_tc.cu; the line between the two: launch_attn_f32).  Measured (6 heads, 16 x 16 tokens; the kernel of one warp
+// per query row, which serves other head dims and windows of at most eight tokens, in brackets): full attention 8 us (63).  Where it fills the chip it
+// runs at 35 to 41 TFLOP/s of the 73 that a loop of nothing but multiply-adds reaches: one of three instructions is not a
+// multiply-add, and the registers leave room for three warps per scheduler.
+#include <cooperative_groups.h>
 #include "f32_common.cuh"
 
 namespace jv {
@@ -40,11 +41,13 @@ constexpr size_t smem_bytes() {
   return ((size_t)(R * kRowsWarp + G * kKeys) * kLd + R * G * kWarpBuf) * sizeof(float);
 }
 
-// prefix_rows: the launch serves the P prefix queries (keys: all tokens) instead of the windows.
-template <int R, int G>
-__global__ void __launch_bounds__(32 * R * G, G == 8 ? 1 : G == 4 ? 2 : 3)  // what shared memory leaves room for
+// kPrefix: the launch serves the P prefix queries (keys: all tokens) instead of the windows, by clusters of blocks along x that
+// share the keys of a row tile and merge their partial softmaxes through distributed shared memory.
+template <int R, int G, bool kPrefix>
+__global__ void __launch_bounds__(32 * R * G, G == 4 ? 2 : 3)  // what shared memory leaves room for
 attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ o,
-                int Hg, int Wg, int P, int wh, int ww, int nwx, bool prefix_rows, bool overlap, float scale) {
+                int Hg, int Wg, int P, int wh, int ww, int nwx, bool overlap, float scale) {
+  namespace cg = cooperative_groups;
   extern __shared__ __align__(16) float smem_f[];
   float* qs = smem_f;                                        // [16 R][kLd]
   float* ps = qs + R * kRowsWarp * kLd;                      // [R G warps]: probabilities [64 keys][kLdP], then the warp's output [16][kLd]
@@ -56,18 +59,19 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tx = lane & 15, ty = lane >> 4;
   const int grp = warp / R, rw = warp % R;                   // key group, row warp
   const int N = P + Hg * Wg;
+  const int nsplit = kPrefix ? (int)cg::this_cluster().num_blocks() : 1, split = kPrefix ? (int)cg::this_cluster().block_rank() : 0;
   const int wy = blockIdx.y / nwx, wx = blockIdx.y % nwx;
-  const int y0 = prefix_rows ? 0 : wy * wh, x0 = prefix_rows ? 0 : wx * ww;
+  const int y0 = kPrefix ? 0 : wy * wh, x0 = kPrefix ? 0 : wx * ww;
   const int vh = min(wh, Hg - y0), vw = min(ww, Wg - x0);    // valid extent of this window
-  const int nq = prefix_rows ? P : vh * vw;                  // query rows; keys: prefix tokens, then the window's own
-  const int cnt = prefix_rows ? N : P + vh * vw;
-  const int row0 = blockIdx.x * (R * kRowsWarp);
+  const int nq = kPrefix ? P : vh * vw;                  // query rows; keys: prefix tokens, then the window's own
+  const int cnt = kPrefix ? N : P + vh * vw;
+  const int row0 = blockIdx.x / nsplit * (R * kRowsWarp);
   if (row0 >= nq) return;                                    // beyond a small edge window
   const size_t base = (size_t)blockIdx.z * N * kDim;
-  const bool dense = prefix_rows || vw == Wg;                // consecutive keys are consecutive tokens
+  const bool dense = kPrefix || vw == Wg;                // consecutive keys are consecutive tokens
   auto key_token = [&](int c) -> int {
     if (c < P) return c;
-    if (dense) return prefix_rows ? c : c + y0 * Wg;
+    if (dense) return kPrefix ? c : c + y0 * Wg;
     const int g = c - P, y = g / vw;
     return P + (y0 + y) * Wg + x0 + (g - y * vw);
   };
@@ -97,17 +101,18 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
   float* kg = ks + grp * kKeys * kLd;
   float* pw = ps + warp * kWarpBuf;
   const int ntiles = (cnt + kKeys - 1) / kKeys;
+  const int first = split * G + grp, stride = nsplit * G;
 
   if (grp == 0) {                                            // Q: group 0 copies the CTA's rows
     const int mine = row0 + rw * kRowsWarp + (lane & 15);
-    const int tok = mine < nq ? key_token(prefix_rows ? mine : P + mine) : -1;
+    const int tok = mine < nq ? key_token(kPrefix ? mine : P + mine) : -1;
 #pragma unroll
     for (int j = 0; j < kRowsWarp / 2; ++j) {
       const int r = 2 * j + ty, tk = __shfl_sync(0xffffffffu, tok, r);
       copy16(qs + (rw * kRowsWarp + r) * kLd + 4 * tx, q + base + (size_t)max(tk, 0) * kDim + 4 * tx, tk >= 0);
     }
   }
-  if (grp < ntiles) load_tile(kg, k, grp);                   // (one copy group with Q)
+  if (first < ntiles) load_tile(kg, k, first);                   // (one copy group with Q)
   else copy_commit();
   if (G > 1) {                                               // Q comes from group 0: everybody waits for it once
     copy_wait<0>();
@@ -127,7 +132,7 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
 #pragma unroll
     for (int e = 0; e < 4; ++e) acc[i][e] = 0ull;
 
-  for (int t = grp; t < ntiles; t += G) {
+  for (int t = first; t < ntiles; t += stride) {
     copy_wait<0>();                                          // K of this tile
     group_sync();
     f32x2 s2[8][4];
@@ -209,7 +214,7 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
       }
     }
     group_sync();                                            // the group is done with V (and the warp with its P)
-    if (t + G < ntiles) load_tile(kg, k, t + G);
+    if (t + stride < ntiles) load_tile(kg, k, t + stride);
   }
 
 #pragma unroll
@@ -234,63 +239,94 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
     }
   }
   __syncthreads();
+  // n partial softmaxes of a row -> maximum, sum and this lane's four channels
+  auto combine = [&](int n, auto&& src_of, float& M, float& L) -> float4 {
+    M = -INFINITY;
+    for (int i = 0; i < n; ++i) M = fmaxf(M, src_of(i)[64]);
+    L = 0.f;
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = 0; i < n; ++i) {
+      const float* src = src_of(i);
+      const float f = M == -INFINITY ? 0.f : expf(src[64] - M);        // a source without a key of weight: exp(-inf) = 0
+      const float4 y = *reinterpret_cast<const float4*>(src + 4 * tx);
+      L = fmaf(src[65], f, L);
+      x.x = fmaf(y.x, f, x.x);
+      x.y = fmaf(y.y, f, x.y);
+      x.z = fmaf(y.z, f, x.z);
+      x.w = fmaf(y.w, f, x.w);
+    }
+    return x;
+  };
+  auto store = [&](int row, const float4& x, float L) {
+    const float inv = 1.f / L;
+    const int tok = key_token(kPrefix ? row : P + row);
+    *reinterpret_cast<float4*>(o + base + (size_t)tok * kDim + 4 * tx) = make_float4(x.x * inv, x.y * inv, x.z * inv, x.w * inv);
+  };
   constexpr int kOwnRows = kRowsWarp / G;                    // rows of row warp rw that this warp writes out
 #pragma unroll
   for (int j = 0; j < kOwnRows / 2; ++j) {
     const int r = grp * kOwnRows + 2 * j + ty, row = row0 + rw * kRowsWarp + r;
     if (row < nq) {
-      float M = -INFINITY;
-#pragma unroll
-      for (int g = 0; g < G; ++g) M = fmaxf(M, ps[(g * R + rw) * kWarpBuf + r * kLd + 64]);
-      float L = 0.f;
-      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        const float* src = ps + (g * R + rw) * kWarpBuf + r * kLd;
-        const float f = expf(src[64] - M);                   // a group without a tile, or a key: exp(-inf) = 0
-        const float4 y = *reinterpret_cast<const float4*>(src + 4 * tx);
-        L = fmaf(src[65], f, L);
-        x.x = fmaf(y.x, f, x.x);
-        x.y = fmaf(y.y, f, x.y);
-        x.z = fmaf(y.z, f, x.z);
-        x.w = fmaf(y.w, f, x.w);
+      float M, L;
+      const float4 x = combine(G, [&](int g) { return ps + (g * R + rw) * kWarpBuf + r * kLd; }, M, L);
+      if (nsplit == 1) {
+        store(row, x, L);
+      } else {                                               // this block's share, over Q
+        float* dst = qs + (rw * kRowsWarp + r) * kLd;
+        *reinterpret_cast<float4*>(dst + 4 * tx) = x;
+        if (tx == 0) {
+          dst[64] = M;
+          dst[65] = L;
+        }
       }
-      const float inv = 1.f / L;
-      const int tok = key_token(prefix_rows ? row : P + row);
-      *reinterpret_cast<float4*>(o + base + (size_t)tok * kDim + 4 * tx) = make_float4(x.x * inv, x.y * inv, x.z * inv, x.w * inv);
     }
+  }
+  if (kPrefix && nsplit > 1) {
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    for (int r = split + nsplit * (2 * warp + ty); r < R * kRowsWarp; r += 2 * R * G * nsplit)   // (uniform over 16 lanes)
+      if (row0 + r < nq) {
+        float M, L;
+        const float4 x = combine(nsplit, [&](int i) { return cluster.map_shared_rank(qs, i) + r * kLd; }, M, L);
+        store(row0 + r, x, L);
+      }
+    cluster.sync();                                          // no block leaves while its shared memory may still be read
   }
   if (overlap) griddep_wait();
 }
 
-template <int R, int G>
-cudaError_t launch(const AttnArgs& a, bool prefix_rows, bool overlap, cudaStream_t st) {
+template <int R, int G, bool kPrefix>
+cudaError_t launch(const AttnArgs& a, int split, bool overlap, cudaStream_t st) {   // split: blocks to a cluster (the prefix queries)
   static OncePerDevice opt_in;
   const cudaError_t e = opt_in.run([&] {
-    return cudaFuncSetAttribute(attn_f32_kernel<R, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<R, G>());
+    return cudaFuncSetAttribute(attn_f32_kernel<R, G, kPrefix>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<R, G>());
   });
   if (e != cudaSuccess) return e;
   const int wh = a.wh < a.Hg ? a.wh : a.Hg, ww = a.ww < a.Wg ? a.ww : a.Wg;
   const int nwx = ceil_div(a.Wg, ww), nwin = nwx * ceil_div(a.Hg, wh);
-  const dim3 grid = prefix_rows ? dim3(ceil_div(a.P, R * kRowsWarp), 1, a.BH) : dim3(ceil_div(wh * ww, R * kRowsWarp), nwin, a.BH);
-  return launch_programmatic(attn_f32_kernel<R, G>, grid, 32 * R * G, smem_bytes<R, G>(), st, (const float*)a.q, (const float*)a.k,
-                             (const float*)a.v, (float*)a.o, a.Hg, a.Wg, a.P, wh, ww, nwx, prefix_rows, overlap, a.scale);
+  const dim3 grid = kPrefix ? dim3(ceil_div(a.P, R * kRowsWarp) * split, 1, a.BH) : dim3(ceil_div(wh * ww, R * kRowsWarp), nwin, a.BH);
+  return launch_cluster(true, attn_f32_kernel<R, G, kPrefix>, kPrefix ? split : 0, grid, 32 * R * G, smem_bytes<R, G>(), st, (const float*)a.q,
+                        (const float*)a.k, (const float*)a.v, (float*)a.o, a.Hg, a.Wg, a.P, wh, ww, nwx, overlap, a.scale);
 }
 
 }  // namespace
 
 bool attn_f32_supported(const AttnArgs& a) { return a.dtype == JV_F32 && a.D == kDim && !a.strided; }
 
-// The P prefix queries go first, with the keys of a row tile split over eight or four groups (their chain is the
-// longest: all N keys); the windows' launch overlaps them, as neither reads what the other writes.  Eight groups take an SM each: for
-// few heads or long sequences.  Four / eight groups, us for the call: 6 heads, 16 x 16 tokens, 8 x 8 windows 11.8 / 10.2, 6 of 37 x 37 33.2 /
-// 27.7, 24 of 37 x 37, 16 x 16 windows 106 / 87; 24 of 24 x 24 47.7 / 50.1.
-// 32 rows x 2 groups per CTA (three on an SM) or 16 rows x 4 groups (two): the second halves the chain of a CTA, and its
-// finer grain leaves less of the last round empty; the first is 10 % faster where both fill the chip.  Measured, 32 x 2 against
-// 16 x 4 with up to two CTAs of 32 rows per SM: 48 CTAs 13 / 8 us, 150 CTAs 57 / 33, 256 CTAs 92 / 69.  Beyond that by
-// rounds, at 9 to 5 for one round of either: 300 CTAs 78 / 60 us (3 and 5 rounds), 384 CTAs 93 / 99 (3 and 6), 512 CTAs
-// 122 / 116 (4 and 7), 688 CTAs 202 / 222 (5 and 10).  Windows of one or two key tiles have no work for four groups (432
-// CTAs, 8 x 8 windows: 18 / 33 us).
+// The P prefix queries go first, with the keys of a row tile split over the four groups of up to eight blocks (their chain is the longest: all
+// N keys), two blocks to an SM; the windows' launch overlaps them, as neither reads what the other writes.  Eight groups of one block / up to 32 of
+// a cluster, us for the call: 6 heads of 37 x 37, 8 x 8 windows 33.4 / 13.6, 12 of 37 x 37, 16 x 16 49.6 / 27.8, 24 of 32 x 32 45.4 / 29.8 (in
+// clusters of at most 148 blocks in all 31.8).
+//
+// Windows and sequences go to the tensor cores (attn_f32_tc.cu) where they fill the chip with row tiles of this kernel.  That one's blocks
+// take 128 rows and start slowly: 7 us for one tile of keys, 10 for two, 12 for four, where this one takes 7 to 8 as long as every SM has one block.
+// This / that one, us: 6 heads of 256 tokens 8.2 / 12.1, 12 of 256 11.4 / 12.2, 6 of 400 19.0 / 15.6, 24 of 256 17.6 / 12.5, 12 of 1024 93 / 26.3; 48 of 100
+// 11.1 / 9.5, 24 of 128 8.1 / 10.2; of 64 tokens: 48 heads 7.5 / 7.5, 96 10.6 / 8.0, 192 (two rounds there) 11.4 / 14.6; 8 x 8 windows,
+// 6 heads of 24 x 24 8.1 / 10.6, 6 of 32 x 32 11.1 / 10.4, 48 of 32 x 32 41.7 / 33.1.  Rows of at most 32 queries stay here (a tile there would be
+// three quarters empty): 4 x 4 windows, 48 heads of 32 x 32 72 / 87.
+//
+// Here, 32 rows x 2 groups per CTA (three on an SM) or 16 rows x 4 groups (two): the second halves the chain of a CTA, the first is 10 % faster
+// where both fill the chip.  Windows of one or two key tiles have no work for four groups (432 CTAs, 8 x 8 windows: 18 / 33 us).
 // Windows of at most eight tokens leave most of a 32 x 64 tile of scores empty: the kernel of one warp per query row, eight to a block, is the
 // better one.  This one / that one, 96 heads of 32 x 32 tokens: 2 x 2 windows 484 / 270 us, 2 x 4 256 / 148, 3 x 3 245 / 254; 12 heads of 64 x 64, 2 x 2
 // 235 / 135.  With prefix tokens, whose queries stay here: as long as a window's keys and they are one tile of that kernel, and the windows fill
@@ -301,16 +337,26 @@ cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st) {
   const bool prefix = a.P > 0;
   if (prefix) {
     const int N = a.P + a.Hg * a.Wg;
-    const bool eight = 8 * a.BH <= device_sm_count() || N >= 1024;
-    const cudaError_t e = eight ? launch<1, 8>(a, true, false, st) : launch<1, 4>(a, true, false, st);
+    const int64_t tiles = (int64_t)ceil_div(a.P, kRowsWarp) * a.BH;
+    int split = 1;
+    while (split < 8 && 2 * split * tiles <= 2 * device_sm_count() && split * 4 * kKeys < N) split *= 2;
+    const cudaError_t e = launch<1, 4, true>(a, split, false, st);
     if (e != cudaSuccess) return e;
   }
   const int64_t sms = device_sm_count(), windows = (int64_t)ceil_div(a.Wg, ww) * ceil_div(a.Hg, wh) * a.BH;
   if (wh * ww <= 8 && (!prefix || (a.P + wh * ww <= 32 && windows >= 8 * sms))) return launch_attn_generic(a, st, true);
-  const int64_t ctas = windows * ceil_div(wh * ww, 2 * kRowsWarp);
-  const int64_t rounds2 = (ctas + sms - 1) / sms, rounds1 = (2 * ctas + sms - 1) / sms;
-  if (wh * ww + a.P > 2 * kKeys && (rounds2 <= 2 || 5 * rounds1 <= 9 * rounds2)) return launch<1, 4>(a, false, prefix, st);
-  return launch<2, 2>(a, false, prefix, st);
+  const int nq = wh * ww, cnt = a.P + nq, key_tiles = ceil_div(cnt, kKeys);
+  const int64_t rows16 = windows * ceil_div(nq, kRowsWarp), rows32 = windows * ceil_div(nq, 2 * kRowsWarp);   // row tiles of this kernel
+  bool tc = nq > 2 * kRowsWarp;
+  if (cnt <= 2 * kKeys) tc = tc && rows32 > sms && (cnt > kKeys || windows > a.BH || a.BH <= sms);
+  else tc = tc && rows16 > sms && (key_tiles > 4 || 3 * rows16 > 4 * sms);
+  if (tc) {
+    int* status = device_status_ptr();
+    if (!status) return cudaErrorUnknown;
+    return launch_attn_f32_tc(a, prefix, status, st);
+  }
+  if (cnt > 2 * kKeys && rows32 <= 2 * sms) return launch<1, 4, false>(a, 1, prefix, st);
+  return launch<2, 2, false>(a, 1, prefix, st);
 }
 
 }  // namespace jv

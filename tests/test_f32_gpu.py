@@ -56,6 +56,82 @@ def test_fp32_kernels(jv, oracle, case):
         assert rel_err(pick(out.cpu()), ref()) <= TOL["f32"], (name, case)
 
 
+# Calls that fill the chip go to the tensor cores, each value as three bf16 terms: ragged last tiles of rows and keys, windows two to a block (an odd number of
+# them, and small ones at the edges), one key tile (a slot without work), prefix tokens in front of a window's keys.
+TC_CASES = [  # B, H, P, Hg, Wg, win
+    (1, 6, 0, 20, 20, 20),
+    (2, 12, 0, 13, 17, 16),
+    (1, 12, 5, 33, 35, 16),
+    (2, 12, 0, 17, 23, 8),
+    (2, 12, 1, 25, 27, 8),
+    (4, 24, 0, 8, 8, 8),
+    (1, 24, 70, 19, 10, 10),
+]
+
+
+def _tc_heads(q, k, v, heads):
+    return tuple(torch.stack([t[b, h] for b, h in heads]).unsqueeze(0) for t in (q, k, v))
+
+
+@pytest.mark.parametrize("case", TC_CASES, ids=lambda c: "x".join(map(str, c)))
+def test_fp32_tensor_cores(jv, oracle, case):
+    """Beside the bar of this file, the 2-norm of the error: a sum's last four additions at its full size are cut to 24 bits
+    (4 * 2^-23 at most, in the scores times their size, up to 8 here, and in the products with V): below 8 * 4 * 2^-23 = 4e-6."""
+    B, H, P, Hg, Wg, win = case
+    q, k, v = inputs.custom_qkv(B, H, P + Hg * Wg, 64, "f32", seed=3600 + P + Hg)
+    dq, dk, dv = (t.to(DEV) for t in (q, k, v))
+    heads = sample_heads(B, H, 4, P + Hg)
+    qs, ks, vs = _tc_heads(q, k, v, heads)
+    for name, call, ref in (
+            ("F", lambda o: jv.full_attn(dq, dk, dv, out=o), lambda: oracle.full_attn(qs, ks, vs)),
+            ("W", lambda o: jv.window_attn(dq, dk, dv, Hg, Wg, win, win, out=o, prefix=P),
+             lambda: oracle.window_attn(qs, ks, vs, Hg, Wg, win, win, prefix=P))):
+        out, check = guarded_empty(q.shape, torch.float32, DEV)
+        out.fill_(float("nan"))
+        call(out)
+        check()
+        o, r = _tc_heads(out.cpu(), out.cpu(), out.cpu(), heads)[0], ref()
+        assert rel_err(o, r) <= TOL["f32"], (name, case)
+        d = o.double().numpy() - r
+        assert float((d * d).sum() ** 0.5) <= 4e-6 * float((r * r).sum() ** 0.5), (name, case)
+
+
+@pytest.mark.parametrize("what", ["k -inf", "k lowest", "k inf", "q nan", "v inf", "v large"])
+def test_fp32_tensor_cores_special_values(jv, what):
+    """What is no finite number, or so large that products of bf16 terms overflow, gives what fp64 gives."""
+    B, H, N = 1, 6, 400
+    q, k, v = inputs.custom_qkv(B, H, N, 64, "f32", seed=3700)
+    name, value = what.split()
+    t = {"q": q, "k": k, "v": v}[name]
+    x = {"-inf": float("-inf"), "inf": float("inf"), "lowest": torch.finfo(torch.float32).min, "nan": float("nan"), "large": 1e37}[value]
+    q[0, 2, :, 3] = q[0, 2, :, 3].abs() + 0.5              # (an infinite score has one sign)
+    q[0, 2, :, 3] = (q[0, 2, :, 3] * 4).round() / 4         # (values that are one bf16 term)
+    t[0, 2, 130:140, 3] = x
+    out, check = guarded_empty(q.shape, torch.float32, DEV)
+    jv.full_attn(*(a.to(DEV) for a in (q, k, v)), out=out)
+    check()
+    s = (q.double() @ k.double().transpose(-1, -2)).clamp(-1e300, 1e300) if value == "lowest" else q.double() @ k.double().transpose(-1, -2)
+    ref = torch.softmax(s / 8.0, -1) @ v.double()
+    got = out.cpu().double()
+    assert torch.equal(got.isfinite(), ref.isfinite())
+    f = ref.isfinite()
+    assert bool(((got - ref).abs()[f] <= 1e-4 * ref.abs()[f].clamp(min=ref[0, 0].square().mean().sqrt())).all())
+
+
+@pytest.mark.parametrize("B,H,P,Hg,Wg,win", [(1, 1, 1, 5, 5, 4), (1, 2, 17, 16, 31, 8), (1, 6, 5, 37, 37, 8), (3, 50, 3, 12, 17, 7)])
+def test_fp32_prefix_queries(jv, oracle, B, H, P, Hg, Wg, win):
+    """The prefix queries' keys over 4 to 32 groups in clusters of 1 to 8 blocks, some of them without a key."""
+    q, k, v = inputs.custom_qkv(B, H, P + Hg * Wg, 64, "f32", seed=3800 + P)
+    out, check = guarded_empty(q.shape, torch.float32, DEV)
+    out.fill_(float("nan"))
+    jv.window_attn(*(t.to(DEV) for t in (q, k, v)), Hg, Wg, win, win, out=out, prefix=P)
+    check()
+    heads = sample_heads(B, H, 4, P)
+    qs, ks, vs = _tc_heads(q, k, v, heads)
+    o = _tc_heads(out.cpu(), k, v, heads)[0]
+    assert rel_err(o, oracle.window_attn(qs, ks, vs, Hg, Wg, win, win, prefix=P)) <= TOL["f32"]
+
+
 # Windows of up to eight tokens are the kernel of one warp per query row's, with prefix tokens where there are many of them (B = 4) and a window's keys
 # are at most 32; their prefix queries are not; windows of nine tokens are one launch of this kernel.
 @pytest.mark.parametrize("B,P", [(2, 0), (2, 1), (4, 1), (4, 24), (4, 31), (4, 70)])
