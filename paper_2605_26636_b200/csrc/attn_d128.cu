@@ -17,14 +17,23 @@
 // Persistent CTAs (one per SM) loop over work items; an item is two consecutive query tiles of one
 // window of one (batch, head) against all key tiles of that window.  Keys outside the grid or the
 // window arrive as zeros or as a neighbour's tokens and are overwritten with -inf in tensor memory
-// before the softmax; query rows outside are not written.  Warp roles (10 warps):
+// before the softmax; query rows outside are not written.  Warp roles (11 warps):
 //   warp 0        TMA producer: two Q tiles per item, K tiles through a ring of three, V tiles through a ring of two
-//   warp 1        MMA issuer, in steps of 64 keys, both tiles: O_t += P_t V of step u, then S_t = Q_t K^T of step u + 2
+//   warps 1, 2    MMA issuers, one per query tile, in steps of 64 keys: O_t += P_t V of step u, then S_t = Q_t K^T of step u + 2
 //                 into the score buffer that P V has just read
-//   warps 2-9     softmax, one thread per query row (warp w: tile (w - 2) / 4, tensor-memory quadrant w % 4):
+//   warps 3-10    softmax, one thread per query row (warp w: tile (w - 3) / 4, tensor-memory quadrant w % 4):
 //                 exact two-pass softmax per step against a lazily raised reference, P as bf16 back into
 //                 tensor memory, final 1/l scaling, rows written straight to global memory (256 contiguous
 //                 bytes per row and thread)
+//
+// What bounds it: the chain of a softmax warp through a step of 64 keys, about 1550 clocks for 270 instructions, with two such warps per
+// sub-core: barrier waits (130 clocks each where there is nothing to wait for), the latencies of tensor memory, and the exponentials, for
+// which the two warps tend to meet at MUFU in phase.  So the fewest waits (the scores' barrier stands for the product before them, too) and
+// three of eight exponentials on the FMA pipe, by a polynomial of degree 4 (2.6e-6: the error against fp64 is not larger than with
+// one of eight of degree 3).  The tensor pipe needs 1294 clocks of a step.  Measured (2 x 8 heads of 4096 tokens / 16 x 16 windows of the
+// same): 133 / 22.3 us with one issuer for both tiles, a wait for every P V and one of eight polynomials; with an issuer each 135 / 22.4;
+// without the waits 127 / 21.3; now 124 / 21.2.  Two of eight 125, four 129.  Two threads per row (four softmax warps per sub-core, maxima
+// exchanged through shared memory: 340 clocks a step) 132 at best.
 //
 // Every mbarrier wait is bounded: a wait that runs out sets the device status word, raises a
 // CTA-wide abort flag, and every role falls through to the common teardown (tensor memory is
@@ -44,15 +53,12 @@ constexpr int kHalfBytes = kTile * kHalfD * 2;   // 16 KB
 constexpr int kTileBytes = 2 * kHalfBytes;       // 32 KB
 constexpr int kQT = 2;                      // query tiles per work item
 constexpr int kKS = 3, kVS = 2;             // K and V ring depths
-constexpr int kWarps = 10;
+constexpr int kWarps = 11;
 constexpr int kThreads = kWarps * 32;
-constexpr int kFirstSoftmaxWarp = 2;
+constexpr int kFirstSoftmaxWarp = 3;
 constexpr uint32_t kTmemCols = 512;
 constexpr int kSub = 64;                    // keys per step
-#ifndef JV_D128_POLY
-#define JV_D128_POLY 1
-#endif
-constexpr int kPolyOf8 = JV_D128_POLY;      // of every 8 score pairs, this many take the polynomial exponential
+constexpr int kPolyOf8 = 3, kPolyDeg = 4;   // of every 8 score pairs, this many take the polynomial exponential, of this degree
 // Tensor-memory columns: score buffer h of tile t (and its P over the first 32 columns) at 128 t + 64 h,
 // O_t at 256 + 128 t
 constexpr uint32_t kColS = 0, kColO = 256;
@@ -101,7 +107,7 @@ struct __align__(8) Barriers {
   uint64_t q_full[kQT], q_empty[kQT];
   uint64_t k_full[kKS], k_empty[kKS], v_full[kVS], v_empty[kVS];
   uint64_t s_full[kQT][2], p_full[kQT][2];   // per query tile and score buffer
-  uint64_t pv_done[kQT];                     // one phase per step: its P V has retired
+  uint64_t pv_done[kQT];                     // two phases per item: its last but one, its last P V has retired
   uint64_t drain;
   uint32_t tmem_base;
   volatile uint32_t abort_flag;
@@ -145,13 +151,13 @@ attn_d128_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     }
     for (int s = 0; s < kKS; ++s) {
       mbar_init(&bar->k_full[s], 1);
-      mbar_init(&bar->k_empty[s], 1);
+      mbar_init(&bar->k_empty[s], 2);         // one commit from each issuer
     }
     for (int s = 0; s < kVS; ++s) {
       mbar_init(&bar->v_full[s], 1);
-      mbar_init(&bar->v_empty[s], 1);
+      mbar_init(&bar->v_empty[s], 2);
     }
-    mbar_init(&bar->drain, 1);
+    mbar_init(&bar->drain, 2);
     bar->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -228,34 +234,45 @@ attn_d128_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         while (!mbar_try(&bar->v_full[g % kVS], (g / kVS) & 1) && globaltimer() - t0 < kWaitLimitNs) {}
       while (globaltimer() - t0 < 1000000ull) {}
     }
-  } else if (warp == 1) {
-    // ================= MMA issuer, both query tiles =================
-    // Per item and query tile t the work is a chain over 64-key steps u (key tile u / 2, half u % 2):
-    //   S_t(u) = Q_t K(u)^T          8 MMAs, M128 N64 K16, operands in shared memory (two channel halves)
-    //   O_t   += P_t(u) V(u)         2 x 4 MMAs, M128 N64 K16, A = P in tensor memory, one per channel half of V
-    // Two score buffers per tile: the scores of steps u and u + 1 are in flight or done while the softmax
-    // works on step u, so it never waits for Q K^T in steady state.  P_t(u) lies over S_t(u) in buffer u % 2,
-    // and S_t(u + 2) is issued into that buffer behind P_t(u) V(u): the tensor pipe executes one thread's
-    // MMAs in issue order.  pv_done tells the softmax warps that a step's P V has retired (O_t quiescent).
+  } else if (warp < kFirstSoftmaxWarp) {
+    // ================= MMA issuer of query tile x =================
+    // Per item the work is a chain over 64-key steps u (key tile u / 2, half u % 2):
+    //   S(u) = Q K(u)^T          8 MMAs, M128 N64 K16, operands in shared memory (two channel halves)
+    //   O   += P(u) V(u)         2 x 4 MMAs, M128 N64 K16, A = P in tensor memory, one per channel half of V
+    // Two score buffers: the scores of steps u and u + 1 are in flight or done while the softmax
+    // works on step u, so it never waits for Q K^T in steady state.  P(u) lies over S(u) in buffer u % 2,
+    // and S(u + 2) is issued into that buffer behind P(u) V(u): the tensor pipe executes one thread's
+    // MMAs in issue order, so the commit that publishes S(u + 1) also says that P(u - 1) V(u - 1) has retired; behind the last
+    // scores pv_done says so.
+    // One warp per tile: a step is up to three waits and 16 MMAs, whose issue the pipe holds back to its own pace (48 clocks each with
+    // both operands in shared memory, 32 with P); both tiles' steps one after the other filled 1800 clocks.
+    const int x = warp - 1;
     bool ok = true;
     int sk = 0, sv = 0;                     // ring stages of the score key tile and of the P V key tile
     uint32_t phk = 0, phv = 0;              // and their "full" parities
-    uint32_t pcnt[2][2] = {{0, 0}, {0, 0}}; // publications seen so far per tile and buffer: parity of p_full
-    uint32_t qcnt[2] = {0, 0};              // items in which the tile existed: parity of q_full
+    uint32_t pcnt[2] = {0, 0};              // publications seen so far per buffer: parity of p_full
+    uint32_t qcnt = 0;                      // items in which the tile existed: parity of q_full
     for (int i = item0; i < p.total_items && ok; i += item_step) {
       const Item it = decode_item(p, i);
       if (it.qt0 >= it.ntiles) continue;
       const int nsteps = 2 * it.ntiles;
-      const bool ex[2] = {true, it.qt0 + 1 < it.ntiles};
-      // Scores of step u: scores_begin waits for the key tile, scores_tile issues tile x's MMAs into buffer
-      // u % 2 (the caller has made sure that the buffer is free: its previous P V has been issued, and one
-      // thread's MMAs execute in issue order), scores_end hands the key tile and the query tiles back.
-      auto scores_begin = [&](int u) -> bool {
-        if ((u & 1) == 0 && !warp_wait<kSuspendNs>(&bar->k_full[sk], phk, &bar->abort_flag, p.status)) return false;
-        tc_fence_after();
-        return true;
-      };
-      auto scores_tile = [&](int u, int x) {
+      if (it.qt0 + x >= it.ntiles) {        // no such tile: its share in handing the key tiles and the query tile back
+        for (int j = 0; j < it.ntiles && ok; ++j) {
+          ok = warp_wait<kSuspendNs>(&bar->k_full[sk], phk, &bar->abort_flag, p.status);
+          if (!ok) break;
+          tc_commit(&bar->k_empty[sk]);
+          if (++sk == kKS) { sk = 0; phk ^= 1; }
+          ok = warp_wait<kSuspendNs>(&bar->v_full[sv], phv, &bar->abort_flag, p.status);
+          if (!ok) break;
+          tc_commit(&bar->v_empty[sv]);
+          if (++sv == kVS) { sv = 0; phv ^= 1; }
+        }
+        tc_commit(&bar->q_empty[x]);        // (behind the item's copies: the producer has seen the phase before this one by then)
+        continue;
+      }
+      // Scores of step u into buffer u % 2 (the caller has made sure that the buffer is free: its previous P V has been issued, and
+      // one thread's MMAs execute in issue order; and that the key tile has landed)
+      auto scores = [&](int u) {
         const uint32_t kb = sK + sk * kTileBytes + (u & 1) * (kSub * kHalfD * 2);   // 64 keys = 8 KB into each half tile
         if (elect_one()) {
 #pragma unroll
@@ -269,68 +286,50 @@ attn_d128_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         }
         __syncwarp();
         tc_commit(&bar->s_full[x][u & 1]);
-      };
-      auto scores_end = [&](int u) {
         if ((u & 1) == 1) {
           tc_commit(&bar->k_empty[sk]);
           if (++sk == kKS) { sk = 0; phk ^= 1; }
         }
-        if (u == nsteps - 1) {              // the item's last scores: its query tiles may be replaced
-          tc_commit(&bar->q_empty[0]);
-          tc_commit(&bar->q_empty[1]);
-        }
+        if (u == nsteps - 1) tc_commit(&bar->q_empty[x]);    // the item's last scores: its query tile may be replaced
       };
-      for (int x = 0; x < 2 && ok; ++x) {
-        if (!ex[x]) continue;
-        ok = warp_wait<kSuspendNs>(&bar->q_full[x], qcnt[x] & 1, &bar->abort_flag, p.status);
-        ++qcnt[x];
-      }
+      auto key_landed = [&](int u) -> bool {
+        return (u & 1) == 1 || warp_wait<kSuspendNs>(&bar->k_full[sk], phk, &bar->abort_flag, p.status);
+      };
+      ok = warp_wait<kSuspendNs>(&bar->q_full[x], qcnt & 1, &bar->abort_flag, p.status);
+      ++qcnt;
       for (int u = 0; u < 2 && ok; ++u) {   // (a key tile is two steps: nsteps >= 2)
-        ok = scores_begin(u);
+        ok = key_landed(u);
         if (!ok) break;
-        for (int x = 0; x < 2; ++x)
-          if (ex[x]) scores_tile(u, x);
-        scores_end(u);
+        tc_fence_after();
+        scores(u);
       }
       for (int u = 0; u < nsteps && ok; ++u) {
         const int hb = u & 1;
         const bool more = u + 2 < nsteps;   // the buffer of step u is free behind its P V: the scores of step u + 2 go there
-        if (hb == 0) {                      // P V of a first half: its V must have landed
-          ok = warp_wait<kSuspendNs>(&bar->v_full[sv], phv, &bar->abort_flag, p.status);
-          if (!ok) break;
-        }
-        if (more) {
-          ok = scores_begin(u + 2);
-          if (!ok) break;
-        }
-        const uint32_t vb = sV + sv * kTileBytes + hb * (kSub * kHalfD * 2);
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-          if (!ex[x]) continue;
-          ok = warp_wait<kSuspendNs>(&bar->p_full[x][hb], pcnt[x][hb] & 1, &bar->abort_flag, p.status);
-          ++pcnt[x][hb];
-          if (!ok) break;
-          tc_fence_after();
-          if (elect_one()) {                 // one lane issues the step's MMAs back to back
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-              const uint64_t dv = smem_desc(vb + half * kHalfBytes);
-#pragma unroll
-              for (int c = 0; c < kSub / 16; ++c)
-                mma_ts_1(tmem + kColO + x * kD + half * kHalfD, tmem + kColS + x * 128 + hb * kSub + c * 8, desc_advance(dv, c * 2048),
-                         kIdescPV, (u > 0 || c > 0) ? 1u : 0u);
-            }
-          }
-          __syncwarp();
-          tc_commit(&bar->pv_done[x]);
-          if (more) scores_tile(u + 2, x);
-        }
+        if (hb == 0) ok = warp_wait<kSuspendNs>(&bar->v_full[sv], phv, &bar->abort_flag, p.status);   // P V of a first half: its V must have landed
+        if (ok && more) ok = key_landed(u + 2);
+        if (ok) ok = warp_wait<kSuspendNs>(&bar->p_full[x][hb], pcnt[hb] & 1, &bar->abort_flag, p.status);
         if (!ok) break;
+        ++pcnt[hb];
+        const uint32_t vb = sV + sv * kTileBytes + hb * (kSub * kHalfD * 2);
+        tc_fence_after();
+        if (elect_one()) {                 // one lane issues the step's MMAs back to back
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            const uint64_t dv = smem_desc(vb + half * kHalfBytes);
+#pragma unroll
+            for (int c = 0; c < kSub / 16; ++c)
+              mma_ts_1(tmem + kColO + x * kD + half * kHalfD, tmem + kColS + x * 128 + hb * kSub + c * 8, desc_advance(dv, c * 2048),
+                       kIdescPV, (u > 0 || c > 0) ? 1u : 0u);
+          }
+        }
+        __syncwarp();
+        if (u >= nsteps - 2) tc_commit(&bar->pv_done[x]);
         if (hb == 1) {                      // both halves of the V tile are in flight or done
           tc_commit(&bar->v_empty[sv]);
           if (++sv == kVS) { sv = 0; phv ^= 1; }
         }
-        if (more) scores_end(u + 2);
+        if (more) scores(u + 2);
       }
     }
     // Teardown: every MMA issued so far must have retired before tensor memory is released.
@@ -351,8 +350,7 @@ attn_d128_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     const float kLazy = 8.f / sl2;                 // the reference maximum moves only when it grew by > 2^8
     const uint64_t sl2x2 = pack2(sl2, sl2);
     bool ok = true;
-    uint32_t scnt[2] = {0, 0};        // steps seen by this tile per score buffer: parity of s_full
-    uint32_t g = 0;                   // steps seen by this tile in all: phase of pv_done
+    uint32_t sc = 0;                  // parity of s_full[t][h] in bit h
 
     for (int i = item0; i < p.total_items && ok; i += item_step) {
       const Item it = decode_item(p, i);
@@ -362,9 +360,9 @@ attn_d128_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
       float m = -INFINITY, l = 0.f;
       for (int u = 0; u < nsteps; ++u) {
         const uint32_t tS = tS0 + (u & 1) * kSub;
-        ok = warp_wait<kSuspendNs>(&bar->s_full[t][u & 1], scnt[u & 1] & 1, &bar->abort_flag, p.status);
+        ok = warp_wait<kSuspendNs>(&bar->s_full[t][u & 1], (sc >> (u & 1)) & 1, &bar->abort_flag, p.status);
         if (!ok) break;
-        ++scnt[u & 1];
+        sc ^= 1u << (u & 1);
         tc_fence_after();
         uint32_t va[32], vb2[32];
         // valid extent of this key tile's box along x and y: a key outside the grid or the window does not exist
@@ -406,7 +404,10 @@ attn_d128_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         max32(va, mx4);
         max32(vb2, mx4);
         const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-        bool pv_seen = u == 0;         // every step looks at the phase of the previous step's P V exactly once
+        if (u == nsteps - 1) {         // (a key tile is two steps: u > 0)
+          ok = warp_wait<kSuspendNs>(&bar->pv_done[t], 0, &bar->abort_flag, p.status);
+          if (!ok) break;
+        }
         float o_scale = 1.f;
         if (mx > m + kLazy) {          // always true on the first step (m = -inf, mx finite)
           o_scale = ex2((m - mx) * sl2);            // first step: exp2(-inf) = 0
@@ -414,11 +415,12 @@ attn_d128_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
           m = mx;
         }
         if (u > 0 && __any_sync(0xffffffffu, o_scale != 1.f)) {
-          // Rare: the reference moved.  O_t may be touched once the previous step's P V has retired
-          // (phase g - 1 of pv_done); the next P V waits for this step's P.
-          ok = warp_wait<kSuspendNs>(&bar->pv_done[t], (g - 1) & 1, &bar->abort_flag, p.status);
-          if (!ok) break;
-          pv_seen = true;
+          // Rare: the reference moved.  O_t may be touched once the previous step's P V has retired, which the next step's scores
+          // say (a look at their barrier; the next step waits for the same phase); the next P V waits for this step's P.
+          if (u < nsteps - 1) {
+            ok = warp_wait<kSuspendNs>(&bar->s_full[t][(u + 1) & 1], (sc >> ((u + 1) & 1)) & 1, &bar->abort_flag, p.status);
+            if (!ok) break;
+          }
           tc_fence_after();
 #pragma unroll 1
           for (int c = 0; c < kD / 32; ++c) {
@@ -436,29 +438,22 @@ attn_d128_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         const uint64_t mnegx2 = pack2(mneg, mneg);
         uint64_t lsum[4] = {0ull, 0ull, 0ull, 0ull};
         uint32_t pk[16];
-        exp32<false, kPolyOf8>(va, sl2x2, mnegx2, lsum, pk, mx4);
+        exp32<false, kPolyOf8, kPolyDeg>(va, sl2x2, mnegx2, lsum, pk, mx4);
         tmem_st16(tS, pk);
-        exp32<false, kPolyOf8>(vb2, sl2x2, mnegx2, lsum, pk, mx4);
+        exp32<false, kPolyOf8, kPolyDeg>(vb2, sl2x2, mnegx2, lsum, pk, mx4);
         tmem_st16(tS + 16, pk);
         float a0, a1, b0, b1;
         unpack2(add2(lsum[0], lsum[1]), a0, a1);
         unpack2(add2(lsum[2], lsum[3]), b0, b1);
         l += (a0 + a1) + (b0 + b1);
-        // A parity wait must not skip a phase: the previous step's P V is waited for here at the latest
-        // (it retired long ago), before this step's P can set the next one going.
-        if (!pv_seen) {
-          ok = warp_wait<kSuspendNs>(&bar->pv_done[t], (g - 1) & 1, &bar->abort_flag, p.status);
-          if (!ok) break;
-        }
         // publish P
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(&bar->p_full[t][u & 1]);
-        ++g;
       }
       if (!ok) break;
       // ---- epilogue: O / l -> bf16 -> this thread's row, 256 contiguous bytes of global memory
-      ok = warp_wait<kSuspendNs>(&bar->pv_done[t], (g - 1) & 1, &bar->abort_flag, p.status);   // the item's last P V
+      ok = warp_wait<kSuspendNs>(&bar->pv_done[t], 1, &bar->abort_flag, p.status);   // the item's last P V
       if (!ok) break;
       tc_fence_after();
       const float inv = 1.f / l;

@@ -274,10 +274,13 @@ __device__ __forceinline__ void max32(const uint32_t (&v)[32], float (&mx)[4]) {
 // exp2 on the FMA pipe, for part of the scores (the MUFU unit, 16 results per clock and SM,
 // is the tightest resource of softmax attention at head_dim 64).  x = n + f with n = round(x),
 // f in [-0.5, 0.5]; 2^f by a degree-3 minimax polynomial (relative error 7.5e-5, well below
-// the bf16 rounding of P); n goes straight into the exponent field.  Valid for x in [-126, 126].
+// the bf16 rounding of P) or of degree 4 (2.6e-6); n goes straight into the exponent field.  Valid for x in [-126, 126].
 constexpr float kPolyC0 = 0.9999280571937561f, kPolyC1 = 0.6932609677314758f;
 constexpr float kPolyC2 = 0.2426111251115799f, kPolyC3 = 0.0551716685295105f;
+constexpr float kPoly4C0 = 0.9999992614457123f, kPoly4C1 = 0.6931218147366893f, kPoly4C2 = 0.24024744827863667f;
+constexpr float kPoly4C3 = 0.055917860319387246f, kPoly4C4 = 0.009570101911169622f;
 constexpr float kRoundMagic = 12582912.f;   // 1.5 * 2^23: adding it leaves round(x) in the low mantissa bits
+template <int kDeg>
 __device__ __forceinline__ void exp2_poly2(uint64_t x, float& p0, float& p1) {
   float x0, x1;
   unpack2(x, x0, x1);
@@ -285,9 +288,17 @@ __device__ __forceinline__ void exp2_poly2(uint64_t x, float& p0, float& p1) {
   const uint64_t t = add2(x, pack2(kRoundMagic, kRoundMagic));
   const uint64_t n = add2(t, pack2(-kRoundMagic, -kRoundMagic));
   const uint64_t f = fma2(n, pack2(-1.f, -1.f), x);
-  uint64_t q = fma2(f, pack2(kPolyC3, kPolyC3), pack2(kPolyC2, kPolyC2));
-  q = fma2(q, f, pack2(kPolyC1, kPolyC1));
-  q = fma2(q, f, pack2(kPolyC0, kPolyC0));
+  uint64_t q;
+  if (kDeg == 3) {
+    q = fma2(f, pack2(kPolyC3, kPolyC3), pack2(kPolyC2, kPolyC2));
+    q = fma2(q, f, pack2(kPolyC1, kPolyC1));
+    q = fma2(q, f, pack2(kPolyC0, kPolyC0));
+  } else {
+    q = fma2(f, pack2(kPoly4C4, kPoly4C4), pack2(kPoly4C3, kPoly4C3));
+    q = fma2(q, f, pack2(kPoly4C2, kPoly4C2));
+    q = fma2(q, f, pack2(kPoly4C1, kPoly4C1));
+    q = fma2(q, f, pack2(kPoly4C0, kPoly4C0));
+  }
   float q0, q1, t0, t1;
   unpack2(q, q0, q1);
   unpack2(t, t0, t1);
@@ -297,8 +308,8 @@ __device__ __forceinline__ void exp2_poly2(uint64_t x, float& p0, float& p1) {
 
 // p = exp2(s * sl2 + mneg) for 32 scores; adds them into four packed partial sums and packs
 // them to bf16 pairs (even key in the low half).  kTrack also folds the scores into mx; of every 8
-// score pairs, kPolyOf8 take the polynomial path.
-template <bool kTrack, int kPolyOf8>
+// score pairs, kPolyOf8 take the polynomial path, of degree kDeg.
+template <bool kTrack, int kPolyOf8, int kDeg = 3>
 __device__ __forceinline__ void exp32(const uint32_t (&v)[32], uint64_t sl2x2, uint64_t mnegx2, uint64_t (&lsum)[4],
                                       uint32_t (&pk)[16], float (&mx)[4]) {
 #pragma unroll
@@ -308,7 +319,7 @@ __device__ __forceinline__ void exp32(const uint32_t (&v)[32], uint64_t sl2x2, u
     const uint64_t x = fma2(pack2(s0, s1), sl2x2, mnegx2);
     float p0, p1;
     if ((i & 7) < kPolyOf8) {
-      exp2_poly2(x, p0, p1);
+      exp2_poly2<kDeg>(x, p0, p1);
     } else {
       float x0, x1;
       unpack2(x, x0, x1);
