@@ -29,25 +29,27 @@ namespace {
 using namespace f32;
 
 constexpr int kDim = 64;
-constexpr int kKeys = 64;        // keys per tile
+constexpr int kTileKeys = 64;    // keys per tile, but for short rows of keys
 constexpr int kRowsWarp = 16;    // query rows per warp
 constexpr int kLd = 68;          // floats per shared-memory row: 16-byte reads of 8 consecutive rows touch all banks
 constexpr int kLdP = 20;         // floats per key of the transposed probabilities (16 rows): 16-byte writes of 8 keys likewise
-constexpr int kWarpBuf = kKeys * kLdP;  // floats of a warp's own buffer
-static_assert(kWarpBuf >= kRowsWarp * kLd, "the buffer takes the warp's output as well");
+// floats of a warp's own buffer: the probabilities of a tile of `keys` keys, then the warp's output
+__host__ __device__ constexpr int warp_buf(int keys) { return keys * kLdP > kRowsWarp * kLd ? keys * kLdP : kRowsWarp * kLd; }
 
-template <int R, int G>
+template <int R, int G, int kKeys>
 constexpr size_t smem_bytes() {
-  return ((size_t)(R * kRowsWarp + G * kKeys) * kLd + R * G * kWarpBuf) * sizeof(float);
+  return ((size_t)(R * kRowsWarp + G * kKeys) * kLd + R * G * warp_buf(kKeys)) * sizeof(float);
 }
 
 // kPrefix: the launch serves the P prefix queries (keys: all tokens) instead of the windows, by clusters of blocks along x that
 // share the keys of a row tile and merge their partial softmaxes through distributed shared memory.
-template <int R, int G, bool kPrefix>
-__global__ void __launch_bounds__(32 * R * G, G == 4 ? 2 : 3)  // what shared memory leaves room for
+// kKeys: keys per tile, 64, or 32 where that leaves no group without one
+template <int R, int G, int kKeys, bool kPrefix>
+__global__ void __launch_bounds__(32 * R * G, G == 2 ? 3 : G == 4 ? 2 : 1)  // what shared memory leaves room for
 attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ o,
                 int Hg, int Wg, int P, int wh, int ww, int nwx, bool overlap, float scale) {
   namespace cg = cooperative_groups;
+  constexpr int kWarpBuf = warp_buf(kKeys), kJ = kKeys / 16;   // a lane's keys of a tile: tx + 16 j
   extern __shared__ __align__(16) float smem_f[];
   float* qs = smem_f;                                        // [16 R][kLd]
   float* ps = qs + R * kRowsWarp * kLd;                      // [R G warps]: probabilities [64 keys][kLdP], then the warp's output [16][kLd]
@@ -135,21 +137,21 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
   for (int t = first; t < ntiles; t += stride) {
     copy_wait<0>();                                          // K of this tile
     group_sync();
-    f32x2 s2[8][4];
+    f32x2 s2[8][kJ];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) s2[i][j] = 0ull;
+      for (int j = 0; j < kJ; ++j) s2[i][j] = 0ull;
 #pragma unroll 4
     for (int c = 0; c < kDim; c += 4) {
-      ulonglong2 kk[4];
+      ulonglong2 kk[kJ];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) kk[j] = *reinterpret_cast<const ulonglong2*>(kg + (tx + 16 * j) * kLd + c);
+      for (int j = 0; j < kJ; ++j) kk[j] = *reinterpret_cast<const ulonglong2*>(kg + (tx + 16 * j) * kLd + c);
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const ulonglong2 qq = *reinterpret_cast<const ulonglong2*>(qr + i * kLd + c);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < kJ; ++j) {
           fma2(s2[i][j], qq.x, kk[j].x);
           fma2(s2[i][j], qq.y, kk[j].y);
         }
@@ -161,18 +163,19 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
     const bool ragged = (t + 1) * kKeys > cnt;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {                            // four rows at a time
-      float p[4][4], alpha[4];                               // [key][row]
+      float p[kJ][4], alpha[4];                              // [key][row]
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         const int i = 4 * h + r;
-        float s[4];
+        float s[kJ];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < kJ; ++j) {
           const float2 e = unpack2(s2[i][j]);
           s[j] = (e.x + e.y) * scale;
           if (ragged && t * kKeys + tx + 16 * j >= cnt) s[j] = -INFINITY;
         }
-        float mx = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
+        float mx = fmaxf(s[0], s[1]);
+        if (kJ == 4) mx = fmaxf(mx, fmaxf(s[2 % kJ], s[3 % kJ]));
 #pragma unroll
         for (int w = 1; w < 16; w <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
         const float mn = fmaxf(m[i], mx);
@@ -181,14 +184,14 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
         m[i] = mn;
         float sum = 0.f;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < kJ; ++j) {
           p[j][r] = expf(s[j] - ref);
           sum += p[j][r];
         }
         l[i] = fmaf(l[i], alpha[r], sum);
       }
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
+      for (int j = 0; j < kJ; ++j)
         *reinterpret_cast<float4*>(pw + (tx + 16 * j) * kLdP + ty * 8 + 4 * h) = make_float4(p[j][0], p[j][1], p[j][2], p[j][3]);
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
@@ -295,17 +298,18 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
   if (overlap) griddep_wait();
 }
 
-template <int R, int G, bool kPrefix>
+template <int R, int G, int kKeys, bool kPrefix>
 cudaError_t launch(const AttnArgs& a, int split, bool overlap, cudaStream_t st) {   // split: blocks to a cluster (the prefix queries)
   static OncePerDevice opt_in;
   const cudaError_t e = opt_in.run([&] {
-    return cudaFuncSetAttribute(attn_f32_kernel<R, G, kPrefix>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<R, G>());
+    return cudaFuncSetAttribute(attn_f32_kernel<R, G, kKeys, kPrefix>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)smem_bytes<R, G, kKeys>());
   });
   if (e != cudaSuccess) return e;
   const int wh = a.wh < a.Hg ? a.wh : a.Hg, ww = a.ww < a.Wg ? a.ww : a.Wg;
   const int nwx = ceil_div(a.Wg, ww), nwin = nwx * ceil_div(a.Hg, wh);
   const dim3 grid = kPrefix ? dim3(ceil_div(a.P, R * kRowsWarp) * split, 1, a.BH) : dim3(ceil_div(wh * ww, R * kRowsWarp), nwin, a.BH);
-  return launch_cluster(true, attn_f32_kernel<R, G, kPrefix>, kPrefix ? split : 0, grid, 32 * R * G, smem_bytes<R, G>(), st, (const float*)a.q,
+  return launch_cluster(true, attn_f32_kernel<R, G, kKeys, kPrefix>, kPrefix ? split : 0, grid, 32 * R * G, smem_bytes<R, G, kKeys>(), st, (const float*)a.q,
                         (const float*)a.k, (const float*)a.v, (float*)a.o, a.Hg, a.Wg, a.P, wh, ww, nwx, overlap, a.scale);
 }
 
@@ -326,7 +330,10 @@ bool attn_f32_supported(const AttnArgs& a) { return a.dtype == JV_F32 && a.D == 
 // three quarters empty): 4 x 4 windows, 48 heads of 32 x 32 72 / 87.
 //
 // Here, 32 rows x 2 groups per CTA (three on an SM) or 16 rows x 4 groups (two): the second halves the chain of a CTA, the first is 10 % faster
-// where both fill the chip.  Windows of one or two key tiles have no work for four groups (432 CTAs, 8 x 8 windows: 18 / 33 us).
+// where both fill the chip.  Short rows of keys (up to 64, 128 and 256) are cut into tiles of 32, so that two, four or eight groups have one each and a
+// CTA's chain is half as long.  Tiles of 64 / of 32, us: 6 heads of 64 tokens 7.5 / 5.4, of 128 8.1 / 5.3, 24 of 128 8.3 / 7.4, 6 of 192 8.1 / 7.1, of 256 8.5 /
+// 8.4; 8 x 8 windows, 6 heads of 16 x 16 8.2 / 5.8, 4 x 4, 24 of 32 x 32 40 / 27.  Eight groups take an SM: only where every row tile gets one (12 heads
+// of 256 tokens 11.7 / 14.8).
 // Windows of at most eight tokens leave most of a 32 x 64 tile of scores empty: the kernel of one warp per query row, eight to a block, is the
 // better one.  This one / that one, 96 heads of 32 x 32 tokens: 2 x 2 windows 484 / 270 us, 2 x 4 256 / 148, 3 x 3 245 / 254; 12 heads of 64 x 64, 2 x 2
 // 235 / 135.  With prefix tokens, whose queries stay here: as long as a window's keys and they are one tile of that kernel, and the windows fill
@@ -339,24 +346,27 @@ cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st) {
     const int N = a.P + a.Hg * a.Wg;
     const int64_t tiles = (int64_t)ceil_div(a.P, kRowsWarp) * a.BH;
     int split = 1;
-    while (split < 8 && 2 * split * tiles <= 2 * device_sm_count() && split * 4 * kKeys < N) split *= 2;
-    const cudaError_t e = launch<1, 4, true>(a, split, false, st);
+    while (split < 8 && 2 * split * tiles <= 2 * device_sm_count() && split * 4 * kTileKeys < N) split *= 2;
+    const cudaError_t e = launch<1, 4, kTileKeys, true>(a, split, false, st);
     if (e != cudaSuccess) return e;
   }
   const int64_t sms = device_sm_count(), windows = (int64_t)ceil_div(a.Wg, ww) * ceil_div(a.Hg, wh) * a.BH;
   if (wh * ww <= 8 && (!prefix || (a.P + wh * ww <= 32 && windows >= 8 * sms))) return launch_attn_generic(a, st, true);
-  const int nq = wh * ww, cnt = a.P + nq, key_tiles = ceil_div(cnt, kKeys);
+  const int nq = wh * ww, cnt = a.P + nq, key_tiles = ceil_div(cnt, kTileKeys);
   const int64_t rows16 = windows * ceil_div(nq, kRowsWarp), rows32 = windows * ceil_div(nq, 2 * kRowsWarp);   // row tiles of this kernel
   bool tc = nq > 2 * kRowsWarp;
-  if (cnt <= 2 * kKeys) tc = tc && rows32 > sms && (cnt > kKeys || windows > a.BH || a.BH <= sms);
+  if (cnt <= 2 * kTileKeys) tc = tc && rows32 > sms && (cnt > kTileKeys || windows > a.BH || a.BH <= sms);
   else tc = tc && rows16 > sms && (key_tiles > 4 || 3 * rows16 > 4 * sms);
   if (tc) {
     int* status = device_status_ptr();
     if (!status) return cudaErrorUnknown;
     return launch_attn_f32_tc(a, prefix, status, st);
   }
-  if (cnt > 2 * kKeys && rows32 <= 2 * sms) return launch<1, 4, false>(a, 1, prefix, st);
-  return launch<2, 2, false>(a, 1, prefix, st);
+  if (cnt <= kTileKeys) return launch<2, 2, 32, false>(a, 1, prefix, st);
+  if (cnt <= 2 * kTileKeys) return launch<1, 4, 32, false>(a, 1, prefix, st);
+  if (cnt <= 4 * kTileKeys && rows16 <= sms) return launch<1, 8, 32, false>(a, 1, prefix, st);
+  if (rows32 <= 2 * sms) return launch<1, 4, kTileKeys, false>(a, 1, prefix, st);
+  return launch<2, 2, kTileKeys, false>(a, 1, prefix, st);
 }
 
 }  // namespace jv

@@ -160,6 +160,17 @@ def test_fp32_short_sequences(jv, oracle, N):
     assert rel_err(out, oracle.full_attn(q, k, v)) <= TOL["f32"]
 
 
+@pytest.mark.parametrize("N", [31, 33, 64, 65, 97, 128, 129, 225, 256, 257])
+def test_fp32_short_rows_of_keys(jv, oracle, N):
+    """Tiles of 32 keys over two, four and eight groups: the last group full, ragged and without a key; one key more than they take."""
+    q, k, v = inputs.custom_qkv(1, 3, N, 64, "f32", seed=3900 + N)
+    out, check = guarded_empty(q.shape, torch.float32, DEV)
+    out.fill_(float("nan"))
+    jv.full_attn(*(t.to(DEV) for t in (q, k, v)), out=out)
+    check()
+    assert rel_err(out, oracle.full_attn(q, k, v)) <= TOL["f32"]
+
+
 @pytest.mark.parametrize("static", [False, True], ids=["squeeze", "static"])
 @pytest.mark.parametrize("case", [(1, 1, 0, 1, 1), (1, 2, 0, 70, 1), (2, 3, 5, 11, 13), (1, 12, 1, 32, 32), (2, 2, 3, 3, 130), (2, 12, 0, 32, 32)],
                          ids=lambda c: "x".join(map(str, c)))
