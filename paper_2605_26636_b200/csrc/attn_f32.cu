@@ -324,7 +324,7 @@ bool attn_f32_supported(const AttnArgs& a) { return a.dtype == JV_F32 && a.D == 
 //
 // Windows and sequences go to the tensor cores (attn_f32_tc.cu) where they fill the chip with row tiles of this kernel.  That one's blocks
 // take 128 rows and start slowly: 7 us for one tile of keys, 10 for two, 12 for four, where this one takes 7 to 8 as long as every SM has one block.
-// This / that one, us: 6 heads of 256 tokens 8.2 / 12.1, 12 of 256 11.4 / 12.2, 6 of 400 19.0 / 15.6, 24 of 256 17.6 / 12.5, 12 of 1024 93 / 26.3; 48 of 100
+// This (with tiles of 64 keys throughout; those of 32 below came later) / that one, us: 6 heads of 256 tokens 8.2 / 12.1, 12 of 256 11.4 / 12.2, 6 of 400 19.0 / 15.6, 24 of 256 17.6 / 12.5, 12 of 1024 93 / 26.3; 48 of 100
 // 11.1 / 9.5, 24 of 128 8.1 / 10.2; of 64 tokens: 48 heads 7.5 / 7.5, 96 10.6 / 8.0, 192 (two rounds there) 11.4 / 14.6; 8 x 8 windows,
 // 6 heads of 24 x 24 8.1 / 10.6, 6 of 32 x 32 11.1 / 10.4, 48 of 32 x 32 41.7 / 33.1.  Rows of at most 32 queries stay here (a tile there would be
 // three quarters empty): 4 x 4 windows, 48 heads of 32 x 32 72 / 87.
