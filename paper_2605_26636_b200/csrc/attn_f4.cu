@@ -364,10 +364,10 @@ attn_f4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         tmem_ld32(tS, va);
         tmem_wait_ld(va);
         max32(va, mx4);
-        const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+        const float mx = max_of(mx4);
         float o_scale = 1.f;
-        if (mx > m + kLazy) {          // always true on the first step (m = -inf, mx finite)
-          o_scale = ex2((m - mx) * sl2);            // first step: exp2(-inf) = 0
+        if (ref_moves(mx, m, kLazy)) { // always true on the first step (m = -inf, mx finite)
+          o_scale = ref_scale(m, mx, sl2);            // first step: 0
           l *= o_scale;
           m = mx;
         }

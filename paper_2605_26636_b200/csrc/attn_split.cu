@@ -289,10 +289,10 @@ attn_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
       tmem_ld32(tS, va);
       tmem_wait_ld(va);
       max32(va, mx4);
-      const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+      const float mx = max_of(mx4);
       float o_scale = 1.f;
-      if (mx > m + kLazy) {          // always true on the first step, unless all of its scores are -inf
-        o_scale = ex2((m - mx) * sl2);
+      if (ref_moves(mx, m, kLazy)) { // always true on the first step, unless all of its scores are -inf
+        o_scale = ref_scale(m, mx, sl2);
         l *= o_scale;
         m = mx;
       }

@@ -383,9 +383,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       max32(va, mx4);
       tmem_wait_ld(vb);
       max32(vb, mx4);
-      const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-      if (mx > m + kLazy) {          // always true on the first step (m = -inf, mx finite)
-        const float alpha = ex2((m - mx) * sl2);   // first step: exp2(-inf) = 0
+      const float mx = max_of(mx4);
+      if (ref_moves(mx, m, kLazy)) { // always true on the first step (m = -inf, mx finite)
+        const float alpha = ref_scale(m, mx, sl2);   // first step: 0
         l *= alpha;
         o_scale *= alpha;
         m = mx;
@@ -408,7 +408,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     // the step's own maximum is tracked on the side.  Any reference value gives the same
     // softmax as long as nothing overflows, so a larger maximum only matters for the steps
     // that follow: it becomes the reference of the next step, which rescales l and O.
-    // A step whose scores exceed the reference by more than 2^kSpecLimit is redone with the
+    // A step whose scores exceed the reference by more than 2^kSpecLimit, or are no numbers, is redone with the
     // two-pass routine (P has not been published yet).
     constexpr float kSpecLimit = 64.f;
     float pend_alpha = 1.f, pend_m = 0.f;
@@ -430,13 +430,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       tmem_wait_ld(vb);
       exp32<true, kPolyOf8>(vb, sl2x2, mnegx2, lsum, pk, mx4);
       tmem_st16(tPb + 16, pk);
-      const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+      const float mx = max_of(mx4);
       float a0, a1, b0, b1;
       unpack2(add2(lsum[0], lsum[1]), a0, a1);
       unpack2(add2(lsum[2], lsum[3]), b0, b1);
       const float grow = (mx - m) * sl2;              // log2 of the largest p of this step
       // one vote for both rare cases: bit 1 = redo this step, bit 0 = some O needs rescaling
-      const unsigned flags = __reduce_or_sync(0xffffffffu, (grow > kSpecLimit ? 2u : 0u) | (o_scale != 1.f ? 1u : 0u));
+      const unsigned flags = __reduce_or_sync(0xffffffffu, (!(grow <= kSpecLimit) ? 2u : 0u) | (o_scale != 1.f ? 1u : 0u));
       if (flags & 2u) return false;                    // redo (whole warp); l untouched
       l += (a0 + a1) + (b0 + b1);
       if (grow > 8.f) {                                // new reference from the next step on

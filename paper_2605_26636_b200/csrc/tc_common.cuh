@@ -237,9 +237,10 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
   return r;
 }
+// the largest; no number if one of them is none
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
 // Two fp32 values in one 64-bit register: the packed fp32x2 arithmetic of sm_100.
@@ -271,10 +272,19 @@ __device__ __forceinline__ void max32(const uint32_t (&v)[32], float (&mx)[4]) {
     for (int u = 0; u < 4; ++u)
       mx[u] = max3(mx[u], __uint_as_float(v[8 * i + 2 * u]), __uint_as_float(v[8 * i + 2 * u + 1]));
 }
+__device__ __forceinline__ float max_of(const float (&mx)[4]) { return max3(max3(mx[0], mx[1], mx[2]), mx[3], mx[3]); }
+
+// The running reference of a row's exponentials.  A score of +inf or no number makes the row no number.  The exponentials do not
+// see to that (the polynomial ones below give 2^-126 for it), so the reference does: such a maximum always moves it, and what has been
+// summed up is then multiplied by no number.
+__device__ __forceinline__ bool ref_moves(float mx, float m, float lazy) { return !(mx <= m + lazy); }
+// factor for what has been summed up against reference m when mx (> m, or no number) takes its place; 0 for m = -inf
+__device__ __forceinline__ float ref_scale(float m, float mx, float sl2) { return ex2((m - mx) * sl2) + (mx - mx); }
+
 // exp2 on the FMA pipe, for part of the scores (the MUFU unit, 16 results per clock and SM,
 // is the tightest resource of softmax attention at head_dim 64).  x = n + f with n = round(x),
 // f in [-0.5, 0.5]; 2^f by a degree-3 minimax polynomial (relative error 7.5e-5, well below
-// the bf16 rounding of P) or of degree 4 (2.6e-6); n goes straight into the exponent field.  Valid for x in [-126, 126].
+// the bf16 rounding of P) or of degree 4 (2.6e-6); n goes straight into the exponent field.  Valid for x in [-126, 126]; below and for no number: 2^-126.
 constexpr float kPolyC0 = 0.9999280571937561f, kPolyC1 = 0.6932609677314758f;
 constexpr float kPolyC2 = 0.2426111251115799f, kPolyC3 = 0.0551716685295105f;
 constexpr float kPoly4C0 = 0.9999992614457123f, kPoly4C1 = 0.6931218147366893f, kPoly4C2 = 0.24024744827863667f;

@@ -1,6 +1,7 @@
 """Keys that are switched off by a score of -inf (a channel of k that is -inf where q's is positive): whole tiles of them for a part of
 the kernel that sees only those at first, a group of warps, a key slot, a warp or half a window.  They weigh nothing; the
-result is the softmax over the other keys."""
+result is the softmax over the other keys.  And keys whose score is +inf or no number: a softmax with one of those is no number,
+wherever the key lies."""
 import pytest
 import torch
 
@@ -17,7 +18,7 @@ def jv():
 
 
 def attend(q, k, v):
-    return torch.softmax(q @ k.transpose(-1, -2) / 8, -1) @ v
+    return torch.softmax(q @ k.transpose(-1, -2) * q.shape[-1] ** -0.5, -1) @ v
 
 
 def reference(q, k, v, Hg, Wg, win, P):
@@ -77,3 +78,69 @@ def test_a_row_without_any_key_is_nan(jv):
     assert bool(torch.isnan(jv.window_attn(q, k, v, 16, 16, 8, 8)).all())
     q, k, v = (t.repeat(1, 1, 3, 1) for t in (q, k, v))
     assert bool(torch.isnan(jv.full_attn(q, k, v)).all())
+
+
+# One call for each kernel (and dtype, head_dim, prefix) that takes exponentials of scores, windows of 0 being full attention
+ROUTES = [  # dtype, D, B, H, P, Hg, Wg, win
+    ("bf16", 64, 1, 48, 0, 1, 1024, 0),                # four query tiles per CTA
+    ("bf16", 64, 1, 24, 0, 1, 1024, 0),                # two
+    ("bf16", 64, 1, 24, 0, 1, 600, 0),                 # keys over four slots
+    ("bf16", 64, 1, 24, 0, 1, 200, 0),                 # short sequences on the window kernel
+    ("bf16", 64, 1, 4, 0, 40, 36, 16),
+    ("bf16", 64, 1, 4, 5, 40, 36, 16),
+    ("bf16", 64, 1, 4, 0, 40, 36, 8),
+    ("bf16", 64, 1, 4, 5, 40, 36, 8),
+    ("bf16", 64, 2, 8, 0, 65, 33, 32),                 # windows of eight tiles
+    ("bf16", 128, 2, 8, 0, 1, 1200, 0),
+    ("bf16", 128, 2, 8, 0, 40, 30, 16),
+    ("f32", 64, 1, 24, 0, 1, 1000, 0),                 # tensor cores
+    ("f32", 64, 2, 12, 1, 25, 27, 8),                  # two windows to a block
+    ("f32", 64, 1, 12, 70, 20, 20, 16),
+    ("f32", 64, 1, 3, 0, 1, 300, 0),                   # multiply-adds
+    ("f32", 64, 1, 3, 5, 20, 20, 16),
+]
+BAR = {"f32": 3e-6, "bf16": 1e-2}      # (as above)
+
+
+def _call(jv, case, seed):
+    dtype, D, B, H, P, Hg, Wg, win = case
+    N = P + Hg * Wg
+    gen = torch.Generator(device=DEV).manual_seed(seed + N)
+    q, k, v = (torch.randn((B, H, N, D), generator=gen, device=DEV) for _ in range(3))
+    q[..., 0] = 1.0
+
+    def run():
+        a = [x.bfloat16() if dtype == "bf16" else x for x in (q, k, v)]
+        o = jv.full_attn(*a) if win == 0 else jv.window_attn(*a, Hg, Wg, win, win, prefix=P)
+        return o.double(), reference(*a, Hg, Wg, win if win else max(Hg, Wg), P)
+    return q, k, v, run
+
+
+def _compare(o, ref, dtype, what):
+    assert torch.equal(torch.isnan(o), torch.isnan(ref)), what
+    f = torch.isfinite(ref)
+    assert bool(torch.isfinite(o[f]).all()), what
+    assert float((o - ref)[f].norm() / ref[f].norm()) <= BAR[dtype], what
+
+
+@pytest.mark.parametrize("case", ROUTES, ids=lambda c: "x".join(map(str, c)))
+@pytest.mark.parametrize("value", [float("nan"), float("inf")], ids=str)
+def test_a_score_that_is_no_number_or_plus_infinity(jv, case, value):
+    """At every position of a tile of 32 scores: in full attention one key per head, a head on, in windows one per window."""
+    dtype, D, B, H, P, Hg, Wg, win = case
+    N = P + Hg * Wg
+    for off in (0, 15, 30, N - 20) if win == 0 else (0, 23):
+        q, k, v, run = _call(jv, case, 7500)
+        kf = k.view(B * H, N, D)
+        for h in range(B * H - 1):
+            if win == 0:
+                kf[h, (off + h) % N, 0] = value
+                continue
+            for w, (y0, x0) in enumerate((y, x) for y in range(0, Hg, win) for x in range(0, Wg, win)):
+                i = (off + 7 * h + w) % (win * win)
+                y, x = y0 + i // win, x0 + i % win
+                if w % 5 != 4 and y < Hg and x < Wg:
+                    kf[h, P + y * Wg + x, 0] = value
+        o, ref = run()
+        assert bool(torch.isnan(ref).any()) and bool(torch.isfinite(ref).any())
+        _compare(o, ref, dtype, off)
