@@ -409,7 +409,7 @@ attn_d128_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
           if (!ok) break;
         }
         float o_scale = 1.f;
-        if (ref_moves(mx, m, kLazy)) { // always true on the first step (m = -inf, mx finite)
+        if (ref_moves(mx, m, kLazy)) { // always true on the first step, unless all of its scores are -inf
           o_scale = ref_scale(m, mx, sl2);            // first step: 0
           l *= o_scale;
           m = mx;
@@ -434,7 +434,7 @@ attn_d128_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
           tmem_wait_st();
         }
         // ---- pass 2: exponentials against the reference, P over the scores just consumed
-        const float mneg = -m * sl2;
+        const float mneg = ref_negative(m, sl2);
         const uint64_t mnegx2 = pack2(mneg, mneg);
         uint64_t lsum[4] = {0ull, 0ull, 0ull, 0ull};
         uint32_t pk[16];
@@ -456,7 +456,7 @@ attn_d128_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
       ok = warp_wait<kSuspendNs>(&bar->pv_done[t], 1, &bar->abort_flag, p.status);   // the item's last P V
       if (!ok) break;
       tc_fence_after();
-      const float inv = 1.f / l;
+      const float inv = ref_inverse(m, l);
       // this thread's token: row r of the tile's box
       const int r = 32 * q4 + lane;
       const int qx = it.x0 + (it.qt0 + t) * p.step_x + (r & (p.box_w - 1)), qy = it.y0 + (it.qt0 + t) * p.step_y + (r >> p.lg_box_w);

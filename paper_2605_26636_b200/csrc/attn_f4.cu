@@ -366,7 +366,7 @@ attn_f4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         max32(va, mx4);
         const float mx = max_of(mx4);
         float o_scale = 1.f;
-        if (ref_moves(mx, m, kLazy)) { // always true on the first step (m = -inf, mx finite)
+        if (ref_moves(mx, m, kLazy)) { // always true on the first step, unless all of its scores are -inf
           o_scale = ref_scale(m, mx, sl2);            // first step: 0
           l *= o_scale;
           m = mx;
@@ -389,7 +389,7 @@ attn_f4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
           tmem_wait_ld(va);
         }
         // ---- pass 2: exponentials against the reference, P over the scores just consumed
-        const float mneg = -m * sl2;
+        const float mneg = ref_negative(m, sl2);
         const uint64_t mnegx2 = pack2(mneg, mneg);
         uint64_t lsum[4] = {0ull, 0ull, 0ull, 0ull};
         uint32_t pk[16];
@@ -414,7 +414,7 @@ attn_f4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       if (!ok) break;
       ++ocnt;
       tc_fence_after();
-      const float inv = 1.f / l;
+      const float inv = ref_inverse(m, l);
       const int tok = (it.qt0 + t) * kTile + 32 * q4;          // first token of this warp's 32 rows
       const bool store = tok < p.N;                            // rows past N inside the box are clipped by the store
       if (store) {

@@ -312,7 +312,7 @@ attn_split_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constan
         tmem_wait_ld(va);
       }
       // pass 2: exponentials against the reference, P over the scores just consumed
-      const float mneg = m == -INFINITY ? 0.f : -m * sl2;    // (all scores of the slot so far -inf: probabilities of 2^-126 at most, not NaN)
+      const float mneg = ref_negative(m, sl2);
       const uint64_t mnegx2 = pack2(mneg, mneg);
       uint64_t lsum[4] = {0ull, 0ull, 0ull, 0ull};
       uint32_t pk[16];

@@ -384,13 +384,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       tmem_wait_ld(vb);
       max32(vb, mx4);
       const float mx = max_of(mx4);
-      if (ref_moves(mx, m, kLazy)) { // always true on the first step (m = -inf, mx finite)
+      if (ref_moves(mx, m, kLazy)) { // always true on the first step, unless all of its scores are -inf
         const float alpha = ref_scale(m, mx, sl2);   // first step: 0
         l *= alpha;
         o_scale *= alpha;
         m = mx;
       }
-      const float mneg = -m * sl2;
+      const float mneg = ref_negative(m, sl2);
       const uint64_t mnegx2 = pack2(mneg, mneg);
       uint64_t lsum[4] = {0ull, 0ull, 0ull, 0ull};
       uint32_t pk[16];
@@ -662,7 +662,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       done.x_end = x_end;
       done.y_end = y_end;
       done.par = n & 1;
-      done.inv = 1.f / l;
+      done.inv = ref_inverse(m, l);
       cur = nxt;
       ++n;
     }

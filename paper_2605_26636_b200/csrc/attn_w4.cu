@@ -527,7 +527,7 @@ attn_w4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         max32(va, mx4);
         const float mx = max_of(mx4);
         float o_scale = 1.f;
-        if (ref_moves(mx, m, kLazy)) { // always true on the first step (m = -inf, mx finite)
+        if (ref_moves(mx, m, kLazy)) { // always true on the first step, unless all of its scores are -inf
           o_scale = ref_scale(m, mx, sl2);            // first step: 0
           l *= o_scale;
           m = mx;
@@ -556,8 +556,7 @@ attn_w4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
           }
         }
         // ---- pass 2: exponentials against the reference, P over the scores just consumed
-        // (kWpt == 2: half a window's scores may all be -inf; probabilities of 2^-126 at most then, not NaN)
-        const float mneg = kWpt == 2 && m == -INFINITY ? 0.f : -m * sl2;
+        const float mneg = ref_negative(m, sl2);
         const uint64_t mnegx2 = pack2(mneg, mneg);
         uint64_t lsum[4] = {0ull, 0ull, 0ull, 0ull};
         uint32_t pk[16];
@@ -594,7 +593,7 @@ attn_w4_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       ok = warp_wait<kSuspendNs>(&bar->o_full[t], n & 1, &bar->abort_flag, p.status);
       if (!ok) break;
       tc_fence_after();
-      const float inv = kWpt == 2 && m == -INFINITY ? __uint_as_float(0x7fc00000u) : 1.f / l;   // no key of any weight: NaN
+      const float inv = ref_inverse(m, l);
       const int wx0 = it.x0, wy0 = it.y0 + x * p.box_h + sub_y;           // origin of this warp's sub-box
       const bool store = wx0 < it.x_end && wy0 < it.y_end;                // else none of its rows exists
       unsigned char* stg = smem + (size_t)(2 * t + (n & 1)) * kTileBytes + q4 * 4096;

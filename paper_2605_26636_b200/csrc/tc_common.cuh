@@ -280,6 +280,10 @@ __device__ __forceinline__ float max_of(const float (&mx)[4]) { return max3(max3
 __device__ __forceinline__ bool ref_moves(float mx, float m, float lazy) { return !(mx <= m + lazy); }
 // factor for what has been summed up against reference m when mx (> m, or no number) takes its place; 0 for m = -inf
 __device__ __forceinline__ float ref_scale(float m, float mx, float sl2) { return ex2((m - mx) * sl2) + (mx - mx); }
+// m = -inf: all scores so far are -inf, and weigh 0 or 2^-126 against any other
+__device__ __forceinline__ float ref_negative(float m, float sl2) { return m == -INFINITY ? 0.f : -m * sl2; }
+// a row without any key of weight is no number
+__device__ __forceinline__ float ref_inverse(float m, float l) { return m == -INFINITY ? __uint_as_float(0x7fc00000u) : 1.f / l; }
 
 // exp2 on the FMA pipe, for part of the scores (the MUFU unit, 16 results per clock and SM,
 // is the tightest resource of softmax attention at head_dim 64).  x = n + f with n = round(x),

@@ -144,3 +144,33 @@ def test_a_score_that_is_no_number_or_plus_infinity(jv, case, value):
         o, ref = run()
         assert bool(torch.isnan(ref).any()) and bool(torch.isfinite(ref).any())
         _compare(o, ref, dtype, off)
+
+
+@pytest.mark.parametrize("case", ROUTES, ids=lambda c: "x".join(map(str, c)))
+def test_first_keys_of_score_minus_infinity(jv, case):
+    """The first steps of a row see no key of weight: 64 keys, and two tiles and a bit; in windows the first 1/4 and all but the last row."""
+    dtype, D, B, H, P, Hg, Wg, win = case
+    N = P + Hg * Wg
+    t = torch.arange(N, device=DEV)
+    y = (t - P).clamp(min=0) // Wg
+    masks = [t < n for n in (64, 128 if N < 300 else 261)] if win == 0 else [(y % win < n) & (t >= P) & (y < Hg - Hg % win) for n in (win // 4, win - 1)]
+    for off in masks + ([t < P + 64] if win and P else []):          # (with the prefix keys, which the prefix queries see first)
+        q, k, v, run = _call(jv, case, 7600)
+        k[:, :, off, 0] = float("-inf")
+        o, ref = run()
+        assert bool(torch.isfinite(ref).any())
+        _compare(o, ref, dtype, int(off.sum()))
+
+
+@pytest.mark.parametrize("case", ROUTES, ids=lambda c: "x".join(map(str, c)))
+def test_rows_without_any_key_are_nan(jv, case):
+    """Every key of the first head, and in windows every key of the first window, its prefix keys included."""
+    dtype, D, B, H, P, Hg, Wg, win = case
+    q, k, v, run = _call(jv, case, 7700)
+    k[0, 0, :, 0] = float("-inf")
+    if win:
+        t = torch.arange(P + Hg * Wg, device=DEV) - P
+        k[:, :, (t < 0) | ((t // Wg < win) & (t % Wg < win)), 0] = float("-inf")
+    o, ref = run()
+    assert bool(torch.isnan(ref).any()) and bool(torch.isfinite(ref).any())
+    _compare(o, ref, dtype, 0)
