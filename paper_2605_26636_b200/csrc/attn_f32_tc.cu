@@ -393,7 +393,7 @@ attn_f32_tc_kernel(const Params p) {
       uint64_t o[32];
 #pragma unroll
       for (int i = 0; i < 32; ++i) o[i] = 0ull;
-      float m = -INFINITY, l = 0.f, alpha = 0.f;               // m: reference, in the exponent's units (times sl2)
+      float m = -INFINITY, l = 0.f, alpha = 0.f;               // m: the largest score so far
       // o = o alpha + the product of step u with V, alpha as that step found it
       auto take_o = [&](int u) -> bool {
         if (!warp_wait<kSuspendNs>(&bar->o_full[s], u & 1, &bar->abort_flag, p.status)) return false;
@@ -441,13 +441,14 @@ attn_f32_tc_kernel(const Params p) {
           tmem_ld32(tSu, v);
           tmem_wait_ld(v);
           max32(v, mx4);
-          const float mn = fmaxf(m, fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * p.sl2);
+          const float mn = fmaxf(m, max_of(mx4));
           const float ref = mn == -INFINITY ? 0.f : mn;                // all scores so far are -inf: weight 0, not NaN
-          const float alpha_u = ex2(m - ref);                          // exp(-inf) = 0 on the first step
+          const float alpha_u = ex2((m - ref) * p.sl2);                // exp(-inf) = 0 on the first step
           m = mn;
           const uint64_t nref2 = pack2(-ref, -ref);
           uint64_t sum[2] = {0ull, 0ull};
-          // probabilities of 32 keys: two planes over their scores, the third in y2
+          // probabilities of 32 keys: two planes over their scores, the third in y2.  The largest score is subtracted before the scale comes in:
+          // the exponent of the largest is 0 however large the scores are (rounded products of scores beyond 2^32 are off by 2^7 and more)
           auto half = [&](int h, uint32_t (&y2)[2][8]) {
 #pragma unroll
             for (int c = 0; c < 2; ++c) {              // 16 keys at a time
@@ -456,7 +457,7 @@ attn_f32_tc_kernel(const Params p) {
               for (int i = 0; i < 8; ++i) {
                 const int e = 16 * c + 2 * i;
                 float x0, x1;
-                unpack2(fma2(pack2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])), sl2x2, nref2), x0, x1);
+                unpack2(mul2(add2(pack2(__uint_as_float(v[e]), __uint_as_float(v[e + 1])), nref2), sl2x2), x0, x1);
                 uint64_t pr = pack2(ex2(x0), ex2(x1));
                 sum[i & 1] = add2(sum[i & 1], pr);
                 y[0][i] = cut2(pr);
@@ -501,7 +502,7 @@ attn_f32_tc_kernel(const Params p) {
       if (ok && row < wq.nq && !bar->abort_flag) {
         const float2 ml = *reinterpret_cast<const float2*>(other + kPartBytes + r * 8);
         const float M = fmaxf(m, ml.x);
-        const float f = ex2(m - M), fo = ex2(ml.x - M);                          // a slot without a key: exp(-inf) = 0
+        const float f = ex2((m - M) * p.sl2), fo = ex2((ml.x - M) * p.sl2);      // a slot without a key: exp(-inf) = 0
         const float inv = 1.f / fmaf(ml.y, fo, l * f);
         float4* dst = reinterpret_cast<float4*>(p.o + base + (size_t)wq.query_token(row) * kD + 32 * s);
 #pragma unroll

@@ -118,6 +118,31 @@ def test_fp32_tensor_cores_special_values(jv, what):
     assert bool(((got - ref).abs()[f] <= 1e-4 * ref.abs()[f].clamp(min=ref[0, 0].square().mean().sqrt())).all())
 
 
+@pytest.mark.parametrize("size", [3e4, 1e5, 1e6, 1e9])
+@pytest.mark.parametrize("sign", [1, -1])
+@pytest.mark.parametrize("H,Hg,Wg", [(3, 24, 16), (24, 24, 16)], ids=["multiply-adds", "tensor cores"])
+def test_fp32_large_scores(jv, H, Hg, Wg, size, sign):
+    """q and k of this size: one key takes all of a row's weight.  sign -1: all scores are negative.  Rows whose two largest scores are closer
+    than the rounding of a sum of 64 products in 32 bits (64 * 2^-24 of the largest at most) need only be finite."""
+    q, k, v = (t.to(DEV) for t in inputs.custom_qkv(1, H, Hg * Wg, 64, "f32", seed=3750))
+    q, k = q * size, k * size
+    if sign < 0:
+        q, k = q.abs(), -k.abs()
+
+    def windows(t):                                          # 8 x 8 windows as heads
+        return t.view(1, H, Hg // 8, 8, Wg // 8, 8, 64).transpose(3, 4).reshape(1, -1, 64, 64)
+
+    for o, (a, b, c) in ((jv.full_attn(q, k, v), (q, k, v)), (windows(jv.window_attn(q, k, v, Hg, Wg, 8, 8)), map(windows, (q, k, v)))):
+        s = a.double() @ b.double().transpose(-1, -2) / 8
+        top = s.topk(2, -1)
+        gap = top.values[..., 0] - top.values[..., 1]
+        clear = (gap > 64 * 2.0 ** -24 * s.abs().amax(-1)) & (gap > 100)
+        assert float(clear.double().mean()) > 0.98
+        assert bool(torch.isfinite(o).all())
+        want = torch.gather(c, 2, top.indices[..., :1].expand(-1, -1, -1, 64))
+        assert float((o - want).abs()[clear].max()) <= 1e-5
+
+
 @pytest.mark.parametrize("B,H,P,Hg,Wg,win", [(1, 1, 1, 5, 5, 4), (1, 2, 17, 16, 31, 8), (1, 6, 5, 37, 37, 8), (3, 50, 3, 12, 17, 7)])
 def test_fp32_prefix_queries(jv, oracle, B, H, P, Hg, Wg, win):
     """The prefix queries' keys over 4 to 32 groups in clusters of 1 to 8 blocks, some of them without a key."""
