@@ -354,7 +354,7 @@ cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st) {
   if (wh * ww <= 8 && (!prefix || (a.P + wh * ww <= 32 && windows >= 8 * sms))) return launch_attn_generic(a, st, true);
   const int nq = wh * ww, cnt = a.P + nq, key_tiles = ceil_div(cnt, kTileKeys);
   const int64_t rows16 = windows * ceil_div(nq, kRowsWarp), rows32 = windows * ceil_div(nq, 2 * kRowsWarp);   // row tiles of this kernel
-  bool tc = nq > 2 * kRowsWarp;
+  bool tc = nq > 2 * kRowsWarp && a.scale <= 0x1p40f;      // (a larger scale: the last bits of very small values of q and k may count)
   if (cnt <= 2 * kTileKeys) tc = tc && rows32 > sms && (cnt > kTileKeys || windows > a.BH || a.BH <= sms);
   else tc = tc && rows16 > sms && (key_tiles > 4 || 3 * rows16 > 4 * sms);
   if (tc) {

@@ -8,7 +8,9 @@
 // step of 64 keys (scores: of 64 channels), where the small terms meet before the large ones, so that four additions at
 // the size of the result are left; the steps' products with V are added up in fp32 registers, rounded to nearest.
 // A CTA that meets an infinity, a NaN or a value beyond 2^60 among its inputs computes its rows again with fp32 multiply-adds, one
-// warp per row (0 * inf, or inf - inf, between terms would make NaN of what is none).
+// warp per row (0 * inf, or inf - inf, between terms would make NaN of what is none).  So does one with a value of V below 2^-100, but for 0:
+// the third term of such a value, or its products, may lie below bf16's and fp32's normal range (2^-126), and the 24 bits get lost from 2^-110 on.
+// What q and k lose there is below 2^-68 of a score: nothing while the softmax scale is at most 2^40 (launch_attn_f32).
 //
 // One CTA serves 128 query rows of one (batch, head) and window, with its key tiles (64 keys) dealt to two slots: a slot
 // has its own four softmax warps (a thread per row), three warps that cut K and V into bf16 planes, MMA issuer and rings, so that
@@ -75,7 +77,7 @@ struct __align__(8) Barriers {
   uint64_t s_full[kSlots][2], p_full[kSlots], o_full[kSlots];
   uint64_t drain;
   uint32_t tmem_base;
-  volatile uint32_t abort_flag, special;      // special: an infinity, a NaN or a very large value among the CTA's inputs
+  volatile uint32_t abort_flag, special;      // special: an infinity, a NaN, a very large or very small value among the CTA's inputs
 };
 constexpr int kOffQ2 = kSlots * kSlotBytes;    // third plane of Q [128][64], 128-byte swizzle
 constexpr size_t kSmemTiles = kOffQ2 + kTile * kD * 2;
@@ -127,6 +129,12 @@ __device__ __forceinline__ bool noted(uint64_t bad) {
   unpack2(bad, b0, b1);
   return !(fabsf(b0) <= 3.4e38f) || !(fabsf(b1) <= 3.4e38f);
 }
+// The smallest magnitude noted but for 0: its bits without the sign, times 2, less 1 (0 becomes the largest value)
+__device__ __forceinline__ void note_small(uint32_t& least, const float4& x) {
+  least = __vimin3_u32(least, 2 * __float_as_uint(x.x) - 1, 2 * __float_as_uint(x.y) - 1);
+  least = __vimin3_u32(least, 2 * __float_as_uint(x.z) - 1, 2 * __float_as_uint(x.w) - 1);
+}
+constexpr uint32_t kSmall = 2 * ((127u - 100u) << 23) - 1;       // of 2^-100
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
                ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
@@ -295,6 +303,7 @@ attn_f32_tc_kernel(const Params p) {
       const int c4 = lane & 15, hi = lane >> 4;               // rows 2 cw + hi + 6 i (from 64 on: none)
       unsigned char* ring = smem + s * kSlotBytes;
       uint64_t bad = 0ull;
+      uint32_t least = 0xffffffffu;
       // token of the row that lanes 16 (j & 1) .. + 15 take as their i = j / 2, looked up by lane j
       auto row_token = [&](int t) -> int {
         const int c = t * kSub + 2 * cw + (lane & 1) + 6 * (lane >> 1);
@@ -326,6 +335,7 @@ attn_f32_tc_kernel(const Params p) {
               if (row < kSub) {                                 // (a row past the tile is loaded and not stored)
                 note(bad, a);
                 note(bad, b);
+                if (kv == 1) note_small(least, x[i]);
                 uint2 y;
                 y.x = cut2(a); y.y = cut2(b);
                 *reinterpret_cast<uint2*>(to) = y;
@@ -344,7 +354,7 @@ attn_f32_tc_kernel(const Params p) {
         }
         tok = next;
       }
-      if (noted(bad)) bar->special = 1;
+      if (noted(bad) || least < kSmall) bar->special = 1;
     } else {
       // ================= softmax: one thread per query row and slot =================
       asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));

@@ -118,6 +118,24 @@ def test_fp32_tensor_cores_special_values(jv, what):
     assert bool(((got - ref).abs()[f] <= 1e-4 * ref.abs()[f].clamp(min=ref[0, 0].square().mean().sqrt())).all())
 
 
+@pytest.mark.parametrize("size", [1e-27, 1e-30, 1e-34, 1e-36, 1e-37])
+@pytest.mark.parametrize("H,Hg,Wg", [(3, 24, 16), (24, 24, 16)], ids=["multiply-adds", "tensor cores"])
+def test_fp32_small_values(jv, H, Hg, Wg, size):
+    """V of this size in some channels, or q against a large k: results as accurate as those of other sizes, down to fp32's subnormals (results of
+    5e-39, in steps of 1.4e-45)."""
+    q, k, v = (t.to(DEV) for t in inputs.custom_qkv(1, H, Hg * Wg, 64, "f32", seed=3770))
+    v[..., 5:60] *= size
+    v[..., 7] = 0.0
+    v[:, 1, 33] = 0.0
+    ref = torch.softmax(q.double() @ k.double().transpose(-1, -2) / 8, -1) @ v.double()
+    o = jv.full_attn(q, k, v).double()
+    for c in (slice(0, 5), slice(5, 60)):
+        assert float((o - ref)[..., c].norm() / ref[..., c].norm()) <= 6e-7
+    assert bool((o[..., 7] == 0).all())
+    o = jv.full_attn(q * size, k * 1e9, v, scale=1 / (8 * size * 1e9)).double()
+    assert float((o - ref).norm() / ref.norm()) <= 6e-7
+
+
 @pytest.mark.parametrize("size", [3e4, 1e5, 1e6, 1e9])
 @pytest.mark.parametrize("sign", [1, -1])
 @pytest.mark.parametrize("H,Hg,Wg", [(3, 24, 16), (24, 24, 16)], ids=["multiply-adds", "tensor cores"])
