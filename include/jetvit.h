@@ -31,17 +31,22 @@
  *             Kernels bound every wait (2 s); one that gives up sets a sticky
  *             per-device status word and returns, and jv_device_status()
  *             reports JV_ERR_TIMEOUT.  While the word is set, the tensor-core
- *             kernels (bf16, D = 64 or 128) that are launched leave WITHOUT
+ *             kernels (bf16, D = 64 or 128; f32 attention at D = 64 but for
+ *             small calls) that are launched leave WITHOUT
  *             writing their output: calls keep returning JV_OK (they only
  *             enqueue) and o keeps its old contents until jv_device_status()
- *             has been called, which reads and clears the word.  A caller that
+ *             has been called, which reads and clears the word.  A call leaves
+ *             o alone or writes all of it.  A caller that
  *             must know that its results are valid calls jv_device_status()
  *             after the work it cares about.  With the environment variable
  *             JETVIT_DEBUG set, a call that returns JV_ERR_CUDA also prints
  *             the CUDA error string to stderr.
  *   Precision bf16 tensors: bf16 tensor-core products with fp32 accumulation,
  *             fp32 softmax / state, round-to-nearest-even output.  f32 tensors:
- *             fp32 arithmetic throughout (no tf32).
+ *             fp32 arithmetic (no tf32).  f32 attention at D = 64 but for small
+ *             calls forms its products on tensor cores, each value as a sum of
+ *             three bf16 terms (all 24 bits of it), sums in fp32: its error is
+ *             no larger than that of fp32 multiply-adds.
  */
 #ifndef JETVIT_H_
 #define JETVIT_H_

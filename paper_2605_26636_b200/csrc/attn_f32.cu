@@ -47,7 +47,7 @@ constexpr size_t smem_bytes() {
 template <int R, int G, int kKeys, bool kPrefix>
 __global__ void __launch_bounds__(32 * R * G, G == 2 ? 3 : G == 4 ? 2 : 1)  // what shared memory leaves room for
 attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ o,
-                int Hg, int Wg, int P, int wh, int ww, int nwx, bool overlap, float scale) {
+                const int* status, int Hg, int Wg, int P, int wh, int ww, int nwx, bool overlap, float scale) {
   namespace cg = cooperative_groups;
   constexpr int kWarpBuf = warp_buf(kKeys), kJ = kKeys / 16;   // a lane's keys of a tile: tx + 16 j
   extern __shared__ __align__(16) float smem_f[];
@@ -57,6 +57,8 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
   // overlap: the launch ahead is that of the prefix queries (it has waited for what came before it); waited for at the end
   if (!overlap) griddep_wait();
   griddep_launch_dependents();
+  // an earlier kernel gave up, and the windows' kernel looks at the word, too: o stays as it is (status null: that one does not)
+  const bool gave_up = kPrefix && status && *reinterpret_cast<const volatile int*>(status) != 0;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tx = lane & 15, ty = lane >> 4;
   const int grp = warp / R, rw = warp % R;                   // key group, row warp
@@ -263,7 +265,7 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
   auto store = [&](int row, const float4& x, float L) {
     const float inv = 1.f / L;
     const int tok = key_token(kPrefix ? row : P + row);
-    *reinterpret_cast<float4*>(o + base + (size_t)tok * kDim + 4 * tx) = make_float4(x.x * inv, x.y * inv, x.z * inv, x.w * inv);
+    if (!gave_up) *reinterpret_cast<float4*>(o + base + (size_t)tok * kDim + 4 * tx) = make_float4(x.x * inv, x.y * inv, x.z * inv, x.w * inv);
   };
   constexpr int kOwnRows = kRowsWarp / G;                    // rows of row warp rw that this warp writes out
 #pragma unroll
@@ -299,7 +301,7 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
 }
 
 template <int R, int G, int kKeys, bool kPrefix>
-cudaError_t launch(const AttnArgs& a, int split, bool overlap, cudaStream_t st) {   // split: blocks to a cluster (the prefix queries)
+cudaError_t launch(const AttnArgs& a, int split, const int* status, bool overlap, cudaStream_t st) {   // split: blocks to a cluster (the prefix queries)
   static OncePerDevice opt_in;
   const cudaError_t e = opt_in.run([&] {
     return cudaFuncSetAttribute(attn_f32_kernel<R, G, kKeys, kPrefix>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -310,7 +312,7 @@ cudaError_t launch(const AttnArgs& a, int split, bool overlap, cudaStream_t st) 
   const int nwx = ceil_div(a.Wg, ww), nwin = nwx * ceil_div(a.Hg, wh);
   const dim3 grid = kPrefix ? dim3(ceil_div(a.P, R * kRowsWarp) * split, 1, a.BH) : dim3(ceil_div(wh * ww, R * kRowsWarp), nwin, a.BH);
   return launch_cluster(true, attn_f32_kernel<R, G, kKeys, kPrefix>, kPrefix ? split : 0, grid, 32 * R * G, smem_bytes<R, G, kKeys>(), st, (const float*)a.q,
-                        (const float*)a.k, (const float*)a.v, (float*)a.o, a.Hg, a.Wg, a.P, wh, ww, nwx, overlap, a.scale);
+                        (const float*)a.k, (const float*)a.v, (float*)a.o, status, a.Hg, a.Wg, a.P, wh, ww, nwx, overlap, a.scale);
 }
 
 }  // namespace
@@ -342,31 +344,29 @@ bool attn_f32_supported(const AttnArgs& a) { return a.dtype == JV_F32 && a.D == 
 cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st) {
   const int wh = a.wh < a.Hg ? a.wh : a.Hg, ww = a.ww < a.Wg ? a.ww : a.Wg;
   const bool prefix = a.P > 0;
-  if (prefix) {
-    const int N = a.P + a.Hg * a.Wg;
-    const int64_t tiles = (int64_t)ceil_div(a.P, kRowsWarp) * a.BH;
-    int split = 1;
-    while (split < 8 && 2 * split * tiles <= 2 * device_sm_count() && split * 4 * kTileKeys < N) split *= 2;
-    const cudaError_t e = launch<1, 4, kTileKeys, true>(a, split, false, st);
-    if (e != cudaSuccess) return e;
-  }
   const int64_t sms = device_sm_count(), windows = (int64_t)ceil_div(a.Wg, ww) * ceil_div(a.Hg, wh) * a.BH;
-  if (wh * ww <= 8 && (!prefix || (a.P + wh * ww <= 32 && windows >= 8 * sms))) return launch_attn_generic(a, st, true);
   const int nq = wh * ww, cnt = a.P + nq, key_tiles = ceil_div(cnt, kTileKeys);
   const int64_t rows16 = windows * ceil_div(nq, kRowsWarp), rows32 = windows * ceil_div(nq, 2 * kRowsWarp);   // row tiles of this kernel
   bool tc = nq > 2 * kRowsWarp && a.scale <= 0x1p40f;      // (a larger scale: the last bits of very small values of q and k may count)
   if (cnt <= 2 * kTileKeys) tc = tc && rows32 > sms && (cnt > kTileKeys || windows > a.BH || a.BH <= sms);
   else tc = tc && rows16 > sms && (key_tiles > 4 || 3 * rows16 > 4 * sms);
-  if (tc) {
-    int* status = device_status_ptr();
-    if (!status) return cudaErrorUnknown;
-    return launch_attn_f32_tc(a, prefix, status, st);
+  int* status = nullptr;                                   // for the kernels of a call that leave o alone while the word is set: all of them, or none
+  if (tc && !(status = device_status_ptr())) return cudaErrorUnknown;
+  if (prefix) {
+    const int N = a.P + a.Hg * a.Wg;
+    const int64_t tiles = (int64_t)ceil_div(a.P, kRowsWarp) * a.BH;
+    int split = 1;
+    while (split < 8 && 2 * split * tiles <= 2 * sms && split * 4 * kTileKeys < N) split *= 2;
+    const cudaError_t e = launch<1, 4, kTileKeys, true>(a, split, status, false, st);
+    if (e != cudaSuccess) return e;
   }
-  if (cnt <= kTileKeys) return launch<2, 2, 32, false>(a, 1, prefix, st);
-  if (cnt <= 2 * kTileKeys) return launch<1, 4, 32, false>(a, 1, prefix, st);
-  if (cnt <= 4 * kTileKeys && rows16 <= sms) return launch<1, 8, 32, false>(a, 1, prefix, st);
-  if (rows32 <= 2 * sms) return launch<1, 4, kTileKeys, false>(a, 1, prefix, st);
-  return launch<2, 2, kTileKeys, false>(a, 1, prefix, st);
+  if (tc) return launch_attn_f32_tc(a, prefix, status, st);
+  if (nq <= 8 && (!prefix || (cnt <= 32 && windows >= 8 * sms))) return launch_attn_generic(a, st, true);
+  if (cnt <= kTileKeys) return launch<2, 2, 32, false>(a, 1, nullptr, prefix, st);
+  if (cnt <= 2 * kTileKeys) return launch<1, 4, 32, false>(a, 1, nullptr, prefix, st);
+  if (cnt <= 4 * kTileKeys && rows16 <= sms) return launch<1, 8, 32, false>(a, 1, nullptr, prefix, st);
+  if (rows32 <= 2 * sms) return launch<1, 4, kTileKeys, false>(a, 1, nullptr, prefix, st);
+  return launch<2, 2, kTileKeys, false>(a, 1, nullptr, prefix, st);
 }
 
 }  // namespace jv

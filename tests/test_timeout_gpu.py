@@ -106,6 +106,10 @@ def test_every_tensor_core_kernel_leaves_at_once(jv):
     mixer("F, head_dim 128", q6, lambda o: jv.full_attn(q6, k6, v6, out=o))
     mixer("W, head_dim 128", q6, lambda o: jv.window_attn(q6, k6, v6, 40, 30, 16, 16, out=o))
     mixer("L, head_dim 128", q6, lambda o: jv.linear_attn(q6, k6, v6, 40, 30, out=o))
+    q7, k7, v7 = (t.to(DEV) for t in inputs.custom_qkv(1, 24, 5 + 33 * 29, 64, "f32", seed=507))
+    mixer("F, fp32", q7, lambda o: jv.full_attn(q7, k7, v7, out=o))
+    for win in (8, 16):
+        mixer(f"W {win} with prefix tokens, fp32", q7, lambda o, win=win: jv.window_attn(q7, k7, v7, 33, 29, win, win, out=o, prefix=5))
     for name, (B, N, H) in (("one CTA", (1, 300, 6)), ("pairs", (3, 3100, 8))):
         x, w, b, wo, bo = proj(B, N, H)
         outs = [torch.empty((B, H, N, 64), dtype=torch.bfloat16, device=DEV) for _ in range(3)]
@@ -210,6 +214,26 @@ def test_prefix_rows_stay_while_the_word_is_set(jv, oracle, P):
     assert jv.device_status() == jv.JV_ERR_TIMEOUT
     assert rel_err(calls[0](outs[0]), oracle.linear_attn(qh, kh, vh, Hg, Wg, dwc=dh, prefix=P)) <= TOL["bf16"]
     assert rel_err(calls[3](outs[3]), oracle.window_attn(qh, kh, vh, Hg, Wg, 16, 16, prefix=P)) <= TOL["bf16"]
+    assert jv.device_status() == jv.JV_OK
+
+
+@pytest.mark.parametrize("H,stays", [(16, True), (1, False)], ids=["tensor cores", "multiply-adds"])
+@pytest.mark.parametrize("P,win", [(1, 8), (5, 16), (40, 8)])
+def test_fp32_windows_stay_whole_while_the_word_is_set(jv, oracle, H, stays, P, win):
+    """Window attention of fp32 tensors, prefix rows and windows: large calls leave all of o alone, small ones write all of it."""
+    Hg, Wg = (33, 29) if stays else (13, 11)
+    qh, kh, vh = inputs.custom_qkv(1, H, P + Hg * Wg, 64, "f32", seed=93 + P)
+    q, k, v = (t.to(DEV) for t in (qh, kh, vh))
+    ref = oracle.window_attn(qh, kh, vh, Hg, Wg, win, win, prefix=P)
+    o = torch.full_like(q, 1234.5)
+    assert jv.device_status() == jv.JV_OK
+    jv.selftest_wait_timeout(1000)
+    for _ in range(2):
+        jv.window_attn(q, k, v, Hg, Wg, win, win, out=o, prefix=P)
+    torch.cuda.synchronize()
+    assert bool((o == 1234.5).all()) if stays else rel_err(o, ref) <= TOL["f32"]
+    assert jv.device_status() == jv.JV_ERR_TIMEOUT
+    assert rel_err(jv.window_attn(q, k, v, Hg, Wg, win, win, out=o, prefix=P), ref) <= TOL["f32"]
     assert jv.device_status() == jv.JV_OK
 
 
