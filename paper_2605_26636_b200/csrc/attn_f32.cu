@@ -347,7 +347,7 @@ cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st) {
   const int64_t sms = device_sm_count(), windows = (int64_t)ceil_div(a.Wg, ww) * ceil_div(a.Hg, wh) * a.BH;
   const int nq = wh * ww, cnt = a.P + nq, key_tiles = ceil_div(cnt, kTileKeys);
   const int64_t rows16 = windows * ceil_div(nq, kRowsWarp), rows32 = windows * ceil_div(nq, 2 * kRowsWarp);   // row tiles of this kernel
-  bool tc = nq > 2 * kRowsWarp && a.scale <= 0x1p40f;      // (a larger scale: the last bits of very small values of q and k may count)
+  bool tc = nq > 2 * kRowsWarp && a.scale >= 0x1p-40f && a.scale <= 0x1p40f;   // (else what its terms do not hold of very small or infinite values may count)
   if (cnt <= 2 * kTileKeys) tc = tc && rows32 > sms && (cnt > kTileKeys || windows > a.BH || a.BH <= sms);
   else tc = tc && rows16 > sms && (key_tiles > 4 || 3 * rows16 > 4 * sms);
   int* status = nullptr;                                   // for the kernels of a call that leave o alone while the word is set: all of them, or none

@@ -7,10 +7,15 @@
 // Sums stay as they were in fp32 multiply-adds or better: the tensor core's accumulator only takes the terms of ONE
 // step of 64 keys (scores: of 64 channels), where the small terms meet before the large ones, so that four additions at
 // the size of the result are left; the steps' products with V are added up in fp32 registers, rounded to nearest.
-// A CTA that meets an infinity, a NaN or a value beyond 2^60 among its inputs computes its rows again with fp32 multiply-adds, one
-// warp per row (0 * inf, or inf - inf, between terms would make NaN of what is none).  So does one with a value of V below 2^-100, but for 0:
-// the third term of such a value, or its products, may lie below bf16's and fp32's normal range (2^-126), and the 24 bits get lost from 2^-110 on.
-// What q and k lose there is below 2^-68 of a score: nothing while the softmax scale is at most 2^40 (launch_attn_f32).
+// An infinity in K (or what rounds to one: finite values from bf16's largest on) is cut as 2^110 of its sign, so that keys switched off by a
+// score of -inf cost next to nothing: such a key's score is below -2^69 and weighs nothing against scores within 2^30.  What the
+// terms cannot hold, the CTA computes again with fp32 multiply-adds, one warp per row:
+//   - a row whose weights or results are no finite numbers (a score of +inf or NaN, no key of weight, infinities in V);
+//   - beside infinities in K: a row of q with a zero in such a channel (a score of NaN), or with values beyond 2^25 or below 2^-40 (the bounds above); a
+//     row whose largest score is beyond 2^30; a key with two infinities or with other values beyond 2^30;
+//   - values of q beyond 2^60, or below 2^-100 but not 0, and such small values of V: their third term, or its products, may lie below 2^-126, the
+//     normal range, and bits get lost from 2^-110 on.  (What k loses there is below 2^-68 of a score: nothing while the softmax
+//     scale is at most 2^40: launch_attn_f32.)
 //
 // One CTA serves 128 query rows of one (batch, head) and window, with its key tiles (64 keys) dealt to two slots: a slot
 // has its own four softmax warps (a thread per row), three warps that cut K and V into bf16 planes, MMA issuer and rings, so that
@@ -77,7 +82,9 @@ struct __align__(8) Barriers {
   uint64_t s_full[kSlots][2], p_full[kSlots], o_full[kSlots];
   uint64_t drain;
   uint32_t tmem_base;
-  volatile uint32_t abort_flag, special;      // special: an infinity, a NaN, a very large or very small value among the CTA's inputs
+  volatile uint32_t abort_flag;
+  volatile uint32_t special, untame;          // the CTA's rows have to be computed with multiply-adds: in any case, or if there are infinities in K
+  uint32_t k_inf[2], q_zero[2];               // channels 32 i .. with an infinity in K, with a zero in Q
 };
 constexpr int kOffQ2 = kSlots * kSlotBytes;    // third plane of Q [128][64], 128-byte swizzle
 constexpr size_t kSmemTiles = kOffQ2 + kTile * kD * 2;
@@ -122,7 +129,7 @@ __device__ __forceinline__ uint32_t last2(uint64_t x) {
   unpack2(x, lo, hi);
   return pack_bf16(lo, hi);
 }
-// Infinite or no number once one of the values noted is, or exceeds 2^60: a product of two smaller ones does not overflow
+// Infinite or no number once one of the values noted is, or exceeds 2^60
 __device__ __forceinline__ void note(uint64_t& bad, uint64_t x) { bad = fma2(x, pack2(0x1p67f, 0x1p67f), bad); }
 __device__ __forceinline__ bool noted(uint64_t bad) {
   float b0, b1;
@@ -134,7 +141,20 @@ __device__ __forceinline__ void note_small(uint32_t& least, const float4& x) {
   least = __vimin3_u32(least, 2 * __float_as_uint(x.x) - 1, 2 * __float_as_uint(x.y) - 1);
   least = __vimin3_u32(least, 2 * __float_as_uint(x.z) - 1, 2 * __float_as_uint(x.w) - 1);
 }
-constexpr uint32_t kSmall = 2 * ((127u - 100u) << 23) - 1;       // of 2^-100
+constexpr uint32_t note_of(int e) { return 2 * ((127u + e) << 23) - 1; }         // of 2^e
+constexpr uint32_t kSmall = note_of(-100), kSmallQ = note_of(-40);
+constexpr float kInfinite = 3.3895e38f;      // bf16's largest value and a little
+__device__ __forceinline__ bool no_number(float x) { return !(fabsf(x) < INFINITY); }
+// Four values in three planes of a ring stage
+__device__ __forceinline__ void store3(unsigned char* to, uint64_t a, uint64_t b) {
+  uint2 y;
+  y.x = cut2(a); y.y = cut2(b);
+  *reinterpret_cast<uint2*>(to) = y;
+  y.x = cut2(a); y.y = cut2(b);
+  *reinterpret_cast<uint2*>(to + kPlane) = y;
+  y.x = last2(a); y.y = last2(b);
+  *reinterpret_cast<uint2*>(to + 2 * kPlane) = y;
+}
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
                ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
@@ -207,7 +227,8 @@ attn_f32_tc_kernel(const Params p) {
     }
     mbar_init(&bar->drain, kSlots);
     bar->abort_flag = 0;
-    bar->special = 0;
+    bar->special = bar->untame = 0;
+    for (int i = 0; i < 2; ++i) bar->k_inf[i] = bar->q_zero[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -302,7 +323,6 @@ attn_f32_tc_kernel(const Params p) {
       const int ntiles = (w.cnt + kSub - 1) / kSub;
       const int c4 = lane & 15, hi = lane >> 4;               // rows 2 cw + hi + 6 i (from 64 on: none)
       unsigned char* ring = smem + s * kSlotBytes;
-      uint64_t bad = 0ull;
       uint32_t least = 0xffffffffu;
       // token of the row that lanes 16 (j & 1) .. + 15 take as their i = j / 2, looked up by lane j
       auto row_token = [&](int t) -> int {
@@ -324,6 +344,7 @@ attn_f32_tc_kernel(const Params p) {
         for (int kv = 0; kv < 2; ++kv) {
           ok = warp_wait<kSuspendNs>(kv == 0 ? &bar->k_empty[s][g] : &bar->v_empty[s][g], ((u / kStages) & 1) ^ 1, &bar->abort_flag, p.status);
           if (!ok) break;
+          uint64_t bad = 0ull;
           unsigned char* dst = ring + (kv * kStages + g) * kStageBytes + (c4 & 1) * 8;
 #pragma unroll
           for (int half = 0; half < 2; ++half) {
@@ -333,28 +354,50 @@ attn_f32_tc_kernel(const Params p) {
               unsigned char* to = dst + row * 128 + (((c4 >> 1) ^ (row & 7)) << 4);
               uint64_t a = pack2(x[i].x, x[i].y), b = pack2(x[i].z, x[i].w);
               if (row < kSub) {                                 // (a row past the tile is loaded and not stored)
-                note(bad, a);
-                note(bad, b);
-                if (kv == 1) note_small(least, x[i]);
-                uint2 y;
-                y.x = cut2(a); y.y = cut2(b);
-                *reinterpret_cast<uint2*>(to) = y;
-                y.x = cut2(a); y.y = cut2(b);
-                *reinterpret_cast<uint2*>(to + kPlane) = y;
-                y.x = last2(a); y.y = last2(b);
-                *reinterpret_cast<uint2*>(to + 2 * kPlane) = y;
+                if (kv == 0) {
+                  note(bad, a);
+                  note(bad, b);
+                } else {
+                  note_small(least, x[i]);
+                }
+                store3(to, a, b);
               }
             }
             // the rows just stored are V's, or the next tile's K's: on their way under the other half
 #pragma unroll
             for (int i = half * 6; i < 6 + half * (kConvRows - 6); ++i) load(i, kv == 0 ? p.v : p.k, kv == 0 ? tok : next);
           }
+          if (kv == 0 && __any_sync(0xffffffffu, noted(bad))) {     // infinities in K: the tile once more (its values have made room for V's)
+#pragma unroll 1
+            for (int i = 0; i < kConvRows; ++i) {
+              const int row = 2 * cw + hi + 6 * i, tk = __shfl_sync(0xffffffffu, tok, 2 * i + hi);
+              float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (tk >= 0) y = __ldcg(reinterpret_cast<const float4*>(p.k + base + (size_t)tk * kD + 4 * c4));
+              float e[4] = {y.x, y.y, y.z, y.w};
+              uint32_t inf = 0;
+              bool big = false;
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const bool is = fabsf(e[j]) >= kInfinite;
+                inf |= (is ? 1u : 0u) << j;
+                big = big || (!is && fabsf(e[j]) > 0x1p30f);
+                if (is) e[j] = copysignf(0x1p110f, e[j]);
+              }
+              const uint32_t of_row = 0xffffu << (16 * hi);         // the lanes that have this row
+              const uint32_t infs = __ballot_sync(0xffffffffu, inf != 0) & of_row, bigs = __ballot_sync(0xffffffffu, big) & of_row;
+              if (inf && row < kSub) {
+                atomicOr(&bar->k_inf[c4 >> 3], inf << (4 * (c4 & 7)));
+                store3(dst + row * 128 + (((c4 >> 1) ^ (row & 7)) << 4), pack2(e[0], e[1]), pack2(e[2], e[3]));
+                if (bigs || __popc(infs) > 1 || __popc(inf) > 1) bar->special = 1;
+              }
+            }
+          }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           mbar_arrive(kv == 0 ? &bar->k_full[s][g] : &bar->v_full[s][g]);
         }
         tok = next;
       }
-      if (noted(bad) || least < kSmall) bar->special = 1;
+      if (least < kSmall) bar->special = 1;
     } else {
       // ================= softmax: one thread per query row and slot =================
       asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
@@ -372,7 +415,8 @@ attn_f32_tc_kernel(const Params p) {
       {
         const bool in = row < wq.nq;
         const float4* src = reinterpret_cast<const float4*>(p.q + base + (size_t)wq.query_token(in ? row : 0) * kD + 32 * s);
-        uint64_t bad = 0ull;
+        uint32_t least = 0xffffffffu, zero = 0;
+        float most = 0.f;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           uint32_t y[3][8];
@@ -380,8 +424,9 @@ attn_f32_tc_kernel(const Params p) {
           for (int i = 0; i < 4; ++i) {
             const float4 x = in ? __ldcg(src + 4 * h + i) : make_float4(0.f, 0.f, 0.f, 0.f);
             uint64_t a = pack2(x.x, x.y), b = pack2(x.z, x.w);
-            note(bad, a);
-            note(bad, b);
+            note_small(least, x);
+            most = max3(max3(most, fabsf(x.x), fabsf(x.y)), fabsf(x.z), fabsf(x.w));
+            zero |= ((x.x == 0.f ? 1u : 0u) | (x.y == 0.f ? 2u : 0u) | (x.z == 0.f ? 4u : 0u) | (x.w == 0.f ? 8u : 0u)) << (16 * h + 4 * i);
             y[0][2 * i] = cut2(a); y[0][2 * i + 1] = cut2(b);
             y[1][2 * i] = cut2(a); y[1][2 * i + 1] = cut2(b);
             y[2][2 * i] = last2(a); y[2][2 * i + 1] = last2(b);
@@ -393,7 +438,9 @@ attn_f32_tc_kernel(const Params p) {
             *reinterpret_cast<uint4*>(smem + kOffQ2 + r * 128 + (((4 * s + 2 * h + i) ^ (r & 7)) << 4)) =
                 make_uint4(y[2][4 * i], y[2][4 * i + 1], y[2][4 * i + 2], y[2][4 * i + 3]);
         }
-        if (noted(bad)) bar->special = 1;
+        if (least < kSmall || !(most <= 0x1p60f)) bar->special = 1;
+        if (least < kSmallQ || !(most <= 0x1p25f)) bar->untame = 1;
+        if (in && zero) atomicOr(&bar->q_zero[s], zero);
         tmem_wait_st();
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_fence_before();
@@ -513,7 +560,8 @@ attn_f32_tc_kernel(const Params p) {
         const float2 ml = *reinterpret_cast<const float2*>(other + kPartBytes + r * 8);
         const float M = fmaxf(m, ml.x);
         const float f = ex2((m - M) * p.sl2), fo = ex2((ml.x - M) * p.sl2);      // a slot without a key: exp(-inf) = 0
-        const float inv = 1.f / fmaf(ml.y, fo, l * f);
+        const float L = fmaf(ml.y, fo, l * f), inv = 1.f / L;
+        uint64_t zeros = 0ull;                                                     // or no number, once one of the results is no finite one
         float4* dst = reinterpret_cast<float4*>(p.o + base + (size_t)wq.query_token(row) * kD + 32 * s);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -521,9 +569,15 @@ attn_f32_tc_kernel(const Params p) {
           float x0, x1, x2, x3;
           unpack2(s == 0 ? o[2 * i] : o[16 + 2 * i], x0, x1);
           unpack2(s == 0 ? o[2 * i + 1] : o[17 + 2 * i], x2, x3);
-          dst[i] = make_float4(fmaf(y.x, fo, x0 * f) * inv, fmaf(y.y, fo, x1 * f) * inv, fmaf(y.z, fo, x2 * f) * inv,
-                               fmaf(y.w, fo, x3 * f) * inv);
+          const float4 z = make_float4(fmaf(y.x, fo, x0 * f) * inv, fmaf(y.y, fo, x1 * f) * inv, fmaf(y.z, fo, x2 * f) * inv,
+                                       fmaf(y.w, fo, x3 * f) * inv);
+          dst[i] = z;
+          zeros = fma2(pack2(z.x, z.y), 0ull, fma2(pack2(z.z, z.w), 0ull, zeros));
         }
+        float z0, z1;
+        unpack2(zeros, z0, z1);
+        if (!(L < INFINITY) || no_number(z0 + z1)) bar->special = 1;
+        if (!(fabsf(M) < 0x1p30f)) bar->untame = 1;
       }
     }
   }
@@ -533,7 +587,9 @@ attn_f32_tc_kernel(const Params p) {
   tc_fence_after();
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
-  if (!skip && warp < kWarpSlot && bar->special && !bar->abort_flag) plain_rows(p, base, warp, lane);   // (the softmax warps: they have the registers)
+  const uint32_t k_inf0 = bar->k_inf[0], k_inf1 = bar->k_inf[1];
+  const bool special = bar->special || ((k_inf0 | k_inf1) && bar->untame) || (k_inf0 & bar->q_zero[0]) || (k_inf1 & bar->q_zero[1]);
+  if (!skip && warp < kWarpSlot && special && !bar->abort_flag) plain_rows(p, base, warp, lane);   // (the softmax warps: they have the registers)
   if (p.overlap) griddep_wait();
 }
 

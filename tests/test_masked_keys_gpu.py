@@ -174,3 +174,47 @@ def test_rows_without_any_key_are_nan(jv, case):
     o, ref = run()
     assert bool(torch.isnan(ref).any()) and bool(torch.isfinite(ref).any())
     _compare(o, ref, dtype, 0)
+
+
+@pytest.mark.parametrize("what", ["q zero", "two channels", "two signs", "beside large", "large q", "larger q", "small q", "tiny q", "large scores", "lowest", "mixed"])
+@pytest.mark.parametrize("case", [c for c in ROUTES if c[0] == "f32"], ids=lambda c: "x".join(map(str, c)))
+def test_infinities_in_fp32_keys(jv, case, what):
+    """Where an infinite channel of k does not simply switch its key off, or does so among values that come close to the bounds of the kernels: the rows
+    that are no numbers are, and the others are as accurate as ever."""
+    dtype, D, B, H, P, Hg, Wg, win = case
+    N = P + Hg * Wg
+    q, k, v, run = _call(jv, case, 7800)
+    t = torch.arange(N, device=DEV)
+    off, rows = t % 9 == 4, t % 5 == 2
+    k[:, :, off, 0] = float("-inf")
+    if what == "q zero":                                   # 0 * inf: no number
+        q[:, :, rows, 0] = 0.0
+        q[..., 1] = 0.0                                    # (and zeros that meet nothing)
+    elif what == "two channels":                           # of one sign or two, by q's
+        k[:, :, t % 90 == 4, 40] = float("-inf")
+    elif what == "two signs":
+        k[:, :2, t % 90 == 4, 40] = float("inf")
+        q[..., 40] = 0.5
+    elif what == "beside large":                           # finite, and against the infinity
+        k[:, :, t % 90 == 4, 40] = 3e38
+        q[..., 40] = 0.5
+    elif what in ("large q", "larger q"):
+        k[:, :, ~off, 0] = 0.0
+        q[:, :, rows, 0] = 5e4 if what == "large q" else 1e9
+    elif what == "small q":
+        q[:, :, rows, 0] = 1e-9
+    elif what == "tiny q":
+        q[:, :, rows, 0] = 1e-36
+    elif what == "large scores":                           # the others are far below
+        k[:, :, ~off, 3], q[..., 3] = -1e12, 0.0
+        q[:, :, rows, 3] = 1e9
+    elif what == "lowest":
+        k[:, :, off, 0] = torch.finfo(torch.float32).min
+    elif what == "mixed":                                  # one key left in some windows and rows
+        k[:, :, t % 8 != 1, 0] = float("-inf")
+    o, ref = run()
+    assert bool(torch.isfinite(ref).any())
+    if what == "large scores":                             # weights of scores of 1e20: only the largest one's counts, and rounding decides which is
+        assert torch.equal(torch.isnan(o), torch.isnan(ref))
+        o, ref = o[:, :, ~rows], ref[:, :, ~rows]
+    _compare(o, ref, dtype, what)
