@@ -28,11 +28,7 @@ namespace {
 
 using namespace f32;
 
-constexpr int kDim = 64;
 constexpr int kTileKeys = 64;    // keys per tile, but for short rows of keys
-constexpr int kRowsWarp = 16;    // query rows per warp
-constexpr int kLd = 68;          // floats per shared-memory row: 16-byte reads of 8 consecutive rows touch all banks
-constexpr int kLdP = 20;         // floats per key of the transposed probabilities (16 rows): 16-byte writes of 8 keys likewise
 // floats of a warp's own buffer: the probabilities of a tile of `keys` keys, then the warp's output
 __host__ __device__ constexpr int warp_buf(int keys) { return keys * kLdP > kRowsWarp * kLd ? keys * kLdP : kRowsWarp * kLd; }
 
@@ -49,11 +45,11 @@ __global__ void __launch_bounds__(32 * R * G, G == 2 ? 3 : G == 4 ? 2 : 1)  // w
 attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ o,
                 const int* status, int Hg, int Wg, int P, int wh, int ww, int nwx, bool overlap, float scale) {
   namespace cg = cooperative_groups;
-  constexpr int kWarpBuf = warp_buf(kKeys), kJ = kKeys / 16;   // a lane's keys of a tile: tx + 16 j
+  constexpr int kWarpBuf = warp_buf(kKeys);
   extern __shared__ __align__(16) float smem_f[];
   float* qs = smem_f;                                        // [16 R][kLd]
-  float* ps = qs + R * kRowsWarp * kLd;                      // [R G warps]: probabilities [64 keys][kLdP], then the warp's output [16][kLd]
-  float* ks = ps + R * G * kWarpBuf;                  // [G][64][kLd]: the group's K tile, then its V tile
+  float* ps = qs + R * kRowsWarp * kLd;                      // [R G warps]: probabilities [kKeys][kLdP], then the warp's output [16][kLd]
+  float* ks = ps + R * G * kWarpBuf;                         // [G][kKeys][kLd]: the group's K tile, then its V tile
   // overlap: the launch ahead is that of the prefix queries (it has waited for what came before it); waited for at the end
   if (!overlap) griddep_wait();
   griddep_launch_dependents();
@@ -124,123 +120,31 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
   }
 
   const float* qr = qs + (rw * kRowsWarp + ty * 8) * kLd;
-  float m[8], l[8];
-  f32x2 acc[4][4];                                           // rows 2 i and 2 i + 1, channel 4 tx + e
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    m[i] = -INFINITY;
-    l[i] = 0.f;
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc[i][e] = 0ull;
-
+  RowTile<kKeys> x;
   for (int t = first; t < ntiles; t += stride) {
     copy_wait<0>();                                          // K of this tile
     group_sync();
-    f32x2 s2[8][kJ];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-      for (int j = 0; j < kJ; ++j) s2[i][j] = 0ull;
-#pragma unroll 4
-    for (int c = 0; c < kDim; c += 4) {
-      ulonglong2 kk[kJ];
-#pragma unroll
-      for (int j = 0; j < kJ; ++j) kk[j] = *reinterpret_cast<const ulonglong2*>(kg + (tx + 16 * j) * kLd + c);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const ulonglong2 qq = *reinterpret_cast<const ulonglong2*>(qr + i * kLd + c);
-#pragma unroll
-        for (int j = 0; j < kJ; ++j) {
-          fma2(s2[i][j], qq.x, kk[j].x);
-          fma2(s2[i][j], qq.y, kk[j].y);
-        }
-      }
-    }
+    x.scores(qr, kg, tx);
     group_sync();                                            // the group is done with K
     load_tile(kg, v, t);                                     // V, under the softmax
 
-    const bool ragged = (t + 1) * kKeys > cnt;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {                            // four rows at a time
-      float p[kJ][4], alpha[4];                              // [key][row]
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int i = 4 * h + r;
-        float s[kJ];
-#pragma unroll
-        for (int j = 0; j < kJ; ++j) {
-          const float2 e = unpack2(s2[i][j]);
-          s[j] = (e.x + e.y) * scale;
-          if (ragged && t * kKeys + tx + 16 * j >= cnt) s[j] = -INFINITY;
-        }
-        float mx = fmaxf(s[0], s[1]);
-        if (kJ == 4) mx = fmaxf(mx, fmaxf(s[2 % kJ], s[3 % kJ]));
-#pragma unroll
-        for (int w = 1; w < 16; w <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
-        const float mn = fmaxf(m[i], mx);
-        const float ref = mn == -INFINITY ? 0.f : mn;        // all scores of this group so far are -inf: weight 0, not NaN
-        alpha[r] = expf(m[i] - ref);                         // exp(-inf) = 0 on the first tile
-        m[i] = mn;
-        float sum = 0.f;
-#pragma unroll
-        for (int j = 0; j < kJ; ++j) {
-          p[j][r] = expf(s[j] - ref);
-          sum += p[j][r];
-        }
-        l[i] = fmaf(l[i], alpha[r], sum);
-      }
-#pragma unroll
-      for (int j = 0; j < kJ; ++j)
-        *reinterpret_cast<float4*>(pw + (tx + 16 * j) * kLdP + ty * 8 + 4 * h) = make_float4(p[j][0], p[j][1], p[j][2], p[j][3]);
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const f32x2 a2 = pack2(alpha[2 * r], alpha[2 * r + 1]);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[2 * h + r][e] = mul2(acc[2 * h + r][e], a2);
-      }
-    }
+    x.softmax(cnt - t * kKeys, scale, pw, tx, ty);
     copy_wait<0>();                                          // V of this tile
     group_sync();                                            // (also orders the warp's own probabilities)
-#pragma unroll 8
-    for (int c = 0; c < kKeys; ++c) {
-      const float4 v4 = *reinterpret_cast<const float4*>(kg + c * kLd + 4 * tx);
-      const ulonglong2 pa = *reinterpret_cast<const ulonglong2*>(pw + c * kLdP + ty * 8);
-      const ulonglong2 pb = *reinterpret_cast<const ulonglong2*>(pw + c * kLdP + ty * 8 + 4);
-      const f32x2 vv[4] = {pack2(v4.x, v4.x), pack2(v4.y, v4.y), pack2(v4.z, v4.z), pack2(v4.w, v4.w)};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        fma2(acc[0][e], pa.x, vv[e]);
-        fma2(acc[1][e], pa.y, vv[e]);
-        fma2(acc[2][e], pb.x, vv[e]);
-        fma2(acc[3][e], pb.y, vv[e]);
-      }
-    }
+    x.values(kg, pw, tx, ty);
     group_sync();                                            // the group is done with V (and the warp with its P)
     if (t + stride < ntiles) load_tile(kg, k, t + stride);
   }
 
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-#pragma unroll
-    for (int w = 1; w < 16; w <<= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], w);
-  }
+  x.finish();
   // Merge the groups through the warps' own buffers: output channels 0..63 of a row, then its maximum and sum.
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     float* dst = pw + (ty * 8 + i) * kLd;
-    float x[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 y = unpack2(acc[i / 2][e]);
-      x[e] = i % 2 ? y.y : y.x;
-    }
-    *reinterpret_cast<float4*>(dst + 4 * tx) = make_float4(x[0], x[1], x[2], x[3]);
+    *reinterpret_cast<float4*>(dst + 4 * tx) = x.row(i);
     if (tx == 0) {
-      dst[64] = m[i];
-      dst[65] = l[i];
+      dst[64] = x.m[i];
+      dst[65] = x.l[i];
     }
   }
   __syncthreads();

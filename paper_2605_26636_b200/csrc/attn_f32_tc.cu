@@ -7,15 +7,16 @@
 // Sums stay as they were in fp32 multiply-adds or better: the tensor core's accumulator only takes the terms of ONE
 // step of 64 keys (scores: of 64 channels), where the small terms meet before the large ones, so that four additions at
 // the size of the result are left; the steps' products with V are added up in fp32 registers, rounded to nearest.
-// An infinity in K (or what rounds to one: finite values from bf16's largest on) is cut as 2^110 of its sign, so that keys switched off by a
-// score of -inf cost next to nothing: such a key's score is below -2^69 and weighs nothing against scores within 2^30.  What the
-// terms cannot hold, the CTA computes again with fp32 multiply-adds, one warp per row:
+// An infinity in K (or what rounds to one: finite values from bf16's largest on) becomes 2^110 of its sign, so that keys switched off by a
+// score of -inf cost little: such a key's score is below -2^69 and weighs nothing against scores within 2^30.  What the
+// terms cannot hold, the CTA computes again with fp32 multiply-adds (plain_rows):
 //   - a row whose weights or results are no finite numbers (a score of +inf or NaN, no key of weight, infinities in V);
-//   - beside infinities in K: a row of q with a zero in such a channel (a score of NaN), or with values beyond 2^25 or below 2^-40 (the bounds above); a
-//     row whose largest score is beyond 2^30; a key with two infinities or with other values beyond 2^30;
-//   - values of q beyond 2^60, or below 2^-100 but not 0, and such small values of V: their third term, or its products, may lie below 2^-126, the
-//     normal range, and bits get lost from 2^-110 on.  (What k loses there is below 2^-68 of a score: nothing while the softmax
-//     scale is at most 2^40: launch_attn_f32.)
+//   - beside infinities in K: a zero of q in such a channel (a score of NaN), values of q beyond 2^25 or below 2^-40 (the bounds above), a row
+//     whose largest score is beyond 2^30, a key with two infinities or with other values beyond 2^30;
+//   - values of q beyond 2^60, or below 2^-100 but not 0; results below 2^-80 beside values of V below 2^-60 but not 0.  The third term of very
+//     small values, or its products, may lie below 2^-126, the normal range, and bits get lost from 2^-110 on.  (What k loses there is
+//     below 2^-68 of a score: nothing while the softmax scale is at most 2^40: launch_attn_f32.)
+// All of this is looked at where it is cheap: K by the sum of its magnitudes and the issuing warp, V by the results.
 //
 // One CTA serves 128 query rows of one (batch, head) and window, with its key tiles (64 keys) dealt to two slots: a slot
 // has its own four softmax warps (a thread per row), three warps that cut K and V into bf16 planes, MMA issuer and rings, so that
@@ -35,6 +36,7 @@
 // (1.8e-7 to 5.2e-7) over 1 to 300 heads of 64 to 1400 tokens.  With terms cut off instead of rounded the terms left out all had
 // the product's sign: 2.3e-7 to 2.8e-7.  With one score buffer per slot 33.1 us in place of 26.3; with the third plane of P in a plane of its own
 // per buffer there is no tensor memory left.
+#include "f32_common.cuh"
 #include "tc_common.cuh"
 
 namespace jv {
@@ -76,6 +78,9 @@ struct Params {
   float scale, sl2;       // softmax scale, and times log2(e)
 };
 
+// What a CTA has met.  kSpecial: its rows have to be computed with multiply-adds; kUntame: if there are infinities in K, too; kInf: there are;
+// kZero: zeros in Q, which matter if they meet one; kLookV: results below 2^-80, which may come of too small values of V; kUnclear: one of these does
+enum : uint32_t { kSpecial = 1, kUntame = 2, kInf = 4, kZero = 8, kLookV = 16, kUnclear = 32 };
 struct __align__(8) Barriers {
   uint64_t q_full;
   uint64_t k_full[kSlots][kStages], k_empty[kSlots][kStages], v_full[kSlots][kStages], v_empty[kSlots][kStages];
@@ -83,8 +88,9 @@ struct __align__(8) Barriers {
   uint64_t drain;
   uint32_t tmem_base;
   volatile uint32_t abort_flag;
-  volatile uint32_t special, untame;          // the CTA's rows have to be computed with multiply-adds: in any case, or if there are infinities in K
-  uint32_t k_inf[2], q_zero[2];               // channels 32 i .. with an infinity in K, with a zero in Q
+  uint32_t flags;                              // kSpecial ..
+  volatile int k_odd[kSlots][kStages];         // 1 + step of a tile of K with values that are no numbers or beyond 2^60
+  uint32_t k_inf[2];                           // channels 32 i .. with an infinity in K
 };
 constexpr int kOffQ2 = kSlots * kSlotBytes;    // third plane of Q [128][64], 128-byte swizzle
 constexpr size_t kSmemTiles = kOffQ2 + kTile * kD * 2;
@@ -129,22 +135,27 @@ __device__ __forceinline__ uint32_t last2(uint64_t x) {
   unpack2(x, lo, hi);
   return pack_bf16(lo, hi);
 }
+__device__ __forceinline__ bool no_number(float x) { return !(fabsf(x) < INFINITY); }
 // Infinite or no number once one of the values noted is, or exceeds 2^60
 __device__ __forceinline__ void note(uint64_t& bad, uint64_t x) { bad = fma2(x, pack2(0x1p67f, 0x1p67f), bad); }
 __device__ __forceinline__ bool noted(uint64_t bad) {
   float b0, b1;
   unpack2(bad, b0, b1);
-  return !(fabsf(b0) <= 3.4e38f) || !(fabsf(b1) <= 3.4e38f);
+  return no_number(b0 + b1);
 }
-// The smallest magnitude noted but for 0: its bits without the sign, times 2, less 1 (0 becomes the largest value)
-__device__ __forceinline__ void note_small(uint32_t& least, const float4& x) {
-  least = __vimin3_u32(least, 2 * __float_as_uint(x.x) - 1, 2 * __float_as_uint(x.y) - 1);
-  least = __vimin3_u32(least, 2 * __float_as_uint(x.z) - 1, 2 * __float_as_uint(x.w) - 1);
+// The smallest and the largest magnitude of values (largest: NaN is passed over)
+__device__ __forceinline__ float min_abs(float m, const float4& x) {
+  asm("{\n.reg .f32 a, b;\nabs.f32 a, %1;\nabs.f32 b, %2;\nmin.f32 %0, %0, a, b;\nabs.f32 a, %3;\nabs.f32 b, %4;\nmin.f32 %0, %0, a, b;\n}"
+      : "+f"(m) : "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w));
+  return m;
 }
-constexpr uint32_t note_of(int e) { return 2 * ((127u + e) << 23) - 1; }         // of 2^e
-constexpr uint32_t kSmall = note_of(-100), kSmallQ = note_of(-40);
-constexpr float kInfinite = 3.3895e38f;      // bf16's largest value and a little
-__device__ __forceinline__ bool no_number(float x) { return !(fabsf(x) < INFINITY); }
+__device__ __forceinline__ float max_abs(float m, const float4& x) {
+  asm("{\n.reg .f32 a, b;\nabs.f32 a, %1;\nabs.f32 b, %2;\nmax.f32 %0, %0, a, b;\nabs.f32 a, %3;\nabs.f32 b, %4;\nmax.f32 %0, %0, a, b;\n}"
+      : "+f"(m) : "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w));
+  return m;
+}
+constexpr float kSmall = 0x1p-100f;
+
 // Four values in three planes of a ring stage
 __device__ __forceinline__ void store3(unsigned char* to, uint64_t a, uint64_t b) {
   uint2 y;
@@ -160,44 +171,128 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
                ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
 }
 
-// The rows of a CTA with fp32 multiply-adds, a warp per query row, a lane per key (scores) and two channels (output)
-__device__ void plain_rows(const Params& p, size_t base, int warp, int lane) {
-  for (int r = warp; r < kTile; r += kWarpSlot) {
-    const Window w(p, p.pair ? 2 * blockIdx.y + (r >> 6) : blockIdx.y);
-    const int row = p.pair ? (r & 63) : blockIdx.x * kTile + r;
-    if (row >= w.nq) continue;
-    const int tok = w.query_token(row);
-    const float q0 = p.q[base + (size_t)tok * kD + lane], q1 = p.q[base + (size_t)tok * kD + 32 + lane];
-    float m = -INFINITY, l = 0.f, o0 = 0.f, o1 = 0.f;
-    for (int c0 = 0; c0 < w.cnt; c0 += 32) {
-      const bool in = c0 + lane < w.cnt;
-      const int kt = w.key_token(in ? c0 + lane : 0);
-      const float* kr = p.k + base + (size_t)kt * kD;
-      float s = 0.f;
-#pragma unroll 8
-      for (int c = 0; c < 32; ++c) {
-        s = fmaf(__shfl_sync(0xffffffffu, q0, c), kr[c], s);
-        s = fmaf(__shfl_sync(0xffffffffu, q1, c), kr[32 + c], s);
-      }
-      s = in ? s * p.scale : -INFINITY;
-      const float mn = fmaxf(m, warp_max(s));
-      const float ref = mn == -INFINITY ? 0.f : mn;          // all scores so far are -inf: weight 0, not NaN
-      const float alpha = expf(m - ref), e = expf(s - ref);
-      m = mn;
-      l = fmaf(l, alpha, warp_sum(e));
-      o0 *= alpha;
-      o1 *= alpha;
-      for (int j = 0; j < 32 && c0 + j < w.cnt; ++j) {
-        const float pj = __shfl_sync(0xffffffffu, e, j);
-        const float* vr = p.v + base + (size_t)__shfl_sync(0xffffffffu, kt, j) * kD;
-        o0 = fmaf(pj, vr[lane], o0);
-        o1 = fmaf(pj, vr[32 + lane], o1);
+// Infinities in a tile of K that has just been cut, by the warp that issues its MMAs: two rows to a lane.  planes: the first of three.
+// (In the warps that cut, even a branch that is never taken cost 5 %, their loads being in flight there.)
+__device__ __forceinline__ void cut_infinities(unsigned char* planes, Barriers* bar, int lane) {
+#pragma unroll 1
+  for (int row = lane; row < kSub; row += 32) {
+    int infs = 0, bigs = 0;                                    // values that are infinite or no number; those and others beyond 2^30
+#pragma unroll 4
+    for (int c = 0; c < kD / 8; ++c) {
+      uint32_t* at = reinterpret_cast<uint32_t*>(planes + row * 128 + ((c ^ (row & 7)) << 4));
+      const uint4 y = *reinterpret_cast<const uint4*>(at);
+      const uint32_t w[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t magnitude = w[j] & 0x7fff7fffu, inf = (magnitude + 0x00800080u) & 0x80008000u;
+        bigs += __popc((magnitude + 0x317f317fu) & 0x80008000u);
+        if (inf == 0) continue;
+        infs += __popc(inf);
+        uint32_t z = w[j];
+#pragma unroll
+        for (int h = 0; h < 32; h += 16)
+          if (((magnitude >> h) & 0xffffu) == 0x7f80u) {
+            z = (z & ~(0x7fffu << h)) | (0x7680u << h);        // 2^110
+            at[j + kPlane / 4] &= ~(0xffffu << h);
+            at[j + 2 * (kPlane / 4)] &= ~(0xffffu << h);
+            const int ch = 8 * c + 2 * j + (h >> 4);
+            atomicOr(&bar->k_inf[ch >> 5], 1u << (ch & 31));
+          }
+        at[j] = z;
       }
     }
-    const float inv = 1.f / l;
-    p.o[base + (size_t)tok * kD + lane] = o0 * inv;
-    p.o[base + (size_t)tok * kD + 32 + lane] = o1 * inv;
+    if (infs) atomicOr(&bar->flags, infs > 1 || bigs > infs ? kInf | kSpecial : kInf);
   }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncwarp();
+}
+// The rows of a CTA with fp32 multiply-adds: 16 rows to each of the softmax warps, in tiles of 32 keys (of 64 the rings have no room), the next one on
+// its way into shared memory under this one.  A pair's windows have their keys each: four warps to either.  12 heads of 1024 tokens: 163 us with the pass on the
+// tensor cores (a warp per row, from global memory: 7.9 ms; the grid of attn_f32.cu, which has more and smaller CTAs: 96).
+constexpr int kPlainKeys = 32;
+constexpr int kPlainTile = kPlainKeys * f32::kLd;               // floats of a tile of K or V
+constexpr int kPlainWarp = kPlainKeys * f32::kLdP;
+static_assert((kTile * f32::kLd + kSlots * 4 * kPlainTile + kWarpSlot * kPlainWarp) * 4 <= kSmemTiles, "over the rings");
+__device__ __forceinline__ void plain_rows(const Params& p, size_t base, int warp, int lane, float* smem) {
+  using namespace f32;
+  const int set = p.pair ? warp >> 2 : 0, nw = p.pair ? 4 : kWarpSlot, tx = lane & 15, ty = lane >> 4;
+  const Window w(p, p.pair ? 2 * blockIdx.y + set : blockIdx.y);
+  if (w.cnt == 0) return;                                       // (a pair's second window that does not exist)
+  const int row0 = p.pair ? 16 * (warp & 3) : blockIdx.x * kTile + 16 * warp;     // this warp's first row of the window
+  float* qs = smem + 16 * warp * kLd;
+  float* kv = smem + kTile * kLd + set * 4 * kPlainTile;        // K, V, K, V
+  float* ps = smem + kTile * kLd + kSlots * 4 * kPlainTile + warp * kPlainWarp;
+  const int ntiles = (w.cnt + kPlainKeys - 1) / kPlainKeys;
+  auto load = [&](int t) {
+    float* dst = kv + (t & 1) * 2 * kPlainTile;
+    for (int r = 2 * (p.pair ? warp & 3 : warp) + ty; r < kPlainKeys; r += 2 * nw) {
+      const bool in = t * kPlainKeys + r < w.cnt;
+      const size_t at = base + (size_t)(in ? w.key_token(t * kPlainKeys + r) : 0) * kD + 4 * tx;
+      copy16(dst + r * kLd + 4 * tx, p.k + at, in);
+      copy16(dst + kPlainTile + r * kLd + 4 * tx, p.v + at, in);
+    }
+    copy_commit();
+  };
+  auto sync = [&]() {
+    if (!p.pair) asm volatile("bar.sync 1, 256;" ::: "memory");
+    else if (set == 0) asm volatile("bar.sync 1, 128;" ::: "memory");
+    else asm volatile("bar.sync 2, 128;" ::: "memory");
+  };
+  for (int r = ty; r < 16; r += 2) {
+    const bool in = row0 + r < w.nq;
+    copy16(qs + r * kLd + 4 * tx, p.q + base + (size_t)(in ? w.query_token(row0 + r) : 0) * kD + 4 * tx, in);
+  }
+  load(0);                                                      // (one copy group with Q)
+  RowTile<kPlainKeys> x;
+  for (int t = 0; t < ntiles; ++t) {
+    if (t + 1 < ntiles) {
+      load(t + 1);
+      copy_wait<1>();
+    } else {
+      copy_wait<0>();
+    }
+    sync();
+    const float* ks = kv + (t & 1) * 2 * kPlainTile;
+    x.scores(qs + 8 * ty * kLd, ks, tx);
+    x.softmax(w.cnt - t * kPlainKeys, p.scale, ps, tx, ty);
+    __syncwarp();
+    x.values(ks + kPlainTile, ps, tx, ty);
+    sync();
+  }
+  x.finish();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int row = row0 + 8 * ty + i;
+    if (row >= w.nq) continue;
+    const float4 y = x.row(i);
+    const float inv = 1.f / x.l[i];
+    *reinterpret_cast<float4*>(p.o + base + (size_t)w.query_token(row) * kD + 4 * tx) = make_float4(y.x * inv, y.y * inv, y.z * inv, y.w * inv);
+  }
+}
+
+// Behind the CTA's last use of its rings, by the softmax warps: its rows once more, where that is needed
+__device__ __forceinline__ void multiply_add(const Params& p, Barriers* bar, uint32_t met, size_t base, int warp, int lane, float* smem) {
+  const int set = p.pair ? warp >> 2 : 0, nw = p.pair ? 4 : kWarpSlot, first = 2 * (p.pair ? warp & 3 : warp) + (lane >> 4), c4 = lane & 15;
+  bool again = (met & kSpecial) || ((met & kInf) && (met & kUntame));
+  const bool look_q = (met & kInf) && (met & kZero), look_v = met & kLookV;
+  if (!again && (look_q || look_v)) {
+    const Window w(p, p.pair ? 2 * blockIdx.y + set : blockIdx.y);
+    const uint32_t inf = bar->k_inf[c4 >> 3] >> (4 * (c4 & 7));                       // of this lane's four channels
+    const int row0 = p.pair ? 0 : blockIdx.x * kTile, rows = look_q ? min(p.pair ? kTile / 2 : kTile, w.nq - row0) : 0;
+#pragma unroll 4
+    for (int r = first; r < rows + (look_v ? w.cnt : 0); r += 2 * nw) {
+      const bool is_q = r < rows;
+      const float* src = is_q ? p.q + base + (size_t)w.query_token(row0 + r) * kD : p.v + base + (size_t)w.key_token(r - rows) * kD;
+      const float4 x = __ldcg(reinterpret_cast<const float4*>(src) + c4);
+      const float e[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) again = again || (is_q ? e[j] == 0.f && ((inf >> j) & 1) : e[j] != 0.f && fabsf(e[j]) < 0x1p-60f);
+    }
+    if (again) atomicOr(&bar->flags, kUnclear);
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    again = *reinterpret_cast<volatile uint32_t*>(&bar->flags) & kUnclear;
+  }
+  if (again) plain_rows(p, base, warp, lane, smem);
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -215,6 +310,7 @@ attn_f32_tc_kernel(const Params p) {
     mbar_init(&bar->q_full, 256);
     for (int s = 0; s < kSlots; ++s) {
       for (int g = 0; g < kStages; ++g) {
+        bar->k_odd[s][g] = 0;
         mbar_init(&bar->k_full[s][g], 96);
         mbar_init(&bar->k_empty[s][g], 1);
         mbar_init(&bar->v_full[s][g], 96);
@@ -227,8 +323,7 @@ attn_f32_tc_kernel(const Params p) {
     }
     mbar_init(&bar->drain, kSlots);
     bar->abort_flag = 0;
-    bar->special = bar->untame = 0;
-    for (int i = 0; i < 2; ++i) bar->k_inf[i] = bar->q_zero[i] = 0;
+    bar->flags = bar->k_inf[0] = bar->k_inf[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -269,6 +364,7 @@ attn_f32_tc_kernel(const Params p) {
           const int g = u % kStages;
           ok = warp_wait<kSuspendNs>(&bar->k_full[s][g], (u / kStages) & 1, &bar->abort_flag, p.status);
           if (!ok) break;
+          if (bar->k_odd[s][g] == u + 1) cut_infinities(smem + s * kSlotBytes + g * kStageBytes, bar, lane);
           tc_fence_after();
           if (elect_one()) {
             const uint64_t dq = smem_desc(sRing + kOffQ2);
@@ -308,6 +404,7 @@ attn_f32_tc_kernel(const Params p) {
           tc_commit(&bar->v_empty[s][g]);
         }
       }
+      asm volatile("bar.arrive 2, 320;" ::: "memory");          // all that this warp has met is noted
       // Teardown: every MMA issued so far must have retired before tensor memory is released.
       tc_commit(&bar->drain);
       if (lane == 0) {
@@ -323,7 +420,6 @@ attn_f32_tc_kernel(const Params p) {
       const int ntiles = (w.cnt + kSub - 1) / kSub;
       const int c4 = lane & 15, hi = lane >> 4;               // rows 2 cw + hi + 6 i (from 64 on: none)
       unsigned char* ring = smem + s * kSlotBytes;
-      uint32_t least = 0xffffffffu;
       // token of the row that lanes 16 (j & 1) .. + 15 take as their i = j / 2, looked up by lane j
       auto row_token = [&](int t) -> int {
         const int c = t * kSub + 2 * cw + (lane & 1) + 6 * (lane >> 1);
@@ -357,8 +453,6 @@ attn_f32_tc_kernel(const Params p) {
                 if (kv == 0) {
                   note(bad, a);
                   note(bad, b);
-                } else {
-                  note_small(least, x[i]);
                 }
                 store3(to, a, b);
               }
@@ -367,37 +461,12 @@ attn_f32_tc_kernel(const Params p) {
 #pragma unroll
             for (int i = half * 6; i < 6 + half * (kConvRows - 6); ++i) load(i, kv == 0 ? p.v : p.k, kv == 0 ? tok : next);
           }
-          if (kv == 0 && __any_sync(0xffffffffu, noted(bad))) {     // infinities in K: the tile once more (its values have made room for V's)
-#pragma unroll 1
-            for (int i = 0; i < kConvRows; ++i) {
-              const int row = 2 * cw + hi + 6 * i, tk = __shfl_sync(0xffffffffu, tok, 2 * i + hi);
-              float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
-              if (tk >= 0) y = __ldcg(reinterpret_cast<const float4*>(p.k + base + (size_t)tk * kD + 4 * c4));
-              float e[4] = {y.x, y.y, y.z, y.w};
-              uint32_t inf = 0;
-              bool big = false;
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const bool is = fabsf(e[j]) >= kInfinite;
-                inf |= (is ? 1u : 0u) << j;
-                big = big || (!is && fabsf(e[j]) > 0x1p30f);
-                if (is) e[j] = copysignf(0x1p110f, e[j]);
-              }
-              const uint32_t of_row = 0xffffu << (16 * hi);         // the lanes that have this row
-              const uint32_t infs = __ballot_sync(0xffffffffu, inf != 0) & of_row, bigs = __ballot_sync(0xffffffffu, big) & of_row;
-              if (inf && row < kSub) {
-                atomicOr(&bar->k_inf[c4 >> 3], inf << (4 * (c4 & 7)));
-                store3(dst + row * 128 + (((c4 >> 1) ^ (row & 7)) << 4), pack2(e[0], e[1]), pack2(e[2], e[3]));
-                if (bigs || __popc(infs) > 1 || __popc(inf) > 1) bar->special = 1;
-              }
-            }
-          }
+          if (kv == 0 && noted(bad)) bar->k_odd[s][g] = u + 1;
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           mbar_arrive(kv == 0 ? &bar->k_full[s][g] : &bar->v_full[s][g]);
         }
         tok = next;
       }
-      if (least < kSmall) bar->special = 1;
     } else {
       // ================= softmax: one thread per query row and slot =================
       asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
@@ -415,8 +484,7 @@ attn_f32_tc_kernel(const Params p) {
       {
         const bool in = row < wq.nq;
         const float4* src = reinterpret_cast<const float4*>(p.q + base + (size_t)wq.query_token(in ? row : 0) * kD + 32 * s);
-        uint32_t least = 0xffffffffu, zero = 0;
-        float most = 0.f;
+        float most = 0.f, least = in ? 1.f : 0.f;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           uint32_t y[3][8];
@@ -424,9 +492,8 @@ attn_f32_tc_kernel(const Params p) {
           for (int i = 0; i < 4; ++i) {
             const float4 x = in ? __ldcg(src + 4 * h + i) : make_float4(0.f, 0.f, 0.f, 0.f);
             uint64_t a = pack2(x.x, x.y), b = pack2(x.z, x.w);
-            note_small(least, x);
-            most = max3(max3(most, fabsf(x.x), fabsf(x.y)), fabsf(x.z), fabsf(x.w));
-            zero |= ((x.x == 0.f ? 1u : 0u) | (x.y == 0.f ? 2u : 0u) | (x.z == 0.f ? 4u : 0u) | (x.w == 0.f ? 8u : 0u)) << (16 * h + 4 * i);
+            most = max_abs(most, x);
+            least = min_abs(least, x);
             y[0][2 * i] = cut2(a); y[0][2 * i + 1] = cut2(b);
             y[1][2 * i] = cut2(a); y[1][2 * i + 1] = cut2(b);
             y[2][2 * i] = last2(a); y[2][2 * i + 1] = last2(b);
@@ -438,9 +505,18 @@ attn_f32_tc_kernel(const Params p) {
             *reinterpret_cast<uint4*>(smem + kOffQ2 + r * 128 + (((4 * s + 2 * h + i) ^ (r & 7)) << 4)) =
                 make_uint4(y[2][4 * i], y[2][4 * i + 1], y[2][4 * i + 2], y[2][4 * i + 3]);
         }
-        if (least < kSmall || !(most <= 0x1p60f)) bar->special = 1;
-        if (least < kSmallQ || !(most <= 0x1p25f)) bar->untame = 1;
-        if (in && zero) atomicOr(&bar->q_zero[s], zero);
+        if (in && (least < 0x1p-40f || most > 0x1p25f)) {
+          uint32_t met = (most > 0x1p60f ? kSpecial : 0u) | (most > 0x1p25f ? kUntame : 0u);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const float4 x = __ldcg(src + i);
+            const float e[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              met |= e[j] == 0.f ? kZero : fabsf(e[j]) < kSmall ? kSpecial : fabsf(e[j]) < 0x1p-40f ? kUntame : 0u;
+          }
+          atomicOr(&bar->flags, met);
+        }
         tmem_wait_st();
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_fence_before();
@@ -562,6 +638,7 @@ attn_f32_tc_kernel(const Params p) {
         const float f = ex2((m - M) * p.sl2), fo = ex2((ml.x - M) * p.sl2);      // a slot without a key: exp(-inf) = 0
         const float L = fmaf(ml.y, fo, l * f), inv = 1.f / L;
         uint64_t zeros = 0ull;                                                     // or no number, once one of the results is no finite one
+        float least = 1.f;
         float4* dst = reinterpret_cast<float4*>(p.o + base + (size_t)wq.query_token(row) * kD + 32 * s);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -573,12 +650,17 @@ attn_f32_tc_kernel(const Params p) {
                                        fmaf(y.w, fo, x3 * f) * inv);
           dst[i] = z;
           zeros = fma2(pack2(z.x, z.y), 0ull, fma2(pack2(z.z, z.w), 0ull, zeros));
+          least = min_abs(least, z);
         }
         float z0, z1;
         unpack2(zeros, z0, z1);
-        if (!(L < INFINITY) || no_number(z0 + z1)) bar->special = 1;
-        if (!(fabsf(M) < 0x1p30f)) bar->untame = 1;
+        const uint32_t met = (!(L < INFINITY) || no_number(z0 + z1) ? kSpecial : 0u) | (least < 0x1p-80f ? kLookV : 0u) | (!(fabsf(M) < 0x1p30f) ? kUntame : 0u);
+        if (met) atomicOr(&bar->flags, met);
       }
+      // (In here the compiler has the softmax warps' registers; behind the roles' end it made the whole kernel 5 % slower.)
+      asm volatile("bar.sync 2, 320;" ::: "memory");
+      const uint32_t met = *reinterpret_cast<volatile uint32_t*>(&bar->flags);
+      if (met && !bar->abort_flag) multiply_add(p, bar, met, base, warp, lane, reinterpret_cast<float*>(smem));
     }
   }
   __syncwarp();
@@ -587,9 +669,6 @@ attn_f32_tc_kernel(const Params p) {
   tc_fence_after();
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
-  const uint32_t k_inf0 = bar->k_inf[0], k_inf1 = bar->k_inf[1];
-  const bool special = bar->special || ((k_inf0 | k_inf1) && bar->untame) || (k_inf0 & bar->q_zero[0]) || (k_inf1 & bar->q_zero[1]);
-  if (!skip && warp < kWarpSlot && special && !bar->abort_flag) plain_rows(p, base, warp, lane);   // (the softmax warps: they have the registers)
   if (p.overlap) griddep_wait();
 }
 
