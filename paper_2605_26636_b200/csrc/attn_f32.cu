@@ -21,6 +21,9 @@
 // runs at 35 to 41 TFLOP/s of the 73 that a loop of nothing but multiply-adds reaches: one of three instructions is not a
 // multiply-add, and the registers leave room for three warps per scheduler.
 #include <cooperative_groups.h>
+
+#include <type_traits>
+
 #include "f32_common.cuh"
 
 namespace jv {
@@ -148,15 +151,24 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
     }
   }
   __syncthreads();
-  // n partial softmaxes of a row -> maximum, sum and this lane's four channels
-  auto combine = [&](int n, auto&& src_of, float& M, float& L) -> float4 {
+  // n <= kMost partial softmaxes of a row -> maximum, sum and this lane's four channels.  Unrolled, so that all of them are on their way at once.
+  auto combine = [&](auto most, int n, auto&& src_of, float& M, float& L) -> float4 {
+    constexpr int kMost = decltype(most)::value;
+    float m[kMost];
     M = -INFINITY;
-    for (int i = 0; i < n; ++i) M = fmaxf(M, src_of(i)[64]);
+#pragma unroll
+    for (int i = 0; i < kMost; ++i) {
+      m[i] = i < n ? src_of(i)[64] : -INFINITY;
+      M = fmaxf(M, m[i]);
+    }
+    const float ref = M == -INFINITY ? 0.f : M;
     L = 0.f;
     float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int i = 0; i < n; ++i) {
+#pragma unroll
+    for (int i = 0; i < kMost; ++i) {
+      if (i >= n) continue;
       const float* src = src_of(i);
-      const float f = M == -INFINITY ? 0.f : expf(src[64] - M);        // a source without a key of weight: exp(-inf) = 0
+      const float f = expf(m[i] - ref);                                // a source without a key of weight: exp(-inf) = 0
       const float4 y = *reinterpret_cast<const float4*>(src + 4 * tx);
       L = fmaf(src[65], f, L);
       x.x = fmaf(y.x, f, x.x);
@@ -177,7 +189,7 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
     const int r = grp * kOwnRows + 2 * j + ty, row = row0 + rw * kRowsWarp + r;
     if (row < nq) {
       float M, L;
-      const float4 x = combine(G, [&](int g) { return ps + (g * R + rw) * kWarpBuf + r * kLd; }, M, L);
+      const float4 x = combine(std::integral_constant<int, G>(), G, [&](int g) { return ps + (g * R + rw) * kWarpBuf + r * kLd; }, M, L);
       if (nsplit == 1) {
         store(row, x, L);
       } else {                                               // this block's share, over Q
@@ -196,7 +208,7 @@ attn_f32_kernel(const float* __restrict__ q, const float* __restrict__ k, const 
     for (int r = split + nsplit * (2 * warp + ty); r < R * kRowsWarp; r += 2 * R * G * nsplit)   // (uniform over 16 lanes)
       if (row0 + r < nq) {
         float M, L;
-        const float4 x = combine(nsplit, [&](int i) { return cluster.map_shared_rank(qs, i) + r * kLd; }, M, L);
+        const float4 x = combine(std::integral_constant<int, 8>(), nsplit, [&](int i) { return cluster.map_shared_rank(qs, i) + r * kLd; }, M, L);
         store(row0 + r, x, L);
       }
     cluster.sync();                                          // no block leaves while its shared memory may still be read
@@ -224,21 +236,30 @@ cudaError_t launch(const AttnArgs& a, int split, const int* status, bool overlap
 bool attn_f32_supported(const AttnArgs& a) { return a.dtype == JV_F32 && a.D == kDim && !a.strided; }
 
 // The P prefix queries go first, with the keys of a row tile split over the four groups of up to eight blocks (their chain is the longest: all
-// N keys), two blocks to an SM; the windows' launch overlaps them, as neither reads what the other writes.  Eight groups of one block / up to 32 of
-// a cluster, us for the call: 6 heads of 37 x 37, 8 x 8 windows 33.4 / 13.6, 12 of 37 x 37, 16 x 16 49.6 / 27.8, 24 of 32 x 32 45.4 / 29.8 (in
-// clusters of at most 148 blocks in all 31.8).
+// N keys), two blocks to an SM; the windows' launch overlaps them, as neither reads what the other writes.  One block of four groups / as many as
+// the rule gives, us for the call with 16 x 16 windows: 6 heads of 37 x 37, 5 prefix tokens 32.8 / 16.5, 24 of 24 x 24 35.3 / 27.7, 48 of 37 x 37 105.8 / 80.8, 192
+// 309 / 309.  More than 16 prefix tokens are several row tiles per head: a second block per SM is worth it only where the groups have more than
+// a tile each (6 heads of 20 x 20, 120 prefix tokens, 5 x 5 windows, one / two blocks per SM 16.4 / 19.7, of 24 x 24, 100, 4 x 4 20.7 / 15.8), and where the tiles
+// alone give most SMs a block, that one has eight groups (12 heads of 24 x 24, 120, 5 x 5, two of four groups / one of eight 37.0 / 35.2; of 32 x 32 54.2 / 49.1).
 //
 // Windows and sequences go to the tensor cores (attn_f32_tc.cu) where they fill the chip with row tiles of this kernel.  That one's blocks
-// take 128 rows and start slowly: 7 us for one tile of keys, 10 for two, 12 for four, where this one takes 7 to 8 as long as every SM has one block.
-// This (with tiles of 64 keys throughout; those of 32 below came later) / that one, us: 6 heads of 256 tokens 8.2 / 12.1, 12 of 256 11.4 / 12.2, 6 of 400 19.0 / 15.6, 24 of 256 17.6 / 12.5, 12 of 1024 93 / 26.3; 48 of 100
-// 11.1 / 9.5, 24 of 128 8.1 / 10.2; of 64 tokens: 48 heads 7.5 / 7.5, 96 10.6 / 8.0, 192 (two rounds there) 11.4 / 14.6; 8 x 8 windows,
-// 6 heads of 24 x 24 8.1 / 10.6, 6 of 32 x 32 11.1 / 10.4, 48 of 32 x 32 41.7 / 33.1.  Rows of at most 32 queries stay here (a tile there would be
-// three quarters empty): 4 x 4 windows, 48 heads of 32 x 32 72 / 87.
+// take 128 rows, or two windows of up to 64, and start slowly: 10 us for two tiles of keys, 12 for four, where this one takes 7 to 8 as long as every SM
+// has one block.  This / that one, us:
+//   up to 64 keys: always here.  96 heads of 64 tokens 7.6 / 8.4, 384 17.8 / 17.8; 8 x 8 windows, 48 heads of 32 x 32 32.0 / 31.7, 192 of 20 x 20
+//     48.0 / 64.4; 7 x 7, 96 of 24 x 24 45.3 / 53.5 (6 x 6, 48 of 24 x 24 30.2 / 28.1);
+//   up to 128: 192 heads of 100 28.5 / 19.7, 48 of 100 11.1 / 9.5; of windows (8 x 8, 5 prefix tokens) 24 heads of 16 x 16 12.9 / 14.3, 12 of 20 x 20
+//     12.7 / 13.4, 24 of 24 x 24 24.6 / 23.4, 48 of 16 x 16 21.5 / 15.1, 192 of 20 x 20 88 / 91;
+//   up to 256: 6 heads of 256 8.2 / 12.5, 12 of 256 11.6 / 12.6, 24 of 256 17.6 / 12.5; 16 x 16 windows, 6 heads of 24 x 24 11.8 / 12.7;
+//   more: 6 heads of 300 12.7 / 14.0, 6 of 400 19.0 / 15.6, 12 of 1024 93 / 27.9.
+// Rows of at most 32 queries stay here (a tile there would be three quarters empty): 4 x 4 windows, 48 heads of 32 x 32 72 / 87.
 //
-// Here, 32 rows x 2 groups per CTA (three on an SM) or 16 rows x 4 groups (two): the second halves the chain of a CTA, the first is 10 % faster
-// where both fill the chip.  Short rows of keys (up to 64, 128 and 256) are cut into tiles of 32, so that two, four or eight groups have one each and a
-// CTA's chain is half as long.  Tiles of 64 / of 32, us: 6 heads of 64 tokens 7.5 / 5.4, of 128 8.1 / 5.3, 24 of 128 8.3 / 7.4, 6 of 192 8.1 / 7.1, of 256 8.5 /
-// 8.4; 8 x 8 windows, 6 heads of 16 x 16 8.2 / 5.8, 4 x 4, 24 of 32 x 32 40 / 27.  Eight groups take an SM: only where every row tile gets one (12 heads
+// Here, 32 rows x 2 groups per CTA (three on an SM) or 16 rows x 4 groups (two): the second halves the chain of a CTA, the first is faster
+// where both fill the chip several times and its 32 rows are filled.  More than 128 keys and 17 to 32 queries, 16 x 4 / 32 x 2 (5 x 5 windows, 120 prefix tokens): 6 heads of
+// 16 x 16 12.5 / 20.8, 12 of 24 x 24 35.1 / 39.5, 12 of 32 x 32 55.1 / 48.9, 192 of 24 x 24 392 / 347.  Up to 128, 24 heads of 16 x 16, 8 x 8 windows,
+// 5 prefix tokens 18.2 / 12.9; 4 x 4 windows, 100, 96 heads of 24 x 24 129 / 159.
+// Short rows of keys (up to 64, 128 and 256) are cut into tiles of 32, so that two, four or eight groups have one each and a
+// CTA's chain is half as long.  Tiles of 64 / of 32, us: 6 heads of 64 tokens 7.5 / 5.4, of 128 8.1 / 5.3, 24 of 128 8.3 / 7.4, 6 of 200 8.0 / 7.4, of 256 8.3 /
+// 8.2; 8 x 8 windows, 6 heads of 16 x 16 8.2 / 5.8, 4 x 4, 24 of 32 x 32 40 / 27.  Eight groups take an SM: only where every row tile gets one (12 heads
 // of 256 tokens 11.7 / 14.8).
 // Windows of at most eight tokens leave most of a 32 x 64 tile of scores empty: the kernel of one warp per query row, eight to a block, is the
 // better one.  This one / that one, 96 heads of 32 x 32 tokens: 2 x 2 windows 484 / 270 us, 2 x 4 256 / 148, 3 x 3 245 / 254; 12 heads of 64 x 64, 2 x 2
@@ -250,26 +271,35 @@ cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st) {
   const bool prefix = a.P > 0;
   const int64_t sms = device_sm_count(), windows = (int64_t)ceil_div(a.Wg, ww) * ceil_div(a.Hg, wh) * a.BH;
   const int nq = wh * ww, cnt = a.P + nq, key_tiles = ceil_div(cnt, kTileKeys);
-  const int64_t rows16 = windows * ceil_div(nq, kRowsWarp), rows32 = windows * ceil_div(nq, 2 * kRowsWarp);   // row tiles of this kernel
+  // row tiles of this kernel: small windows at the edges have fewer
+  auto row_tiles = [&](int rows) -> int64_t {
+    const int ny = a.Hg / wh, nx = a.Wg / ww, eh = a.Hg % wh, ew = a.Wg % ww;
+    return a.BH * ((int64_t)ny * nx * ceil_div(nq, rows) + (int64_t)nx * ceil_div(eh * ww, rows) + (int64_t)ny * ceil_div(wh * ew, rows) + ceil_div(eh * ew, rows));
+  };
+  const int64_t rows16 = row_tiles(kRowsWarp), rows32 = row_tiles(2 * kRowsWarp);
   bool tc = nq > 2 * kRowsWarp && a.scale >= 0x1p-40f && a.scale <= 0x1p40f;   // (else what its terms do not hold of very small or infinite values may count)
-  if (cnt <= 2 * kTileKeys) tc = tc && rows32 > sms && (cnt > kTileKeys || windows > a.BH || a.BH <= sms);
-  else tc = tc && rows16 > sms && (key_tiles > 4 || 3 * rows16 > 4 * sms);
+  if (cnt <= kTileKeys) tc = false;
+  else if (cnt <= 2 * kTileKeys) tc = tc && rows32 > sms && (nq > kTileKeys || rows32 > 2 * sms);
+  else tc = tc && rows16 > sms && (key_tiles > 4 || 2 * rows16 > 3 * sms);
   int* status = nullptr;                                   // for the kernels of a call that leave o alone while the word is set: all of them, or none
   if (tc && !(status = device_status_ptr())) return cudaErrorUnknown;
   if (prefix) {
     const int N = a.P + a.Hg * a.Wg;
     const int64_t tiles = (int64_t)ceil_div(a.P, kRowsWarp) * a.BH;
     int split = 1;
-    while (split < 8 && 2 * split * tiles <= 2 * sms && split * 4 * kTileKeys < N) split *= 2;
-    const cudaError_t e = launch<1, 4, kTileKeys, true>(a, split, status, false, st);
+    while (split < 8 && split * tiles <= sms && split * 4 * kTileKeys < N &&
+           (a.P <= kRowsWarp || 2 * split * tiles <= sms || split * 5 * kTileKeys <= N)) split *= 2;
+    const bool eight = a.P > kRowsWarp && 2 * tiles > sms && tiles <= sms;
+    const cudaError_t e = eight ? launch<1, 8, kTileKeys, true>(a, 1, status, false, st) : launch<1, 4, kTileKeys, true>(a, split, status, false, st);
     if (e != cudaSuccess) return e;
   }
   if (tc) return launch_attn_f32_tc(a, prefix, status, st);
   if (nq <= 8 && (!prefix || (cnt <= 32 && windows >= 8 * sms))) return launch_attn_generic(a, st, true);
   if (cnt <= kTileKeys) return launch<2, 2, 32, false>(a, 1, nullptr, prefix, st);
-  if (cnt <= 2 * kTileKeys) return launch<1, 4, 32, false>(a, 1, nullptr, prefix, st);
+  if (cnt <= 2 * kTileKeys && (nq <= kRowsWarp || rows16 <= 2 * sms)) return launch<1, 4, 32, false>(a, 1, nullptr, prefix, st);
   if (cnt <= 4 * kTileKeys && rows16 <= sms) return launch<1, 8, 32, false>(a, 1, nullptr, prefix, st);
-  if (rows32 <= 2 * sms) return launch<1, 4, kTileKeys, false>(a, 1, nullptr, prefix, st);
+  const int64_t rounds2 = (windows * ceil_div(nq, 2 * kRowsWarp) + sms - 1) / sms, rounds1 = (windows * ceil_div(nq, kRowsWarp) + sms - 1) / sms;
+  if (cnt > 2 * kTileKeys && (rounds2 <= 2 || 5 * rounds1 <= 9 * rounds2)) return launch<1, 4, kTileKeys, false>(a, 1, nullptr, prefix, st);
   return launch<2, 2, kTileKeys, false>(a, 1, nullptr, prefix, st);
 }
 
