@@ -2,7 +2,7 @@
 // multiply-adds throughout, register-tiled.
 //
 // What bounds it: the FMA pipes (4 * 64 flop per query-key pair; 128 multiply-adds per clock and SM).  A warp
-// owns 16 query rows and walks tiles of 64 keys; a lane owns 8 rows x 4 keys of the scores (keys lane % 16 + 16 j)
+// owns 16 query rows and walks tiles of 64 keys (short rows of keys: 32); a lane owns 8 rows x 4 keys of the scores (keys lane % 16 + 16 j)
 // and 8 rows x 4 channels of the output.  Multiply-adds are packed pairs (fma.rn.f32x2: even and odd channels
 // in QK^T, two neighbouring rows in PV), fed by 128-bit shared-memory loads: 12 loads per 64 packed
 // multiply-adds, three quarters of what the shared-memory port could deliver.  The rows of a
@@ -15,7 +15,7 @@
 // place: with three CTAs on an SM the others compute while one waits for a copy), and the groups' partial softmaxes are
 // merged at the end.
 //
-// It serves what does not fill the chip with its row tiles, short rows of queries and the prefix queries of windows; the rest goes to the
+// It serves what does not fill the chip with its row tiles, rows of up to 64 keys, short rows of queries and the prefix queries of windows; the rest goes to the
 // tensor cores (attn_f32_tc.cu; the line between the two: launch_attn_f32).  Measured (6 heads, 16 x 16 tokens; the kernel of one warp
 // per query row, which serves other head dims and windows of at most eight tokens, in brackets): full attention 8 us (63).  Where it fills the chip it
 // runs at 35 to 41 TFLOP/s of the 73 that a loop of nothing but multiply-adds reaches: one of three instructions is not a

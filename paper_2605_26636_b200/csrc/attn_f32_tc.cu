@@ -29,12 +29,13 @@
 // and 64 of the step's product with V.  The scores of step u + 1 are computed while the softmax works on step u.
 //
 // What bounds it: the tensor pipe, 48 MMAs of M128 N64 K16 per step (1536 clocks), with the exponentials and the cutting of P, K
-// and V (about 1370 issue slots a step and sub-core) right behind; a pair of steps, one per slot, takes 4000 clocks.  Two slots cost 2.2 us
-// for 128 keys, a CTA 8.5 us besides (launch, first loads, first step, merge).
-// Measured (the kernel of fp32 multiply-adds, attn_f32.cu, in brackets): full attention, 12 heads of 32 x 32 tokens 26.3 us (93.3), 24 of 37 x 37 68
-// (282), 192 of 1024 300 (1175); 16 x 16 windows, 12 heads of 32 x 32 13.1 (27.1), 96 84 (166).  Error against fp64, 2-norm: 1.5e-7 to 2.1e-7
-// (1.8e-7 to 5.2e-7) over 1 to 300 heads of 64 to 1400 tokens.  With terms cut off instead of rounded the terms left out all had
-// the product's sign: 2.3e-7 to 2.8e-7.  With one score buffer per slot 33.1 us in place of 26.3; with the third plane of P in a plane of its own
+// and V (about 1370 issue slots a step and sub-core) right behind; a pair of steps, one per slot, takes 4000 clocks.  A call of one round of CTAs takes
+// 10 us for 128 keys (launch, first loads, first step, merge) and 2.4 for every further 128.
+// Measured (the kernel of fp32 multiply-adds, attn_f32.cu, in brackets): full attention, 12 heads of 32 x 32 tokens 27.9 us (93.9), 24 of 37 x 37 65.9
+// (279), 192 of 1024 309 (1177); 16 x 16 windows, 12 heads of 32 x 32 13.8 (27.3), 96 83.5 (166).  Without the looks at what three terms cannot hold, and with the
+// scale in the exponent's multiply-add, 26.6, 64.0, 300; 13.4, 80.  Error against fp64, 2-norm: 1.6e-7 to 2.1e-7
+// (2.1e-7 to 5.1e-7) over 6 to 192 heads of 64 to 1400 tokens, with q four times as large 2.3e-7 to 3.1e-7 (3.4e-7 to 6.7e-7).  With terms cut off instead of rounded the
+// terms left out all had the product's sign: 2.3e-7 to 2.8e-7.  With one score buffer per slot 33.1 us in place of 26.3; with the third plane of P in a plane of its own
 // per buffer there is no tensor memory left.
 #include "f32_common.cuh"
 #include "tc_common.cuh"

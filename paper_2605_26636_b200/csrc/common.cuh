@@ -164,7 +164,7 @@ cudaError_t launch_attn_prefix(const AttnArgs& a, int free_sms, const int* statu
 // fp32 tensors at D == 64: register-tiled fp32 kernel (full and windowed attention, prefix tokens)
 bool attn_f32_supported(const AttnArgs& a);
 cudaError_t launch_attn_f32(const AttnArgs& a, cudaStream_t st);
-// the same arithmetic on the tensor cores, fp32 values as sums of three bf16 terms (without the prefix queries, whose launch
+// on the tensor cores, fp32 values as sums of three bf16 terms, six of their nine products, sums in fp32 (without the prefix queries, whose launch
 // it overlaps if that is the one ahead)
 cudaError_t launch_attn_f32_tc(const AttnArgs& a, bool overlap, int* status, cudaStream_t st);
 // tcgen05 path: bf16, D == 64.  full = true: F over all N tokens; else W with (wh, ww)

@@ -218,3 +218,23 @@ def test_infinities_in_fp32_keys(jv, case, what):
         assert torch.equal(torch.isnan(o), torch.isnan(ref))
         o, ref = o[:, :, ~rows], ref[:, :, ~rows]
     _compare(o, ref, dtype, what)
+
+
+@pytest.mark.parametrize("what", ["v inf", "v nan", "v 1e35", "v 1e-37", "q inf", "q nan"])
+@pytest.mark.parametrize("case", [c for c in ROUTES if c[0] == "f32"], ids=lambda c: "x".join(map(str, c)))
+def test_fp32_values_beyond_the_ordinary(jv, case, what):
+    """In one channel, of every 50th token or (very small ones) of all: what comes out infinite or no number is where fp64 has it, the rest, channel by channel, as
+    accurate as ever."""
+    dtype, D, B, H, P, Hg, Wg, win = case
+    q, k, v, run = _call(jv, case, 7900)
+    name, value = what.split()
+    t = q if name == "q" else v
+    if value == "1e-37":
+        t[..., 3] *= 1e-37
+    else:
+        t[:, ::2, 7::50, 3] = float(value)
+    o, ref = run()
+    assert torch.equal(torch.isnan(o), torch.isnan(ref)) and torch.equal(torch.isinf(o), torch.isinf(ref))
+    for c in (slice(3, 4), slice(4, D)):
+        f = torch.isfinite(ref[..., c])
+        assert float((o - ref)[..., c][f].norm()) <= BAR[dtype] * float(ref[..., c][f].norm())
